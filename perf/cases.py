@@ -129,17 +129,15 @@ def tolerance(case):
     return {"rel": 0.01, "max": 0.08} if c["sharp"] != 1.0 else {"rel": 0.008, "max": 0.036}
 
 
-def prepare(case, seed):
-    c = case
+def _inputs(c, seed):
+    """Images, tokens before and after the features move on, and weights, from the seed alone."""
     scene = "trajectory" if c["frames"] >= 100 else "polygons"
     wl = Workload("case", c["frames"], c["grid_h"], c["grid_w"], c["ratio"], scene, 1, 6, 1000 + 7919 * int(seed))
     dev = torch.device("cuda")
     kind = c["kind"]
     bf = torch.bfloat16
-    ctx = LiteVGGT(wl.frames, wl.grid_h, wl.grid_w, wl.merge_ratio, qkv_dtype=1 if c["fp8"] else 0)
     images = make_images(wl, dev)
-    x = make_tokens(wl, images)
-    s = dict(kind=kind, ctx=ctx, ext=c["ext"])
+    s = dict(images=images, x=make_tokens(wl, images))
     w_qkv, b_qkv, w_o, b_o = make_attention_weights(wl, 0, dev)
     if c["sharp"] != 1.0:
         w_qkv[:D] *= c["sharp"]
@@ -154,26 +152,43 @@ def prepare(case, seed):
         s["local"] = make_block_weights(wl, 0, dev)
     if kind == "block":
         s["global"] = make_block_weights(wl, 1, dev)
+    if kind in ("first", "refresh"):
+        s["drift_seed"] = wl.seed + 901
+    return s
+
+
+def _drift(s):
+    # the features have moved on since the plan at hand was built
+    x = s["x"]
+    g = torch.Generator(device=x.device)
+    g.manual_seed(s.pop("drift_seed"))
+    for i in range(0, x.shape[0], 1 << 17):
+        part = x[i:i + (1 << 17)]
+        part += (0.05 * torch.randn(part.shape, generator=g, device=x.device)).to(x.dtype)
+
+
+def prepare(case, seed):
+    c = case
+    kind = c["kind"]
+    ctx = LiteVGGT(c["frames"], c["grid_h"], c["grid_w"], c["ratio"], qkv_dtype=1 if c["fp8"] else 0)
+    s = _inputs(c, seed)
+    s.update(kind=kind, ctx=ctx, ext=c["ext"])
+    x = s["x"]
     if kind != "local":
         # the indices an earlier layer of the same sequence left behind
-        s["grad"] = ctx.grad_map(images)
+        s["grad"] = ctx.grad_map(s["images"])
         s["plan"] = ctx.merge_plan(x, s["grad"])
-        s["xm"] = torch.empty(ctx.n_merged, D, dtype=bf, device=dev)
+        s["xm"] = torch.empty(ctx.n_merged, D, dtype=x.dtype, device=x.device)
         s["ym"] = torch.empty_like(s["xm"])
     if kind in ("first", "refresh"):
-        s["images"] = images
-        # the features have moved on since that plan was built
-        g = torch.Generator(device=dev)
-        g.manual_seed(wl.seed + 901)
-        for i in range(0, x.shape[0], 1 << 17):
-            part = x[i:i + (1 << 17)]
-            part += (0.05 * torch.randn(part.shape, generator=g, device=dev)).to(bf)
+        _drift(s)
+    else:
+        del s["images"]
     if kind == "host":
         s["x"] = x.to("cpu").pin_memory()
         s["out"] = torch.empty_like(s["x"]).pin_memory()
         torch.cuda.synchronize()
     else:
-        s["x"] = x
         s["out"] = torch.empty_like(x)
     if kind in ("local", "block"):
         s["normed"] = torch.empty_like(x)
@@ -224,3 +239,152 @@ def run(state):
     ctx.global_layer_host_pipelined(s["plan"], x, *s["attn"], out)
     ctx.host_drain()
     return out
+
+
+# ---- the same passes in 64 bits, plain torch ------------------------------------------------------
+def _plan64(c, x, grad):
+    """dst_of, kept_idx of the merge plan: GA scores, anchors, cosine matches, the R best merged."""
+    f, gh, gw = c["frames"], c["grid_h"], c["grid_w"]
+    p, dev = gh * gw, x.device
+    t, n, m, n_src, n_dst = _sizes(c)
+    var = torch.empty(f, gh, gw, dtype=torch.float64, device=dev)
+    for i in range(0, f, 8):
+        g = x.view(f, t, D)[i:i + 8, SPECIAL:].double().view(-1, gh, gw, D).permute(0, 3, 1, 2)
+        mean = torch.nn.functional.avg_pool2d(g, 3, 1, 1, count_include_pad=False)
+        square = torch.nn.functional.avg_pool2d(g * g, 3, 1, 1, count_include_pad=False)
+        var[i:i + 8] = (square - mean * mean).mean(1)
+
+    def unit(v):
+        low, high = v.amin((1, 2), keepdim=True), v.amax((1, 2), keepdim=True)
+        return (v - low) / (high - low + 1e-6)
+
+    score = 0.5 * unit(grad) + 0.5 * unit(var)
+    ids = torch.arange(p, device=dev).view(1, gh, gw)
+    ch, cw = (gh + 1) // 2, (gw + 1) // 2
+    padded = torch.full((f, 2 * ch, 2 * cw), math.inf, dtype=torch.float64, device=dev)
+    padded[:, :gh, :gw] = score
+    padded_ids = torch.zeros(1, 2 * ch, 2 * cw, dtype=torch.long, device=dev)
+    padded_ids[:, :gh, :gw] = ids
+    cells = padded.view(f, ch, 2, cw, 2).transpose(2, 3).reshape(f, ch * cw, 4)
+    cell_ids = padded_ids.view(1, ch, 2, cw, 2).transpose(2, 3).reshape(1, ch * cw, 4).expand(f, -1, -1)
+    anchors = cell_ids.gather(2, cells.argmin(2, keepdim=True)).squeeze(2)
+    is_dst = torch.zeros(f, p, dtype=torch.bool, device=dev).scatter_(1, anchors, True)
+    n_ga = min(int(0.1 * p + 1e-9), p - ch * cw)
+    kept = torch.zeros_like(is_dst)
+    if n_ga:
+        top = score.view(f, p).masked_fill(is_dst, -math.inf).topk(n_ga, 1).indices
+        kept.scatter_(1, top, True)
+    is_src = ~(is_dst | kept)
+    is_src[0], is_dst[0] = False, True
+    token = (torch.arange(f, device=dev)[:, None] * t + SPECIAL + torch.arange(p, device=dev)[None])
+    src, dst = token[is_src], token[is_dst]
+    assert src.numel() == n_src and dst.numel() == n_dst
+    b = x[dst].double()
+    b /= b.norm(dim=1, keepdim=True).clamp_min(1e-12)
+    best, sim = torch.empty_like(src), torch.empty(n_src, dtype=torch.float64, device=dev)
+    for i in range(0, n_src, 2048):
+        a = x[src[i:i + 2048]].double()
+        s = (a / a.norm(dim=1, keepdim=True).clamp_min(1e-12)) @ b.T
+        sim[i:i + 2048], j = s.max(1)
+        best[i:i + 2048] = dst[j]
+    merged = sim.sort(descending=True, stable=True).indices[:n - m]
+    own = torch.ones(n, dtype=torch.bool, device=dev)
+    own[src[merged]] = False
+    kept_idx = own.nonzero().squeeze(1)
+    dst_of = torch.cumsum(own.long(), 0) - 1
+    dst_of[src[merged]] = dst_of[best[merged]]
+    return dst_of, kept_idx
+
+
+def _grad64(images):
+    f, _, h, w = images.shape
+    out = torch.empty(f, h // 14, w // 14, dtype=torch.float64, device=images.device)
+    kx = torch.tensor([[-1.0, 0.0, 1.0], [-2.0, 0.0, 2.0], [-1.0, 0.0, 1.0]], dtype=torch.float64, device=images.device)
+    kernel = torch.stack((kx, kx.T))[:, None]
+    for i in range(0, f, 16):
+        grey = images[i:i + 16].double().mean(1, keepdim=True)
+        g = torch.nn.functional.conv2d(torch.nn.functional.pad(grey, (1, 1, 1, 1), mode="replicate"), kernel)
+        out[i:i + 16] = torch.nn.functional.avg_pool2d(g.pow(2).sum(1, keepdim=True).sqrt(), 14).squeeze(1)
+    return out
+
+
+def _attention64(x, weights, frames=1, q_norm=None, k_norm=None, pos=None):
+    w_qkv, b_qkv, w_o, b_o = (v.double() for v in weights)
+    n = x.shape[0]
+    q, k, v = ((x @ w_qkv.T + b_qkv).view(frames, n // frames, 3, 16, 64).permute(2, 0, 3, 1, 4))
+
+    def normed(u, affine):
+        gamma, beta = affine
+        return torch.nn.functional.layer_norm(u, (64,), gamma.double(), beta.double(), 1e-5)
+
+    def turned(u):  # 32 channels by the row, 32 by the column; channel i and i + 16 form a plane
+        theta = 100.0 ** (-torch.arange(16, dtype=torch.float64, device=x.device) / 16)
+        out = torch.empty_like(u)
+        for axis in range(2):
+            angle = pos[:, axis, None] * theta
+            a, b = u[..., 32 * axis:32 * axis + 16], u[..., 32 * axis + 16:32 * axis + 32]
+            out[..., 32 * axis:32 * axis + 16] = a * angle.cos() - b * angle.sin()
+            out[..., 32 * axis + 16:32 * axis + 32] = b * angle.cos() + a * angle.sin()
+        return out
+
+    if q_norm is not None:
+        q, k = normed(q, q_norm), normed(k, k_norm)
+    if pos is not None:
+        q, k = turned(q), turned(k)
+    o = torch.empty(frames, n // frames, 16, 64, dtype=torch.float64, device=x.device)
+    for i in range(frames):
+        for h in range(16):
+            for r in range(0, n // frames, 8192):
+                o[i, r:r + 8192, h] = torch.softmax(q[i, h, r:r + 8192] @ k[i, h].T / 8.0, 1) @ v[i, h]
+    return o.view(n, D) @ w_o.T + b_o
+
+
+def _global64(c, s, x, residual, plan):
+    dst_of, kept_idx = plan
+    m = kept_idx.numel()
+    total = torch.zeros(m, D, dtype=torch.float64, device=x.device).index_add_(0, dst_of, x)
+    xm = total / torch.bincount(dst_of, minlength=m)[:, None]
+    norm = {}
+    if c["ext"]:
+        t = c["grid_h"] * c["grid_w"] + SPECIAL
+        patch = kept_idx % t - SPECIAL
+        pos = torch.stack((patch // c["grid_w"], patch % c["grid_w"]), 1) + 1
+        norm = dict(q_norm=s["q_norm"], k_norm=s["k_norm"], pos=torch.where(patch[:, None] < 0, 0, pos).double())
+    return xm, lambda: residual + _attention64(xm, s["attn"], **norm)[dst_of]
+
+
+def _norm64(x, affine):
+    return torch.nn.functional.layer_norm(x, (D,), affine[0].double(), affine[1].double(), 1e-6)
+
+
+def _mlp64(x, weights):
+    w1, b1, w2, b2 = (v.double() for v in weights)
+    return torch.cat([torch.nn.functional.gelu(p @ w1.T + b1) @ w2.T + b2 for p in x.split(1 << 15)])
+
+
+def exact(case, seed):
+    """What run returns, in 64 bits and with nothing quantised; the longer cases would take minutes."""
+    c = case
+    if _flops(c) > 5e12:
+        return None
+    s = _inputs(c, seed)
+    kind = c["kind"]
+    if kind != "local":
+        grad = _grad64(s["images"])
+        if kind in ("first", "refresh"):
+            _drift(s)
+        plan = _plan64(c, s["x"], grad)
+    x = s["x"].double()
+    if kind in ("local", "block"):
+        w = s["local"]
+        x = x + _attention64(_norm64(x, w["ln1"]), w["attn"], c["frames"])
+        x = x + _mlp64(_norm64(x, w["ln2"]), w["mlp"])
+        if kind == "local":
+            return x
+        w = s["global"]
+        x = _global64(c, s, _norm64(x, w["ln1"]), x, plan)[1]()
+        return x + _mlp64(_norm64(x, w["ln2"]), w["mlp"])
+    xm, layer = _global64(c, s, x, x, plan)
+    if kind == "refresh":
+        return grad, xm
+    return (grad, layer()) if kind == "first" else layer().cpu() if kind == "host" else layer()
