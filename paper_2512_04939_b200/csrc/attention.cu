@@ -4,7 +4,15 @@
 // computed flash-style: scores never leave the SM.
 //
 // One CTA = 256 query rows (two tiles of 128) of one head, sweeping all keys in tiles of
-// 128 that are consumed as two halves of 64 ("steps").  Warp roles (20 warps):
+// 128 that are consumed as two halves of 64 ("steps").  Sequences of up to kFaOneTileRows rows
+// take CTAs of one tile instead, two to an SM, with half of everything below: the set-up and the
+// write-back of one CTA then run under the sweep of the other, and a sequence pays for ceil(rows /
+// 128) tiles and not for an even number of them.  What a sequence of 1041 rows (a 28 x 37 frame) spends
+// outside its nine key tiles bounded it; the frame-local layer of 200 such frames, projections
+// included, went from 3.09 to 2.58 ms.  The pair of tiles reads every K/V tile once for 256 rows and
+// is the faster one when the sweep is long and the chip runs into its power cap: 297 us (one tile)
+// against 304 at 8.3 K rows, 1.80 ms each at 22 K, 10.6 to 11.1 ms against 10.3 to 10.7 at 52 K, 28.6
+// against 28.2 at 83 K.  Warp roles of the pair (20 warps):
 //   warps 0-15  softmax.  Warp w works on query tile t = w / 8, TMEM lane quarter w % 4 (one
 //               thread = one query row) and the column half c = (w / 4) % 2 of every step:
 //               32 of the step's 64 scores per row.  The two threads of a row swap their
@@ -44,8 +52,8 @@
 // thread handles per step; 7 measured best in the kernel (on register data alone, 4 warps per
 // scheduler: 6 pairs take 182 clocks per 32 scores against 257 with the special-function unit only,
 // 8 pairs 220).
-// Shared memory: K ring, V ring, and behind the V ring a block of the same size that holds the
-// ones column of the P V operand for every ring position (see the kernel).
+// Shared memory: K ring, V ring, and behind the V ring a 2 KB block that holds the ones column of
+// the P V operand (see the kernel).
 //
 // Key chunks.  All CTAs of a head stream the same K/V, but they drift apart, so their combined
 // working set is the head's whole K/V; beyond about a quarter of the L2 that no longer stays
@@ -70,10 +78,17 @@
 // B <= kFaFixedRefLimit runs the sweep with a constant reference (in fact with none: the constant
 // cancels, see the kernel): no row maximum, no exchange between the two threads of a row, no
 // rescaling, and - the softmax scale 1/sqrt(64) log2(e) arriving folded into K - no arithmetic
-// between the tensor core's scores and the exponential.  Rows with larger B (scores that could span more than
-// the exponent range allows) take the online form: base-2 softmax with a lazily updated reference
+// between the tensor core's scores and the exponential.
+// Rows with larger B need a reference other than zero, but seldom a running one: the largest score s0
+// among the first 64 keys bounds the row maximum from below as B does from above, and wherever a
+// whole number m lies close enough to both (kFaShiftUp, kFaShiftDown) it serves the whole sweep - the
+// shifted form, at the cost of a subtraction or a clamp per score, both of which the bound spares the
+// fixed form.  Trained projections attend that sharply (query weights x 16 on the generator's tokens:
+// B up to 213, 98.6 % of the warps): 31,751 rows went from 4.69 to 4.36 ms there, and from 5.35
+// to 4.0 ms on Gaussian rows, where the online form rescales more.
+// What remains takes the online form: base-2 softmax with a lazily updated reference
 // maximum, the running output rescaled only when a row maximum grows by more than 2^8 over the
-// reference (the threads then first wait until the tile's last P V has retired).  Both forms equal
+// reference (the threads then first wait until the tile's last P V has retired).  All three equal
 // the plain softmax up to rounding.
 #include "common.cuh"
 #include "runtime.h"
@@ -84,6 +99,7 @@ constexpr int kFaStages = 4;
 constexpr int kFaSoftmaxWarps = 16;
 constexpr int kFaThreads = (kFaSoftmaxWarps + 4) * 32;
 constexpr int kFaTileBytes = 128 * 64 * 2;
+constexpr int kFaOnesBytes = 16 * 128;  // 16 key rows of the ones column block
 constexpr uint32_t kFaColS = 0, kFaColO = 256, kFaColQ = 416;
 constexpr uint32_t kFaOCols = 80;  // 64 output channels, the row sum, 15 unused columns
 constexpr float kFaRescaleThreshold = 8.0f;
@@ -105,21 +121,50 @@ constexpr int kFaChunkTiles = LV_FA_CHUNK_TILES;  // 65536 keys: K and V of one 
 #define LV_FA_POLY_PAIRS 7
 #endif
 constexpr int kFaPolyPairs = LV_FA_POLY_PAIRS;
+// The same in the shifted-reference form, whose polynomial pairs also need a clamp and whose other
+// pairs a subtraction.  At 31,751 rows, time over that of the QKV projection in the same run (the
+// clock moves under the power cap): 0 pairs 30.3, 3: 29.9, 4: 28.5, 5: 28.3, 7: 28.0.
+#ifndef LV_FA_SHIFT_POLY_PAIRS
+#define LV_FA_SHIFT_POLY_PAIRS 5
+#endif
+constexpr int kFaShiftPolyPairs = LV_FA_SHIFT_POLY_PAIRS;
+// Shifted reference m of a row with score bound B and a known score s0: B - m <= kFaShiftUp keeps row sums
+// over 2^20 keys and |v| <= 2^20 below 2^124; m - s0 <= kFaShiftDown leaves 34 binades between the row's
+// largest probability and the smallest normal number, so that even 2^20 keys that are rounded to
+// zero hold less than 2^-14 of the row's mass (the probabilities' own rounding is 2^-9).
+constexpr float kFaShiftUp = 84.0f, kFaShiftDown = 92.0f;
+// Sequences of at most this many rows take CTAs of one query tile, two to an SM (figures at the top).
+#ifndef LV_FA_ONE_TILE_ROWS
+#define LV_FA_ONE_TILE_ROWS 16384
+#endif
+constexpr long long kFaOneTileRows = LV_FA_ONE_TILE_ROWS;
 
+template <int kStages>
 struct FaBarriers {
   uint64_t q_ready;
-  uint64_t k_full[kFaStages], k_empty[kFaStages];
-  uint64_t v_full[kFaStages], v_empty[kFaStages];
+  uint64_t k_full[kStages], k_empty[kStages];
+  uint64_t v_full[kStages], v_empty[kStages];
   uint64_t s_full[2][2], p_ready[2][2], pv_done[2], o_done[2];
   uint64_t teardown[2];
   uint32_t tmem_base;
   uint32_t abort_flag;
 };
 // partial row maxima swapped between the two threads of a row: [step parity][tile][column half][row]
+template <int kTiles>
 struct FaExchange {
-  float row_max[2][2][2][128];
+  float row_max[2][kTiles][2][128];
 };
-constexpr int kFaSmemBytes = 3 * kFaStages * kFaTileBytes + (int)sizeof(FaExchange) + 512 + 1024;
+// What differs between the CTA of two query tiles (one CTA per SM) and that of one (two per SM).
+template <int kTiles>
+struct FaShape {
+  static constexpr int kSoftmaxWarps = 8 * kTiles;
+  static constexpr int kThreads = (kSoftmaxWarps + (kTiles == 2 ? 4 : 2)) * 32;
+  static constexpr int kStages = kTiles == 2 ? 4 : 3;
+  static constexpr uint32_t kTmemCols = 256 * kTiles;
+  static constexpr uint32_t kColS = 0, kColO = 128 * kTiles, kColQ = (128 + 80) * kTiles;
+  static constexpr int kSmemBytes =
+      2 * kStages * kFaTileBytes + kFaOnesBytes + (int)sizeof(FaExchange<kTiles>) + 512 + 1024;
+};
 
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;
@@ -127,13 +172,13 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
-// 2^x for a pair of arguments on the FMA pipes.  Adding 1.5 * 2^23 rounds x to the nearest
-// integer n in the low mantissa bits; 2^(x - n) comes from a cubic fitted on [-1/2, 1/2] and
-// n is added to the exponent field.  Valid for arguments in [-120, 120].
-__device__ __forceinline__ float2 poly_exp2_pair(float2 x) {
-  const float2 magic = make_float2(12582912.0f, 12582912.0f);
+// 2^(x - m) for a pair of arguments on the FMA pipes, `magic` = 1.5 * 2^23 - m with m a whole number.
+// Adding it rounds x to the nearest integer and leaves n = that integer - m in the low mantissa
+// bits; the fraction's power comes from a cubic fitted on [-1/2, 1/2] and n is added to the exponent
+// field.  Valid for x - m in [-120, 120].
+__device__ __forceinline__ float2 poly_exp2_pair(float2 x, float2 magic, float2 neg_magic) {
   const float2 t = __fadd2_rn(x, magic);
-  const float2 n = __fadd2_rn(t, make_float2(-12582912.0f, -12582912.0f));
+  const float2 n = __fadd2_rn(t, neg_magic);
   const float2 f = __ffma2_rn(n, make_float2(-1.0f, -1.0f), x);
   float2 p = __ffma2_rn(make_float2(0.0551716648f, 0.0551716648f), f, make_float2(0.2426111251f, 0.2426111251f));
   p = __ffma2_rn(p, f, make_float2(0.6932609677f, 0.6932609677f));
@@ -143,17 +188,21 @@ __device__ __forceinline__ float2 poly_exp2_pair(float2 x) {
   r.y = __uint_as_float(__float_as_uint(p.y) + (__float_as_uint(t.y) << 23));
   return r;
 }
+__device__ __forceinline__ float2 poly_exp2_pair(float2 x) {
+  return poly_exp2_pair(x, make_float2(12582912.0f, 12582912.0f), make_float2(-12582912.0f, -12582912.0f));
+}
 
 // Wait until the most recent loads into a ring (up to one per stage) have landed.
-// `issued` counts the loads issued into the ring so far; load i uses stage i % kFaStages and
-// completes the phase with parity (i / kFaStages) & 1.  Not sensitive to the abort flag: the
+// `issued` counts the loads issued into the ring so far; load i uses stage i % kStages and
+// completes the phase with parity (i / kStages) & 1.  Not sensitive to the abort flag: the
 // copies are in flight and must finish before the shared memory can be given up.
+template <int kStages>
 __device__ __forceinline__ void drain_ring(uint64_t* full, uint32_t issued, uint32_t* status) {
-  const uint32_t n_drain = issued < (uint32_t)kFaStages ? issued : (uint32_t)kFaStages;
+  const uint32_t n_drain = issued < (uint32_t)kStages ? issued : (uint32_t)kStages;
   for (uint32_t i = 0; i < n_drain; ++i) {
     const uint32_t idx = issued - 1 - i;
     const long long t0 = clock64();
-    while (!mbar_try_wait(&full[idx % kFaStages], (idx / kFaStages) & 1u)) {
+    while (!mbar_try_wait(&full[idx % kStages], (idx / kStages) & 1u)) {
       if (clock64() - t0 > kTimeoutCycles) { atomicOr(status, kStatusTimeout); break; }
     }
   }
@@ -197,13 +246,51 @@ __device__ __forceinline__ void exp2_chunk(const uint32_t (&s)[32], uint32_t (&p
   }
 }
 
+// The same for a reference m that is a whole number, |m| <= 2^20: p = 2^(s - m).  For the polynomial
+// pairs the subtraction is free, m being part of the constant that rounds to the nearest integer; they
+// clamp at m - 120, below which the exponent field would wrap.
+template <int kPoly>
+__device__ __forceinline__ void exp2_chunk_shifted(const uint32_t (&s)[32], float m, uint32_t (&packed)[16]) {
+  const float2 neg_m = make_float2(-m, -m);
+  const float floor_s = m - 120.0f, magic = 12582912.0f - m;  // exact: 1.5 * 2^23 -+ 2^20 keeps its exponent
+  const float2 magic2 = make_float2(magic, magic), neg_magic2 = make_float2(-magic, -magic);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    float2 p;
+    if (i < kPoly) {
+      const float2 x = make_float2(fmaxf(__uint_as_float(s[2 * i]), floor_s), fmaxf(__uint_as_float(s[2 * i + 1]), floor_s));
+      p = poly_exp2_pair(x, magic2, neg_magic2);
+    } else {
+      const float2 x = __fadd2_rn(make_float2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), neg_m);
+      p.x = fast_exp2(x.x);
+      p.y = fast_exp2(x.y);
+    }
+    packed[i] = pack_bf16(p.x, p.y);
+  }
+}
+
+// Largest of a thread's 32 scores.
+__device__ __forceinline__ float max32(const uint32_t (&s)[32]) {
+  float mx[4];
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    const uint32_t* sc = &s[g * 8];
+    mx[g] = fmax3(__uint_as_float(sc[0]), __uint_as_float(sc[1]), __uint_as_float(sc[2]));
+    mx[g] = fmax3(mx[g], __uint_as_float(sc[3]), __uint_as_float(sc[4]));
+    mx[g] = fmax3(mx[g], __uint_as_float(sc[5]), __uint_as_float(sc[6]));
+    mx[g] = fmaxf(mx[g], __uint_as_float(sc[7]));
+  }
+  return fmaxf(fmax3(mx[0], mx[1], mx[2]), mx[3]);
+}
+
 __device__ __forceinline__ void pair_barrier(int id) {  // the two warps of one (tile, lane quarter)
   asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory");
 }
 
 // kFirst / kLast: this launch holds the first / the last key chunk of the sweep.
-template <bool kFirst, bool kLast>
-__global__ void __launch_bounds__(kFaThreads, 1)
+// kTiles: query tiles of the CTA.
+template <int kTiles, bool kFirst, bool kLast>
+__global__ void __launch_bounds__(FaShape<kTiles>::kThreads, kTiles == 2 ? 1 : 2)
 flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_bfloat16* __restrict__ qkv,
                        __nv_bfloat16* __restrict__ o, float* __restrict__ o_state, float* __restrict__ ml_state,
                        const float* __restrict__ k_norm2_max, int seq_len, int dim, int tile_begin, int tile_end,
@@ -211,31 +298,36 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* smem_k = smem;
-  uint8_t* smem_v = smem_k + kFaStages * kFaTileBytes;
-  uint8_t* smem_ones = smem_v + kFaStages * kFaTileBytes;  // mirrors the V ring, see below
-  FaExchange* xchg = reinterpret_cast<FaExchange*>(smem_ones + kFaStages * kFaTileBytes);
-  FaBarriers* bars = reinterpret_cast<FaBarriers*>(xchg + 1);
+  using Shape = FaShape<kTiles>;
+  constexpr int kStages = Shape::kStages;
+  uint8_t* smem_v = smem_k + kStages * kFaTileBytes;
+  uint8_t* smem_ones = smem_v + kStages * kFaTileBytes;  // see below
+  FaExchange<kTiles>* xchg = reinterpret_cast<FaExchange<kTiles>*>(smem_ones + kFaOnesBytes);
+  FaBarriers<kStages>* bars = reinterpret_cast<FaBarriers<kStages>*>(xchg + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // blockIdx.z selects one of the independent sequences of seq_len rows laid back to back (the
   // global layer has one; a frame-local layer has one per frame)
   const int row_base = blockIdx.z * seq_len;
-  const int q0 = blockIdx.x * 256;  // within the sequence
+  const int q0 = blockIdx.x * (128 * kTiles);  // within the sequence
   const int head = blockIdx.y;
   // this launch covers key tiles [tile_begin, tile_end) of ceil(seq_len / 128); local tile j is
   // key tile tile_begin + j, step n = local tile n/2, half n%2
   const int n_kv = tile_end - tile_begin;
-  const int n_steps = 2 * n_kv;
+  // a last key tile with at most 64 keys has no second half
+  const bool half_tail = kLast && seq_len - (tile_end - 1) * 128 <= 64;
+  const int n_steps = 2 * n_kv - (half_tail ? 1 : 0);
+  const int n_tiles_live = kTiles == 2 && q0 + 128 < seq_len ? 2 : 1;  // a tile without rows takes no part
   constexpr bool first_chunk = kFirst;
   constexpr bool last_chunk = kLast;
 
   if (threadIdx.x == 0) {
-    mbar_init(&bars->q_ready, kFaSoftmaxWarps);
-    for (int s = 0; s < kFaStages; ++s) {
+    mbar_init(&bars->q_ready, 8 * n_tiles_live);
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(&bars->k_full[s], 1);
-      mbar_init(&bars->k_empty[s], 2);  // both MMA issuers release a stage
+      mbar_init(&bars->k_empty[s], n_tiles_live);  // every live tile's MMA issuer releases a stage
       mbar_init(&bars->v_full[s], 1);
-      mbar_init(&bars->v_empty[s], 2);
+      mbar_init(&bars->v_empty[s], n_tiles_live);
     }
     for (int t = 0; t < 2; ++t) {
       for (int h = 0; h < 2; ++h) {
@@ -252,18 +344,20 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
     tma_prefetch_desc(&tmap_qkv);
   }
   // The row sums come out of the second MMA: its B operand is 80 columns wide, V's 64 channels and,
-  // one descriptor stride (the size of the V ring) further on, a block whose first column is 1 and
-  // whose other columns are 0, so accumulator column 64 collects sum_k P[row, k] of exactly the bf16
-  // probabilities that multiply V.  The block is laid out like a V tile (128-byte rows, 16-byte
-  // chunks XOR-swizzled with the row index modulo 8) and repeated for every ring position.
-  for (int i = threadIdx.x; i < kFaStages * kFaTileBytes / 16; i += kFaThreads) {
-    const int r = i >> 3, chunk = i & 7;  // 128-byte row, 16-byte chunk within it
+  // one descriptor stride further on, a block whose first column is 1 and whose other columns are 0,
+  // so accumulator column 64 collects sum_k P[row, k] of exactly the bf16 probabilities that multiply
+  // V.  The block is 16 key rows (one instruction's worth) laid out like a V tile (128-byte rows,
+  // 16-byte chunks XOR-swizzled with the row index modulo 8); every instruction's descriptor carries
+  // the stride from its own V rows to this one block.
+  if (threadIdx.x < kFaOnesBytes / 16) {
+    const int r = threadIdx.x >> 3, chunk = threadIdx.x & 7;  // 128-byte row, 16-byte chunk within it
     const uint32_t first = chunk == (r & 7) ? 0x00003f80u : 0u;  // bf16 1.0 in logical column 0
-    reinterpret_cast<uint4*>(smem_ones)[i] = make_uint4(first, 0u, 0u, 0u);
+    reinterpret_cast<uint4*>(smem_ones)[threadIdx.x] = make_uint4(first, 0u, 0u, 0u);
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes, read by the MMA
-  if (warp == 16) {
-    tmem_alloc(&bars->tmem_base, 512);
+  constexpr int kIssuerWarp = Shape::kSoftmaxWarps;  // of tile 0; then the TMA producer, the issuer of tile 1
+  if (warp == kIssuerWarp) {
+    tmem_alloc(&bars->tmem_base, Shape::kTmemCols);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -272,13 +366,13 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
   const uint32_t tmem_base = bars->tmem_base;
   const WaitCtl ctl{&bars->abort_flag, status};
 
-  if (warp == 17) {
+  if (warp == kIssuerWarp + 1) {
     // ------------------------------------------------------------------ TMA producer
     if (elect_one()) {
       uint32_t k_issued = 0, v_issued = 0;
       for (int j = 0; j < n_kv; ++j) {
-        const int stage = j % kFaStages;
-        const uint32_t phase = (uint32_t)(j / kFaStages) & 1u;
+        const int stage = j % kStages;
+        const uint32_t phase = (uint32_t)(j / kStages) & 1u;
         if (!mbar_wait(&bars->k_empty[stage], phase ^ 1u, ctl)) break;
         mbar_expect_tx(&bars->k_full[stage], kFaTileBytes);
         tma_load_2d(smem_k + stage * kFaTileBytes, &tmap_qkv, &bars->k_full[stage], dim + head * 64,
@@ -291,23 +385,26 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         ++v_issued;
       }
       // every load issued by this thread must have landed before the CTA may exit
-      drain_ring(bars->k_full, k_issued, status);
-      drain_ring(bars->v_full, v_issued, status);
+      drain_ring<kStages>(bars->k_full, k_issued, status);
+      drain_ring<kStages>(bars->v_full, v_issued, status);
     }
-  } else if (warp == 16 || warp == 18) {
+  } else if (warp == kIssuerWarp || (n_tiles_live == 2 && warp == kIssuerWarp + 2)) {
     // ------------------------------------------------------------------ MMA issuer of tile t
     if (elect_one()) {
-      const int t = warp == 16 ? 0 : 1;
+      const int t = warp == kIssuerWarp ? 0 : 1;
       constexpr uint32_t idesc_qk = umma_idesc_bf16(128, 64, false, false);
       constexpr uint32_t idesc_pv = umma_idesc_bf16(128, kFaOCols, false, true);
-      const uint32_t s_col = tmem_base + kFaColS + t * 128;
-      const uint32_t o_col = tmem_base + kFaColO + t * kFaOCols;
-      const uint32_t q_col = tmem_base + kFaColQ + t * 32;
+      const uint32_t s_col = tmem_base + Shape::kColS + t * 128;
+      const uint32_t o_col = tmem_base + Shape::kColO + t * kFaOCols;
+      const uint32_t q_col = tmem_base + Shape::kColQ + t * 32;
       // S_h = Q (tensor memory) x K[64h .. 64h+63]^T (shared memory, K-major); 4 steps of 16 channels
       // the descriptors are linear in the shared-memory address (its 16-byte units sit in the low
       // bits and cannot carry out of their field), so a stage / half is one addition away
       const uint64_t k_desc0 = smem_desc_sw128(smem_u32(smem_k), 16, 1024);
-      const uint64_t v_desc0 = smem_desc_sw128(smem_u32(smem_v), kFaStages * kFaTileBytes, 1024);
+      const uint64_t v_desc0 = smem_desc_sw128(smem_u32(smem_v), kStages * kFaTileBytes, 1024);
+      // x 16-byte units into the V ring: the address grows and the stride to the ones block (bits
+      // 16-29, never below zero because that block lies behind the ring) shrinks by the same amount
+      auto v_desc_at = [&](uint32_t x) { return v_desc0 + (uint64_t)x - ((uint64_t)x << 16); };
       auto issue_qk = [&](int h, int stage) {
         const uint64_t b_desc = k_desc0 + (uint64_t)((stage * kFaTileBytes + h * 8192) >> 4);
 #pragma unroll
@@ -319,7 +416,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       if (ok) {
         tc_fence_after();
         issue_qk(0, 0);
-        issue_qk(1, 0);
+        if (n_steps > 1) issue_qk(1, 0);
         umma_commit(&bars->k_empty[0]);
       }
       int stage = 0;
@@ -327,27 +424,29 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       for (int j = 0; j < n_kv && ok; ++j) {
         int next_stage = stage + 1;
         uint32_t next_phase = phase;
-        if (next_stage == kFaStages) { next_stage = 0; next_phase ^= 1u; }
+        if (next_stage == kStages) { next_stage = 0; next_phase ^= 1u; }
         const bool last = j + 1 == n_kv;
         if (!mbar_wait(&bars->v_full[stage], phase, ctl)) { ok = false; break; }
         if (!last && !mbar_wait(&bars->k_full[next_stage], next_phase, ctl)) { ok = false; break; }
         for (int h = 0; h < 2; ++h) {
+          if (last && h == 1 && half_tail) break;
           if (!mbar_wait(&bars->p_ready[t][h], j & 1, ctl)) { ok = false; break; }
           tc_fence_after();
           // 64 keys of V_j (64 rows of 128 bytes = 8192 bytes per half), 16 keys per instruction:
           // 8 TMEM columns of P (keys 0-31 in columns [0,16) of the half, keys 32-63 in [32,48)),
-          // 2048 bytes of V
-          // second 64-column block of B = the ones block, one V ring further on
-          const uint64_t v_desc = v_desc0 + (uint64_t)((stage * kFaTileBytes + h * 8192) >> 4);
+          // 2048 bytes of V; second 64-column block of B = the ones block
+          const uint32_t v_at = (uint32_t)((stage * kFaTileBytes + h * 8192) >> 4);
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            umma_ts(o_col, s_col + h * 64 + (k >> 1) * 32 + (k & 1) * 8, v_desc + 128 * k, idesc_pv,
+            umma_ts(o_col, s_col + h * 64 + (k >> 1) * 32 + (k & 1) * 8, v_desc_at(v_at + 128 * k), idesc_pv,
                     (j | h | k) != 0 ? 1u : 0u);  // every launch starts its accumulators from zero
           if (last) {
             // no further Q K^T follows whose completion would tell the softmax threads that this
             // P V has retired
             umma_commit(&bars->pv_done[t]);
-            if (h == 1) umma_commit(&bars->o_done[t]);
+            if (h == 1 || half_tail) umma_commit(&bars->o_done[t]);
+          } else if (h == 1 && half_tail && j + 2 == n_kv) {
+            umma_commit(&bars->pv_done[t]);  // the half that would follow does not exist
           } else {
             issue_qk(h, next_stage);
           }
@@ -366,7 +465,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         }
       }
     }
-  } else if (warp < kFaSoftmaxWarps) {
+  } else if (warp < 8 * n_tiles_live) {
     // ------------------------------------------------------------------ softmax warps
     const int t = warp >> 3;
     const int c = (warp >> 2) & 1;
@@ -377,11 +476,12 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
     const int row_local = q0 + t * 128 + row_in_tile;
     const bool row_live = row_local < seq_len;
     const int row = row_base + row_local;  // global row of qkv / o
-    const uint32_t s_addr = tmem_base + lane_base + kFaColS + t * 128;
-    const uint32_t o_addr = tmem_base + lane_base + kFaColO + t * kFaOCols + c * 32;
-    const uint32_t l_addr = tmem_base + lane_base + kFaColO + t * kFaOCols + 64;  // row sum column (+15 unused)
+    const uint32_t s_addr = tmem_base + lane_base + Shape::kColS + t * 128;
+    const uint32_t o_addr = tmem_base + lane_base + Shape::kColO + t * kFaOCols + c * 32;
+    const uint32_t l_addr = tmem_base + lane_base + Shape::kColO + t * kFaOCols + 64;  // row sum column (+15 unused)
     float q_norm2 = 0.0f;  // |q|^2 of the whole row, summed in the same order by both of its threads
     bool fixed_ref;
+    float score_bound;
     {
       // this thread's half (32 channels) of its query row goes to tensor memory
       uint32_t qreg[16];
@@ -406,9 +506,9 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       // Cauchy-Schwarz bound on this row's scores (K carries the softmax scale, so the scores are in
       // base-2 units already); both threads of a row hold the same value, and both warps of a pair
       // vote over the same 32 rows, so they agree on the form they run
-      const float score_bound = sqrtf(q_norm2 * k_norm2_max[blockIdx.z * gridDim.y + head]);
+      score_bound = sqrtf(q_norm2 * k_norm2_max[blockIdx.z * gridDim.y + head]);
       fixed_ref = __all_sync(0xffffffffu, score_bound <= kFaFixedRefLimit ? 1 : 0) != 0;
-      tmem_st16(tmem_base + lane_base + kFaColQ + t * 32 + c * 16, qreg);
+      tmem_st16(tmem_base + lane_base + Shape::kColQ + t * 32 + c * 16, qreg);
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
@@ -417,7 +517,14 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
     float m_ref = -INFINITY;  // reference, in the scores' own (base-2) units
     bool ok = true;
     int pair_syncs = 0;  // both warps of a pair must pass the same number of pair barriers
-    if (fixed_ref) {
+    if (q0 + t * 128 + (int)quarter * 32 >= seq_len) {
+      // ---- no live row in this warp (nor in its partner): the issuer needs the hand-over, nobody the result
+      pair_syncs = n_steps;
+      for (int n = 0; n < n_steps && ok; ++n) {
+        ok = mbar_wait_warp(&bars->s_full[t][n & 1], (uint32_t)(n >> 1) & 1u, ctl);
+        if (ok && lane == 0) mbar_arrive(&bars->p_ready[t][n & 1]);
+      }
+    } else if (fixed_ref) {
       // ---- fixed reference.  The scores all lie inside [-score_bound, score_bound]; the constant
       // 2^-score_bound that would bring the exponents to [-2 score_bound, 0] cancels between numerator
       // and row sum, so it is not applied: reference 0, and the scores go into the exponential as
@@ -451,8 +558,65 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         return true;
       };
       for (int j = 0; j + 1 < n_kv && ok; ++j) ok = step(j, 0, false) && step(j, 1, false);
-      if (ok && n_kv > 0) ok = step(n_kv - 1, 0, true) && step(n_kv - 1, 1, true);
+      if (ok && n_kv > 0) ok = step(n_kv - 1, 0, true) && (half_tail || step(n_kv - 1, 1, true));
     } else {
+    // ---- a reference that is not zero.  The first step's scores are looked at once (they stay where
+    // they are for the sweep): their maximum is a lower bound of the row maximum, score_bound an upper one.
+    bool shifted = false;
+    if (mbar_wait_warp(&bars->s_full[t][0], 0, ctl)) {
+      tc_fence_after();
+      uint32_t s[32];
+      tmem_ld32(s_addr + c * 32, s);
+      tmem_ld_wait();
+      const int valid = seq_len - tile_begin * 128 - c * 32;
+      if (valid < 32) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+          if (i >= valid) s[i] = 0xff800000u;  // -inf
+      }
+      const float mx_own = max32(s);
+      xchg->row_max[1][t][c][row_in_tile] = mx_own;  // the sweep's first exchange uses the other slot
+      pair_barrier(barrier_id);
+      const float mx_first = fmaxf(mx_own, xchg->row_max[1][t][c ^ 1][row_in_tile]);
+      const float m = ceilf(fmaxf(score_bound - kFaShiftUp, mx_first));
+      shifted = __all_sync(0xffffffffu, m - mx_first <= kFaShiftDown && fabsf(m) <= 1048576.0f ? 1 : 0) != 0;
+      if (shifted) m_ref = m;
+    } else {
+      xchg->row_max[1][t][c][row_in_tile] = INFINITY;  // sends the partner to the form that keeps meeting this warp
+      pair_barrier(barrier_id);
+      ok = false;
+    }
+    if (shifted) {
+    // ---- shifted reference, kept for the whole launch: a whole number m (see kFaShiftUp) under which
+    // nothing overflows and the row's largest probability is not small, so no running maximum is
+    // needed.
+    pair_syncs = n_steps;
+    auto step = [&](int j, int h, bool may_mask) -> bool {
+      if (!mbar_wait_warp(&bars->s_full[t][h], j & 1, ctl)) return false;
+      tc_fence_after();
+      uint32_t s[32];
+      tmem_ld32(s_addr + h * 64 + c * 32, s);
+      tmem_ld_wait();
+      uint32_t packed[16];
+      const int valid = may_mask ? seq_len - ((tile_begin + j) * 2 + h) * 64 - c * 32 : 32;
+      if (may_mask && valid < 32) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+          if (i >= valid) s[i] = 0xff800000u;  // -inf: probability 0 (the polynomial cannot take it)
+        exp2_chunk_shifted<0>(s, m_ref, packed);
+      } else {
+        exp2_chunk_shifted<kFaShiftPolyPairs>(s, m_ref, packed);
+      }
+      tmem_st16(s_addr + h * 64 + c * 32, packed);  // over the start of the columns just read
+      tmem_st_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->p_ready[t][h]);
+      return true;
+    };
+    for (int j = 0; j + 1 < n_kv && ok; ++j) ok = step(j, 0, false) && step(j, 1, false);
+    if (ok && n_kv > 0) ok = step(n_kv - 1, 0, true) && (half_tail || step(n_kv - 1, 1, true));
+    } else if (ok) {
     // ---- online form; the same two written-out halves per key tile as above
     auto step = [&](int j, int h, bool may_mask) -> bool {
       if (!mbar_wait_warp(&bars->s_full[t][h], j & 1, ctl)) return false;
@@ -468,16 +632,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
             if (i >= valid) s[i] = 0xff800000u;  // -inf
         }
       }
-      float mx[4];
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        const uint32_t* sc = &s[g * 8];
-        mx[g] = fmax3(__uint_as_float(sc[0]), __uint_as_float(sc[1]), __uint_as_float(sc[2]));
-        mx[g] = fmax3(mx[g], __uint_as_float(sc[3]), __uint_as_float(sc[4]));
-        mx[g] = fmax3(mx[g], __uint_as_float(sc[5]), __uint_as_float(sc[6]));
-        mx[g] = fmaxf(mx[g], __uint_as_float(sc[7]));
-      }
-      const float mx_own = fmaxf(fmax3(mx[0], mx[1], mx[2]), mx[3]);
+      const float mx_own = max32(s);
       // swap with the thread that holds the other 32 scores of this row
       xchg->row_max[h][t][c][row_in_tile] = mx_own;
       pair_barrier(barrier_id);
@@ -490,9 +645,9 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         if (__any_sync(0xffffffffu, grow ? 1 : 0)) {
           // O_t may still be the target of the previous step's P V.  The issuer follows that P V
           // with the Q K^T that refills the other half's scores, so their arrival tells that it
-          // has retired; after the last key tile, where nothing follows, pv_done does.
+          // has retired; where nothing follows (the last key tile, a half that does not exist), pv_done does.
           const int jp = h == 1 ? j : j - 1;  // key tile of step n-1 (its half is h^1)
-          const bool waited = jp + 1 < n_kv
+          const bool waited = 2 * (jp + 1) + (h ^ 1) < n_steps
                                   ? mbar_wait_warp(&bars->s_full[t][h ^ 1], (uint32_t)(jp + 1) & 1u, ctl)
                                   : mbar_wait_warp(&bars->pv_done[t], 0, ctl);
           if (!waited) return false;
@@ -526,7 +681,8 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       return true;
     };
     for (int j = 0; j + 1 < n_kv && ok; ++j) ok = step(j, 0, false) && step(j, 1, false);
-    if (ok && n_kv > 0) ok = step(n_kv - 1, 0, true) && step(n_kv - 1, 1, true);
+    if (ok && n_kv > 0) ok = step(n_kv - 1, 0, true) && (half_tail || step(n_kv - 1, 1, true));
+    }
     }
     // a warp that gave up early still meets its partner at every barrier the partner may be in
     for (; pair_syncs < n_steps; ++pair_syncs) pair_barrier(barrier_id);
@@ -589,9 +745,9 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 16) {
+  if (warp == kIssuerWarp) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, 512);
+    tmem_dealloc(tmem_base, Shape::kTmemCols);
   }
 }
 
@@ -616,7 +772,7 @@ constexpr int kFa8VTileBytes = 64 * 128;           // 64 channels x 128 key byte
 constexpr int kFa8VStageBytes = kFa8VTileBytes + 16 * 128;  // + the ones rows
 constexpr uint32_t kFa8ColQ = 416;                 // Q_0, Q_1: 16 columns of 4 bytes each
 constexpr float kFa8Headroom = 8.0f;               // the row maximum maps to 2^8 of E4M3's 448
-constexpr int kFa8SmemBytes = kFaStages * (kFa8KTileBytes + kFa8VStageBytes) + (int)sizeof(FaExchange) + 512 + 1024;
+constexpr int kFa8SmemBytes = kFaStages * (kFa8KTileBytes + kFa8VStageBytes) + (int)sizeof(FaExchange<2>) + 512 + 1024;
 
 template <bool kFirst, bool kLast>
 __global__ void __launch_bounds__(kFaThreads, 1)
@@ -628,8 +784,8 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* smem_k = smem;
   uint8_t* smem_v = smem_k + kFaStages * kFa8KTileBytes;
-  FaExchange* xchg = reinterpret_cast<FaExchange*>(smem_v + kFaStages * kFa8VStageBytes);
-  FaBarriers* bars = reinterpret_cast<FaBarriers*>(xchg + 1);
+  FaExchange<2>* xchg = reinterpret_cast<FaExchange<2>*>(smem_v + kFaStages * kFa8VStageBytes);
+  FaBarriers<kFaStages>* bars = reinterpret_cast<FaBarriers<kFaStages>*>(xchg + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q0 = blockIdx.x * 256;
@@ -696,8 +852,8 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
         tma_load_2d(smem_v + stage * kFa8VStageBytes, &tmap_v8t, &bars->v_full[stage], (tile_begin + j) * 128, head * 64);
         ++v_issued;
       }
-      drain_ring(bars->k_full, k_issued, status);
-      drain_ring(bars->v_full, v_issued, status);
+      drain_ring<kFaStages>(bars->k_full, k_issued, status);
+      drain_ring<kFaStages>(bars->v_full, v_issued, status);
     }
   } else if (warp == 16 || warp == 18) {
     // ------------------------------------------------------------------ MMA issuer of tile t
@@ -819,16 +975,7 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
             if (i >= valid) s[i] = 0xff800000u;  // -inf
         }
       }
-      float mx[4];
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        const uint32_t* sc = &s[g * 8];
-        mx[g] = fmax3(__uint_as_float(sc[0]), __uint_as_float(sc[1]), __uint_as_float(sc[2]));
-        mx[g] = fmax3(mx[g], __uint_as_float(sc[3]), __uint_as_float(sc[4]));
-        mx[g] = fmax3(mx[g], __uint_as_float(sc[5]), __uint_as_float(sc[6]));
-        mx[g] = fmaxf(mx[g], __uint_as_float(sc[7]));
-      }
-      const float mx_own = fmaxf(fmax3(mx[0], mx[1], mx[2]), mx[3]);
+      const float mx_own = max32(s);
       xchg->row_max[h][t][c][row_in_tile] = mx_own;
       pair_barrier(barrier_id);
       ++pair_syncs;
@@ -1030,15 +1177,15 @@ cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, 
     return cudaErrorInvalidValue;
   using Kernel = void (*)(const CUtensorMap, const __nv_bfloat16*, __nv_bfloat16*, float*, float*, const float*, int,
                           int, int, int, uint32_t*);
-  const Kernel kernels[2][2] = {{flash_attention_kernel<false, false>, flash_attention_kernel<false, true>},
-                                {flash_attention_kernel<true, false>, flash_attention_kernel<true, true>}};
-  static std::atomic<unsigned long long> smem_set[2][2];
-  for (int a = 0; a < 2; ++a)
-    for (int b = 0; b < 2; ++b) {
-      cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(kernels[a][b]), kFaSmemBytes, smem_set[a][b]);
-      if (e != cudaSuccess) return e;
-    }
-  const dim3 grid((unsigned)((seq_len + 255) / 256), (unsigned)ctx->sz.heads, (unsigned)n_seq);
+  // [query tiles of a CTA - 1][first chunk][last chunk]
+  const Kernel kernels[2][2][2] = {
+      {{flash_attention_kernel<1, false, false>, flash_attention_kernel<1, false, true>},
+       {flash_attention_kernel<1, true, false>, flash_attention_kernel<1, true, true>}},
+      {{flash_attention_kernel<2, false, false>, flash_attention_kernel<2, false, true>},
+       {flash_attention_kernel<2, true, false>, flash_attention_kernel<2, true, true>}}};
+  const int smem_bytes[2] = {FaShape<1>::kSmemBytes, FaShape<2>::kSmemBytes};
+  static std::atomic<unsigned long long> smem_set[2][2][2];
+  const int tiles = seq_len <= kFaOneTileRows ? 1 : 2;
   // balanced chunks of at most kFaChunkTiles key tiles; more than one needs the state buffers (which
   // are sized for the single long sequence of the global layer)
   const int n_tiles = (int)((seq_len + 127) / 128);
@@ -1046,9 +1193,14 @@ cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, 
   const int per_chunk = (n_tiles + n_chunks - 1) / n_chunks;
   if (n_chunks > 1 && (n_seq != 1 || ctx->ws.attn_o_state == nullptr || ctx->ws.attn_ml_state == nullptr))
     return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)((n_tiles + tiles - 1) / tiles), (unsigned)ctx->sz.heads, (unsigned)n_seq);
+  const int threads = tiles == 2 ? FaShape<2>::kThreads : FaShape<1>::kThreads;
   for (int begin = 0; begin < n_tiles; begin += per_chunk) {
     const int end = begin + per_chunk < n_tiles ? begin + per_chunk : n_tiles;
-    kernels[begin == 0][end == n_tiles]<<<grid, kFaThreads, kFaSmemBytes, s>>>(
+    const int a = tiles - 1, b = begin == 0, c = end == n_tiles;
+    cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(kernels[a][b][c]), smem_bytes[a], smem_set[a][b][c]);
+    if (e != cudaSuccess) return e;
+    kernels[a][b][c]<<<grid, threads, smem_bytes[a], s>>>(
         tmap, qkv, o, ctx->ws.attn_o_state, ctx->ws.attn_ml_state, ctx->ws.attn_kmax, (int)seq_len, dim, begin, end,
         ctx->ws.status);
     ++*launches;

@@ -332,6 +332,7 @@ def score_bounds(qkv, heads=16):
 
 
 FIXED_REF_LIMIT = 80.0  # the library's kFaFixedRefLimit
+SHIFT_UP, SHIFT_DOWN = 84.0, 92.0  # and its kFaShiftUp, kFaShiftDown
 
 
 @pytest.mark.parametrize("wl", [WORKLOADS["C1"], MID], ids=lambda w: w.name)
@@ -407,6 +408,80 @@ def test_attention_core_with_peaked_softmax(lib, grid, sharpness, form):
 
 
 # ------------------------------------------------------------------ Q/K normalisation and rotary embedding
+def softmax_forms(qkv, heads=16, limit=FIXED_REF_LIMIT):
+    """Which of the kernel's three softmax forms every warp of 32 rows takes, per head: "fixed" where all
+    its rows have a score bound under the limit, "shifted" where bound and the maximum over the first
+    64 keys leave room for one whole-number reference, else "online"."""
+    m, d = qkv.shape[0], qkv.shape[1] // 3
+    b = score_bounds(qkv, heads)
+    forms = {}
+    for h in range(heads):
+        q, k = qkv[:, h * 64:h * 64 + 64], qkv[:, d + h * 64:d + h * 64 + 64]
+        first = (q @ k[:64].T).max(1)
+        shift = np.ceil(np.maximum(b[:, h] - SHIFT_UP, first)) - first <= SHIFT_DOWN
+        for w in range(0, m, 32):
+            if (b[w:w + 32, h] <= limit).all():
+                form = "fixed"
+            else:
+                form = "shifted" if shift[w:w + 32].all() else "online"
+            forms[form] = forms.get(form, 0) + 1
+    return forms
+
+
+@pytest.mark.parametrize("frames,grid,sharpness,form", [
+    (1, (1, 1), 1.0, "fixed"), (1, (1, 59), 16.0, "shifted"), (1, (2, 30), 16.0, "shifted"), (1, (3, 41), 64.0, "online"),
+    (1, (2, 62), 1.0, "fixed"), (1, (11, 17), 64.0, "online"), (1, (4, 47), 64.0, "online"), (1, (14, 18), 16.0, "shifted"),
+    (4, (64, 64), 1.0, "fixed"), (4, (64, 64), 16.0, "shifted"), (4, (64, 64), 64.0, "online")])
+def test_attention_core_at_tile_edges_in_every_softmax_form(lib, frames, grid, sharpness, form):
+    """Sequence lengths around the 64-key halves, the 128-row tiles and (16,404 rows: 129 tiles, the last
+    with 20 rows and without a second half) the pairs of tiles of a CTA."""
+    ctx = lib.LiteVGGT(frames, grid[0], grid[1], 0.0)
+    m = ctx.n_merged
+    g = torch.Generator().manual_seed(77 + m)
+    x = torch.randn(m, 1024, generator=g).to(torch.bfloat16)
+    w_qkv, b_qkv, w_o, b_o = make_attention_weights(WORKLOADS["C1"], 3)
+    w_qkv[:1024] *= sharpness
+    ctx.global_attn(x.cuda(), w_qkv.cuda(), b_qkv.cuda(), w_o.cuda(), b_o.cuda())
+    ctx.poll()
+    qkv = to_f64(ctx.debug_buffer(0))
+    assert softmax_forms(qkv).get(form, 0) > 0
+    rows = np.arange(m) if m < 4096 else np.r_[0:40, 8190:8230, m - 40:m]
+    ref_o = O.attention_core(unfold_k(qkv), heads=16, rows=rows)
+    # The probabilities are rounded to bf16, each off by at most 2^-9 relative, and the row sum is formed
+    # from the rounded values: an output moves by 2^-9 sum_i d_i p_i (v_i - o), |d_i| <= 1.  Rows of random
+    # keys do not average that away, so it is bounded per entry: Hoeffding's inequality for independent
+    # d_i, taken where 1e7 entries together exceed it with a chance of 1e-6 (a factor sqrt(2 ln 2e13) = 7.8).
+    u, worst = unfold_k(qkv), 0.0
+    for h in range(16):
+        q, k, v = (u[:, i * 1024 + h * 64:i * 1024 + h * 64 + 64] for i in range(3))
+        s = q[rows] @ k.T / 8.0
+        p = np.exp(s - s.max(1, keepdims=True))
+        p2 = (p / p.sum(1, keepdims=True)) ** 2
+        o = ref_o[:, h * 64:h * 64 + 64]
+        worst = max(worst, float((p2 @ (v * v) - 2 * o * (p2 @ v) + o * o * p2.sum(1, keepdims=True)).max()))
+    noise = 7.8 * 2.0 ** -9 * np.sqrt(worst) / float(np.sqrt(np.mean(ref_o * ref_o)))
+    check_bf16(f"edges m={m} s={sharpness}: attention core", to_f64(ctx.debug_buffer(1))[rows], ref_o, noise=noise,
+               sampled=m >= 4096)
+    ctx.close()
+
+
+@pytest.mark.parametrize("grid", [(1, 1), (1, 59), (4, 15), (3, 41), (4, 31)], ids=lambda g: f"{g[0]}x{g[1]}")
+def test_frame_attention_at_tile_edges(lib, grid):
+    """6, 64, 65, 128 and 129 tokens a frame.  The rows share a common part, as a frame's tokens do:
+    LAYER_NOISE is stated against the RMS of outputs that do not average out to sigma / sqrt(rows), where
+    the rounding of p (2^-9 per key, relative to sigma / sqrt(rows) too) would be of the output's own size."""
+    ctx = lib.LiteVGGT(3, grid[0], grid[1], 0.5)
+    n = ctx.n_tokens
+    g = torch.Generator().manual_seed(5 + n)
+    x = (torch.randn(1, 1024, generator=g) + 0.5 * torch.randn(n, 1024, generator=g)).to(torch.bfloat16)
+    w = make_attention_weights(WORKLOADS["C1"], 4)
+    y = ctx.frame_attn(x.cuda(), *[t.cuda() for t in w])
+    ctx.poll()
+    ref = O.frame_attention(to_f64(x), 3, *[to_f64(t) for t in w])
+    check_bf16(f"frame attention, {n // 3} tokens a frame", to_f64(y), ref, noise=LAYER_NOISE)
+    ctx.close()
+
+
 @pytest.mark.parametrize("wl", [WORKLOADS["C1"], ODD], ids=lambda w: w.name)
 @pytest.mark.parametrize("mode", ["norm", "rope", "both"])
 def test_global_attention_with_qk_norm_and_rope(lib, wl, mode):
