@@ -236,6 +236,18 @@ litevggt_status ensure_block_ws(litevggt_ctx* ctx) {
   return LITEVGGT_OK;
 }
 
+// What the global layer's attention core needs to know about Q, K and V before it starts.
+LinearStat core_stat(const litevggt_ctx* ctx, long long m) {
+  LinearStat st;
+  if (ctx->cfg.qkv_dtype == 1) {
+    st.amax = ctx->ws.qkv_amax;
+  } else {
+    st.key_norm = ctx->ws.attn_kmax;
+    st.seq_len = m;
+  }
+  return st;
+}
+
 }  // namespace
 
 extern "C" {
@@ -548,11 +560,11 @@ litevggt_status litevggt_global_attn(litevggt_ctx* ctx, const void* x_merged, in
     StepTimer t(ctx, 6, s);
     e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x_merged), m, d,
                              static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
-                             2 * d, kKeyScaleLog2e, ctx->ws.qkv, s, &n);
+                             2 * d, kKeyScaleLog2e, core_stat(ctx, m), ctx->ws.qkv, s, &n);
   }
   if (e == cudaSuccess && ctx->cfg.qkv_dtype == 1) {
     StepTimer t(ctx, 14, s);
-    e = launch_qkv_quantize(ctx, ctx->ws.qkv, m, s, &n);
+    e = launch_qkv_quantize(ctx, ctx->ws.qkv, m, true, s, &n);
   }
   if (e == cudaSuccess) {
     StepTimer t(ctx, 7, s);
@@ -590,14 +602,16 @@ litevggt_status litevggt_global_attn_ext(litevggt_ctx* ctx, const litevggt_plan*
     if (plan == nullptr) return LITEVGGT_ERR_NULL;
     if (!plan_ok(plan) || plan->owner != ctx || !plan->built) return LITEVGGT_ERR_STALE_PLAN;
   }
+  const bool embeds = given == 4 || ext->rope != 0, fp8 = ctx->cfg.qkv_dtype == 1;
   const int d = ctx->sz.dim;
   cudaStream_t s = (cudaStream_t)stream;
   int n = 0;
   cudaError_t e;
   {
     StepTimer t(ctx, 6, s);
-    e = launch_linear(ctx, static_cast<const __nv_bfloat16*>(x_merged), m, d, static_cast<const __nv_bfloat16*>(w_qkv),
-                      3 * d, static_cast<const __nv_bfloat16*>(b_qkv), ctx->ws.qkv, s, &n);
+    e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x_merged), m, d,
+                             static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
+                             2 * d, 1.0f, embeds ? LinearStat{} : core_stat(ctx, m), ctx->ws.qkv, s, &n);
   }
   if (e == cudaSuccess) {
     StepTimer t(ctx, 13, s);
@@ -606,11 +620,11 @@ litevggt_status litevggt_global_attn_ext(litevggt_ctx* ctx, const litevggt_plan*
                         static_cast<const __nv_bfloat16*>(ext->q_norm_beta),
                         static_cast<const __nv_bfloat16*>(ext->k_norm_gamma),
                         static_cast<const __nv_bfloat16*>(ext->k_norm_beta), ext->norm_eps, ext->rope != 0,
-                        ext->rope_base, s, &n);
+                        ext->rope_base, fp8 ? nullptr : ctx->ws.attn_kmax, s, &n);
   }
   if (e == cudaSuccess && ctx->cfg.qkv_dtype == 1) {
     StepTimer t(ctx, 14, s);
-    e = launch_qkv_quantize(ctx, ctx->ws.qkv, m, s, &n);
+    e = launch_qkv_quantize(ctx, ctx->ws.qkv, m, !embeds, s, &n);
   }
   if (e == cudaSuccess) {
     StepTimer t(ctx, 7, s);
@@ -661,7 +675,8 @@ litevggt_status litevggt_frame_attn(litevggt_ctx* ctx, const void* x, const void
     StepTimer t(ctx, 11, s);
     e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x), z.n_tokens, d,
                              static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
-                             2 * d, kKeyScaleLog2e, ctx->ws.blk_qkv, s, &n);
+                             2 * d, kKeyScaleLog2e, LinearStat{ctx->ws.attn_kmax, z.tokens_frame, nullptr},
+                             ctx->ws.blk_qkv, s, &n);
     if (e == cudaSuccess) e = launch_flash_attention(ctx, ctx->ws.blk_qkv, z.tokens_frame, z.frames, ctx->ws.blk_o, s, &n);
     if (e == cudaSuccess)
       e = launch_linear_mlp(ctx, ctx->ws.blk_o, z.n_tokens, d, static_cast<const __nv_bfloat16*>(w_o), d,

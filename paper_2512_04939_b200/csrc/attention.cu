@@ -73,7 +73,7 @@
 // every score of a row is at most B = |q| max_k |k| (K carrying the softmax scale: base-2 units), so
 // with m = B all exponents lie in [-2B, 0]; while 2B stays well inside the exponent range of
 // fp32 nothing underflows, every probability keeps its 8 significant bits and the fp32
-// accumulators their 24.  A small pass over K finds max_k |k|^2 per head before the sweep, each
+// accumulators their 24.  The pass that rounds K last leaves max_k |k|^2 per head behind, each
 // softmax thread takes |q|^2 of its row while loading Q, and a warp pair whose rows all have
 // B <= kFaFixedRefLimit runs the sweep with a constant reference (in fact with none: the constant
 // cancels, see the kernel): no row maximum, no exchange between the two threads of a row, no
@@ -1121,56 +1121,11 @@ cudaError_t launch_flash_attention_fp8(litevggt_ctx* ctx, long long m, __nv_bflo
   return cudaGetLastError();
 }
 
-// max_k |k|^2 per (sequence, head), for the Cauchy-Schwarz bound on a row's scores.  Warp per key
-// row: the 128 16-byte pieces of a K row go to the lanes in four passes, eight neighbouring lanes
-// share a head.  Non-negative floats order like their bit patterns, so the maximum is an integer
-// atomicMax on a zeroed array.
-constexpr int kKnormWarps = 8;
-__global__ void __launch_bounds__(kKnormWarps * 32)
-key_norm_max_kernel(const __nv_bfloat16* __restrict__ qkv, int seq_len, int dim, float* __restrict__ k_norm2_max) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int seq = blockIdx.y, heads = dim / 64;
-  float best[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  for (int r = blockIdx.x * kKnormWarps + warp; r < seq_len; r += gridDim.x * kKnormWarps) {
-    const uint4* src = reinterpret_cast<const uint4*>(qkv + ((size_t)seq * seq_len + r) * 3 * dim + dim);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint4 v = __ldg(src + lane + 32 * j);
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-      float sum = 0.0f;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        sum = fmaf(bf16_lo(w[e]), bf16_lo(w[e]), sum);
-        sum = fmaf(bf16_hi(w[e]), bf16_hi(w[e]), sum);
-      }
-      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-      sum += __shfl_xor_sync(0xffffffffu, sum, 4);
-      best[j] = fmaxf(best[j], sum);
-    }
-  }
-  if ((lane & 7) == 0) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      atomicMax(reinterpret_cast<unsigned int*>(k_norm2_max) + seq * heads + (lane >> 3) + 4 * j,
-                __float_as_uint(best[j]));
-  }
-}
-
 cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long seq_len, int n_seq,
                                    __nv_bfloat16* o, cudaStream_t s, int* launches) {
   if (seq_len == 0 || n_seq == 0) return cudaSuccess;
   const int dim = ctx->sz.dim;
   if (dim != 1024 || ctx->ws.attn_kmax == nullptr) return cudaErrorInvalidValue;
-  {
-    cudaError_t e = cudaMemsetAsync(ctx->ws.attn_kmax, 0, (size_t)n_seq * ctx->sz.heads * sizeof(float), s);
-    if (e != cudaSuccess) return e;
-    long long blocks = (seq_len + 63) / 64;
-    if (blocks > 2048) blocks = 2048;
-    key_norm_max_kernel<<<dim3((unsigned)blocks, (unsigned)n_seq), kKnormWarps * 32, 0, s>>>(qkv, (int)seq_len, dim,
-                                                                                            ctx->ws.attn_kmax);
-    ++*launches;
-  }
   const long long rows = seq_len * n_seq;
   CUtensorMap tmap;
   if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap, qkv, (uint64_t)3 * dim, (uint64_t)rows, (uint64_t)3 * dim, 64, 128))

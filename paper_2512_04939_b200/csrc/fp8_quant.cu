@@ -12,7 +12,8 @@ namespace lv {
 
 constexpr int kAmaxWarps = 8;
 
-// Largest magnitude per (tensor, head).  Warp per row: the row's 384 16-byte pieces go to the lanes
+// Largest magnitude per (tensor, head), where Q and K changed after the projection (whose epilogue
+// takes it otherwise).  Warp per row: the row's 384 16-byte pieces go to the lanes
 // in 12 passes, 8 neighbouring lanes share a head.  Magnitudes are non-negative floats, which
 // order like their bit patterns: integer atomicMax on a zeroed array.
 __global__ void __launch_bounds__(kAmaxWarps * 32)
@@ -102,16 +103,20 @@ qkv_quantize_kernel(const __nv_bfloat16* __restrict__ qkv, long long m, long lon
   dv[1] = sv[1];
 }
 
-cudaError_t launch_qkv_quantize(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long m, cudaStream_t s, int* launches) {
+cudaError_t launch_qkv_quantize(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long m, bool have_amax, cudaStream_t s,
+                                int* launches) {
   if (m == 0) return cudaSuccess;
   Workspace& ws = ctx->ws;
   if (ws.q8 == nullptr || ctx->sz.dim != 1024 || ctx->sz.heads != 16) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemsetAsync(ws.qkv_amax, 0, 48 * sizeof(float), s);
-  if (e != cudaSuccess) return e;
-  long long blocks = (m + kAmaxWarps - 1) / kAmaxWarps;
-  if (blocks > 4096) blocks = 4096;
-  qkv_amax_kernel<<<(unsigned)blocks, kAmaxWarps * 32, 0, s>>>(qkv, m, ws.qkv_amax);
-  ++*launches;
+  if (!have_amax) {
+    cudaError_t e = cudaMemsetAsync(ws.qkv_amax, 0, 48 * sizeof(float), s);
+    if (e != cudaSuccess) return e;
+    // few blocks: every one sends 48 atomics per warp, and all of them meet on the same 48 words
+    long long blocks = (m + kAmaxWarps - 1) / kAmaxWarps;
+    if (blocks > 4ll * ctx->num_sms) blocks = 4ll * ctx->num_sms;
+    qkv_amax_kernel<<<(unsigned)blocks, kAmaxWarps * 32, 0, s>>>(qkv, m, ws.qkv_amax);
+    ++*launches;
+  }
   const long long m_pad = round_up(m, 128);
   qkv_quantize_kernel<<<dim3((unsigned)(m_pad / 128), 16), 256, 0, s>>>(qkv, m, m_pad, ws.qkv_amax, ws.q8, ws.k8, ws.v8t);
   ++*launches;

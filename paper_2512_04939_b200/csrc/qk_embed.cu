@@ -12,6 +12,9 @@
 //                  (kept_idx[r]); special tokens sit at (0, 0), the patch at grid row py, column
 //                  px at (py + 1, px + 1)
 //
+// The largest |k|^2 of every head, which the attention kernel's softmax reference needs, is taken on the
+// way: every block keeps it for the rows it walks over.
+//
 // One warp per row, HBM-bound: a lane owns 8 consecutive channels (16 bytes), 8 lanes cover a head,
 // one warp instruction moves four heads.  Statistics need three shuffles over the 8 lanes of a
 // head; the rotation partner of a lane is two lanes away.  All arithmetic in fp32, one rounding.
@@ -32,16 +35,20 @@ struct EmbedParams {
   int rope;                      // 0: no rotation
   float log2_base;
   int tokens_frame, n_special, grid_w;
+  float* key_norm;               // [16] or null: largest |k|^2 per head of the rounded result, starts at zero
 };
 
 __global__ void __launch_bounds__(kEmbedThreads)
 qk_embed_kernel(__nv_bfloat16* __restrict__ qkv, const int* __restrict__ kept_idx, long long m_rows,
                 long long n_tokens, EmbedParams p, uint32_t* status) {
   const int lane = threadIdx.x & 31;
-  const long long row = (long long)blockIdx.x * kEmbedRowsPerCta + (threadIdx.x >> 5);
-  if (row >= m_rows) return;
   const int j = lane & 7;  // which 8 channels of the head: 8j .. 8j+7
-
+  float theta[8];  // angle per position of this lane's 8 channels
+#pragma unroll
+  for (int e = 0; e < 8; ++e) theta[e] = exp2f(-(float)(8 * (j & 1) + e) * (1.0f / 16.0f) * p.log2_base);  // plane i in 0..15
+  float best[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // largest |k|^2 of heads (lane / 8) + 4 i
+  for (long long row = (long long)blockIdx.x * kEmbedRowsPerCta + (threadIdx.x >> 5); row < m_rows;
+       row += (long long)gridDim.x * kEmbedRowsPerCta) {
   // rotation of this lane's 8 channels: the same for every head and for queries and keys
   float cs[8], sn[8];
   const bool first = (j & 2) == 0;  // channels 0..15 of their half: out = v cos - partner sin
@@ -59,11 +66,9 @@ qk_embed_kernel(__nv_bfloat16* __restrict__ qkv, const int* __restrict__ kept_id
     }
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const int plane = 8 * (j & 1) + e;  // i in 0..15
-      const float theta = exp2f(-(float)plane * (1.0f / 16.0f) * p.log2_base);
       // angles stay below 2^8 rad (grids of at most 128 x 64), where the fast path is good to ~1e-5 absolute,
       // two orders under the rounding of the bf16 result
-      __sincosf((float)pos * theta, &sn[e], &cs[e]);
+      __sincosf((float)pos * theta[e], &sn[e], &cs[e]);
       if (first) sn[e] = -sn[e];
     }
   }
@@ -132,15 +137,36 @@ qk_embed_kernel(__nv_bfloat16* __restrict__ qkv, const int* __restrict__ kept_id
 #pragma unroll
       for (int e = 0; e < 8; ++e) v[e] *= kKeyScaleLog2e;
     }
-    base[step * 32 + lane] = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
-                                        pack_bf16(v[6], v[7]));
+    const uint4 packed = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+    base[step * 32 + lane] = packed;
+    if (is_k && p.key_norm != nullptr) {
+      const uint32_t w2[4] = {packed.x, packed.y, packed.z, packed.w};
+      float sum = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) sum = fmaf(bf16_hi(w2[i]), bf16_hi(w2[i]), fmaf(bf16_lo(w2[i]), bf16_lo(w2[i]), sum));
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      best[step - 4] = fmaxf(best[step - 4], sum);  // fmaxf drops a NaN
+    }
+  }
+  }
+  if (p.key_norm != nullptr) {
+    __shared__ unsigned int block_best[16];  // non-negative floats order like their bit patterns
+    if (threadIdx.x < 16) block_best[threadIdx.x] = 0u;
+    __syncthreads();
+    if (j == 0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) atomicMax(&block_best[4 * i + (lane >> 3)], __float_as_uint(best[i]));
+    }
+    __syncthreads();
+    if (threadIdx.x < 16) atomicMax(reinterpret_cast<unsigned int*>(p.key_norm) + threadIdx.x, block_best[threadIdx.x]);
   }
 }
 
 cudaError_t launch_qk_embed(const litevggt_ctx* ctx, __nv_bfloat16* qkv, const int* kept_idx, long long m,
                             const __nv_bfloat16* q_gamma, const __nv_bfloat16* q_beta, const __nv_bfloat16* k_gamma,
-                            const __nv_bfloat16* k_beta, float eps, int rope, float rope_base, cudaStream_t s,
-                            int* launches) {
+                            const __nv_bfloat16* k_beta, float eps, int rope, float rope_base, float* key_norm,
+                            cudaStream_t s, int* launches) {
   if (m == 0 || (q_gamma == nullptr && !rope)) return cudaSuccess;
   const Sizes& z = ctx->sz;
   EmbedParams p;
@@ -154,8 +180,15 @@ cudaError_t launch_qk_embed(const litevggt_ctx* ctx, __nv_bfloat16* qkv, const i
   p.tokens_frame = z.tokens_frame;
   p.n_special = (int)z.n_special;
   p.grid_w = (int)z.grid_w;
-  const unsigned blocks = (unsigned)((m + kEmbedRowsPerCta - 1) / kEmbedRowsPerCta);
-  qk_embed_kernel<<<blocks, kEmbedThreads, 0, s>>>(qkv, kept_idx, m, z.n_tokens, p, ctx->ws.status);
+  p.key_norm = key_norm;
+  if (key_norm != nullptr) {
+    cudaError_t e = cudaMemsetAsync(key_norm, 0, 16 * sizeof(float), s);
+    if (e != cudaSuccess) return e;
+  }
+  // as many blocks as an SM holds at a time: the key norms of a block's rows meet in one atomic per head
+  long long blocks = (m + kEmbedRowsPerCta - 1) / kEmbedRowsPerCta;
+  if (blocks > 8ll * ctx->num_sms) blocks = 8ll * ctx->num_sms;
+  qk_embed_kernel<<<(unsigned)blocks, kEmbedThreads, 0, s>>>(qkv, kept_idx, m, z.n_tokens, p, ctx->ws.status);
   ++*launches;
   return cudaGetLastError();
 }

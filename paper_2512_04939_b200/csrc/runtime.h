@@ -193,9 +193,16 @@ cudaError_t launch_linear(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m
                           long long n, const __nv_bfloat16* bias, __nv_bfloat16* out, cudaStream_t s, int* launches);
 // The same with output columns [scale_begin, scale_end) (multiples of 64) multiplied by `scale` in
 // fp32 before the one rounding to bf16: the QKV projection of an attention layer scales its K columns.
+// It also leaves behind one of two statistics of the rounded output, zeroed here first:
+struct LinearStat {
+  float* key_norm = nullptr;  // [sequences, heads] largest |k|^2 over the columns [scale_begin, scale_end) ...
+  long long seq_len = 0;      // ... of sequences of this many rows
+  float* amax = nullptr;      // [n / 64] largest magnitude of every 64 columns
+};
 cudaError_t launch_linear_scaled(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k,
                                  const __nv_bfloat16* w, long long n, const __nv_bfloat16* bias, int scale_begin,
-                                 int scale_end, float scale, __nv_bfloat16* out, cudaStream_t s, int* launches);
+                                 int scale_end, float scale, const LinearStat& stat, __nv_bfloat16* out, cudaStream_t s,
+                                 int* launches);
 
 cudaError_t launch_linear_mlp(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k,
                               const __nv_bfloat16* w, long long n, const __nv_bfloat16* bias, int gelu,
@@ -212,14 +219,18 @@ cudaError_t launch_bounded_wait_selftest(litevggt_ctx* ctx, long long limit_cycl
 // qk_embed.cu: optional per-head LayerNorm and 2-D rotary embedding of Q and K, in place on [m, 3D]
 cudaError_t launch_qk_embed(const litevggt_ctx* ctx, __nv_bfloat16* qkv, const int* kept_idx, long long m,
                             const __nv_bfloat16* q_gamma, const __nv_bfloat16* q_beta, const __nv_bfloat16* k_gamma,
-                            const __nv_bfloat16* k_beta, float eps, int rope, float rope_base, cudaStream_t s,
-                            int* launches);
+                            const __nv_bfloat16* k_beta, float eps, int rope, float rope_base, float* key_norm,
+                            cudaStream_t s, int* launches);
+// ctx->ws.attn_kmax holds the largest |k|^2 per sequence and head (left there by whichever pass rounded
+// K last: the projection or qk_embed)
 cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long seq_len, int n_seq,
                                    __nv_bfloat16* o, cudaStream_t s, int* launches);
 size_t attention_state_bytes(long long m, int dim, int heads, size_t* ml_offset);
-// E4M3 variant: per-head amax of Q, K, V and their quantised copies (fp8_quant.cu), then the
-// attention core on those (attention.cu); one sequence of m rows
-cudaError_t launch_qkv_quantize(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long m, cudaStream_t s, int* launches);
+// E4M3 variant: quantised copies of Q, K, V by the per-head magnitudes in ctx->ws.qkv_amax - taken from
+// qkv here first unless the projection has left them there - (fp8_quant.cu), then the attention core on
+// those (attention.cu); one sequence of m rows
+cudaError_t launch_qkv_quantize(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long m, bool have_amax, cudaStream_t s,
+                                int* launches);
 cudaError_t launch_flash_attention_fp8(litevggt_ctx* ctx, long long m, __nv_bfloat16* o, cudaStream_t s, int* launches);
 
 }  // namespace lv
