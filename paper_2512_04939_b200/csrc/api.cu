@@ -301,6 +301,7 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
   const size_t o_src = c.take<int>(z.n_src), o_dst = c.take<int>(z.n_dst);
   const size_t o_ps = c.take<__nv_bfloat16>(z.n_src * z.dim), o_pd = c.take<__nv_bfloat16>(z.n_dst * z.dim);
   const size_t o_ns = c.take<float>(z.n_src), o_nd = c.take<float>(round_up(z.n_dst, 256));
+  const size_t o_match = c.take<unsigned long long>(z.n_src);
   const size_t o_keys = c.take<unsigned long long>(cap);
   const size_t o_tmp = c.take<int>(z.n_tokens + 1), o_blk = c.take<int>(2048), o_row = c.take<int>(z.n_tokens);
   const size_t o_qkv = c.take<__nv_bfloat16>(z.n_merged * 3 * z.dim), o_o = c.take<__nv_bfloat16>(z.n_merged * z.dim);
@@ -329,6 +330,7 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
   ws.panel_dst = reinterpret_cast<__nv_bfloat16*>(ws.base + o_pd);
   ws.inv_norm_src = reinterpret_cast<float*>(ws.base + o_ns);
   ws.inv_norm_dst = reinterpret_cast<float*>(ws.base + o_nd);
+  ws.match_keys = reinterpret_cast<unsigned long long*>(ws.base + o_match);
   ws.sort_keys = reinterpret_cast<unsigned long long*>(ws.base + o_keys);
   ws.scan_tmp = reinterpret_cast<int*>(ws.base + o_tmp);
   ws.scan_blocks = reinterpret_cast<int*>(ws.base + o_blk);

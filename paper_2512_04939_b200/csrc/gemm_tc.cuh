@@ -6,26 +6,41 @@
 // round to bf16, store) and (b) the src->anchor cosine matching (epilogue keeps a
 // running row argmax, so the |Src| x |Dst| score matrix never exists in memory).
 //
-// Shape of one CTA:
-//   warp 0      TMA producer (one elected lane): A tile 128 x 64 and B tile 256 x 64 per
-//               k-block into a 4-stage shared-memory ring (128-byte swizzle)
-//   warp 1      MMA issuer (one elected lane): 4 x tcgen05.mma M128 N256 K16 per k-block
-//               into one of two 256-column fp32 accumulators in tensor memory
+// Mostly two CTAs (a cluster, the two SMs of a TPC) share a tile of 256 rows x kBN columns: each holds its
+// own 128 rows of A and half of the tile's rows of B, and one tcgen05.mma.cta_group::2 per 16 of K
+// reads both halves of B from both SMs.  What bounds the mainloop is the stream from L2 into shared
+// memory, and a pair needs 32 KB per CTA and k-block of a 256-column tile where a CTA of its own
+// needs 48 KB for the same arithmetic: 1322 -> 1434 TFLOP/s on 52,050 rows x 1024 x 3072, 1465 -> 1535 at
+// k = 4096 and 104 K rows.  Narrow tiles fill the chip where rows are few (543 rows x 1024 x 1024: 10.1 -> 7.6 us).
+// A CTA of its own with 128 x 256 tiles (kCtas = 1) remains
+// where its finer rows save a wave (3360 rows x 1024 x 4096: 23.6 us against 27.1) and for short k,
+// where the epilogue bounds the launch and a pair would drain in step.
+//
+// Shape of one CTA of the pair:
+//   warp 0      TMA producer (one elected lane): A tile 128 x 64 and B tile kBN/2 x 64 per
+//               k-block into a shared-memory ring (128-byte swizzle); both CTAs' loads count
+//               towards the `full` barrier of the leader (the CTA of even rank)
+//   warp 1      leader only: MMA issuer (one elected lane), 4 x tcgen05.mma M256 K16 per k-block
+//               into one of two kBN-column fp32 accumulators in both SMs' tensor memory; its
+//               commits arrive on the barriers of both CTAs
 //   warps 2..   epilogue: each thread owns one accumulator row (one TMEM lane) and
 //               walks its columns in chunks while the issuer already fills the other
 //               accumulator.  An epilogue with per-row state (the argmax) runs on four
-//               warps, one per 32-lane quarter, over all 256 columns.  An epilogue that
-//               writes a matrix runs on eight (two per quarter, 128 columns each) and
+//               warps, one per 32-lane quarter, over all columns.  An epilogue that
+//               writes a matrix runs on eight (two per quarter, every other 64 columns) and
 //               hands every 64-column chunk back as bf16; the warp parks its 32 x 64
 //               block in shared memory (128-byte swizzle) and one lane sends it to
 //               global memory as a TMA store, so rows leave the SM as whole 128-byte
 //               lines
-// Tile order.  With a row-state epilogue each CTA owns a block of 128 rows at a time and
-// sweeps all column tiles in ascending order (the state stays in registers); row blocks
-// are handed out round-robin over a grid of at most one CTA per SM.  With a matrix
-// epilogue tiles are numbered row block major and dealt round-robin, so the CTAs running
-// at one moment share a few row blocks of A and the whole of B stays in L2 - with the
-// row-block order and K = 4096 the 148 resident A panels (1 MB each) outgrew L2.
+// Tile order.  With a row-state epilogue each pair owns a block of 256 rows at a time and
+// sweeps all column tiles in ascending order (the state stays in registers); all pairs sweep
+// in step, so a tile of B comes from HBM once for all of them.  Row blocks are handed out
+// round-robin as long as there is one for every pair; the rest, a last wave that would
+// leave most of the chip idle (1 block for 74 pairs at 200 frames of 28 x 37, 32 at 32 of 37 x 37), is dealt
+// out in equal runs of column tiles, and the epilogue combines what it found in parts of a
+// row's sweep.  With a matrix epilogue tiles are numbered row block major and dealt
+// round-robin, so the CTAs running at one moment share a few row blocks of A and the whole
+// of B stays in L2 - with the row-block order and K = 4096 the resident A panels outgrew L2.
 #pragma once
 
 #include <cuda.h>
@@ -34,10 +49,8 @@
 
 namespace lv {
 
-constexpr int kGemmBM = 128;
-constexpr int kGemmBN = 256;
+constexpr int kGemmBM = 128;  // rows of a CTA
 constexpr int kGemmBK = 64;
-constexpr int kGemmStages = 4;
 constexpr int kGemmMaxThreads = 320;  // 2 + 8 warps
 // Threads of a launch: TMA warp + MMA warp + 4 (row-state epilogue) or 8 (matrix epilogue) warps.
 template <class Epi>
@@ -45,67 +58,100 @@ constexpr int gemm_threads() {
   return 64 + (Epi::kTileOut ? 256 : 128);
 }
 constexpr int kGemmTileABytes = kGemmBM * kGemmBK * 2;
-constexpr int kGemmTileBBytes = kGemmBN * kGemmBK * 2;
-constexpr int kGemmStageBytes = kGemmTileABytes + kGemmTileBBytes;
 constexpr int kGemmOutChunkCols = 64;                                   // columns per staged output block
 constexpr int kGemmOutBlockBytes = 32 * kGemmOutChunkCols * 2;          // one warp's 32 rows x 64 columns
 constexpr int kGemmOutBytes = 8 * kGemmOutBlockBytes;                   // one block per epilogue warp
-constexpr int kGemmSmemBytes = kGemmStages * kGemmStageBytes + kGemmOutBytes + 256 + 1024;  // + barriers + slack
 
+// Ring geometry of a tile of kBN columns shared by kCtas CTAs.
+template <int kBN, int kCtas>
+struct GemmShape {
+  static constexpr int kTileBBytes = kBN / kCtas * kGemmBK * 2;
+  static constexpr int kStageBytes = kGemmTileABytes + kTileBBytes;
+  static constexpr int kStages = 6 * 32768 / kStageBytes;  // a pair: 6 at 256 columns, 9 at 64; one CTA: 4 at 256
+  static constexpr uint32_t kTmemCols = kBN > 128 ? 512 : 2 * kBN;  // two accumulators, a power of two
+  static constexpr int kSmemBytes = kStages * kStageBytes + kGemmOutBytes + 512 + 1024;  // + barriers + slack
+};
+
+template <int kStages>
 struct GemmBarriers {
-  uint64_t full[kGemmStages];
-  uint64_t empty[kGemmStages];
+  uint64_t full[kStages];   // used in the leader
+  uint64_t empty[kStages];
   uint64_t tmem_full[2];
-  uint64_t tmem_empty[2];
+  uint64_t tmem_empty[2];   // used in the leader
   uint64_t teardown;
   uint32_t tmem_base;
   uint32_t abort_flag;
 };
 
-// The i-th tile of this CTA; false once the CTA has run out of tiles.
+// The i-th tile of a pair (or of a CTA of its own); false once it has run out of tiles.  `first` / `last`:
+// the tile begins / ends the pair's run through this row block.
+struct GemmTile {
+  int mb, nt;
+  bool first, last;
+};
 template <bool kRoundRobinTiles>
-__device__ __forceinline__ bool gemm_tile_at(int i, int num_m_blocks, int num_n_tiles, int& mb, int& nt) {
+__device__ __forceinline__ bool gemm_tile_at(int i, int pair, int pairs, int num_m_blocks, int num_n_tiles, GemmTile& tile) {
   if constexpr (kRoundRobinTiles) {
-    const long long t = (long long)blockIdx.x + (long long)i * gridDim.x;
+    const long long t = (long long)pair + (long long)i * pairs;
     if (t >= (long long)num_m_blocks * num_n_tiles) return false;
-    mb = (int)(t / num_n_tiles);
-    nt = (int)(t % num_n_tiles);
+    tile.mb = (int)(t / num_n_tiles);
+    tile.nt = (int)(t % num_n_tiles);
     return true;
   } else {
-    const long long b = (long long)blockIdx.x + (long long)(i / num_n_tiles) * gridDim.x;
-    if (b >= num_m_blocks) return false;
-    mb = (int)b;
-    nt = i % num_n_tiles;
+    const int full = num_m_blocks / pairs;  // sweeps with a row block for every pair
+    if (i < full * num_n_tiles) {
+      tile.mb = pair + i / num_n_tiles * pairs;
+      tile.nt = i % num_n_tiles;
+      tile.first = tile.nt == 0;
+      tile.last = tile.nt == num_n_tiles - 1;
+      return true;
+    }
+    const long long rest = (long long)(num_m_blocks - full * pairs) * num_n_tiles;
+    const long long lo = rest * pair / pairs, hi = rest * (pair + 1) / pairs;
+    const long long t = lo + (i - full * num_n_tiles);
+    if (t >= hi) return false;
+    tile.mb = full * pairs + (int)(t / num_n_tiles);
+    tile.nt = (int)(t % num_n_tiles);
+    tile.first = tile.nt == 0 || t == lo;
+    tile.last = tile.nt == num_n_tiles - 1 || t == hi - 1;
     return true;
   }
 }
 
-template <class Epi>
+template <class Epi, int kBN, int kCtas>
 __global__ void __launch_bounds__(kGemmMaxThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                const __grid_constant__ CUtensorMap tmap_out, int m_rows, int n_cols, int k_dim, Epi epi,
                uint32_t* status) {
+  using Shape = GemmShape<kBN, kCtas>;
+  constexpr int kStages = Shape::kStages;
+  constexpr bool kPair = kCtas == 2;
+  static_assert(kPair || Epi::kTileOut, "the row-state epilogue runs on pairs");
   extern __shared__ uint8_t smem_raw[];
+  // the same offset in both CTAs of a pair: the leader's descriptors address the other CTA's tiles too
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* smem_a = smem;
-  uint8_t* smem_b = smem + kGemmStages * kGemmTileABytes;
-  uint8_t* smem_out = smem + kGemmStages * kGemmStageBytes;
-  GemmBarriers* bars = reinterpret_cast<GemmBarriers*>(smem_out + kGemmOutBytes);
+  uint8_t* smem_b = smem + kStages * kGemmTileABytes;
+  uint8_t* smem_out = smem + kStages * Shape::kStageBytes;
+  GemmBarriers<kStages>* bars = reinterpret_cast<GemmBarriers<kStages>*>(smem_out + kGemmOutBytes);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int num_m_blocks = (m_rows + kGemmBM - 1) / kGemmBM;
-  const int num_n_tiles = (n_cols + kGemmBN - 1) / kGemmBN;
+  const uint32_t rank = kPair ? cluster_ctarank() : 0u;
+  const bool leader = rank == 0;
+  const int pair = blockIdx.x / kCtas, pairs = gridDim.x / kCtas;
+  const int num_m_blocks = (m_rows + kCtas * kGemmBM - 1) / (kCtas * kGemmBM);
+  const int num_n_tiles = (n_cols + kBN - 1) / kBN;
   const int num_kb = k_dim / kGemmBK;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kGemmStages; ++s) {
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(&bars->full[s], 1);
       mbar_init(&bars->empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&bars->tmem_full[b], 1);
-      mbar_init(&bars->tmem_empty[b], Epi::kTileOut ? 8 : 4);
+      mbar_init(&bars->tmem_empty[b], (Epi::kTileOut ? 8 : 4) * kCtas);  // the epilogue warps of both CTAs
     }
     mbar_init(&bars->teardown, 1);
     bars->abort_flag = 0;
@@ -115,11 +161,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     if constexpr (Epi::kTileOut) tma_prefetch_desc(&tmap_out);
   }
   if (warp == 1) {
-    tmem_alloc(&bars->tmem_base, 512);
-    tmem_relinquish();
+    if constexpr (kPair) {
+      tmem_alloc_pair(&bars->tmem_base, Shape::kTmemCols);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(&bars->tmem_base, Shape::kTmemCols);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
-  __syncthreads();
+  if constexpr (kPair) cluster_sync(); else __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = bars->tmem_base;
   const WaitCtl ctl{&bars->abort_flag, status};
@@ -131,63 +182,82 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       uint32_t phase = 0;
       uint32_t issued = 0;
       bool ok = true;
-      int mb, nt;
-      for (int i = 0; ok && gemm_tile_at<Epi::kTileOut>(i, num_m_blocks, num_n_tiles, mb, nt); ++i) {
+      GemmTile tile;
+      for (int i = 0; ok && gemm_tile_at<Epi::kTileOut>(i, pair, pairs, num_m_blocks, num_n_tiles, tile); ++i) {
+        const int row = (kCtas * tile.mb + (int)rank) * kGemmBM, col = tile.nt * kBN + (int)rank * (kBN / kCtas);
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!mbar_wait(&bars->empty[stage], phase ^ 1u, ctl)) { ok = false; break; }
-          mbar_expect_tx(&bars->full[stage], kGemmStageBytes);
-          tma_load_2d(smem_a + stage * kGemmTileABytes, &tmap_a, &bars->full[stage], kb * kGemmBK, mb * kGemmBM);
-          tma_load_2d(smem_b + stage * kGemmTileBBytes, &tmap_b, &bars->full[stage], kb * kGemmBK, nt * kGemmBN);
+          if (leader) mbar_expect_tx(&bars->full[stage], kCtas * Shape::kStageBytes);
+          uint8_t* dst_a = smem_a + stage * kGemmTileABytes;
+          uint8_t* dst_b = smem_b + stage * Shape::kTileBBytes;
+          if constexpr (kPair) {
+            const uint32_t full = mapa_u32(smem_u32(&bars->full[stage]), 0);
+            tma_load_2d_pair(dst_a, &tmap_a, full, kb * kGemmBK, row);
+            tma_load_2d_pair(dst_b, &tmap_b, full, kb * kGemmBK, col);
+          } else {
+            tma_load_2d(dst_a, &tmap_a, &bars->full[stage], kb * kGemmBK, row);
+            tma_load_2d(dst_b, &tmap_b, &bars->full[stage], kb * kGemmBK, col);
+          }
           ++issued;
-          if (++stage == kGemmStages) { stage = 0; phase ^= 1u; }
+          if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
       }
-      // Drain: every load this thread issued must have landed before the CTA may exit.
-      const uint32_t n_drain = issued < (uint32_t)kGemmStages ? issued : (uint32_t)kGemmStages;
+      // Drain: every load this thread issued must have landed and been consumed (and the commit that says
+      // so have arrived here) before the CTA may exit; a pair that gave up still waits for its loads.
+      const uint32_t n_drain = issued < (uint32_t)kStages ? issued : (uint32_t)kStages;
       for (uint32_t i = 0; i < n_drain; ++i) {
         // walk back over the most recently used stages
         int s = stage - 1 - (int)i;
         uint32_t ph = phase;
-        while (s < 0) { s += kGemmStages; ph ^= 1u; }
+        while (s < 0) { s += kStages; ph ^= 1u; }
         const long long t0 = clock64();
-        while (!mbar_try_wait(&bars->full[s], ph)) {
+        while (!mbar_try_wait(&bars->empty[s], ph)) {
+          // (the other CTA's barrier counts this one's bytes: without it, give them a million cycles)
+          if (*ctl.abort_flag != 0u && (leader ? mbar_try_wait(&bars->full[s], ph) : clock64() - t0 > (1ll << 20))) break;
           if (clock64() - t0 > kTimeoutCycles) { atomicOr(status, kStatusTimeout); break; }
         }
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (elect_one()) {
-      constexpr uint32_t idesc = umma_idesc_bf16(kGemmBM, kGemmBN, false, false);
+    if (leader && elect_one()) {
+      constexpr uint32_t idesc = umma_idesc_bf16(kCtas * kGemmBM, kBN, false, false);
+      auto commit = [](uint64_t* bar, uint16_t ctas) {
+        if constexpr (kPair) umma_commit_pair(bar, ctas); else umma_commit(bar);
+      };
+      const uint64_t a_desc0 = smem_desc_sw128(smem_u32(smem_a), 16, 1024);
+      const uint64_t b_desc0 = smem_desc_sw128(smem_u32(smem_b), 16, 1024);
       int stage = 0;
       uint32_t phase = 0;
       uint32_t tile_iter = 0;
       bool ok = true;
-      int mb, nt;
-      for (int i = 0; ok && gemm_tile_at<Epi::kTileOut>(i, num_m_blocks, num_n_tiles, mb, nt); ++i, ++tile_iter) {
+      GemmTile tile;
+      for (int i = 0; ok && gemm_tile_at<Epi::kTileOut>(i, pair, pairs, num_m_blocks, num_n_tiles, tile); ++i, ++tile_iter) {
         const uint32_t ab = tile_iter & 1u;
         const uint32_t ab_phase = (tile_iter >> 1) & 1u;
         if (!mbar_wait(&bars->tmem_empty[ab], ab_phase ^ 1u, ctl)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + ab * kGemmBN;
+        const uint32_t d_tmem = tmem_base + ab * kBN;
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!mbar_wait(&bars->full[stage], phase, ctl)) { ok = false; break; }
           tc_fence_after();
-          const uint64_t a_desc = smem_desc_sw128(smem_u32(smem_a + stage * kGemmTileABytes), 16, 1024);
-          const uint64_t b_desc = smem_desc_sw128(smem_u32(smem_b + stage * kGemmTileBBytes), 16, 1024);
+          // the descriptors are linear in the shared-memory address (16-byte units in the low bits)
+          const uint64_t a_desc = a_desc0 + (uint64_t)(stage * (kGemmTileABytes >> 4));
+          const uint64_t b_desc = b_desc0 + (uint64_t)(stage * (Shape::kTileBBytes >> 4));
 #pragma unroll
           for (int k = 0; k < kGemmBK / 16; ++k) {
             // +32 bytes along K inside the swizzled row = +2 in descriptor units
-            umma_ss(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
+            if constexpr (kPair) umma_ss_pair(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
+            else umma_ss(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
           }
-          umma_commit(&bars->empty[stage]);
-          if (++stage == kGemmStages) { stage = 0; phase ^= 1u; }
+          commit(&bars->empty[stage], 3);
+          if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
-        if (ok) umma_commit(&bars->tmem_full[ab]);
+        if (ok) commit(&bars->tmem_full[ab], 3);
       }
       if (!ok) {
         // make sure no MMA is still in flight before tensor memory is released
-        umma_commit(&bars->teardown);
+        commit(&bars->teardown, 1);
         const long long t0 = clock64();
         while (!mbar_try_wait(&bars->teardown, 0)) {
           if (clock64() - t0 > kTimeoutCycles) break;
@@ -197,26 +267,29 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   } else {
     // ------------------------------------------------------------------ epilogue warps
     const uint32_t quarter = warp & 3u;  // TMEM lanes 32*quarter .. 32*quarter+31
-    const uint32_t half = (uint32_t)(warp - 2) >> 2;  // which 128 columns (matrix epilogue only)
+    const int half = (warp - 2) >> 2;    // even or odd 64-column chunks (matrix epilogue only)
     const int row_in_tile = quarter * 32 + lane;
     uint32_t tile_iter = 0;
     uint32_t chunk_iter = 0;
     typename Epi::State st;
-    int mb, nt;
-    for (int i = 0; gemm_tile_at<Epi::kTileOut>(i, num_m_blocks, num_n_tiles, mb, nt); ++i, ++tile_iter) {
-      const int row = mb * kGemmBM + row_in_tile;
-      if (nt == 0) epi.begin(st, row);
+    GemmTile tile;
+    for (int i = 0; gemm_tile_at<Epi::kTileOut>(i, pair, pairs, num_m_blocks, num_n_tiles, tile); ++i, ++tile_iter) {
+      const int row0 = (kCtas * tile.mb + (int)rank) * kGemmBM;
+      const int row = row0 + row_in_tile;
+      if constexpr (!Epi::kTileOut) {
+        if (tile.first) epi.begin(st, row);
+      }
       const uint32_t ab = tile_iter & 1u;
       const uint32_t ab_phase = (tile_iter >> 1) & 1u;
       if (!mbar_wait_warp(&bars->tmem_full[ab], ab_phase, ctl)) break;
       tc_fence_after();
-      const uint32_t t_addr = tmem_base + ((quarter * 32u) << 16) + ab * kGemmBN;
+      const uint32_t t_addr = tmem_base + ((quarter * 32u) << 16) + ab * kBN;
       if constexpr (Epi::kTileOut) {
-        const int warp_row0 = mb * kGemmBM + (int)quarter * 32;
+        const int warp_row0 = row0 + (int)quarter * 32;
         uint8_t* block = smem_out + (warp - 2) * kGemmOutBlockBytes;
 #pragma unroll 1
-        for (int c = (int)half * 2; c < (int)half * 2 + 2; ++c) {
-          const int col0 = nt * kGemmBN + c * kGemmOutChunkCols;
+        for (int c = half; c < kBN / kGemmOutChunkCols; c += 2) {
+          const int col0 = tile.nt * kBN + c * kGemmOutChunkCols;
           if (col0 >= n_cols || warp_row0 >= m_rows) break;  // nothing of this block exists (warp-uniform)
           uint32_t acc[64];
           tmem_ld32(t_addr + c * 64, reinterpret_cast<uint32_t(&)[32]>(acc[0]));
@@ -246,17 +319,22 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         }
       } else {
 #pragma unroll 1
-        for (int c = 0; c < kGemmBN / 32; ++c) {
+        for (int c = 0; c < kBN / 32; ++c) {
           uint32_t acc[32];
           tmem_ld32(t_addr + c * 32, acc);
           tmem_ld_wait();
-          epi.consume(st, row, nt * kGemmBN + c * 32, acc);
+          epi.consume(st, row, tile.nt * kBN + c * 32, acc);
         }
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->tmem_empty[ab]);
-      if (nt == num_n_tiles - 1) epi.finish(st, row);
+      if (lane == 0) {
+        if constexpr (kPair) mbar_arrive_cluster(mapa_u32(smem_u32(&bars->tmem_empty[ab]), 0));
+        else mbar_arrive(&bars->tmem_empty[ab]);
+      }
+      if constexpr (!Epi::kTileOut) {
+        if (tile.last) epi.finish(st, row);
+      }
     }
     // Shared memory must outlive every store that still reads it.
     if constexpr (Epi::kTileOut) {
@@ -264,12 +342,48 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     }
   }
 
+  // neither CTA may exit while the other can still arrive on its barriers or its tiles are being read
+  __syncwarp();
   tc_fence_before();
-  __syncthreads();
+  if constexpr (kPair) cluster_sync(); else __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, 512);
+    if constexpr (kPair) tmem_dealloc_pair(tmem_base, Shape::kTmemCols); else tmem_dealloc(tmem_base, Shape::kTmemCols);
   }
+}
+
+// One launch of the mainloop on at most one CTA per SM; `work` bounds the pairs (or CTAs) that find something
+// to do.
+template <class Epi, int kBN, int kCtas>
+cudaError_t gemm_launch(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& out, long long m, long long n,
+                        long long k, const Epi& epi, long long work, int num_sms, uint32_t* status, cudaStream_t s) {
+  using Shape = GemmShape<kBN, kCtas>;
+  static std::atomic<unsigned long long> smem_set{0};
+  cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(gemm_tc_kernel<Epi, kBN, kCtas>), Shape::kSmemBytes,
+                                            smem_set);
+  if (e != cudaSuccess) return e;
+  const long long groups = work < num_sms / kCtas ? work : num_sms / kCtas;
+  cudaLaunchAttribute cluster;
+  cluster.id = cudaLaunchAttributeClusterDimension;
+  cluster.val.clusterDim.x = kCtas;
+  cluster.val.clusterDim.y = 1;
+  cluster.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(kCtas * groups));
+  cfg.blockDim = dim3(gemm_threads<Epi>());
+  cfg.dynamicSmemBytes = Shape::kSmemBytes;
+  cfg.stream = s;
+  cfg.attrs = &cluster;
+  cfg.numAttrs = kCtas > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<Epi, kBN, kCtas>, a, b, out, (int)m, (int)n, (int)k, epi, status);
+}
+
+// What a launch costs, in units of what one column of a tile costs per k-block, times k: every wave pays
+// about 150 columns' worth for the 128 rows of A that each CTA loads, a pair about 90 x 1024 once
+// for its cluster-wide hand-overs.  (us at k = 1024, one wave / every further one: a pair at 256 columns 11.3 /
+// 5.3, 192: 9.8 / 4.6, 128: 8.0 / 3.75, 64: 7.6 / 2.8; one CTA at 256 columns 10.6 / 6.2.)
+inline long long gemm_cost(long long waves, int bn, long long k, bool pair) {
+  return pair ? waves * (150 + bn) * k + 90 * 1024 : waves * (184 + bn) * k;
 }
 
 // ----------------------------------------------------------------------------------------
@@ -296,8 +410,6 @@ struct LinearEpilogue {
   int seq_len;
   float* stat;
 
-  __device__ __forceinline__ void begin(State&, int) const {}
-  __device__ __forceinline__ void finish(State&, int) const {}
   // 64 accumulator columns of one row -> 32 bf16 pairs
   __device__ __forceinline__ void transform(int row, int col0, const uint32_t (&acc)[64], uint32_t (&packed)[32]) const {
     convert(col0, acc, packed);
@@ -381,8 +493,6 @@ struct MlpEpilogue {
   long long ld_res;
   int gelu;
 
-  __device__ __forceinline__ void begin(State&, int) const {}
-  __device__ __forceinline__ void finish(State&, int) const {}
   __device__ __forceinline__ void transform(int row, int col0, const uint32_t (&acc)[64],
                                             uint32_t (&packed)[32]) const {
     const bool has_res = residual != nullptr && row < m_rows;
@@ -421,21 +531,26 @@ struct MlpEpilogue {
   }
 };
 
-// Epilogue: running argmax over columns of acc[row, col] * inv_norm_b[col]; at the end
-// best_idx[row] = col_ids[argmax], best_val[row] = max * inv_norm_a[row].
-// Columns are visited in ascending order and only a strictly larger value replaces the
-// current best, so exact ties resolve to the lowest column.
+// Epilogue: running argmax over columns of acc[row, col] * inv_norm_b[col].  What a pair found in its
+// run through a row block's columns goes into key[row] by an atomic maximum: the value's bits in an
+// order-preserving form above the complement of the column, so the largest value wins and of equal
+// ones the lowest column, whatever the runs and their order.  Keys start at zero, below every
+// value.  Within a run columns are visited in ascending order and only a strictly larger value replaces
+// the current best.
+__host__ __device__ __forceinline__ unsigned ordered_bits(unsigned u) {  // monotone float bits -> unsigned
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__host__ __device__ __forceinline__ unsigned unordered_bits(unsigned u) {  // its inverse
+  return (u & 0x80000000u) ? (u & 0x7fffffffu) : ~u;
+}
 struct ArgmaxEpilogue {
   static constexpr bool kTileOut = false;
   struct State {
     float best;
     int best_col;
   };
-  const float* inv_norm_a;  // [m_rows]
   const float* inv_norm_b;  // [n_cols rounded up to 256], padding = 0
-  const int* col_ids;       // [n_cols]
-  int* best_idx;            // [m_rows]
-  float* best_val;          // [m_rows]
+  unsigned long long* key;  // [m_rows]
   int m_rows;
   int n_cols;
 
@@ -464,8 +579,8 @@ struct ArgmaxEpilogue {
   }
   __device__ __forceinline__ void finish(State& st, int row) const {
     if (row >= m_rows) return;
-    best_idx[row] = col_ids[st.best_col];
-    best_val[row] = st.best * inv_norm_a[row];
+    const float v = st.best + 0.0f;  // -0 and +0 are the same value
+    atomicMax(&key[row], (unsigned long long)ordered_bits(__float_as_uint(v)) << 32 | (unsigned)~st.best_col);
   }
 };
 

@@ -159,7 +159,7 @@ static cudaError_t exclusive_scan(const int* in, int* out, int* block_sums, long
 }
 
 // ------------------------------------------------------------------------------ element-wise steps
-__device__ __forceinline__ unsigned ordered_bits(float f) {  // monotone float -> unsigned
+__device__ __forceinline__ unsigned sim_bits(float f) {  // monotone float -> unsigned
   const unsigned u = __float_as_uint(f);
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
@@ -169,7 +169,7 @@ __global__ void make_sim_keys_kernel(const float* __restrict__ best_sim, unsigne
                                      long long n_src, long long cap) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= cap) return;
-  keys[i] = i < n_src ? ((unsigned long long)(~ordered_bits(best_sim[i])) << 32) | (unsigned)i : ~0ull;
+  keys[i] = i < n_src ? ((unsigned long long)(~sim_bits(best_sim[i])) << 32) | (unsigned)i : ~0ull;
 }
 
 __global__ void fill_int_kernel(int* __restrict__ p, int v, long long n) {

@@ -7,6 +7,50 @@
 
 namespace lv {
 
+// Columns of a pair's tile, or 0: CTAs of their own, 256 columns.  Narrower tiles win where wider ones
+// would leave pairs idle in the only or the last wave, CTAs of their own where 128 rows a block save a wave,
+// and below k = 512 (104,100 rows x 128 x 320: 36 us, a pair 50).
+static int tile_columns(long long m, long long n, long long k, int num_sms) {
+  if (k < 512) return 0;
+  auto waves = [&](int rows, int bn, int groups) {
+    return (((m + rows - 1) / rows) * ((n + bn - 1) / bn) + groups - 1) / groups;
+  };
+  int best = 0;
+  long long best_cost = gemm_cost(waves(kGemmBM, 256, num_sms), 256, k, false);
+  for (int bn = 256; bn >= 64; bn -= 64) {
+    const long long cost = gemm_cost(waves(2 * kGemmBM, bn, num_sms / 2), bn, k, true);
+    if (cost < best_cost) {
+      best = bn;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
+// out [m, n] = epi(a [m, k] w [n, k]^T)
+template <class Epi>
+static cudaError_t launch_gemm_out(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k,
+                                   const __nv_bfloat16* w, long long n, __nv_bfloat16* out, const Epi& epi, cudaStream_t s,
+                                   int* launches) {
+  const int columns = tile_columns(m, n, k, ctx->num_sms), bn = columns != 0 ? columns : 256;
+  CUtensorMap tmap_a, tmap_b, tmap_out;
+  if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap_a, a, (uint64_t)k, (uint64_t)m, (uint64_t)k, kGemmBK, kGemmBM) ||
+      !make_tmap_bf16_2d(ctx->encode_tiled, &tmap_b, w, (uint64_t)k, (uint64_t)n, (uint64_t)k, kGemmBK, columns != 0 ? bn / 2 : bn) ||
+      !make_tmap_bf16_2d(ctx->encode_tiled, &tmap_out, out, (uint64_t)n, (uint64_t)m, (uint64_t)n, kGemmOutChunkCols,
+                         32))
+    return cudaErrorInvalidValue;
+  const long long rows = columns != 0 ? 2 * kGemmBM : kGemmBM, tiles = ((m + rows - 1) / rows) * ((n + bn - 1) / bn);
+  ++*launches;
+  auto run = [&](auto launch) { return launch(tmap_a, tmap_b, tmap_out, m, n, k, epi, tiles, ctx->num_sms, ctx->ws.status, s); };
+  switch (columns) {
+    case 0: return run(gemm_launch<Epi, 256, 1>);
+    case 64: return run(gemm_launch<Epi, 64, 2>);
+    case 128: return run(gemm_launch<Epi, 128, 2>);
+    case 192: return run(gemm_launch<Epi, 192, 2>);
+    default: return run(gemm_launch<Epi, 256, 2>);
+  }
+}
+
 cudaError_t launch_linear(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k, const __nv_bfloat16* w,
                           long long n, const __nv_bfloat16* bias, __nv_bfloat16* out, cudaStream_t s, int* launches) {
   return launch_linear_scaled(ctx, a, m, k, w, n, bias, 0, 0, 1.0f, LinearStat{}, out, s, launches);
@@ -25,12 +69,6 @@ cudaError_t launch_linear_scaled(litevggt_ctx* ctx, const __nv_bfloat16* a, long
     cudaError_t e = cudaMemsetAsync(stat.key_norm != nullptr ? stat.key_norm : stat.amax, 0, words * sizeof(float), s);
     if (e != cudaSuccess) return e;
   }
-  CUtensorMap tmap_a, tmap_b, tmap_out;
-  if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap_a, a, (uint64_t)k, (uint64_t)m, (uint64_t)k, kGemmBK, kGemmBM) ||
-      !make_tmap_bf16_2d(ctx->encode_tiled, &tmap_b, w, (uint64_t)k, (uint64_t)n, (uint64_t)k, kGemmBK, kGemmBN) ||
-      !make_tmap_bf16_2d(ctx->encode_tiled, &tmap_out, out, (uint64_t)n, (uint64_t)m, (uint64_t)n, kGemmOutChunkCols,
-                         32))
-    return cudaErrorInvalidValue;
   LinearEpilogue epi;
   epi.bias = bias;
   epi.m_rows = (int)m;
@@ -41,16 +79,7 @@ cudaError_t launch_linear_scaled(litevggt_ctx* ctx, const __nv_bfloat16* a, long
   epi.stat_kind = stat.key_norm != nullptr ? kStatKeyNorm : stat.amax != nullptr ? kStatAmax : kStatNone;
   epi.seq_len = (int)stat.seq_len;
   epi.stat = stat.key_norm != nullptr ? stat.key_norm : stat.amax;
-  static std::atomic<unsigned long long> smem_set{0};
-  cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(gemm_tc_kernel<LinearEpilogue>), kGemmSmemBytes,
-                                            smem_set);
-  if (e != cudaSuccess) return e;
-  const long long tiles = ((m + kGemmBM - 1) / kGemmBM) * ((n + kGemmBN - 1) / kGemmBN);
-  const int grid = tiles < ctx->num_sms ? (int)tiles : ctx->num_sms;
-  gemm_tc_kernel<LinearEpilogue><<<grid, gemm_threads<LinearEpilogue>(), kGemmSmemBytes, s>>>(tmap_a, tmap_b, tmap_out, (int)m, (int)n,
-                                                                            (int)k, epi, ctx->ws.status);
-  ++*launches;
-  return cudaGetLastError();
+  return launch_gemm_out(ctx, a, m, k, w, n, out, epi, s, launches);
 }
 
 // out = act(a w^T + bias) + residual, the two layers of the transformer MLP (fc1: GELU, no residual;
@@ -59,12 +88,6 @@ cudaError_t launch_linear_mlp(litevggt_ctx* ctx, const __nv_bfloat16* a, long lo
                               const __nv_bfloat16* w, long long n, const __nv_bfloat16* bias, int gelu,
                               const __nv_bfloat16* residual, __nv_bfloat16* out, cudaStream_t s, int* launches) {
   if (m == 0) return cudaSuccess;
-  CUtensorMap tmap_a, tmap_b, tmap_out;
-  if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap_a, a, (uint64_t)k, (uint64_t)m, (uint64_t)k, kGemmBK, kGemmBM) ||
-      !make_tmap_bf16_2d(ctx->encode_tiled, &tmap_b, w, (uint64_t)k, (uint64_t)n, (uint64_t)k, kGemmBK, kGemmBN) ||
-      !make_tmap_bf16_2d(ctx->encode_tiled, &tmap_out, out, (uint64_t)n, (uint64_t)m, (uint64_t)n, kGemmOutChunkCols,
-                         32))
-    return cudaErrorInvalidValue;
   MlpEpilogue epi;
   epi.bias = bias;
   epi.residual = residual;
@@ -72,16 +95,7 @@ cudaError_t launch_linear_mlp(litevggt_ctx* ctx, const __nv_bfloat16* a, long lo
   epi.n_cols = (int)n;
   epi.ld_res = n;
   epi.gelu = gelu;
-  static std::atomic<unsigned long long> smem_set{0};
-  cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(gemm_tc_kernel<MlpEpilogue>), kGemmSmemBytes,
-                                            smem_set);
-  if (e != cudaSuccess) return e;
-  const long long tiles = ((m + kGemmBM - 1) / kGemmBM) * ((n + kGemmBN - 1) / kGemmBN);
-  const int grid = tiles < ctx->num_sms ? (int)tiles : ctx->num_sms;
-  gemm_tc_kernel<MlpEpilogue><<<grid, gemm_threads<MlpEpilogue>(), kGemmSmemBytes, s>>>(tmap_a, tmap_b, tmap_out, (int)m, (int)n,
-                                                                         (int)k, epi, ctx->ws.status);
-  ++*launches;
-  return cudaGetLastError();
+  return launch_gemm_out(ctx, a, m, k, w, n, out, epi, s, launches);
 }
 
 }  // namespace lv

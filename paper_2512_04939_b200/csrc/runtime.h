@@ -63,6 +63,7 @@ struct Workspace {
   __nv_bfloat16* panel_dst = nullptr;  // [|Dst|, D]
   float* inv_norm_src = nullptr;       // [|Src|]
   float* inv_norm_dst = nullptr;       // [round_up(|Dst|,256)]
+  unsigned long long* match_keys = nullptr;  // [|Src|] best (cosine, anchor) so far, as one ordered word
   // index build
   unsigned long long* sort_keys = nullptr;  // [pow2 >= max(|Src|, R)]
   int* scan_tmp = nullptr;                  // [N] kept flags / scan output

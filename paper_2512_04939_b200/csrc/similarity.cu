@@ -20,7 +20,8 @@ __global__ void __launch_bounds__(kPackThreads)
 pack_rows_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ src_list,
                  const int* __restrict__ dst_list, long long n_src, long long n_dst, long long n_dst_padded,
                  long long n_tokens, __nv_bfloat16* __restrict__ panel_src, __nv_bfloat16* __restrict__ panel_dst,
-                 float* __restrict__ inv_norm_src, float* __restrict__ inv_norm_dst, uint32_t* status) {
+                 float* __restrict__ inv_norm_src, float* __restrict__ inv_norm_dst, unsigned long long* __restrict__ key,
+                 uint32_t* status) {
   const int lane = threadIdx.x & 31;
   const long long row = (long long)blockIdx.x * (kPackThreads / 32) + (threadIdx.x >> 5);
   if (row >= n_src + n_dst_padded) return;
@@ -55,7 +56,24 @@ pack_rows_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ sr
   if (lane == 0) {
     const float inv = 1.0f / fmaxf(sqrtf(ss), 1e-12f);
     (is_src ? inv_norm_src : inv_norm_dst)[r] = inv;
+    if (is_src) key[r] = 0ull;  // below the key of every value
   }
+}
+
+// keys of the argmax -> anchor token and cosine of every src row
+__global__ void unpack_matches_kernel(const unsigned long long* __restrict__ key, const int* __restrict__ dst_list,
+                                      const float* __restrict__ inv_norm_src, int* __restrict__ best_dst,
+                                      float* __restrict__ best_sim, long long n_src, long long n_dst, uint32_t* status) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n_src) return;
+  const unsigned long long k = key[i];
+  unsigned col = ~(unsigned)k;
+  if (col >= n_dst) {
+    atomicOr(status, kStatusBounds);
+    col = 0;
+  }
+  best_dst[i] = dst_list[col];
+  best_sim[i] = __uint_as_float(unordered_bits((unsigned)(k >> 32))) * inv_norm_src[i];
 }
 
 cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, int* best_dst, float* best_sim, cudaStream_t s,
@@ -68,31 +86,40 @@ cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, int* best_ds
   const int warps = kPackThreads / 32;
   pack_rows_kernel<<<(unsigned)((rows + warps - 1) / warps), kPackThreads, 0, s>>>(
       x, ws.src_list, ws.dst_list, z.n_src, z.n_dst, n_dst_padded, z.n_tokens, ws.panel_src, ws.panel_dst,
-      ws.inv_norm_src, ws.inv_norm_dst, ws.status);
+      ws.inv_norm_src, ws.inv_norm_dst, ws.match_keys, ws.status);
   ++*launches;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
 
+  // columns of a tile: 256, unless narrower ones spread few rows over more of the chip
+  const long long row_blocks = (z.n_src + 2 * kGemmBM - 1) / (2 * kGemmBM), pairs = ctx->num_sms / 2;
+  int bn = 256;
+  for (int c = 128; c >= 64; c -= 64) {
+    auto cost = [&](int cols) {
+      return gemm_cost((row_blocks * ((z.n_dst + cols - 1) / cols) + pairs - 1) / pairs, cols, 1024, true);
+    };
+    if (cost(c) < cost(bn)) bn = c;
+  }
   CUtensorMap tmap_a, tmap_b;
   if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap_a, ws.panel_src, 1024, (uint64_t)z.n_src, 1024, kGemmBK, kGemmBM) ||
-      !make_tmap_bf16_2d(ctx->encode_tiled, &tmap_b, ws.panel_dst, 1024, (uint64_t)z.n_dst, 1024, kGemmBK, kGemmBN))
+      !make_tmap_bf16_2d(ctx->encode_tiled, &tmap_b, ws.panel_dst, 1024, (uint64_t)z.n_dst, 1024, kGemmBK, bn / 2))
     return cudaErrorInvalidValue;
   ArgmaxEpilogue epi;
-  epi.inv_norm_a = ws.inv_norm_src;
   epi.inv_norm_b = ws.inv_norm_dst;
-  epi.col_ids = ws.dst_list;
-  epi.best_idx = best_dst;
-  epi.best_val = best_sim;
+  epi.key = ws.match_keys;
   epi.m_rows = (int)z.n_src;
   epi.n_cols = (int)z.n_dst;
-  static std::atomic<unsigned long long> smem_set{0};
-  e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(gemm_tc_kernel<ArgmaxEpilogue>), kGemmSmemBytes, smem_set);
-  if (e != cudaSuccess) return e;
-  const int m_blocks = (int)((z.n_src + kGemmBM - 1) / kGemmBM);
-  const int grid = m_blocks < ctx->num_sms ? m_blocks : ctx->num_sms;
+  const long long tiles = row_blocks * ((z.n_dst + bn - 1) / bn);
   // the argmax epilogue writes no matrix: the store map is never read, any valid map fills the slot
-  gemm_tc_kernel<ArgmaxEpilogue><<<grid, gemm_threads<ArgmaxEpilogue>(), kGemmSmemBytes, s>>>(tmap_a, tmap_b, tmap_a, (int)z.n_src,
-                                                                            (int)z.n_dst, 1024, epi, ws.status);
+  auto run = [&](auto launch) {
+    return launch(tmap_a, tmap_b, tmap_a, z.n_src, z.n_dst, 1024, epi, tiles, ctx->num_sms, ws.status, s);
+  };
+  e = bn == 256 ? run(gemm_launch<ArgmaxEpilogue, 256, 2>)
+                : bn == 128 ? run(gemm_launch<ArgmaxEpilogue, 128, 2>) : run(gemm_launch<ArgmaxEpilogue, 64, 2>);
+  ++*launches;
+  if (e != cudaSuccess) return e;
+  unpack_matches_kernel<<<(unsigned)((z.n_src + 255) / 256), 256, 0, s>>>(ws.match_keys, ws.dst_list, ws.inv_norm_src,
+                                                                         best_dst, best_sim, z.n_src, z.n_dst, ws.status);
   ++*launches;
   return cudaGetLastError();
 }
