@@ -140,11 +140,11 @@ litevggt_status plan_from_classes(litevggt_ctx* ctx, const __nv_bfloat16* x, lit
   cudaError_t e;
   {
     StepTimer t(ctx, 2, s);
-    e = launch_build_lists(ctx, ctx->ws.cls, ctx->ws.src_list, ctx->ws.dst_list, s, &n);
+    e = launch_build_lists(ctx, ctx->ws.cls, ctx->ws.src_list, ctx->ws.dst_list, ctx->ws.src_pos, s, &n);
   }
   if (e == cudaSuccess) {
     StepTimer t(ctx, 3, s);
-    e = launch_match(ctx, x, plan->best_dst, plan->best_sim, s, &n);
+    e = launch_match(ctx, x, s, &n);
   }
   if (e == cudaSuccess) {
     StepTimer t(ctx, 4, s);
@@ -296,14 +296,12 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
   }
   Carver c;
   const long long fp = (long long)z.frames * z.patches;
-  const long long cap = (long long)sort_capacity(z.n_src);
   const size_t o_var = c.take<float>(fp), o_ga = c.take<float>(fp), o_cls = c.take<uint8_t>(z.n_tokens);
   const size_t o_src = c.take<int>(z.n_src), o_dst = c.take<int>(z.n_dst);
   const size_t o_ps = c.take<__nv_bfloat16>(z.n_src * z.dim), o_pd = c.take<__nv_bfloat16>(z.n_dst * z.dim);
   const size_t o_ns = c.take<float>(z.n_src), o_nd = c.take<float>(round_up(z.n_dst, 256));
   const size_t o_match = c.take<unsigned long long>(z.n_src);
-  const size_t o_keys = c.take<unsigned long long>(cap);
-  const size_t o_tmp = c.take<int>(z.n_tokens + 1), o_blk = c.take<int>(2048), o_row = c.take<int>(z.n_tokens);
+  const size_t o_pos = c.take<int>(z.n_tokens), o_idx = c.take<int>(index_scratch_words(z));
   const size_t o_qkv = c.take<__nv_bfloat16>(z.n_merged * 3 * z.dim), o_o = c.take<__nv_bfloat16>(z.n_merged * z.dim);
   size_t ml_off = 0;
   const size_t state_bytes = attention_state_bytes(z.n_merged, z.dim, z.heads, &ml_off);
@@ -331,10 +329,8 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
   ws.inv_norm_src = reinterpret_cast<float*>(ws.base + o_ns);
   ws.inv_norm_dst = reinterpret_cast<float*>(ws.base + o_nd);
   ws.match_keys = reinterpret_cast<unsigned long long*>(ws.base + o_match);
-  ws.sort_keys = reinterpret_cast<unsigned long long*>(ws.base + o_keys);
-  ws.scan_tmp = reinterpret_cast<int*>(ws.base + o_tmp);
-  ws.scan_blocks = reinterpret_cast<int*>(ws.base + o_blk);
-  ws.row_of = reinterpret_cast<int*>(ws.base + o_row);
+  ws.src_pos = reinterpret_cast<int*>(ws.base + o_pos);
+  ws.index_scratch = reinterpret_cast<int*>(ws.base + o_idx);
   ws.qkv = reinterpret_cast<__nv_bfloat16*>(ws.base + o_qkv);
   ws.attn_o = reinterpret_cast<__nv_bfloat16*>(ws.base + o_o);
   if (state_bytes > 0) {

@@ -540,9 +540,6 @@ struct MlpEpilogue {
 __host__ __device__ __forceinline__ unsigned ordered_bits(unsigned u) {  // monotone float bits -> unsigned
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
-__host__ __device__ __forceinline__ unsigned unordered_bits(unsigned u) {  // its inverse
-  return (u & 0x80000000u) ? (u & 0x7fffffffu) : ~u;
-}
 struct ArgmaxEpilogue {
   static constexpr bool kTileOut = false;
   struct State {

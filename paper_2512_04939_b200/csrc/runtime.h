@@ -65,10 +65,8 @@ struct Workspace {
   float* inv_norm_dst = nullptr;       // [round_up(|Dst|,256)]
   unsigned long long* match_keys = nullptr;  // [|Src|] best (cosine, anchor) so far, as one ordered word
   // index build
-  unsigned long long* sort_keys = nullptr;  // [pow2 >= max(|Src|, R)]
-  int* scan_tmp = nullptr;                  // [N] kept flags / scan output
-  int* scan_blocks = nullptr;               // block sums
-  int* row_of = nullptr;                    // [N]
+  int* src_pos = nullptr;        // [N] a token's index in src_list, -1 for tokens of the other classes
+  int* index_scratch = nullptr;  // histograms, counts and the merged tokens on their way (index_build.cu)
   // attention
   __nv_bfloat16* qkv = nullptr;    // [M, 3D]
   __nv_bfloat16* attn_o = nullptr; // [M, D]
@@ -172,16 +170,15 @@ cudaError_t launch_var_map(const litevggt_ctx* ctx, const __nv_bfloat16* x, floa
                            cudaStream_t s, int* launches);
 cudaError_t launch_partition(const litevggt_ctx* ctx, const float* grad, const float* var, float* ga, uint8_t* cls,
                              cudaStream_t s, int* launches);
-cudaError_t launch_build_lists(const litevggt_ctx* ctx, const uint8_t* cls, int* src_list, int* dst_list,
+cudaError_t launch_build_lists(const litevggt_ctx* ctx, const uint8_t* cls, int* src_list, int* dst_list, int* src_pos,
                                cudaStream_t s, int* launches);
 
-// similarity.cu
-cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, int* best_dst, float* best_sim, cudaStream_t s,
-                         int* launches);
+// similarity.cu: leaves every src row's best anchor in ctx->ws.match_keys
+cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, cudaStream_t s, int* launches);
 
 // index_build.cu
 cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStream_t s, int* launches);
-size_t sort_capacity(long long n);
+long long index_scratch_words(const Sizes& z);
 
 // merge_unmerge.cu
 cudaError_t launch_merge(const litevggt_ctx* ctx, const litevggt_plan* plan, const __nv_bfloat16* x,

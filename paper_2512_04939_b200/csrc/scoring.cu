@@ -449,6 +449,12 @@ __device__ __forceinline__ float block_reduce_minmax(float v, bool is_max, float
   return r;
 }
 
+// Scores as unsigned words of the same order; -0 and +0 are the same score.
+__device__ __forceinline__ unsigned score_key(float v) {
+  const unsigned u = __float_as_uint(v + 0.0f);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
 __global__ void __launch_bounds__(kPartThreads)
 partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, float* __restrict__ ga,
                  uint8_t* __restrict__ cls, int grid_h, int grid_w, int n_special, int n_ga, int cell_h, int cell_w,
@@ -458,6 +464,7 @@ partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, 
   float* score = part_smem;                                        // [P]
   uint8_t* is_dst = reinterpret_cast<uint8_t*>(score + p_count);   // [P]
   __shared__ float scratch[kPartThreads / 32];
+  __shared__ int hist[256], found_bin, found_need;
   const int f = blockIdx.x;
   const float* g = grad + (size_t)f * p_count;
   const float* v = var + (size_t)f * p_count;
@@ -498,16 +505,81 @@ partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, 
     is_dst[best] = 1;
   }
   __syncthreads();
-  for (int p = threadIdx.x; p < p_count; p += kPartThreads) {
+  // The n_ga highest of the other scores, ties towards the lower index: the threshold is found eight
+  // bits at a time from the highest (a histogram of the scores that share the bits fixed so far), the
+  // scores equal to it are numbered in index order.  (Ranking every patch against every other was 131 of the
+  // 147 us that 200 frames of 28 x 37 took; 9 now.)  A score that is not a number is kept as it is: GA.
+  unsigned prefix = 0u, mask = 0u;
+  int need = n_ga;
+  for (int shift = 24; shift >= 0 && n_ga > 0; shift -= 8) {
+    for (int i = threadIdx.x; i < 256; i += kPartThreads) hist[i] = 0;
+    __syncthreads();
+    for (int p = threadIdx.x; p < p_count; p += kPartThreads)
+      if (!is_dst[p] && score[p] == score[p]) {
+        const unsigned k = score_key(score[p]);
+        if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & 255u], 1);
+      }
+    __syncthreads();
+    if (threadIdx.x < 32) {  // eight bins a lane, from the highest
+      int c[8], sum = 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        c[i] = hist[255 - (threadIdx.x * 8 + i)];
+        sum += c[i];
+      }
+      int incl = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if ((int)threadIdx.x >= o) incl += t;
+      }
+      int above = incl - sum;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if (above < need && above + c[i] >= need) {
+          found_bin = 255 - (threadIdx.x * 8 + i);
+          found_need = need - above;
+        }
+        above += c[i];
+      }
+      if (threadIdx.x == 31 && incl < need) found_bin = -1;  // fewer scores than asked for: all of them
+    }
+    __syncthreads();
+    const int bin = found_bin;
+    if (bin < 0) break;
+    need = found_need;
+    prefix |= (unsigned)bin << shift;
+    mask |= 255u << shift;
+    __syncthreads();
+  }
+  const bool all = n_ga > 0 && mask != 0xffffffffu;  // (only a search that ran out leaves bits open)
+  // a run of patches per thread, so that ties are numbered in index order
+  const int per = (p_count + kPartThreads - 1) / kPartThreads;
+  const int p0 = threadIdx.x * per, p1 = min(p_count, p0 + per);
+  int ties = 0;
+  if (n_ga > 0 && !all)
+    for (int p = p0; p < p1; ++p) ties += !is_dst[p] && score[p] == score[p] && score_key(score[p]) == prefix ? 1 : 0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int incl = ties;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) hist[warp] = incl;
+  __syncthreads();
+  int tie = incl - ties;
+  for (int i = 0; i < warp; ++i) tie += hist[i];
+  for (int p = p0; p < p1; ++p) {
     uint8_t c = LITEVGGT_CLS_DST;
     if (!is_dst[p]) {
       const float sp = score[p];
-      int rank = 0;
-      for (int q = 0; q < p_count; ++q) {
-        const float sq = score[q];
-        rank += (!is_dst[q] && (sq > sp || (sq == sp && q < p))) ? 1 : 0;
+      bool ga_token = n_ga > 0 && (sp != sp || all);
+      if (!ga_token && n_ga > 0) {
+        const unsigned k = score_key(sp);
+        ga_token = k > prefix || (k == prefix && tie++ < need);
       }
-      c = rank < n_ga ? LITEVGGT_CLS_GA : LITEVGGT_CLS_SRC;
+      c = ga_token ? LITEVGGT_CLS_GA : LITEVGGT_CLS_SRC;
     }
     out[p] = c;
   }
@@ -535,7 +607,7 @@ constexpr int kListThreads = 256;
 
 __global__ void __launch_bounds__(kListThreads)
 build_lists_kernel(const uint8_t* __restrict__ cls, int* __restrict__ src_list, int* __restrict__ dst_list,
-                   int p_count, int n_special, int n_src_frame, int n_dst_frame, uint32_t* status) {
+                   int* __restrict__ src_pos, int p_count, int n_special, int n_src_frame, int n_dst_frame, uint32_t* status) {
   __shared__ int warp_src[kListThreads / 32], warp_dst[kListThreads / 32];
   const int f = blockIdx.x;
   const int tokens_frame = p_count + n_special;
@@ -572,23 +644,28 @@ build_lists_kernel(const uint8_t* __restrict__ cls, int* __restrict__ src_list, 
   }
   for (int t = t0; t < t1; ++t) {
     const uint8_t c = cls[token0 + t];
+    int pos = -1;
     if (c == LITEVGGT_CLS_SRC) {
-      if (off_s < exp_src) src_list[src_base + off_s] = token0 + t;
+      if (off_s < exp_src) {
+        src_list[src_base + off_s] = token0 + t;
+        pos = (int)src_base + off_s;
+      }
       ++off_s;
     } else if (c == LITEVGGT_CLS_DST) {
       if (off_d < exp_dst) dst_list[dst_base + off_d] = token0 + t;
       ++off_d;
     }
+    src_pos[token0 + t] = pos;
   }
   // a short frame (flagged above) still gets valid token indices in its unused slots
   for (int i = tot_s + (int)threadIdx.x; i < exp_src; i += kListThreads) src_list[src_base + i] = token0;
   for (int i = tot_d + (int)threadIdx.x; i < exp_dst; i += kListThreads) dst_list[dst_base + i] = token0;
 }
 
-cudaError_t launch_build_lists(const litevggt_ctx* ctx, const uint8_t* cls, int* src_list, int* dst_list,
+cudaError_t launch_build_lists(const litevggt_ctx* ctx, const uint8_t* cls, int* src_list, int* dst_list, int* src_pos,
                                cudaStream_t s, int* launches) {
   const Sizes& z = ctx->sz;
-  build_lists_kernel<<<z.frames, kListThreads, 0, s>>>(cls, src_list, dst_list, z.patches, z.n_special,
+  build_lists_kernel<<<z.frames, kListThreads, 0, s>>>(cls, src_list, dst_list, src_pos, z.patches, z.n_special,
                                                        z.n_src_frame, z.n_dst_frame, ctx->ws.status);
   ++*launches;
   return cudaGetLastError();

@@ -60,24 +60,7 @@ pack_rows_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ sr
   }
 }
 
-// keys of the argmax -> anchor token and cosine of every src row
-__global__ void unpack_matches_kernel(const unsigned long long* __restrict__ key, const int* __restrict__ dst_list,
-                                      const float* __restrict__ inv_norm_src, int* __restrict__ best_dst,
-                                      float* __restrict__ best_sim, long long n_src, long long n_dst, uint32_t* status) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_src) return;
-  const unsigned long long k = key[i];
-  unsigned col = ~(unsigned)k;
-  if (col >= n_dst) {
-    atomicOr(status, kStatusBounds);
-    col = 0;
-  }
-  best_dst[i] = dst_list[col];
-  best_sim[i] = __uint_as_float(unordered_bits((unsigned)(k >> 32))) * inv_norm_src[i];
-}
-
-cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, int* best_dst, float* best_sim, cudaStream_t s,
-                         int* launches) {
+cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, cudaStream_t s, int* launches) {
   const Sizes& z = ctx->sz;
   Workspace& ws = ctx->ws;
   if (z.n_src == 0) return cudaSuccess;
@@ -117,11 +100,7 @@ cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, int* best_ds
   e = bn == 256 ? run(gemm_launch<ArgmaxEpilogue, 256, 2>)
                 : bn == 128 ? run(gemm_launch<ArgmaxEpilogue, 128, 2>) : run(gemm_launch<ArgmaxEpilogue, 64, 2>);
   ++*launches;
-  if (e != cudaSuccess) return e;
-  unpack_matches_kernel<<<(unsigned)((z.n_src + 255) / 256), 256, 0, s>>>(ws.match_keys, ws.dst_list, ws.inv_norm_src,
-                                                                         best_dst, best_sim, z.n_src, z.n_dst, ws.status);
-  ++*launches;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace lv

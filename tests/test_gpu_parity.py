@@ -177,6 +177,55 @@ def test_index_build_bit_exact_given_same_matches(lib, wl):
     ctx.close()
 
 
+@pytest.mark.parametrize("frames,grid,ratio,cell,keep,kind", [
+    (1, (5, 7), 0.5, 2, 0.1, "random"),     # no src token
+    (2, (9, 9), 0.3, 2, 0.6, "random"),     # few src tokens, all of them merged
+    (5, (9, 11), 0.45, 2, 0.1, "tied"),     # every cosine equal to many others
+    (7, (19, 25), 0.45, 2, 0.0, "equal"),   # one anchor takes 1512 tokens: a long segment, single block
+    (6, (35, 39), 0.2, 8, 0.1, "tied"),     # 8,220 tokens: the smallest plan of several launches
+    (9, (37, 37), 0.45, 2, 0.1, "random"),  # three blocks of tokens, two passes of the 148 pairs' column runs
+    (8, (37, 37), 1.0, 16, 0.0, "equal")])  # one segment of 9,583, every src token merged
+def test_partition_and_index_build_on_degenerate_inputs(lib, frames, grid, ratio, cell, keep, kind):
+    """Ties everywhere, segments longer than a block ranks by comparison, everything or nothing merged."""
+    ctx = lib.LiteVGGT(frames, grid[0], grid[1], ratio, cell_h=cell, cell_w=cell, ga_keep_frac=keep)
+    n = ctx.n_tokens
+    g = torch.Generator().manual_seed(n)
+    if kind == "random":
+        x, grad = torch.randn(n, 1024, generator=g), torch.rand(frames, *grid, generator=g)
+    elif kind == "tied":
+        x = torch.randn(13, 1024, generator=g)[torch.randint(0, 13, (n,), generator=g)]
+        grad = torch.randint(0, 3, (frames, *grid), generator=g).float()
+    else:
+        x, grad = torch.ones(n, 1024), torch.zeros(frames, *grid)
+    x = x.to(torch.bfloat16)
+    plan = ctx.merge_plan(x.cuda(), grad.cuda())
+    ctx.merge_plan(x.cuda(), grad.cuda(), plan)  # and once more in place
+    ctx.poll()
+    ex = ctx.plan_export(plan)
+    assert np.array_equal(ex["cls"], O.partition(ex["ga"], ga_keep_frac=keep, cell_h=cell, cell_w=cell))
+    removed = n - ctx.n_merged
+    dst_of, size, kept = O.select_and_index(ex["cls"], ex["best_dst"], ex["best_sim"], removed)
+    assert np.array_equal(ex["dst_of"], dst_of)
+    assert np.array_equal(ex["size"], size)
+    assert np.array_equal(ex["kept_idx"], kept)
+    src, dst = np.flatnonzero(ex["cls"] == O.CLS_SRC), np.flatnonzero(ex["cls"] == O.CLS_DST)
+    if src.size:
+        rows = np.arange(src.size) if src.size < 2048 else np.r_[0:512, src.size - 512:src.size]
+        best, sim, second = O.match(to_f64(x), src, dst, rows=rows)
+        if kind != "random":  # equal rows have equal products: the lowest anchor wins every tie
+            assert np.array_equal(to_f64(x)[ex["best_dst"][rows]], to_f64(x)[best])
+            assert (ex["best_dst"][rows] <= best).all()
+        else:
+            assert np.array_equal(ex["best_dst"][rows][sim - second > 1e-5], best[sim - second > 1e-5])
+    # the segments hold their tokens in ascending order: the mean of a row is summed in that order
+    xm = ctx.merge(plan, x.cuda())
+    ctx.poll()
+    if kind == "equal":
+        assert bool((xm == 1).all())
+    plan.destroy()
+    ctx.close()
+
+
 def test_identity_at_ratio_zero_and_reuse_equals_recompute(lib):
     wl = WORKLOADS["C1"]
     img, tok = _inputs(wl)
