@@ -305,18 +305,18 @@ litevggt_status litevggt_poll_device_status(litevggt_ctx* ctx, void* stream);
 litevggt_status litevggt_selftest_bounded_wait(litevggt_ctx* ctx, int64_t limit_cycles, uint32_t* outcome,
                                                void* stream);
 
-/* Device-time stopwatches.  Each step of the path is bracketed by CUDA events recorded on
- * the launching stream: which = 0 grad map, 1 var map, 2 partition + token lists, 3 cosine
+/* Device-time stopwatches.  The kernels of each step of the path note on the device's clock when the
+ * first of them started and the last one ended: which = 0 grad map, 1 var map, 2 partition + token lists, 3 cosine
  * matching (pack + GEMM/argmax), 4 selection + index build, 5 merge, 6 qkv projection,
  * 7 attention core, 8 output projection, 9 unmerge, 10 LayerNorm, 11 frame-local attention layer,
  * 12 MLP, 13 Q/K normalisation + rotary embedding, 14 E4M3 quantisation of Q/K/V.
  * litevggt_timers_reset forgets all
- * records; litevggt_timer_read synchronises on the recorded events and returns the summed
+ * records; litevggt_timer_read synchronises the device and returns the summed
  * device time (ms) and the number of records (at most 64 are kept per step). */
 litevggt_status litevggt_timers_reset(litevggt_ctx* ctx);
 litevggt_status litevggt_timer_read(litevggt_ctx* ctx, int which, float* total_ms, int32_t* count);
 /* The individual records of one stopwatch, oldest first: up to `capacity` device times (ms) are
- * written to `ms` (host), *count receives how many.  Synchronises on the recorded events. */
+ * written to `ms` (host), *count receives how many.  Synchronises the device. */
 litevggt_status litevggt_timer_samples(litevggt_ctx* ctx, int which, float* ms, int32_t capacity, int32_t* count);
 
 /* Number of kernels this library has launched on behalf of ctx since creation. */

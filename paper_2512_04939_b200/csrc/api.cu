@@ -78,20 +78,17 @@ struct Carver {
 
 void bump(litevggt_ctx* ctx, int n) { ctx->launches += n; }
 
-// Brackets the launches of one step with an event pair on the launching stream.
+// Hands the launches of one step the stopwatch slot that their kernels write.
 struct StepTimer {
   litevggt_ctx* ctx;
-  cudaStream_t s;
-  int which, slot;
-  StepTimer(litevggt_ctx* c, int w, cudaStream_t st) : ctx(c), s(st), which(w), slot(-1) {
-    Timers& t = ctx->timers;
-    if (!t.created) return;
-    slot = t.used[which] % kTimerSlots;
-    cudaEventRecord(t.start[which][slot], s);
+  int which;
+  StepTimer(litevggt_ctx* c, int w) : ctx(c), which(w) {
+    unsigned long long* slot = c->timers.stamps + 2 * (w * kTimerSlots + c->timers.used[w] % kTimerSlots);
+    c->step.start = slot;
+    c->step.stop = slot + 1;
   }
   ~StepTimer() {
-    if (slot < 0) return;
-    cudaEventRecord(ctx->timers.stop[which][slot], s);
+    ctx->step = Stamp{};
     ++ctx->timers.used[which];
   }
 };
@@ -139,15 +136,15 @@ litevggt_status plan_from_classes(litevggt_ctx* ctx, const __nv_bfloat16* x, lit
   int n = 0;
   cudaError_t e;
   {
-    StepTimer t(ctx, 2, s);
+    StepTimer t(ctx, 2);
     e = launch_build_lists(ctx, ctx->ws.cls, ctx->ws.src_list, ctx->ws.dst_list, ctx->ws.src_pos, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 3, s);
+    StepTimer t(ctx, 3);
     e = launch_match(ctx, x, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 4, s);
+    StepTimer t(ctx, 4);
     e = launch_index_build(ctx, plan, s, &n);
   }
   bump(ctx, n);
@@ -289,7 +286,6 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
   ctx->num_sms = prop.multiProcessorCount;
   ctx->launches = 0;
   ctx->encode_tiled = nullptr;
-  ctx->timers.created = false;
   if (!resolve_encode_tiled(&ctx->encode_tiled)) {
     delete ctx;
     return LITEVGGT_ERR_CUDA;
@@ -311,6 +307,7 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
   const long long m_pad = round_up(z.n_merged, 128);
   const size_t o_q8 = c.take<uint8_t>(fp8 ? z.n_merged * z.dim : 0), o_k8 = c.take<uint8_t>(fp8 ? z.n_merged * z.dim : 0);
   const size_t o_v8 = c.take<uint8_t>(fp8 ? m_pad * z.dim : 0), o_amax = c.take<float>(48);
+  const size_t o_stamps = c.take<unsigned long long>(2 * kNumTimers * kTimerSlots);
   const size_t o_status = c.take<uint32_t>(4);
   Workspace& ws = ctx->ws;
   if (cudaMalloc(&ws.base, c.off) != cudaSuccess) {
@@ -344,21 +341,14 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
     ws.v8t = ws.base + o_v8;
     ws.qkv_amax = reinterpret_cast<float*>(ws.base + o_amax);
   }
+  ctx->timers.stamps = reinterpret_cast<unsigned long long*>(ws.base + o_stamps);
   ws.status = reinterpret_cast<uint32_t*>(ws.base + o_status);
   if (cudaMemset(ws.base + o_var, 0, o_src - o_var) != cudaSuccess ||
-      cudaMemset(ws.status, 0, 16) != cudaSuccess) {
+      cudaMemset(ctx->timers.stamps, 0, o_status - o_stamps) != cudaSuccess || cudaMemset(ws.status, 0, 16) != cudaSuccess) {
     (void)cudaGetLastError();
     cudaFree(ws.base);
     delete ctx;
     return LITEVGGT_ERR_CUDA;
-  }
-  Timers& tm = ctx->timers;
-  tm.created = true;
-  for (int w = 0; w < kNumTimers; ++w) {
-    tm.used[w] = 0;
-    for (int i = 0; i < kTimerSlots; ++i)
-      if (cudaEventCreate(&tm.start[w][i]) != cudaSuccess || cudaEventCreate(&tm.stop[w][i]) != cudaSuccess)
-        tm.created = false;
   }
   (void)cudaGetLastError();
   *out = ctx;
@@ -371,41 +361,49 @@ litevggt_status litevggt_timers_reset(litevggt_ctx* ctx) {
   return LITEVGGT_OK;
 }
 
+static litevggt_status read_stamps(litevggt_ctx* ctx, int which, float (&ms)[kTimerSlots], int* kept) {
+  // the ring keeps the latest kTimerSlots records; slot i holds record i, i + kTimerSlots, ...
+  const int used = ctx->timers.used[which];
+  *kept = used < kTimerSlots ? used : kTimerSlots;
+  if (*kept == 0) return LITEVGGT_OK;
+  DeviceGuard g(ctx->device);
+  if (!g.ok) return LITEVGGT_ERR_CUDA;
+  unsigned long long t[kTimerSlots][2];
+  cudaError_t e = cudaDeviceSynchronize();
+  if (e == cudaSuccess)
+    e = cudaMemcpy(t, ctx->timers.stamps + 2 * kTimerSlots * which, sizeof(t), cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) return cuda_status(e);
+  for (int i = 0; i < *kept; ++i) {
+    const unsigned long long* r = t[(used - *kept + i) % kTimerSlots];
+    ms[i] = r[1] > r[0] ? (float)((double)(r[1] - r[0]) * 1e-6) : 0.0f;  // a step without kernels took no time
+  }
+  return LITEVGGT_OK;
+}
+
 litevggt_status litevggt_timer_read(litevggt_ctx* ctx, int which, float* total_ms, int32_t* count) {
   if (!ctx_ok(ctx) || total_ms == nullptr || count == nullptr) return LITEVGGT_ERR_NULL;
   if (which < 0 || which >= kNumTimers) return LITEVGGT_ERR_SHAPE;
-  Timers& tm = ctx->timers;
   *total_ms = 0.0f;
   *count = 0;
-  if (!tm.created) return LITEVGGT_ERR_CUDA;
-  const int n = tm.used[which] < kTimerSlots ? tm.used[which] : kTimerSlots;
-  for (int i = 0; i < n; ++i) {
-    float ms = 0.0f;
-    if (cudaEventSynchronize(tm.stop[which][i]) != cudaSuccess ||
-        cudaEventElapsedTime(&ms, tm.start[which][i], tm.stop[which][i]) != cudaSuccess)
-      return cuda_status(cudaGetLastError());
-    *total_ms += ms;
-  }
-  *count = n;
+  float ms[kTimerSlots];
+  int kept = 0;
+  const litevggt_status st = read_stamps(ctx, which, ms, &kept);
+  if (st != LITEVGGT_OK) return st;
+  for (int i = 0; i < kept; ++i) *total_ms += ms[i];
+  *count = kept;
   return LITEVGGT_OK;
 }
 
 litevggt_status litevggt_timer_samples(litevggt_ctx* ctx, int which, float* ms, int32_t capacity, int32_t* count) {
   if (!ctx_ok(ctx) || ms == nullptr || count == nullptr) return LITEVGGT_ERR_NULL;
   if (which < 0 || which >= kNumTimers || capacity < 0) return LITEVGGT_ERR_SHAPE;
-  Timers& tm = ctx->timers;
   *count = 0;
-  if (!tm.created) return LITEVGGT_ERR_CUDA;
-  // the ring keeps the latest kTimerSlots records; slot i holds record i, i + kTimerSlots, ...
-  const int used = tm.used[which];
-  const int kept = used < kTimerSlots ? used : kTimerSlots;
+  float all[kTimerSlots];
+  int kept = 0;
+  const litevggt_status st = read_stamps(ctx, which, all, &kept);
+  if (st != LITEVGGT_OK) return st;
   const int n = kept < capacity ? kept : capacity;
-  for (int i = 0; i < n; ++i) {
-    const int slot = (used - kept + i) % kTimerSlots;
-    if (cudaEventSynchronize(tm.stop[which][slot]) != cudaSuccess ||
-        cudaEventElapsedTime(&ms[i], tm.start[which][slot], tm.stop[which][slot]) != cudaSuccess)
-      return cuda_status(cudaGetLastError());
-  }
+  for (int i = 0; i < n; ++i) ms[i] = all[i];
   *count = n;
   return LITEVGGT_OK;
 }
@@ -415,12 +413,6 @@ litevggt_status litevggt_destroy(litevggt_ctx* ctx) {
   if (!ctx_ok(ctx)) return LITEVGGT_ERR_NULL;
   DeviceGuard g(ctx->device);
   cudaDeviceSynchronize();
-  if (ctx->timers.created)
-    for (int w = 0; w < kNumTimers; ++w)
-      for (int i = 0; i < kTimerSlots; ++i) {
-        cudaEventDestroy(ctx->timers.start[w][i]);
-        cudaEventDestroy(ctx->timers.stop[w][i]);
-      }
   if (ctx->pipe.created) {
     cudaStreamDestroy(ctx->pipe.copy_in);
     cudaStreamDestroy(ctx->pipe.copy_out);
@@ -458,7 +450,7 @@ litevggt_status litevggt_grad_map(litevggt_ctx* ctx, const float* images, float*
   int n = 0;
   cudaError_t e;
   {
-    StepTimer t(ctx, 0, (cudaStream_t)stream);
+    StepTimer t(ctx, 0);
     e = launch_grad_map(ctx, images, grad, (cudaStream_t)stream, &n);
   }
   bump(ctx, n);
@@ -480,11 +472,11 @@ litevggt_status litevggt_merge_plan(litevggt_ctx* ctx, const void* x, const floa
   int n = 0;
   cudaError_t e;
   {
-    StepTimer t(ctx, 1, s);
+    StepTimer t(ctx, 1);
     e = launch_var_map(ctx, xb, ctx->ws.var_map, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 2, s);
+    StepTimer t(ctx, 2);
     e = launch_partition(ctx, grad, ctx->ws.var_map, ctx->ws.ga_score, ctx->ws.cls, s, &n);
   }
   bump(ctx, n);
@@ -518,7 +510,7 @@ litevggt_status litevggt_merge(litevggt_ctx* ctx, const litevggt_plan* plan, con
   int n = 0;
   cudaError_t e;
   {
-    StepTimer t(ctx, 5, (cudaStream_t)stream);
+    StepTimer t(ctx, 5);
     e = launch_merge(ctx, plan, static_cast<const __nv_bfloat16*>(x), static_cast<__nv_bfloat16*>(x_merged),
                      (cudaStream_t)stream, &n);
   }
@@ -555,22 +547,22 @@ litevggt_status litevggt_global_attn(litevggt_ctx* ctx, const void* x_merged, in
   int n = 0;
   cudaError_t e;
   {
-    StepTimer t(ctx, 6, s);
+    StepTimer t(ctx, 6);
     e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x_merged), m, d,
                              static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
                              2 * d, kKeyScaleLog2e, core_stat(ctx, m), ctx->ws.qkv, s, &n);
   }
   if (e == cudaSuccess && ctx->cfg.qkv_dtype == 1) {
-    StepTimer t(ctx, 14, s);
+    StepTimer t(ctx, 14);
     e = launch_qkv_quantize(ctx, ctx->ws.qkv, m, true, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 7, s);
+    StepTimer t(ctx, 7);
     e = ctx->cfg.qkv_dtype == 1 ? launch_flash_attention_fp8(ctx, m, ctx->ws.attn_o, s, &n)
                                 : launch_flash_attention(ctx, ctx->ws.qkv, m, 1, ctx->ws.attn_o, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 8, s);
+    StepTimer t(ctx, 8);
     e = launch_linear(ctx, ctx->ws.attn_o, m, d, static_cast<const __nv_bfloat16*>(w_o), d,
                       static_cast<const __nv_bfloat16*>(b_o), static_cast<__nv_bfloat16*>(y_merged), s, &n);
   }
@@ -606,13 +598,13 @@ litevggt_status litevggt_global_attn_ext(litevggt_ctx* ctx, const litevggt_plan*
   int n = 0;
   cudaError_t e;
   {
-    StepTimer t(ctx, 6, s);
+    StepTimer t(ctx, 6);
     e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x_merged), m, d,
                              static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
                              2 * d, 1.0f, embeds ? LinearStat{} : core_stat(ctx, m), ctx->ws.qkv, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 13, s);
+    StepTimer t(ctx, 13);
     e = launch_qk_embed(ctx, ctx->ws.qkv, ext->rope != 0 ? plan->kept_idx : nullptr, m,
                         static_cast<const __nv_bfloat16*>(ext->q_norm_gamma),
                         static_cast<const __nv_bfloat16*>(ext->q_norm_beta),
@@ -621,16 +613,16 @@ litevggt_status litevggt_global_attn_ext(litevggt_ctx* ctx, const litevggt_plan*
                         ext->rope_base, fp8 ? nullptr : ctx->ws.attn_kmax, s, &n);
   }
   if (e == cudaSuccess && ctx->cfg.qkv_dtype == 1) {
-    StepTimer t(ctx, 14, s);
+    StepTimer t(ctx, 14);
     e = launch_qkv_quantize(ctx, ctx->ws.qkv, m, !embeds, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 7, s);
+    StepTimer t(ctx, 7);
     e = ctx->cfg.qkv_dtype == 1 ? launch_flash_attention_fp8(ctx, m, ctx->ws.attn_o, s, &n)
                                 : launch_flash_attention(ctx, ctx->ws.qkv, m, 1, ctx->ws.attn_o, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 8, s);
+    StepTimer t(ctx, 8);
     e = launch_linear(ctx, ctx->ws.attn_o, m, d, static_cast<const __nv_bfloat16*>(w_o), d,
                       static_cast<const __nv_bfloat16*>(b_o), static_cast<__nv_bfloat16*>(y_merged), s, &n);
   }
@@ -646,10 +638,10 @@ litevggt_status litevggt_layernorm(litevggt_ctx* ctx, const void* x, int64_t row
   int n = 0;
   cudaError_t e;
   {
-    StepTimer t(ctx, 10, (cudaStream_t)stream);
+    StepTimer t(ctx, 10);
     e = launch_layernorm(static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(gamma),
                          static_cast<const __nv_bfloat16*>(beta), static_cast<__nv_bfloat16*>(out), rows, eps,
-                         (cudaStream_t)stream, &n);
+                         next_stamp(ctx), (cudaStream_t)stream, &n);
   }
   bump(ctx, n);
   return cuda_status(e);
@@ -670,7 +662,7 @@ litevggt_status litevggt_frame_attn(litevggt_ctx* ctx, const void* x, const void
   int n = 0;
   cudaError_t e;
   {
-    StepTimer t(ctx, 11, s);
+    StepTimer t(ctx, 11);
     e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x), z.n_tokens, d,
                              static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
                              2 * d, kKeyScaleLog2e, LinearStat{ctx->ws.attn_kmax, z.tokens_frame, nullptr},
@@ -702,7 +694,7 @@ litevggt_status litevggt_mlp(litevggt_ctx* ctx, const void* x, int64_t rows, con
   int n = 0;
   cudaError_t e = cudaSuccess;
   {
-    StepTimer t(ctx, 12, s);
+    StepTimer t(ctx, 12);
     for (long long r0 = 0; r0 < rows && e == cudaSuccess; r0 += kMlpChunkRows) {
       const long long nr = rows - r0 < kMlpChunkRows ? rows - r0 : kMlpChunkRows;
       e = launch_linear_mlp(ctx, xb + r0 * d, nr, d, static_cast<const __nv_bfloat16*>(w1), 4 * d,
@@ -726,7 +718,7 @@ litevggt_status litevggt_unmerge(litevggt_ctx* ctx, const litevggt_plan* plan, c
   int n = 0;
   cudaError_t e;
   {
-    StepTimer t(ctx, 9, (cudaStream_t)stream);
+    StepTimer t(ctx, 9);
     e = launch_unmerge(ctx, plan, static_cast<const __nv_bfloat16*>(y_merged),
                        static_cast<const __nv_bfloat16*>(residual), static_cast<__nv_bfloat16*>(out),
                        (cudaStream_t)stream, &n);

@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(FaShape<kTiles>::kThreads, kTiles == 2 ? 1 : 2
 flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_bfloat16* __restrict__ qkv,
                        __nv_bfloat16* __restrict__ o, float* __restrict__ o_state, float* __restrict__ ml_state,
                        const float* __restrict__ k_norm2_max, int seq_len, int dim, int tile_begin, int tile_end,
-                       uint32_t* status) {
+                       uint32_t* status, Stamp stamp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* smem_k = smem;
@@ -365,6 +365,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
   tc_fence_after();
   const uint32_t tmem_base = bars->tmem_base;
   const WaitCtl ctl{&bars->abort_flag, status};
+  const Span span(stamp);
 
   if (warp == kIssuerWarp + 1) {
     // ------------------------------------------------------------------ TMA producer
@@ -779,7 +780,7 @@ __global__ void __launch_bounds__(kFaThreads, 1)
 flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __grid_constant__ CUtensorMap tmap_v8t,
                            const uint8_t* __restrict__ q8, const float* __restrict__ amax, __nv_bfloat16* __restrict__ o,
                            float* __restrict__ o_state, float* __restrict__ ml_state, int seq_len, int dim, int tile_begin,
-                           int tile_end, uint32_t* status) {
+                           int tile_end, uint32_t* status, Stamp stamp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* smem_k = smem;
@@ -835,6 +836,7 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
   tc_fence_after();
   const uint32_t tmem_base = bars->tmem_base;
   const WaitCtl ctl{&bars->abort_flag, status};
+  const Span span(stamp);
 
   if (warp == 17) {
     // ------------------------------------------------------------------ TMA producer
@@ -1098,7 +1100,7 @@ cudaError_t launch_flash_attention_fp8(litevggt_ctx* ctx, long long m, __nv_bflo
       !make_tmap_u8_2d(ctx->encode_tiled, &tmap_v, ws.v8t, (uint64_t)m_pad, (uint64_t)dim, (uint64_t)m_pad, 128, 64))
     return cudaErrorInvalidValue;
   using Kernel = void (*)(const CUtensorMap, const CUtensorMap, const uint8_t*, const float*, __nv_bfloat16*, float*,
-                          float*, int, int, int, int, uint32_t*);
+                          float*, int, int, int, int, uint32_t*, Stamp);
   const Kernel kernels[2][2] = {{flash_attention_fp8_kernel<false, false>, flash_attention_fp8_kernel<false, true>},
                                 {flash_attention_fp8_kernel<true, false>, flash_attention_fp8_kernel<true, true>}};
   static std::atomic<unsigned long long> smem_set[2][2];
@@ -1115,7 +1117,8 @@ cudaError_t launch_flash_attention_fp8(litevggt_ctx* ctx, long long m, __nv_bflo
   for (int begin = 0; begin < n_tiles; begin += per_chunk) {
     const int end = begin + per_chunk < n_tiles ? begin + per_chunk : n_tiles;
     kernels[begin == 0][end == n_tiles]<<<grid, kFaThreads, kFa8SmemBytes, s>>>(
-        tmap_k, tmap_v, ws.q8, ws.qkv_amax, o, ws.attn_o_state, ws.attn_ml_state, (int)m, dim, begin, end, ws.status);
+        tmap_k, tmap_v, ws.q8, ws.qkv_amax, o, ws.attn_o_state, ws.attn_ml_state, (int)m, dim, begin, end, ws.status,
+        next_stamp(ctx));
     ++*launches;
   }
   return cudaGetLastError();
@@ -1131,7 +1134,7 @@ cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, 
   if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap, qkv, (uint64_t)3 * dim, (uint64_t)rows, (uint64_t)3 * dim, 64, 128))
     return cudaErrorInvalidValue;
   using Kernel = void (*)(const CUtensorMap, const __nv_bfloat16*, __nv_bfloat16*, float*, float*, const float*, int,
-                          int, int, int, uint32_t*);
+                          int, int, int, uint32_t*, Stamp);
   // [query tiles of a CTA - 1][first chunk][last chunk]
   const Kernel kernels[2][2][2] = {
       {{flash_attention_kernel<1, false, false>, flash_attention_kernel<1, false, true>},
@@ -1157,7 +1160,7 @@ cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, 
     if (e != cudaSuccess) return e;
     kernels[a][b][c]<<<grid, threads, smem_bytes[a], s>>>(
         tmap, qkv, o, ctx->ws.attn_o_state, ctx->ws.attn_ml_state, ctx->ws.attn_kmax, (int)seq_len, dim, begin, end,
-        ctx->ws.status);
+        ctx->ws.status, next_stamp(ctx));
     ++*launches;
   }
   return cudaGetLastError();

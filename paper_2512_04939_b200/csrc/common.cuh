@@ -18,6 +18,34 @@ namespace lv {
 
 constexpr long long kTimeoutCycles = 1ll << 32;  // about two seconds at 1.9 GHz
 
+// ----------------------------------------------------------------------------- step stopwatches
+__device__ __forceinline__ unsigned long long global_timer() {  // nanoseconds, the same clock on every SM
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+// A kernel's presence on the device, written into its step's stopwatch: the first block's arrival, and the
+// latest departure of the blocks that can be among the last to leave (blocks start in order, and no more
+// than kSpanBlocks are resident at a time).  Two stores to memory in place of two events between
+// kernels, which held the stream for about 2.7 us each: 72 -> 45 us for the layer of four small frames.
+constexpr long long kSpanBlocks = 148 * 32;
+struct Span {
+  const Stamp& stamp;  // a kernel parameter: nothing is held in registers meanwhile
+  __device__ __forceinline__ static long long block() {
+    return blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
+  }
+  __device__ __forceinline__ explicit Span(const Stamp& s) : stamp(s) {
+    if (threadIdx.x == 0 && stamp.start != nullptr && block() == 0) *stamp.start = global_timer();
+  }
+  __device__ __forceinline__ ~Span() {
+    if (threadIdx.x == 0 && stamp.stop != nullptr &&
+        block() + kSpanBlocks >= (long long)gridDim.x * gridDim.y * gridDim.z)
+      atomicMax(stamp.stop, global_timer());
+  }
+  Span(const Span&) = delete;
+  Span& operator=(const Span&) = delete;
+};
+
 // ----------------------------------------------------------------------------- bf16
 __device__ __forceinline__ float bf16_lo(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }

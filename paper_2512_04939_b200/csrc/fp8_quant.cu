@@ -17,7 +17,8 @@ constexpr int kAmaxWarps = 8;
 // in 12 passes, 8 neighbouring lanes share a head.  Magnitudes are non-negative floats, which
 // order like their bit patterns: integer atomicMax on a zeroed array.
 __global__ void __launch_bounds__(kAmaxWarps * 32)
-qkv_amax_kernel(const __nv_bfloat16* __restrict__ qkv, long long m, float* __restrict__ amax) {
+qkv_amax_kernel(const __nv_bfloat16* __restrict__ qkv, long long m, float* __restrict__ amax, Stamp stamp) {
+  const Span span(stamp);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float best[12];
 #pragma unroll
@@ -69,7 +70,8 @@ __device__ __forceinline__ void quantize32(const __nv_bfloat16* src, float inv, 
 // keys, and a padded key must not carry anything that is not finite).
 __global__ void __launch_bounds__(256)
 qkv_quantize_kernel(const __nv_bfloat16* __restrict__ qkv, long long m, long long m_pad, const float* __restrict__ amax,
-                    uint8_t* __restrict__ q8, uint8_t* __restrict__ k8, uint8_t* __restrict__ v8t) {
+                    uint8_t* __restrict__ q8, uint8_t* __restrict__ k8, uint8_t* __restrict__ v8t, Stamp stamp) {
+  const Span span(stamp);
   __shared__ __align__(16) uint8_t v_tile[64][128 + 16];
   const int head = blockIdx.y;
   const long long row0 = (long long)blockIdx.x * 128;
@@ -114,11 +116,11 @@ cudaError_t launch_qkv_quantize(litevggt_ctx* ctx, const __nv_bfloat16* qkv, lon
     // few blocks: every one sends 48 atomics per warp, and all of them meet on the same 48 words
     long long blocks = (m + kAmaxWarps - 1) / kAmaxWarps;
     if (blocks > 4ll * ctx->num_sms) blocks = 4ll * ctx->num_sms;
-    qkv_amax_kernel<<<(unsigned)blocks, kAmaxWarps * 32, 0, s>>>(qkv, m, ws.qkv_amax);
+    qkv_amax_kernel<<<(unsigned)blocks, kAmaxWarps * 32, 0, s>>>(qkv, m, ws.qkv_amax, next_stamp(ctx));
     ++*launches;
   }
   const long long m_pad = round_up(m, 128);
-  qkv_quantize_kernel<<<dim3((unsigned)(m_pad / 128), 16), 256, 0, s>>>(qkv, m, m_pad, ws.qkv_amax, ws.q8, ws.k8, ws.v8t);
+  qkv_quantize_kernel<<<dim3((unsigned)(m_pad / 128), 16), 256, 0, s>>>(qkv, m, m_pad, ws.qkv_amax, ws.q8, ws.k8, ws.v8t, next_stamp(ctx));
   ++*launches;
   return cudaGetLastError();
 }

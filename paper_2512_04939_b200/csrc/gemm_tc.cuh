@@ -122,7 +122,7 @@ template <class Epi, int kBN, int kCtas>
 __global__ void __launch_bounds__(kGemmMaxThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                const __grid_constant__ CUtensorMap tmap_out, int m_rows, int n_cols, int k_dim, Epi epi,
-               uint32_t* status) {
+               uint32_t* status, Stamp stamp) {
   using Shape = GemmShape<kBN, kCtas>;
   constexpr int kStages = Shape::kStages;
   constexpr bool kPair = kCtas == 2;
@@ -174,6 +174,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   tc_fence_after();
   const uint32_t tmem_base = bars->tmem_base;
   const WaitCtl ctl{&bars->abort_flag, status};
+  const Span span(stamp);
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -356,7 +357,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 // to do.
 template <class Epi, int kBN, int kCtas>
 cudaError_t gemm_launch(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& out, long long m, long long n,
-                        long long k, const Epi& epi, long long work, int num_sms, uint32_t* status, cudaStream_t s) {
+                        long long k, const Epi& epi, long long work, int num_sms, uint32_t* status,
+                        const Stamp& stamp, cudaStream_t s) {
   using Shape = GemmShape<kBN, kCtas>;
   static std::atomic<unsigned long long> smem_set{0};
   cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(gemm_tc_kernel<Epi, kBN, kCtas>), Shape::kSmemBytes,
@@ -375,7 +377,7 @@ cudaError_t gemm_launch(const CUtensorMap& a, const CUtensorMap& b, const CUtens
   cfg.stream = s;
   cfg.attrs = &cluster;
   cfg.numAttrs = kCtas > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<Epi, kBN, kCtas>, a, b, out, (int)m, (int)n, (int)k, epi, status);
+  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<Epi, kBN, kCtas>, a, b, out, (int)m, (int)n, (int)k, epi, status, stamp);
 }
 
 // What a launch costs, in units of what one column of a tile costs per k-block, times k: every wave pays

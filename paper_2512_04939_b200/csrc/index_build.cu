@@ -96,6 +96,7 @@ struct IndexArgs {
   int *rem_token, *rem_anchor, *rem_row, *rem_slot, *seg_tmp;  // [R] merged tokens; tokens by slot
   long long n_src, n_dst, n_tokens, n_merged, n_remove;
   uint32_t* status;
+  Stamp stamp;
 };
 
 // Fixes the bits of pass `pass` from its histogram.  Called by a whole block of kIdxThreads threads.
@@ -377,6 +378,7 @@ static __host__ __device__ inline int phase_blocks(int phase, const IndexArgs& a
 
 template <int phase>
 __global__ void __launch_bounds__(kIdxThreads) index_phase_kernel(const IndexArgs a) {
+  const Span span(a.stamp);
   run_phase<phase>(blockIdx.x, gridDim.x, a);
 }
 
@@ -391,19 +393,21 @@ __device__ __forceinline__ void run_phases_from(const IndexArgs& a) {
   if constexpr (phase < kOrder) run_phases_from<phase + 1>(a);
 }
 __global__ void __launch_bounds__(kIdxThreads, 1) index_small_kernel(const IndexArgs a, int* zeroed, int zeroed_words) {
+  const Span span(a.stamp);
   for (int i = threadIdx.x; i < zeroed_words; i += kIdxThreads) zeroed[i] = 0;
   __syncthreads();
   run_phases_from<kSelect0>(a);
 }
 
 template <int phase>
-static void launch_phases_from(const IndexArgs& a, int select_blocks, cudaStream_t s, int* launches) {
+static void launch_phases_from(const litevggt_ctx* ctx, IndexArgs& a, int select_blocks, cudaStream_t s, int* launches) {
   const int blocks = phase_blocks(phase, a, select_blocks);
   if (blocks > 0) {
+    a.stamp = next_stamp(ctx);
     index_phase_kernel<phase><<<(unsigned)blocks, kIdxThreads, 0, s>>>(a);
     ++*launches;
   }
-  if constexpr (phase < kOrder) launch_phases_from<phase + 1>(a, select_blocks, s, launches);
+  if constexpr (phase < kOrder) launch_phases_from<phase + 1>(ctx, a, select_blocks, s, launches);
 }
 
 // [ 3 histograms | long segments: count, rows | merged tokens per row ], zeroed for every plan
@@ -457,6 +461,7 @@ cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStrea
   a.n_remove = r;
   a.status = ws.status;
   if (z.n_tokens <= kSmallTokens) {
+    a.stamp = next_stamp(ctx);
     index_small_kernel<<<1, kIdxThreads, 0, s>>>(a, zero, (int)zeroed);
     ++*launches;
     return cudaGetLastError();
@@ -468,7 +473,7 @@ cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStrea
   long long select_blocks = (z.n_src + 4 * kIdxThreads - 1) / (4 * kIdxThreads);
   if (select_blocks > 2 * ctx->num_sms) select_blocks = 2 * ctx->num_sms;
   if (select_blocks < 2) select_blocks = 2;
-  launch_phases_from<kSelect0>(a, (int)select_blocks, s, launches);
+  launch_phases_from<kSelect0>(ctx, a, (int)select_blocks, s, launches);
   return cudaGetLastError();
 }
 

@@ -41,7 +41,7 @@ static cudaError_t launch_gemm_out(litevggt_ctx* ctx, const __nv_bfloat16* a, lo
     return cudaErrorInvalidValue;
   const long long rows = columns != 0 ? 2 * kGemmBM : kGemmBM, tiles = ((m + rows - 1) / rows) * ((n + bn - 1) / bn);
   ++*launches;
-  auto run = [&](auto launch) { return launch(tmap_a, tmap_b, tmap_out, m, n, k, epi, tiles, ctx->num_sms, ctx->ws.status, s); };
+  auto run = [&](auto launch) { return launch(tmap_a, tmap_b, tmap_out, m, n, k, epi, tiles, ctx->num_sms, ctx->ws.status, next_stamp(ctx), s); };
   switch (columns) {
     case 0: return run(gemm_launch<Epi, 256, 1>);
     case 64: return run(gemm_launch<Epi, 64, 2>);

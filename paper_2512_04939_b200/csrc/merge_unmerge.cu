@@ -35,7 +35,8 @@ __device__ __forceinline__ void load_row(uint4 (&v)[4], const __nv_bfloat16* row
 __global__ void __launch_bounds__(kRowThreads)
 merge_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ kept_idx, const int* __restrict__ seg_off,
              const int* __restrict__ seg_src, __nv_bfloat16* __restrict__ xm, long long n_merged,
-             long long n_tokens, long long n_remove, uint32_t* status) {
+             long long n_tokens, long long n_remove, uint32_t* status, Stamp stamp) {
+  const Span span(stamp);
   const int lane = threadIdx.x & 31;
   const long long j = (long long)blockIdx.x * kRowsPerCta + (threadIdx.x >> 5);
   if (j >= n_merged) return;
@@ -96,7 +97,8 @@ merge_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ kept_i
 __global__ void __launch_bounds__(kRowThreads)
 unmerge_kernel(const __nv_bfloat16* __restrict__ ym, const int* __restrict__ dst_of,
                const __nv_bfloat16* __restrict__ residual, __nv_bfloat16* __restrict__ out, long long n_tokens,
-               long long n_merged, uint32_t* status) {
+               long long n_merged, uint32_t* status, Stamp stamp) {
+  const Span span(stamp);
   const int lane = threadIdx.x & 31;
   const long long i = (long long)blockIdx.x * kRowsPerCta + (threadIdx.x >> 5);
   if (i >= n_tokens) return;
@@ -131,7 +133,9 @@ unmerge_kernel(const __nv_bfloat16* __restrict__ ym, const int* __restrict__ dst
 // in registers, fp32, one rounding.  One warp per row like the kernels above.
 __global__ void __launch_bounds__(kRowThreads)
 layernorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gamma,
-                 const __nv_bfloat16* __restrict__ beta, __nv_bfloat16* __restrict__ out, long long rows, float eps) {
+                 const __nv_bfloat16* __restrict__ beta, __nv_bfloat16* __restrict__ out, long long rows, float eps,
+                 Stamp stamp) {
+  const Span span(stamp);
   const int lane = threadIdx.x & 31;
   const long long i = (long long)blockIdx.x * kRowsPerCta + (threadIdx.x >> 5);
   if (i >= rows) return;
@@ -179,10 +183,11 @@ layernorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __res
 }
 
 cudaError_t launch_layernorm(const __nv_bfloat16* x, const __nv_bfloat16* gamma, const __nv_bfloat16* beta,
-                             __nv_bfloat16* out, long long rows, float eps, cudaStream_t s, int* launches) {
+                             __nv_bfloat16* out, long long rows, float eps, const Stamp& stamp, cudaStream_t s,
+                             int* launches) {
   if (rows == 0) return cudaSuccess;
   const unsigned blocks = (unsigned)((rows + kRowsPerCta - 1) / kRowsPerCta);
-  layernorm_kernel<<<blocks, kRowThreads, 0, s>>>(x, gamma, beta, out, rows, eps);
+  layernorm_kernel<<<blocks, kRowThreads, 0, s>>>(x, gamma, beta, out, rows, eps, stamp);
   ++*launches;
   return cudaGetLastError();
 }
@@ -192,7 +197,7 @@ cudaError_t launch_merge(const litevggt_ctx* ctx, const litevggt_plan* plan, con
   const Sizes& z = ctx->sz;
   const unsigned blocks = (unsigned)((z.n_merged + kRowsPerCta - 1) / kRowsPerCta);
   merge_kernel<<<blocks, kRowThreads, 0, s>>>(x, plan->kept_idx, plan->seg_off, plan->seg_src, xm, z.n_merged,
-                                              z.n_tokens, z.n_remove, ctx->ws.status);
+                                              z.n_tokens, z.n_remove, ctx->ws.status, next_stamp(ctx));
   ++*launches;
   return cudaGetLastError();
 }
@@ -202,7 +207,7 @@ cudaError_t launch_unmerge(const litevggt_ctx* ctx, const litevggt_plan* plan, c
   const Sizes& z = ctx->sz;
   const unsigned blocks = (unsigned)((z.n_tokens + kRowsPerCta - 1) / kRowsPerCta);
   unmerge_kernel<<<blocks, kRowThreads, 0, s>>>(ym, plan->dst_of, residual, out, z.n_tokens, z.n_merged,
-                                                ctx->ws.status);
+                                                ctx->ws.status, next_stamp(ctx));
   ++*launches;
   return cudaGetLastError();
 }

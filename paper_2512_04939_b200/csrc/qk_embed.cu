@@ -40,7 +40,8 @@ struct EmbedParams {
 
 __global__ void __launch_bounds__(kEmbedThreads)
 qk_embed_kernel(__nv_bfloat16* __restrict__ qkv, const int* __restrict__ kept_idx, long long m_rows,
-                long long n_tokens, EmbedParams p, uint32_t* status) {
+                long long n_tokens, EmbedParams p, uint32_t* status, Stamp stamp) {
+  const Span span(stamp);
   const int lane = threadIdx.x & 31;
   const int j = lane & 7;  // which 8 channels of the head: 8j .. 8j+7
   float theta[8];  // angle per position of this lane's 8 channels
@@ -188,7 +189,7 @@ cudaError_t launch_qk_embed(const litevggt_ctx* ctx, __nv_bfloat16* qkv, const i
   // as many blocks as an SM holds at a time: the key norms of a block's rows meet in one atomic per head
   long long blocks = (m + kEmbedRowsPerCta - 1) / kEmbedRowsPerCta;
   if (blocks > 8ll * ctx->num_sms) blocks = 8ll * ctx->num_sms;
-  qk_embed_kernel<<<(unsigned)blocks, kEmbedThreads, 0, s>>>(qkv, kept_idx, m, z.n_tokens, p, ctx->ws.status);
+  qk_embed_kernel<<<(unsigned)blocks, kEmbedThreads, 0, s>>>(qkv, kept_idx, m, z.n_tokens, p, ctx->ws.status, next_stamp(ctx));
   ++*launches;
   return cudaGetLastError();
 }

@@ -93,15 +93,18 @@ struct Workspace {
 }  // namespace lv
 
 namespace lv {
-// Device-time stopwatches, one per step of the path: CUDA event pairs recorded on the
-// launching stream around the step's kernels, kept in a small ring per step.
+// Where a kernel notes when it was on the device (common.cuh: Span).
+struct Stamp {
+  unsigned long long* start = nullptr;  // only the step's first kernel
+  unsigned long long* stop = nullptr;   // every kernel of the step; the latest time stays
+};
+// Device-time stopwatches, one per step of the path: the times at which the step's kernels came
+// and went, by the device's own clock, kept in a small ring per step.
 constexpr int kNumTimers = 15;
 constexpr int kTimerSlots = 64;
 struct Timers {
-  cudaEvent_t start[kNumTimers][kTimerSlots];
-  cudaEvent_t stop[kNumTimers][kTimerSlots];
-  int used[kNumTimers];  // launches recorded since the last reset
-  bool created;
+  unsigned long long* stamps = nullptr;  // device [kNumTimers][kTimerSlots]{start, stop}, in the workspace
+  int used[kNumTimers] = {};             // launches recorded since the last reset
 };
 }  // namespace lv
 
@@ -127,6 +130,7 @@ struct litevggt_ctx {
   long long launches;
   void* encode_tiled;  // cuTensorMapEncodeTiled, resolved at run time
   lv::Timers timers;
+  mutable lv::Stamp step;  // of the step whose kernels are being launched
   HostPipe pipe;
 };
 
@@ -147,6 +151,13 @@ struct litevggt_plan {
 };
 
 namespace lv {
+
+// The stamp of the step's next kernel.
+inline Stamp next_stamp(const litevggt_ctx* ctx) {
+  const Stamp s = ctx->step;
+  ctx->step.start = nullptr;
+  return s;
+}
 
 // bits of the device status word
 constexpr uint32_t kStatusTimeout = 1u;
@@ -206,7 +217,8 @@ cudaError_t launch_linear_mlp(litevggt_ctx* ctx, const __nv_bfloat16* a, long lo
                               const __nv_bfloat16* w, long long n, const __nv_bfloat16* bias, int gelu,
                               const __nv_bfloat16* residual, __nv_bfloat16* out, cudaStream_t s, int* launches);
 cudaError_t launch_layernorm(const __nv_bfloat16* x, const __nv_bfloat16* gamma, const __nv_bfloat16* beta,
-                             __nv_bfloat16* out, long long rows, float eps, cudaStream_t s, int* launches);
+                             __nv_bfloat16* out, long long rows, float eps, const Stamp& stamp, cudaStream_t s,
+                             int* launches);
 
 // selftest.cu: one CTA waits on a barrier that nobody arrives on, with the given cycle limit
 cudaError_t launch_bounded_wait_selftest(litevggt_ctx* ctx, long long limit_cycles, uint32_t* outcome, cudaStream_t s,

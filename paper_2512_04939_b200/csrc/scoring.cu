@@ -38,7 +38,8 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 }
 
 __global__ void __launch_bounds__(kGradThreads)
-grad_map_kernel(const float* __restrict__ images, float* __restrict__ grad, int grid_h, int grid_w, int patch) {
+grad_map_kernel(const float* __restrict__ images, float* __restrict__ grad, int grid_h, int grid_w, int patch, Stamp stamp) {
+  const Span span(stamp);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int pps = 30 / patch;  // patches per strip (patch <= 30)
   const int strips = (grid_w + pps - 1) / pps;
@@ -113,7 +114,8 @@ grad_map_kernel(const float* __restrict__ images, float* __restrict__ grad, int 
 // per-row bookkeeping (row counters, queue index, end-of-patch test) is gone.  kAhead divides kPatch.
 template <int kPatch, int kAhead>
 __global__ void __launch_bounds__(kGradThreads)
-grad_map_patch_kernel(const float* __restrict__ images, float* __restrict__ grad, int grid_h, int grid_w) {
+grad_map_patch_kernel(const float* __restrict__ images, float* __restrict__ grad, int grid_h, int grid_w, Stamp stamp) {
+  const Span span(stamp);
   static_assert(kPatch % kAhead == 0 && kPatch <= 30 && kAhead >= 2, "queue slots must be static");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int pps = 30 / kPatch;
@@ -192,9 +194,9 @@ cudaError_t launch_grad_map(const litevggt_ctx* ctx, const float* images, float*
   const dim3 grid((unsigned)((strips + kGradThreads / 32 - 1) / (kGradThreads / 32)),
                   (unsigned)((z.grid_h + kGradPatchRows - 1) / kGradPatchRows), (unsigned)z.frames);
   if (patch == 14)
-    grad_map_patch_kernel<14, LV_GRAD_AHEAD14><<<grid, kGradThreads, 0, s>>>(images, grad, z.grid_h, z.grid_w);
+    grad_map_patch_kernel<14, LV_GRAD_AHEAD14><<<grid, kGradThreads, 0, s>>>(images, grad, z.grid_h, z.grid_w, next_stamp(ctx));
   else
-    grad_map_kernel<<<grid, kGradThreads, 0, s>>>(images, grad, z.grid_h, z.grid_w, patch);
+    grad_map_kernel<<<grid, kGradThreads, 0, s>>>(images, grad, z.grid_h, z.grid_w, patch, next_stamp(ctx));
   ++*launches;
   return cudaGetLastError();
 }
@@ -306,7 +308,9 @@ __device__ __forceinline__ float var_reduce_rows(const float (&v)[kVarRows], int
 }
 
 __global__ void __launch_bounds__(kVarThreads, LV_VAR_OCC)
-var_map_kernel(const __nv_bfloat16* __restrict__ x, float* __restrict__ var, int grid_h, int grid_w, int n_special) {
+var_map_kernel(const __nv_bfloat16* __restrict__ x, float* __restrict__ var, int grid_h, int grid_w, int n_special,
+               Stamp stamp) {
+  const Span span(stamp);
   __shared__ float part[kVarWarps][kVarRows][kVarMaxW];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int f = blockIdx.y, row_base = blockIdx.x * kVarRows;
@@ -422,7 +426,7 @@ cudaError_t launch_var_map(const litevggt_ctx* ctx, const __nv_bfloat16* x, floa
   const Sizes& z = ctx->sz;
   if (z.grid_w > kVarMaxW) return cudaErrorInvalidValue;
   const unsigned strips = (unsigned)((z.grid_h + kVarRows - 1) / kVarRows);
-  var_map_kernel<<<dim3(strips, z.frames), kVarThreads, 0, s>>>(x, var, z.grid_h, z.grid_w, z.n_special);
+  var_map_kernel<<<dim3(strips, z.frames), kVarThreads, 0, s>>>(x, var, z.grid_h, z.grid_w, z.n_special, next_stamp(ctx));
   ++*launches;
   return cudaGetLastError();
 }
@@ -458,7 +462,8 @@ __device__ __forceinline__ unsigned score_key(float v) {
 __global__ void __launch_bounds__(kPartThreads)
 partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, float* __restrict__ ga,
                  uint8_t* __restrict__ cls, int grid_h, int grid_w, int n_special, int n_ga, int cell_h, int cell_w,
-                 float alpha, float beta) {
+                 float alpha, float beta, Stamp stamp) {
+  const Span span(stamp);
   extern __shared__ float part_smem[];
   const int p_count = grid_h * grid_w;
   float* score = part_smem;                                        // [P]
@@ -593,7 +598,7 @@ cudaError_t launch_partition(const litevggt_ctx* ctx, const float* grad, const f
   if (e != cudaSuccess) return e;
   partition_kernel<<<z.frames, kPartThreads, smem, s>>>(grad, var, ga, cls, z.grid_h, z.grid_w, z.n_special,
                                                         z.n_ga_frame, ctx->cfg.cell_h, ctx->cfg.cell_w,
-                                                        ctx->cfg.alpha, ctx->cfg.beta);
+                                                        ctx->cfg.alpha, ctx->cfg.beta, next_stamp(ctx));
   ++*launches;
   return cudaGetLastError();
 }
@@ -607,7 +612,8 @@ constexpr int kListThreads = 256;
 
 __global__ void __launch_bounds__(kListThreads)
 build_lists_kernel(const uint8_t* __restrict__ cls, int* __restrict__ src_list, int* __restrict__ dst_list,
-                   int* __restrict__ src_pos, int p_count, int n_special, int n_src_frame, int n_dst_frame, uint32_t* status) {
+                   int* __restrict__ src_pos, int p_count, int n_special, int n_src_frame, int n_dst_frame, uint32_t* status, Stamp stamp) {
+  const Span span(stamp);
   __shared__ int warp_src[kListThreads / 32], warp_dst[kListThreads / 32];
   const int f = blockIdx.x;
   const int tokens_frame = p_count + n_special;
@@ -666,7 +672,7 @@ cudaError_t launch_build_lists(const litevggt_ctx* ctx, const uint8_t* cls, int*
                                cudaStream_t s, int* launches) {
   const Sizes& z = ctx->sz;
   build_lists_kernel<<<z.frames, kListThreads, 0, s>>>(cls, src_list, dst_list, src_pos, z.patches, z.n_special,
-                                                       z.n_src_frame, z.n_dst_frame, ctx->ws.status);
+                                                       z.n_src_frame, z.n_dst_frame, ctx->ws.status, next_stamp(ctx));
   ++*launches;
   return cudaGetLastError();
 }

@@ -21,7 +21,8 @@ pack_rows_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ sr
                  const int* __restrict__ dst_list, long long n_src, long long n_dst, long long n_dst_padded,
                  long long n_tokens, __nv_bfloat16* __restrict__ panel_src, __nv_bfloat16* __restrict__ panel_dst,
                  float* __restrict__ inv_norm_src, float* __restrict__ inv_norm_dst, unsigned long long* __restrict__ key,
-                 uint32_t* status) {
+                 uint32_t* status, Stamp stamp) {
+  const Span span(stamp);
   const int lane = threadIdx.x & 31;
   const long long row = (long long)blockIdx.x * (kPackThreads / 32) + (threadIdx.x >> 5);
   if (row >= n_src + n_dst_padded) return;
@@ -69,7 +70,7 @@ cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, cudaStream_t
   const int warps = kPackThreads / 32;
   pack_rows_kernel<<<(unsigned)((rows + warps - 1) / warps), kPackThreads, 0, s>>>(
       x, ws.src_list, ws.dst_list, z.n_src, z.n_dst, n_dst_padded, z.n_tokens, ws.panel_src, ws.panel_dst,
-      ws.inv_norm_src, ws.inv_norm_dst, ws.match_keys, ws.status);
+      ws.inv_norm_src, ws.inv_norm_dst, ws.match_keys, ws.status, next_stamp(ctx));
   ++*launches;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -95,7 +96,7 @@ cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, cudaStream_t
   const long long tiles = row_blocks * ((z.n_dst + bn - 1) / bn);
   // the argmax epilogue writes no matrix: the store map is never read, any valid map fills the slot
   auto run = [&](auto launch) {
-    return launch(tmap_a, tmap_b, tmap_a, z.n_src, z.n_dst, 1024, epi, tiles, ctx->num_sms, ws.status, s);
+    return launch(tmap_a, tmap_b, tmap_a, z.n_src, z.n_dst, 1024, epi, tiles, ctx->num_sms, ws.status, next_stamp(ctx), s);
   };
   e = bn == 256 ? run(gemm_launch<ArgmaxEpilogue, 256, 2>)
                 : bn == 128 ? run(gemm_launch<ArgmaxEpilogue, 128, 2>) : run(gemm_launch<ArgmaxEpilogue, 64, 2>);
