@@ -233,6 +233,11 @@ litevggt_status ensure_block_ws(litevggt_ctx* ctx) {
   return LITEVGGT_OK;
 }
 
+// The key norms of `sequences` sequences, which an output projection leaves zero for the next layer.
+ZeroWords kmax_words(const litevggt_ctx* ctx, long long sequences) {
+  return ZeroWords{reinterpret_cast<uint32_t*>(ctx->ws.attn_kmax), sequences * ctx->sz.heads};
+}
+
 // What the global layer's attention core needs to know about Q, K and V before it starts.
 LinearStat core_stat(const litevggt_ctx* ctx, long long m) {
   LinearStat st;
@@ -344,6 +349,7 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
   ctx->timers.stamps = reinterpret_cast<unsigned long long*>(ws.base + o_stamps);
   ws.status = reinterpret_cast<uint32_t*>(ws.base + o_status);
   if (cudaMemset(ws.base + o_var, 0, o_src - o_var) != cudaSuccess ||
+      cudaMemset(ws.attn_kmax, 0, sizeof(float) * (size_t)z.frames * z.heads) != cudaSuccess ||
       cudaMemset(ctx->timers.stamps, 0, o_status - o_stamps) != cudaSuccess || cudaMemset(ws.status, 0, 16) != cudaSuccess) {
     (void)cudaGetLastError();
     cudaFree(ws.base);
@@ -527,7 +533,7 @@ litevggt_status litevggt_linear(litevggt_ctx* ctx, const void* a, int64_t m, int
     return LITEVGGT_ERR_ALIGN;
   int nl = 0;
   cudaError_t e = launch_linear(ctx, static_cast<const __nv_bfloat16*>(a), m, k, static_cast<const __nv_bfloat16*>(w),
-                                n, static_cast<const __nv_bfloat16*>(bias), static_cast<__nv_bfloat16*>(out),
+                                n, static_cast<const __nv_bfloat16*>(bias), ZeroWords{}, static_cast<__nv_bfloat16*>(out),
                                 (cudaStream_t)stream, &nl);
   bump(ctx, nl);
   return cuda_status(e);
@@ -564,7 +570,7 @@ litevggt_status litevggt_global_attn(litevggt_ctx* ctx, const void* x_merged, in
   if (e == cudaSuccess) {
     StepTimer t(ctx, 8);
     e = launch_linear(ctx, ctx->ws.attn_o, m, d, static_cast<const __nv_bfloat16*>(w_o), d,
-                      static_cast<const __nv_bfloat16*>(b_o), static_cast<__nv_bfloat16*>(y_merged), s, &n);
+                      static_cast<const __nv_bfloat16*>(b_o), kmax_words(ctx, 1), static_cast<__nv_bfloat16*>(y_merged), s, &n);
   }
   bump(ctx, n);
   return cuda_status(e);
@@ -624,7 +630,7 @@ litevggt_status litevggt_global_attn_ext(litevggt_ctx* ctx, const litevggt_plan*
   if (e == cudaSuccess) {
     StepTimer t(ctx, 8);
     e = launch_linear(ctx, ctx->ws.attn_o, m, d, static_cast<const __nv_bfloat16*>(w_o), d,
-                      static_cast<const __nv_bfloat16*>(b_o), static_cast<__nv_bfloat16*>(y_merged), s, &n);
+                      static_cast<const __nv_bfloat16*>(b_o), kmax_words(ctx, 1), static_cast<__nv_bfloat16*>(y_merged), s, &n);
   }
   bump(ctx, n);
   return cuda_status(e);
@@ -671,7 +677,7 @@ litevggt_status litevggt_frame_attn(litevggt_ctx* ctx, const void* x, const void
     if (e == cudaSuccess)
       e = launch_linear_mlp(ctx, ctx->ws.blk_o, z.n_tokens, d, static_cast<const __nv_bfloat16*>(w_o), d,
                             static_cast<const __nv_bfloat16*>(b_o), 0, static_cast<const __nv_bfloat16*>(residual),
-                            static_cast<__nv_bfloat16*>(y), s, &n);
+                            kmax_words(ctx, z.frames), static_cast<__nv_bfloat16*>(y), s, &n);
   }
   bump(ctx, n);
   return cuda_status(e);
@@ -698,11 +704,11 @@ litevggt_status litevggt_mlp(litevggt_ctx* ctx, const void* x, int64_t rows, con
     for (long long r0 = 0; r0 < rows && e == cudaSuccess; r0 += kMlpChunkRows) {
       const long long nr = rows - r0 < kMlpChunkRows ? rows - r0 : kMlpChunkRows;
       e = launch_linear_mlp(ctx, xb + r0 * d, nr, d, static_cast<const __nv_bfloat16*>(w1), 4 * d,
-                            static_cast<const __nv_bfloat16*>(b1), 1, nullptr, ctx->ws.blk_hidden, s, &n);
+                            static_cast<const __nv_bfloat16*>(b1), 1, nullptr, ZeroWords{}, ctx->ws.blk_hidden, s, &n);
       if (e == cudaSuccess)
         e = launch_linear_mlp(ctx, ctx->ws.blk_hidden, nr, 4 * d, static_cast<const __nv_bfloat16*>(w2), d,
                               static_cast<const __nv_bfloat16*>(b2), 0, rb != nullptr ? rb + r0 * d : nullptr,
-                              yb + r0 * d, s, &n);
+                              ZeroWords{}, yb + r0 * d, s, &n);
     }
   }
   bump(ctx, n);

@@ -105,7 +105,7 @@ extern "C" litevggt_status litevggt_global_attn_static(const void* x_merged, int
   local.sz.dim = kStaticDim;
   local.sz.heads = kStaticHeads;
   local.ws.status = status;
-  local.ws.attn_kmax = reinterpret_cast<float*>(dev->scratch + 64);  // zeroed by the projection's launcher
+  local.ws.attn_kmax = reinterpret_cast<float*>(dev->scratch + 64);  // zero at load and after every call
   int n = 0;
   cudaError_t e = lv::launch_linear_scaled(&local, static_cast<const __nv_bfloat16*>(x_merged), m, kStaticDim,
                                            static_cast<const __nv_bfloat16*>(w_qkv), 3 * kStaticDim,
@@ -114,7 +114,9 @@ extern "C" litevggt_status litevggt_global_attn_static(const void* x_merged, int
   if (e == cudaSuccess) e = lv::launch_flash_attention(&local, qkv, m, 1, o, s, &n);
   if (e == cudaSuccess)
     e = lv::launch_linear(&local, o, m, kStaticDim, static_cast<const __nv_bfloat16*>(w_o), kStaticDim,
-                          static_cast<const __nv_bfloat16*>(b_o), static_cast<__nv_bfloat16*>(y_merged), s, &n);
+                          static_cast<const __nv_bfloat16*>(b_o),
+                          lv::ZeroWords{reinterpret_cast<uint32_t*>(local.ws.attn_kmax), kStaticHeads},
+                          static_cast<__nv_bfloat16*>(y_merged), s, &n);
   if (e != cudaSuccess) {
     (void)cudaGetLastError();
     return LITEVGGT_ERR_CUDA;

@@ -24,6 +24,15 @@ __device__ __forceinline__ unsigned long long global_timer() {  // nanoseconds, 
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
+// First in every kernel of the library, before anything that another kernel may have written or may still
+// read: the launch of a small grid did not wait for the kernel before it to end (runtime.h: launch), so the
+// set-up above this - barriers, tensor memory, descriptors - runs under that kernel's last blocks.
+__device__ __forceinline__ void wait_for_previous_kernel() {
+  if ((long long)gridDim.x * gridDim.y * gridDim.z > kOverlapBlocks) return;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // and the next one may set itself up
+}
+
 // A kernel's presence on the device, written into its step's stopwatch: the first block's arrival, and the
 // latest departure of the blocks that can be among the last to leave (blocks start in order, and no more
 // than kSpanBlocks are resident at a time).  Two stores to memory in place of two events between
@@ -35,6 +44,7 @@ struct Span {
     return blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
   }
   __device__ __forceinline__ explicit Span(const Stamp& s) : stamp(s) {
+    wait_for_previous_kernel();
     if (threadIdx.x == 0 && stamp.start != nullptr && block() == 0) *stamp.start = global_timer();
   }
   __device__ __forceinline__ ~Span() {

@@ -116,13 +116,14 @@ cudaError_t launch_qkv_quantize(litevggt_ctx* ctx, const __nv_bfloat16* qkv, lon
     // few blocks: every one sends 48 atomics per warp, and all of them meet on the same 48 words
     long long blocks = (m + kAmaxWarps - 1) / kAmaxWarps;
     if (blocks > 4ll * ctx->num_sms) blocks = 4ll * ctx->num_sms;
-    qkv_amax_kernel<<<(unsigned)blocks, kAmaxWarps * 32, 0, s>>>(qkv, m, ws.qkv_amax, next_stamp(ctx));
+    e = launch(qkv_amax_kernel, dim3((unsigned)blocks), kAmaxWarps * 32, 0, s, qkv, m, ws.qkv_amax, next_stamp(ctx));
+    if (e != cudaSuccess) return e;
     ++*launches;
   }
   const long long m_pad = round_up(m, 128);
-  qkv_quantize_kernel<<<dim3((unsigned)(m_pad / 128), 16), 256, 0, s>>>(qkv, m, m_pad, ws.qkv_amax, ws.q8, ws.k8, ws.v8t, next_stamp(ctx));
   ++*launches;
-  return cudaGetLastError();
+  return launch(qkv_quantize_kernel, dim3((unsigned)(m_pad / 128), 16), 256, 0, s, qkv, m, m_pad, ws.qkv_amax, ws.q8, ws.k8, ws.v8t,
+                next_stamp(ctx));
 }
 
 }  // namespace lv

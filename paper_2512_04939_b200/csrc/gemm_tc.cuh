@@ -122,7 +122,7 @@ template <class Epi, int kBN, int kCtas>
 __global__ void __launch_bounds__(kGemmMaxThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                const __grid_constant__ CUtensorMap tmap_out, int m_rows, int n_cols, int k_dim, Epi epi,
-               uint32_t* status, Stamp stamp) {
+               uint32_t* status, ZeroWords zero, Stamp stamp) {
   using Shape = GemmShape<kBN, kCtas>;
   constexpr int kStages = Shape::kStages;
   constexpr bool kPair = kCtas == 2;
@@ -175,6 +175,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   const uint32_t tmem_base = bars->tmem_base;
   const WaitCtl ctl{&bars->abort_flag, status};
   const Span span(stamp);
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < zero.count; i += (long long)gridDim.x * blockDim.x)
+    zero.words[i] = 0u;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -358,26 +360,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 template <class Epi, int kBN, int kCtas>
 cudaError_t gemm_launch(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& out, long long m, long long n,
                         long long k, const Epi& epi, long long work, int num_sms, uint32_t* status,
-                        const Stamp& stamp, cudaStream_t s) {
+                        const ZeroWords& zero, const Stamp& stamp, cudaStream_t s) {
   using Shape = GemmShape<kBN, kCtas>;
   static std::atomic<unsigned long long> smem_set{0};
   cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(gemm_tc_kernel<Epi, kBN, kCtas>), Shape::kSmemBytes,
                                             smem_set);
   if (e != cudaSuccess) return e;
   const long long groups = work < num_sms / kCtas ? work : num_sms / kCtas;
-  cudaLaunchAttribute cluster;
-  cluster.id = cudaLaunchAttributeClusterDimension;
-  cluster.val.clusterDim.x = kCtas;
-  cluster.val.clusterDim.y = 1;
-  cluster.val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(kCtas * groups));
-  cfg.blockDim = dim3(gemm_threads<Epi>());
-  cfg.dynamicSmemBytes = Shape::kSmemBytes;
-  cfg.stream = s;
-  cfg.attrs = &cluster;
-  cfg.numAttrs = kCtas > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<Epi, kBN, kCtas>, a, b, out, (int)m, (int)n, (int)k, epi, status, stamp);
+  return launch_clusters(kCtas, true, gemm_tc_kernel<Epi, kBN, kCtas>, dim3((unsigned)(kCtas * groups)), gemm_threads<Epi>(),
+                         Shape::kSmemBytes, s, a, b, out, (int)m, (int)n, (int)k, epi, status, zero, stamp);
 }
 
 // What a launch costs, in units of what one column of a tile costs per k-block, times k: every wave pays

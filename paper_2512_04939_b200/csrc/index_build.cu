@@ -15,7 +15,7 @@
 //   group     merged tokens count into their rows (the count's old value is a slot), a scan over the
 //             rows gives the segments, each token goes to its slot and then to its rank among its
 //             segment's tokens.  Which slot a token got depends on scheduling, its rank does not.
-// Ten launches and one memset, or - up to kSmallTokens tokens, where a launch costs more than what it does -
+// Ten launches, or - up to kSmallTokens tokens, where a launch costs more than what it does -
 // one launch of one block.  The two bitonic sorts of 64-bit keys that came before took 92 launches at 200
 // frames of 28 x 37 (418 us, 77 now) and 23 at four of 16 x 16 (82 us, 19 now; 50 as ten launches).
 // No host synchronisation: all counts follow from the config.
@@ -400,22 +400,30 @@ __global__ void __launch_bounds__(kIdxThreads, 1) index_small_kernel(const Index
 }
 
 template <int phase>
-static void launch_phases_from(const litevggt_ctx* ctx, IndexArgs& a, int select_blocks, cudaStream_t s, int* launches) {
+static cudaError_t launch_phases_from(const litevggt_ctx* ctx, IndexArgs& a, int select_blocks, cudaStream_t s, int* launches) {
   const int blocks = phase_blocks(phase, a, select_blocks);
   if (blocks > 0) {
     a.stamp = next_stamp(ctx);
-    index_phase_kernel<phase><<<(unsigned)blocks, kIdxThreads, 0, s>>>(a);
+    const cudaError_t e = launch(index_phase_kernel<phase>, dim3((unsigned)blocks), kIdxThreads, 0, s, a);
+    if (e != cudaSuccess) return e;
     ++*launches;
   }
-  if constexpr (phase < kOrder) launch_phases_from<phase + 1>(ctx, a, select_blocks, s, launches);
+  if constexpr (phase < kOrder) return launch_phases_from<phase + 1>(ctx, a, select_blocks, s, launches);
+  return cudaSuccess;
 }
 
-// [ 3 histograms | long segments: count, rows | merged tokens per row ], zeroed for every plan
+// [ 3 histograms | long segments: count, rows | merged tokens per row ], first in the scratch array and zero
+// when a plan's build starts
 static long long zero_words(const Sizes& z) { return 3 * kSelBins + 1 + z.n_remove / kLongSegment + 1 + z.n_merged; }
 
 // Words of the index build's scratch array.
 long long index_scratch_words(const Sizes& z) {
   return round_up(zero_words(z), 4) + 8 + 2 * kIdxThreads + kIdxThreads + round_up(z.n_src, 4) + 5 * round_up(z.n_remove, 4);
+}
+
+ZeroWords index_zero_words(const litevggt_ctx* ctx) {
+  if (ctx->sz.n_tokens <= kSmallTokens) return ZeroWords{};  // the single block does it
+  return ZeroWords{reinterpret_cast<uint32_t*>(ctx->ws.index_scratch), zero_words(ctx->sz)};
 }
 
 cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStream_t s, int* launches) {
@@ -462,19 +470,19 @@ cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStrea
   a.status = ws.status;
   if (z.n_tokens <= kSmallTokens) {
     a.stamp = next_stamp(ctx);
-    index_small_kernel<<<1, kIdxThreads, 0, s>>>(a, zero, (int)zeroed);
     ++*launches;
-    return cudaGetLastError();
+    return launch(index_small_kernel, dim3(1), kIdxThreads, 0, s, a, zero, (int)zeroed);
   }
-  cudaError_t e = cudaMemsetAsync(zero, 0, (size_t)zeroed * 4, s);
-  if (e != cudaSuccess) return e;
+  if (z.n_src == 0) {  // no matching ran
+    cudaError_t e = cudaMemsetAsync(zero, 0, (size_t)zeroed * 4, s);
+    if (e != cudaSuccess) return e;
+  }
   // at most as many blocks as run at a time, and at least two (one means the single-block kernel): each
   // flushes a histogram
   long long select_blocks = (z.n_src + 4 * kIdxThreads - 1) / (4 * kIdxThreads);
   if (select_blocks > 2 * ctx->num_sms) select_blocks = 2 * ctx->num_sms;
   if (select_blocks < 2) select_blocks = 2;
-  launch_phases_from<kSelect0>(ctx, a, (int)select_blocks, s, launches);
-  return cudaGetLastError();
+  return launch_phases_from<kSelect0>(ctx, a, (int)select_blocks, s, launches);
 }
 
 }  // namespace lv

@@ -30,8 +30,8 @@ static int tile_columns(long long m, long long n, long long k, int num_sms) {
 // out [m, n] = epi(a [m, k] w [n, k]^T)
 template <class Epi>
 static cudaError_t launch_gemm_out(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k,
-                                   const __nv_bfloat16* w, long long n, __nv_bfloat16* out, const Epi& epi, cudaStream_t s,
-                                   int* launches) {
+                                   const __nv_bfloat16* w, long long n, __nv_bfloat16* out, const Epi& epi,
+                                   const ZeroWords& zero, cudaStream_t s, int* launches) {
   const int columns = tile_columns(m, n, k, ctx->num_sms), bn = columns != 0 ? columns : 256;
   CUtensorMap tmap_a, tmap_b, tmap_out;
   if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap_a, a, (uint64_t)k, (uint64_t)m, (uint64_t)k, kGemmBK, kGemmBM) ||
@@ -41,7 +41,7 @@ static cudaError_t launch_gemm_out(litevggt_ctx* ctx, const __nv_bfloat16* a, lo
     return cudaErrorInvalidValue;
   const long long rows = columns != 0 ? 2 * kGemmBM : kGemmBM, tiles = ((m + rows - 1) / rows) * ((n + bn - 1) / bn);
   ++*launches;
-  auto run = [&](auto launch) { return launch(tmap_a, tmap_b, tmap_out, m, n, k, epi, tiles, ctx->num_sms, ctx->ws.status, next_stamp(ctx), s); };
+  auto run = [&](auto launch) { return launch(tmap_a, tmap_b, tmap_out, m, n, k, epi, tiles, ctx->num_sms, ctx->ws.status, zero, next_stamp(ctx), s); };
   switch (columns) {
     case 0: return run(gemm_launch<Epi, 256, 1>);
     case 64: return run(gemm_launch<Epi, 64, 2>);
@@ -52,8 +52,15 @@ static cudaError_t launch_gemm_out(litevggt_ctx* ctx, const __nv_bfloat16* a, lo
 }
 
 cudaError_t launch_linear(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k, const __nv_bfloat16* w,
-                          long long n, const __nv_bfloat16* bias, __nv_bfloat16* out, cudaStream_t s, int* launches) {
-  return launch_linear_scaled(ctx, a, m, k, w, n, bias, 0, 0, 1.0f, LinearStat{}, out, s, launches);
+                          long long n, const __nv_bfloat16* bias, const ZeroWords& zero, __nv_bfloat16* out, cudaStream_t s,
+                          int* launches) {
+  if (m == 0) return cudaSuccess;
+  LinearEpilogue epi = {};
+  epi.bias = bias;
+  epi.m_rows = (int)m;
+  epi.n_cols = (int)n;
+  epi.scale = 1.0f;
+  return launch_gemm_out(ctx, a, m, k, w, n, out, epi, zero, s, launches);
 }
 
 cudaError_t launch_linear_scaled(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k,
@@ -62,11 +69,9 @@ cudaError_t launch_linear_scaled(litevggt_ctx* ctx, const __nv_bfloat16* a, long
                                  int* launches) {
   if (m == 0) return cudaSuccess;
   if (scale_begin % 64 != 0 || scale_end % 64 != 0) return cudaErrorInvalidValue;
-  if (stat.key_norm != nullptr || stat.amax != nullptr) {
-    if (stat.key_norm != nullptr && stat.seq_len <= 0) return cudaErrorInvalidValue;
-    const size_t words = stat.key_norm != nullptr ? (size_t)((m + stat.seq_len - 1) / stat.seq_len) * ((scale_end - scale_begin) / 64)
-                                                  : (size_t)(n / 64);
-    cudaError_t e = cudaMemsetAsync(stat.key_norm != nullptr ? stat.key_norm : stat.amax, 0, words * sizeof(float), s);
+  if (stat.key_norm != nullptr && stat.seq_len <= 0) return cudaErrorInvalidValue;
+  if (stat.amax != nullptr) {
+    cudaError_t e = cudaMemsetAsync(stat.amax, 0, (size_t)(n / 64) * sizeof(float), s);
     if (e != cudaSuccess) return e;
   }
   LinearEpilogue epi;
@@ -79,14 +84,15 @@ cudaError_t launch_linear_scaled(litevggt_ctx* ctx, const __nv_bfloat16* a, long
   epi.stat_kind = stat.key_norm != nullptr ? kStatKeyNorm : stat.amax != nullptr ? kStatAmax : kStatNone;
   epi.seq_len = (int)stat.seq_len;
   epi.stat = stat.key_norm != nullptr ? stat.key_norm : stat.amax;
-  return launch_gemm_out(ctx, a, m, k, w, n, out, epi, s, launches);
+  return launch_gemm_out(ctx, a, m, k, w, n, out, epi, ZeroWords{}, s, launches);
 }
 
 // out = act(a w^T + bias) + residual, the two layers of the transformer MLP (fc1: GELU, no residual;
 // fc2: identity, residual = the block's input).
 cudaError_t launch_linear_mlp(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k,
                               const __nv_bfloat16* w, long long n, const __nv_bfloat16* bias, int gelu,
-                              const __nv_bfloat16* residual, __nv_bfloat16* out, cudaStream_t s, int* launches) {
+                              const __nv_bfloat16* residual, const ZeroWords& zero, __nv_bfloat16* out, cudaStream_t s,
+                              int* launches) {
   if (m == 0) return cudaSuccess;
   MlpEpilogue epi;
   epi.bias = bias;
@@ -95,7 +101,7 @@ cudaError_t launch_linear_mlp(litevggt_ctx* ctx, const __nv_bfloat16* a, long lo
   epi.n_cols = (int)n;
   epi.ld_res = n;
   epi.gelu = gelu;
-  return launch_gemm_out(ctx, a, m, k, w, n, out, epi, s, launches);
+  return launch_gemm_out(ctx, a, m, k, w, n, out, epi, zero, s, launches);
 }
 
 }  // namespace lv

@@ -187,29 +187,26 @@ cudaError_t launch_layernorm(const __nv_bfloat16* x, const __nv_bfloat16* gamma,
                              int* launches) {
   if (rows == 0) return cudaSuccess;
   const unsigned blocks = (unsigned)((rows + kRowsPerCta - 1) / kRowsPerCta);
-  layernorm_kernel<<<blocks, kRowThreads, 0, s>>>(x, gamma, beta, out, rows, eps, stamp);
   ++*launches;
-  return cudaGetLastError();
+  return launch(layernorm_kernel, dim3(blocks), kRowThreads, 0, s, x, gamma, beta, out, rows, eps, stamp);
 }
 
 cudaError_t launch_merge(const litevggt_ctx* ctx, const litevggt_plan* plan, const __nv_bfloat16* x,
                          __nv_bfloat16* xm, cudaStream_t s, int* launches) {
   const Sizes& z = ctx->sz;
   const unsigned blocks = (unsigned)((z.n_merged + kRowsPerCta - 1) / kRowsPerCta);
-  merge_kernel<<<blocks, kRowThreads, 0, s>>>(x, plan->kept_idx, plan->seg_off, plan->seg_src, xm, z.n_merged,
-                                              z.n_tokens, z.n_remove, ctx->ws.status, next_stamp(ctx));
   ++*launches;
-  return cudaGetLastError();
+  return launch(merge_kernel, dim3(blocks), kRowThreads, 0, s, x, plan->kept_idx, plan->seg_off, plan->seg_src, xm, z.n_merged,
+                z.n_tokens, z.n_remove, ctx->ws.status, next_stamp(ctx));
 }
 
 cudaError_t launch_unmerge(const litevggt_ctx* ctx, const litevggt_plan* plan, const __nv_bfloat16* ym,
                            const __nv_bfloat16* residual, __nv_bfloat16* out, cudaStream_t s, int* launches) {
   const Sizes& z = ctx->sz;
   const unsigned blocks = (unsigned)((z.n_tokens + kRowsPerCta - 1) / kRowsPerCta);
-  unmerge_kernel<<<blocks, kRowThreads, 0, s>>>(ym, plan->dst_of, residual, out, z.n_tokens, z.n_merged,
-                                                ctx->ws.status, next_stamp(ctx));
   ++*launches;
-  return cudaGetLastError();
+  return launch(unmerge_kernel, dim3(blocks), kRowThreads, 0, s, ym, plan->dst_of, residual, out, z.n_tokens, z.n_merged,
+                ctx->ws.status, next_stamp(ctx));
 }
 
 }  // namespace lv

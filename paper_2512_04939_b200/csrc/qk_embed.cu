@@ -182,16 +182,12 @@ cudaError_t launch_qk_embed(const litevggt_ctx* ctx, __nv_bfloat16* qkv, const i
   p.n_special = (int)z.n_special;
   p.grid_w = (int)z.grid_w;
   p.key_norm = key_norm;
-  if (key_norm != nullptr) {
-    cudaError_t e = cudaMemsetAsync(key_norm, 0, 16 * sizeof(float), s);
-    if (e != cudaSuccess) return e;
-  }
   // as many blocks as an SM holds at a time: the key norms of a block's rows meet in one atomic per head
   long long blocks = (m + kEmbedRowsPerCta - 1) / kEmbedRowsPerCta;
   if (blocks > 8ll * ctx->num_sms) blocks = 8ll * ctx->num_sms;
-  qk_embed_kernel<<<(unsigned)blocks, kEmbedThreads, 0, s>>>(qkv, kept_idx, m, z.n_tokens, p, ctx->ws.status, next_stamp(ctx));
   ++*launches;
-  return cudaGetLastError();
+  return launch(qk_embed_kernel, dim3((unsigned)blocks), kEmbedThreads, 0, s, qkv, kept_idx, m, z.n_tokens, p, ctx->ws.status,
+                next_stamp(ctx));
 }
 
 }  // namespace lv

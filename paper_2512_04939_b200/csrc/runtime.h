@@ -152,6 +152,42 @@ struct litevggt_plan {
 
 namespace lv {
 
+// Enqueues a kernel of this library on `s`, `cluster` CTAs to a cluster.  With `overlap` and a grid of at most
+// kOverlapBlocks blocks it may start before the kernel in front of it has ended - each calls
+// wait_for_previous_kernel (common.cuh) before it touches memory, so what overlaps is launch latency and
+// set-up: 288 -> 255 us for a block over seven frames, 116 -> 94 us for the first layer of four small
+// ones.  Larger grids gain nothing by it, and asking costs their short blocks time (LayerNorm of 208 K
+// rows: 145 -> 181 us).
+constexpr long long kOverlapBlocks = 148 * 8;
+template <class... P, class... A>
+inline cudaError_t launch_clusters(int cluster, bool overlap, void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem,
+                                   cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute attrs[2];
+  unsigned n = 0;
+  if (overlap && (long long)grid.x * grid.y * grid.z <= kOverlapBlocks) {
+    attrs[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attrs[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attrs[n].id = cudaLaunchAttributeClusterDimension;
+    attrs[n].val.clusterDim.x = (unsigned)cluster;
+    attrs[n].val.clusterDim.y = 1;
+    attrs[n++].val.clusterDim.z = 1;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attrs;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(args)...);
+}
+template <class... P, class... A>
+inline cudaError_t launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A&&... args) {
+  return launch_clusters(1, true, kernel, grid, threads, smem, s, static_cast<A&&>(args)...);
+}
+
 // The stamp of the step's next kernel.
 inline Stamp next_stamp(const litevggt_ctx* ctx) {
   const Stamp s = ctx->step;
@@ -165,6 +201,12 @@ constexpr uint32_t kStatusBounds = 2u;
 
 constexpr uint32_t kCtxMagic = 0x4c564358u;
 constexpr uint32_t kPlanMagic = 0x4c56504cu;
+
+// Words that a launch sets to zero for whoever comes after it.
+struct ZeroWords {
+  uint32_t* words = nullptr;
+  long long count = 0;
+};
 
 // tensor_map.cu
 bool resolve_encode_tiled(void** fn);
@@ -190,6 +232,8 @@ cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, cudaStream_t
 // index_build.cu
 cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStream_t s, int* launches);
 long long index_scratch_words(const Sizes& z);
+// the part of the scratch array that has to be zero before launch_index_build; the matching sees to it
+ZeroWords index_zero_words(const litevggt_ctx* ctx);
 
 // merge_unmerge.cu
 cudaError_t launch_merge(const litevggt_ctx* ctx, const litevggt_plan* plan, const __nv_bfloat16* x,
@@ -199,14 +243,17 @@ cudaError_t launch_unmerge(const litevggt_ctx* ctx, const litevggt_plan* plan, c
 
 // linear.cu
 cudaError_t launch_linear(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k, const __nv_bfloat16* w,
-                          long long n, const __nv_bfloat16* bias, __nv_bfloat16* out, cudaStream_t s, int* launches);
+                          long long n, const __nv_bfloat16* bias, const ZeroWords& zero, __nv_bfloat16* out, cudaStream_t s,
+                          int* launches);
 // The same with output columns [scale_begin, scale_end) (multiples of 64) multiplied by `scale` in
 // fp32 before the one rounding to bf16: the QKV projection of an attention layer scales its K columns.
-// It also leaves behind one of two statistics of the rounded output, zeroed here first:
+// It also leaves behind one of two statistics
+// of the rounded output.  Zeroing the key norms takes no launch: they are zero between calls, because
+// the output projection, which runs after their last reader, leaves them so.
 struct LinearStat {
   float* key_norm = nullptr;  // [sequences, heads] largest |k|^2 over the columns [scale_begin, scale_end) ...
   long long seq_len = 0;      // ... of sequences of this many rows
-  float* amax = nullptr;      // [n / 64] largest magnitude of every 64 columns
+  float* amax = nullptr;      // [n / 64] largest magnitude of every 64 columns, zeroed here first
 };
 cudaError_t launch_linear_scaled(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k,
                                  const __nv_bfloat16* w, long long n, const __nv_bfloat16* bias, int scale_begin,
@@ -215,7 +262,8 @@ cudaError_t launch_linear_scaled(litevggt_ctx* ctx, const __nv_bfloat16* a, long
 
 cudaError_t launch_linear_mlp(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k,
                               const __nv_bfloat16* w, long long n, const __nv_bfloat16* bias, int gelu,
-                              const __nv_bfloat16* residual, __nv_bfloat16* out, cudaStream_t s, int* launches);
+                              const __nv_bfloat16* residual, const ZeroWords& zero, __nv_bfloat16* out, cudaStream_t s,
+                              int* launches);
 cudaError_t launch_layernorm(const __nv_bfloat16* x, const __nv_bfloat16* gamma, const __nv_bfloat16* beta,
                              __nv_bfloat16* out, long long rows, float eps, const Stamp& stamp, cudaStream_t s,
                              int* launches);

@@ -193,12 +193,11 @@ cudaError_t launch_grad_map(const litevggt_ctx* ctx, const float* images, float*
   const int strips = (z.grid_w + pps - 1) / pps;
   const dim3 grid((unsigned)((strips + kGradThreads / 32 - 1) / (kGradThreads / 32)),
                   (unsigned)((z.grid_h + kGradPatchRows - 1) / kGradPatchRows), (unsigned)z.frames);
-  if (patch == 14)
-    grad_map_patch_kernel<14, LV_GRAD_AHEAD14><<<grid, kGradThreads, 0, s>>>(images, grad, z.grid_h, z.grid_w, next_stamp(ctx));
-  else
-    grad_map_kernel<<<grid, kGradThreads, 0, s>>>(images, grad, z.grid_h, z.grid_w, patch, next_stamp(ctx));
   ++*launches;
-  return cudaGetLastError();
+  if (patch == 14)
+    return launch(grad_map_patch_kernel<14, LV_GRAD_AHEAD14>, grid, kGradThreads, 0, s, images, grad, z.grid_h, z.grid_w,
+                  next_stamp(ctx));
+  return launch(grad_map_kernel, grid, kGradThreads, 0, s, images, grad, z.grid_h, z.grid_w, patch, next_stamp(ctx));
 }
 
 // ----------------------------------------------------------------------------------------
@@ -426,9 +425,9 @@ cudaError_t launch_var_map(const litevggt_ctx* ctx, const __nv_bfloat16* x, floa
   const Sizes& z = ctx->sz;
   if (z.grid_w > kVarMaxW) return cudaErrorInvalidValue;
   const unsigned strips = (unsigned)((z.grid_h + kVarRows - 1) / kVarRows);
-  var_map_kernel<<<dim3(strips, z.frames), kVarThreads, 0, s>>>(x, var, z.grid_h, z.grid_w, z.n_special, next_stamp(ctx));
   ++*launches;
-  return cudaGetLastError();
+  return launch(var_map_kernel, dim3(strips, z.frames), kVarThreads, 0, s, x, var, z.grid_h, z.grid_w, z.n_special,
+                next_stamp(ctx));
 }
 
 // ----------------------------------------------------------------------------------------
@@ -593,14 +592,10 @@ partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, 
 cudaError_t launch_partition(const litevggt_ctx* ctx, const float* grad, const float* var, float* ga, uint8_t* cls,
                              cudaStream_t s, int* launches) {
   const Sizes& z = ctx->sz;
-  const size_t smem = (size_t)z.patches * (sizeof(float) + 1) + 16;
-  cudaError_t e = cudaFuncSetAttribute(partition_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  partition_kernel<<<z.frames, kPartThreads, smem, s>>>(grad, var, ga, cls, z.grid_h, z.grid_w, z.n_special,
-                                                        z.n_ga_frame, ctx->cfg.cell_h, ctx->cfg.cell_w,
-                                                        ctx->cfg.alpha, ctx->cfg.beta, next_stamp(ctx));
+  const size_t smem = (size_t)z.patches * (sizeof(float) + 1) + 16;  // at most 41 KB (8192 patches)
   ++*launches;
-  return cudaGetLastError();
+  return launch(partition_kernel, dim3(z.frames), kPartThreads, smem, s, grad, var, ga, cls, z.grid_h, z.grid_w, z.n_special,
+                z.n_ga_frame, (int)ctx->cfg.cell_h, (int)ctx->cfg.cell_w, ctx->cfg.alpha, ctx->cfg.beta, next_stamp(ctx));
 }
 
 // ----------------------------------------------------------------------------------------
@@ -671,10 +666,9 @@ build_lists_kernel(const uint8_t* __restrict__ cls, int* __restrict__ src_list, 
 cudaError_t launch_build_lists(const litevggt_ctx* ctx, const uint8_t* cls, int* src_list, int* dst_list, int* src_pos,
                                cudaStream_t s, int* launches) {
   const Sizes& z = ctx->sz;
-  build_lists_kernel<<<z.frames, kListThreads, 0, s>>>(cls, src_list, dst_list, src_pos, z.patches, z.n_special,
-                                                       z.n_src_frame, z.n_dst_frame, ctx->ws.status, next_stamp(ctx));
   ++*launches;
-  return cudaGetLastError();
+  return launch(build_lists_kernel, dim3(z.frames), kListThreads, 0, s, cls, src_list, dst_list, src_pos, z.patches, z.n_special,
+                z.n_src_frame, z.n_dst_frame, ctx->ws.status, next_stamp(ctx));
 }
 
 }  // namespace lv

@@ -68,11 +68,9 @@ cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, cudaStream_t
   const long long n_dst_padded = round_up(z.n_dst, 256);
   const long long rows = z.n_src + n_dst_padded;
   const int warps = kPackThreads / 32;
-  pack_rows_kernel<<<(unsigned)((rows + warps - 1) / warps), kPackThreads, 0, s>>>(
-      x, ws.src_list, ws.dst_list, z.n_src, z.n_dst, n_dst_padded, z.n_tokens, ws.panel_src, ws.panel_dst,
+  cudaError_t e = launch(pack_rows_kernel, dim3((unsigned)((rows + warps - 1) / warps)), kPackThreads, 0, s, x, ws.src_list, ws.dst_list, z.n_src, z.n_dst, n_dst_padded, z.n_tokens, ws.panel_src, ws.panel_dst,
       ws.inv_norm_src, ws.inv_norm_dst, ws.match_keys, ws.status, next_stamp(ctx));
   ++*launches;
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
 
   // columns of a tile: 256, unless narrower ones spread few rows over more of the chip
@@ -94,9 +92,10 @@ cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, cudaStream_t
   epi.m_rows = (int)z.n_src;
   epi.n_cols = (int)z.n_dst;
   const long long tiles = row_blocks * ((z.n_dst + bn - 1) / bn);
+  const ZeroWords zero = index_zero_words(ctx);
   // the argmax epilogue writes no matrix: the store map is never read, any valid map fills the slot
   auto run = [&](auto launch) {
-    return launch(tmap_a, tmap_b, tmap_a, z.n_src, z.n_dst, 1024, epi, tiles, ctx->num_sms, ws.status, next_stamp(ctx), s);
+    return launch(tmap_a, tmap_b, tmap_a, z.n_src, z.n_dst, 1024, epi, tiles, ctx->num_sms, ws.status, zero, next_stamp(ctx), s);
   };
   e = bn == 256 ? run(gemm_launch<ArgmaxEpilogue, 256, 2>)
                 : bn == 128 ? run(gemm_launch<ArgmaxEpilogue, 128, 2>) : run(gemm_launch<ArgmaxEpilogue, 64, 2>);
