@@ -10,14 +10,14 @@
 // 128) tiles and not for an even number of them.  What a sequence of 1041 rows (a 28 x 37 frame) spends
 // outside its nine key tiles bounded it; the frame-local layer of 200 such frames, projections
 // included, went from 3.09 to 2.58 ms.  The pair of tiles reads every K/V tile once for 256 rows and
-// is the faster one when the sweep is long and the chip runs into its power cap: 297 us (one tile)
-// against 304 at 8.3 K rows, 1.80 ms each at 22 K, 10.6 to 11.1 ms against 10.3 to 10.7 at 52 K, 28.6
-// against 28.2 at 83 K.  Warp roles of the pair (20 warps):
-//   warps 0-15  softmax.  Warp w works on query tile t = w / 8, TMEM lane quarter w % 4 (one
-//               thread = one query row) and the column half c = (w / 4) % 2 of every step:
-//               32 of the step's 64 scores per row.  The two threads of a row swap their
-//               partial row maxima through shared memory once per step.  Four softmax warps
-//               per scheduler keep the special-function unit busy while others wait.
+// is the faster one when the sweep is longer: 286 us (one tile) against 279 at 8.3 K rows, 80 each at
+// 4.2 K.  Warp roles of the pair (20 warps):
+//   warps 0-15  softmax.  Warp w works on query tile t = w / 8 and TMEM lane quarter w % 4 (one
+//               thread = one query row); the two warps of a (tile, quarter), c = (w / 4) % 2, either
+//               take every other step whole or share each, 32 of its 64 scores per row and warp
+//               (see the sweep in the kernel).  In the online form, which shares, the two threads of
+//               a row swap their partial row maxima through shared memory once per step.  Four
+//               softmax warps per scheduler keep the special-function unit busy while others wait.
 //   warp  16    MMA issuer of tile 0 (one elected lane):  S_h = Q K_jh^T  and  O += P_h V_jh
 //   warp  17    TMA producer (one elected lane): K_j / V_j through two 4-stage shared-memory rings
 //   warp  18    MMA issuer of tile 1 (issuing costs tens of cycles per instruction, so one
@@ -90,6 +90,8 @@
 // maximum, the running output rescaled only when a row maximum grows by more than 2^8 over the
 // reference (the threads then first wait until the tile's last P V has retired).  All three equal
 // the plain softmax up to rounding.
+#include <type_traits>
+
 #include "common.cuh"
 #include "runtime.h"
 
@@ -135,7 +137,7 @@ constexpr int kFaShiftPolyPairs = LV_FA_SHIFT_POLY_PAIRS;
 constexpr float kFaShiftUp = 84.0f, kFaShiftDown = 92.0f;
 // Sequences of at most this many rows take CTAs of one query tile, two to an SM (figures at the top).
 #ifndef LV_FA_ONE_TILE_ROWS
-#define LV_FA_ONE_TILE_ROWS 16384
+#define LV_FA_ONE_TILE_ROWS 4096
 #endif
 constexpr long long kFaOneTileRows = LV_FA_ONE_TILE_ROWS;
 
@@ -518,6 +520,53 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
     float m_ref = -INFINITY;  // reference, in the scores' own (base-2) units
     bool ok = true;
     int pair_syncs = 0;  // both warps of a pair must pass the same number of pair barriers
+    // The sweep of a row whose reference stays what it is: `exps` turns 32 scores into 16 bf16 pairs.  The two
+    // warps of a pair need nothing from each other here, so in the CTA of two tiles (kWide) each takes every
+    // other step whole - one wait and one hand-over for 64 scores a thread where sharing a step pays for
+    // both twice: 1.85 -> 1.79 ms at 22 K rows, 3.73 -> 3.62 at 32 K, 11.2 -> 10.7 at 52 K, 28.9 -> 27.9 at
+    // 83 K.  With one tile, where a sweep is short, sharing gives the shorter step: 286 us either way at 8.3
+    // K rows, 20.4 against 21.7 at 1.8 K.  (Loading 16 or 32 scores ahead of the exponentials
+    // measured the same or, where it spilled, less.)
+    // Only the last tile of a launch can reach past the sequence, so the steps before it need no masking;
+    // shared steps are written out per half so that barrier and tensor-memory addresses are constants of
+    // the loop.
+    constexpr bool kWide = kTiles == 2;
+    auto sweep = [&](auto exps) {
+      auto step = [&](int j, int h, bool may_mask) -> bool {
+        if (!mbar_wait_warp(&bars->s_full[t][h], j & 1, ctl)) return false;
+        tc_fence_after();
+#pragma unroll
+        for (int i = 0; i < (kWide ? 2 : 1); ++i) {
+          const int g = kWide ? i : c;  // columns [32 g, 32 g + 32) of the half
+          const uint32_t addr = s_addr + h * 64 + g * 32;
+          uint32_t s[32], packed[16];
+          tmem_ld32(addr, s);
+          tmem_ld_wait();
+          const int valid = may_mask ? seq_len - ((tile_begin + j) * 2 + h) * 64 - g * 32 : 32;
+          if (may_mask && valid < 32) {
+#pragma unroll
+            for (int k = 0; k < 32; ++k)
+              if (k >= valid) s[k] = 0xff800000u;  // -inf: probability 0
+            exps(s, packed, std::true_type{});
+          } else {
+            exps(s, packed, std::false_type{});
+          }
+          tmem_st16(addr, packed);  // over the start of the columns just read
+        }
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_count(&bars->p_ready[t][h], kWide ? 2 : 1);
+        return true;
+      };
+      if constexpr (kWide) {
+        for (int j = 0; j + 1 < n_kv && ok; ++j) ok = step(j, c, false);
+        if (ok && n_kv > 0 && !(half_tail && c == 1)) ok = step(n_kv - 1, c, true);
+      } else {
+        for (int j = 0; j + 1 < n_kv && ok; ++j) ok = step(j, 0, false) && step(j, 1, false);
+        if (ok && n_kv > 0) ok = step(n_kv - 1, 0, true) && (half_tail || step(n_kv - 1, 1, true));
+      }
+    };
     if (q0 + t * 128 + (int)quarter * 32 >= seq_len) {
       // ---- no live row in this warp (nor in its partner): the issuer needs the hand-over, nobody the result
       pair_syncs = n_steps;
@@ -532,34 +581,9 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       // they come out of the tensor core.
       m_ref = 0.0f;
       pair_syncs = n_steps;  // this form has no pair barriers
-      // One step = this thread's 32 scores of one half of a key tile.  Only the last tile of a
-      // launch can reach past the sequence, so the steps before it need no masking; the two halves
-      // are written out so that barrier and tensor-memory addresses are constants of the loop.
-      auto step = [&](int j, int h, bool may_mask) -> bool {
-        if (!mbar_wait_warp(&bars->s_full[t][h], j & 1, ctl)) return false;
-        tc_fence_after();
-        uint32_t s[32];
-        tmem_ld32(s_addr + h * 64 + c * 32, s);
-        tmem_ld_wait();
-        uint32_t packed[16];
-        const int valid = may_mask ? seq_len - ((tile_begin + j) * 2 + h) * 64 - c * 32 : 32;
-        if (may_mask && valid < 32) {
-#pragma unroll
-          for (int i = 0; i < 32; ++i)
-            if (i >= valid) s[i] = 0xff800000u;  // -inf: probability 0 (the polynomial cannot take it)
-          exp2_chunk<0>(s, packed);
-        } else {
-          exp2_chunk<kFaPolyPairs>(s, packed);
-        }
-        tmem_st16(s_addr + h * 64 + c * 32, packed);  // over the start of the columns just read
-        tmem_st_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bars->p_ready[t][h]);
-        return true;
-      };
-      for (int j = 0; j + 1 < n_kv && ok; ++j) ok = step(j, 0, false) && step(j, 1, false);
-      if (ok && n_kv > 0) ok = step(n_kv - 1, 0, true) && (half_tail || step(n_kv - 1, 1, true));
+      sweep([](const uint32_t (&s)[32], uint32_t (&packed)[16], auto masked) {
+        exp2_chunk<decltype(masked)::value ? 0 : kFaPolyPairs>(s, packed);  // (the polynomial cannot take -inf)
+      });
     } else {
     // ---- a reference that is not zero.  The first step's scores are looked at once (they stay where
     // they are for the sweep): their maximum is a lower bound of the row maximum, score_bound an upper one.
@@ -592,31 +616,10 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
     // nothing overflows and the row's largest probability is not small, so no running maximum is
     // needed.
     pair_syncs = n_steps;
-    auto step = [&](int j, int h, bool may_mask) -> bool {
-      if (!mbar_wait_warp(&bars->s_full[t][h], j & 1, ctl)) return false;
-      tc_fence_after();
-      uint32_t s[32];
-      tmem_ld32(s_addr + h * 64 + c * 32, s);
-      tmem_ld_wait();
-      uint32_t packed[16];
-      const int valid = may_mask ? seq_len - ((tile_begin + j) * 2 + h) * 64 - c * 32 : 32;
-      if (may_mask && valid < 32) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-          if (i >= valid) s[i] = 0xff800000u;  // -inf: probability 0 (the polynomial cannot take it)
-        exp2_chunk_shifted<0>(s, m_ref, packed);
-      } else {
-        exp2_chunk_shifted<kFaShiftPolyPairs>(s, m_ref, packed);
-      }
-      tmem_st16(s_addr + h * 64 + c * 32, packed);  // over the start of the columns just read
-      tmem_st_wait();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->p_ready[t][h]);
-      return true;
-    };
-    for (int j = 0; j + 1 < n_kv && ok; ++j) ok = step(j, 0, false) && step(j, 1, false);
-    if (ok && n_kv > 0) ok = step(n_kv - 1, 0, true) && (half_tail || step(n_kv - 1, 1, true));
+    const float m = m_ref;
+    sweep([m](const uint32_t (&s)[32], uint32_t (&packed)[16], auto masked) {
+      exp2_chunk_shifted<decltype(masked)::value ? 0 : kFaShiftPolyPairs>(s, m, packed);
+    });
     } else if (ok) {
     // ---- online form; the same two written-out halves per key tile as above
     auto step = [&](int j, int h, bool may_mask) -> bool {
@@ -765,7 +768,8 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
 //     sit at the top of that range: every row runs the online form with the reference kept 8 below
 //     the running row maximum (the largest probability of a row is 2^8 when the reference is set
 //     and may grow to 2^8.75 before the row is rescaled), which leaves 17 binades below the row
-//     maximum before a probability is rounded to zero;
+//     maximum before a probability is rounded to zero; the two warps of a pair take a half of
+//     every key tile each and pass the reference on from step to step;
 //   * scores are multiplied by scale_q scale_k (K arrives with the softmax scale folded in, which its
 //     per-head scale absorbs), the output by scale_v, in fp32.
 constexpr int kFa8KTileBytes = 128 * 64;           // 128 keys x 64 channel bytes
@@ -773,7 +777,42 @@ constexpr int kFa8VTileBytes = 64 * 128;           // 64 channels x 128 key byte
 constexpr int kFa8VStageBytes = kFa8VTileBytes + 16 * 128;  // + the ones rows
 constexpr uint32_t kFa8ColQ = 416;                 // Q_0, Q_1: 16 columns of 4 bytes each
 constexpr float kFa8Headroom = 8.0f;               // the row maximum maps to 2^8 of E4M3's 448
-constexpr int kFa8SmemBytes = kFaStages * (kFa8KTileBytes + kFa8VStageBytes) + (int)sizeof(FaExchange<2>) + 512 + 1024;
+// What the two warps of a pair hand each other: the reference of their 32 rows after every step, and the
+// barriers that say so.
+struct Fa8Refs {
+  float m_ref[2][2][128];       // [column of steps][tile][row]
+  uint64_t ready[2][2][4];      // [column of steps][tile][quarter]
+};
+constexpr int kFa8SmemBytes = kFaStages * (kFa8KTileBytes + kFa8VStageBytes) + (int)sizeof(Fa8Refs) + 512 + 1024;
+
+// Of the 16 pairs of 32 scores, this many take the polynomial exponential.  Core at 21,984 rows: 4 pairs
+// 2.20 ms, 5: 2.14, 6: 2.14, 7: 2.16 (0, with both halves read twice: 2.32); 2.22 when the two warps of a
+// pair shared every step and swapped row maxima in it.
+#ifndef LV_FA8_POLY_PAIRS
+#define LV_FA8_POLY_PAIRS 6
+#endif
+constexpr int kFa8PolyPairs = LV_FA8_POLY_PAIRS;
+
+// 32 scores -> 32 E4M3 probabilities 2^(s * scale - m)
+__device__ __forceinline__ void exp2_chunk_e4m3(const uint32_t (&s)[32], float2 scale2, float2 neg_m2, uint32_t (&packed)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    float2 p[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int pair = 2 * i + k;
+      float2 x = __ffma2_rn(make_float2(__uint_as_float(s[2 * pair]), __uint_as_float(s[2 * pair + 1])), scale2, neg_m2);
+      if (pair < kFa8PolyPairs) {
+        // (below 2^-10 an E4M3 probability is zero; the polynomial takes arguments down to -120)
+        p[k] = poly_exp2_pair(make_float2(fmaxf(x.x, -64.0f), fmaxf(x.y, -64.0f)));
+      } else {
+        p[k].x = fast_exp2(x.x);
+        p[k].y = fast_exp2(x.y);
+      }
+    }
+    packed[i] = pack_e4m3x4(p[0].x, p[0].y, p[1].x, p[1].y);
+  }
+}
 
 template <bool kFirst, bool kLast>
 __global__ void __launch_bounds__(kFaThreads, 1)
@@ -785,14 +824,13 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* smem_k = smem;
   uint8_t* smem_v = smem_k + kFaStages * kFa8KTileBytes;
-  FaExchange<2>* xchg = reinterpret_cast<FaExchange<2>*>(smem_v + kFaStages * kFa8VStageBytes);
-  FaBarriers<kFaStages>* bars = reinterpret_cast<FaBarriers<kFaStages>*>(xchg + 1);
+  Fa8Refs* refs = reinterpret_cast<Fa8Refs*>(smem_v + kFaStages * kFa8VStageBytes);
+  FaBarriers<kFaStages>* bars = reinterpret_cast<FaBarriers<kFaStages>*>(refs + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q0 = blockIdx.x * 256;
   const int head = blockIdx.y;
   const int n_kv = tile_end - tile_begin;
-  const int n_steps = 2 * n_kv;
   constexpr bool first_chunk = kFirst;
   constexpr bool last_chunk = kLast;
 
@@ -812,6 +850,7 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
       mbar_init(&bars->pv_done[t], 1);
       mbar_init(&bars->o_done[t], 1);
     }
+    for (int i = 0; i < 16; ++i) mbar_init(&refs->ready[0][0][0] + i, 1);
     mbar_init(&bars->teardown[0], 1);
     mbar_init(&bars->teardown[1], 1);
     bars->abort_flag = 0;
@@ -926,14 +965,13 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
     const int t = warp >> 3;
     const int c = (warp >> 2) & 1;
     const uint32_t quarter = warp & 3u;
-    const int barrier_id = 1 + t * 4 + (int)quarter;
     const int row_in_tile = (int)quarter * 32 + lane;
     const uint32_t lane_base = (quarter * 32u) << 16;
     const int row_local = q0 + t * 128 + row_in_tile;
     const bool row_live = row_local < seq_len;
     const int row = row_local;
     const uint32_t s_addr = tmem_base + lane_base + kFaColS + t * 128;
-    const uint32_t o_addr = tmem_base + lane_base + kFaColO + t * kFaOCols + c * 32;
+    const uint32_t o_row = tmem_base + lane_base + kFaColO + t * kFaOCols, o_addr = o_row + c * 32;
     const uint32_t l_addr = tmem_base + lane_base + kFaColO + t * kFaOCols + 64;
     {
       // this thread's 32 channels (32 bytes) of its query row
@@ -960,75 +998,79 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
     const float2 scale2 = make_float2(scale_log2e, scale_log2e);
     float m_ref = -INFINITY;
     bool ok = true;
-    int pair_syncs = 0;
-    // the two halves of a key tile are written out (barrier and tensor-memory addresses constant);
-    // only the last tile of a launch can reach past the sequence
-    auto step = [&](int j, int h, bool may_mask) -> bool {
-      if (!mbar_wait_warp(&bars->s_full[t][h], j & 1, ctl)) return false;
+    // Warp c of a pair takes half c of every key tile whole (64 scores a thread) and they alternate: each
+    // step starts from the reference the partner's step before it left, and leaves its own as soon as the
+    // step's maximum is known - before its exponentials, so the partner does not wait for those.  Only
+    // the last tile of a launch can reach past the sequence.
+    auto step = [&](int j, bool may_mask) -> bool {
+      if (!mbar_wait_warp(&bars->s_full[t][c], j & 1, ctl)) return false;
       tc_fence_after();
-      uint32_t s[32];
-      tmem_ld32(s_addr + h * 64 + c * 32, s);
-      tmem_ld_wait();
-      if (may_mask) {
-        const int valid = seq_len - ((tile_begin + j) * 2 + h) * 64 - c * 32;
-        if (valid < 32) {
+      const uint32_t base = s_addr + c * 64;
+      const int valid = may_mask ? seq_len - ((tile_begin + j) * 2 + c) * 64 : 64;
+      auto load = [&](int g, uint32_t (&s)[32]) {
+        tmem_ld32(base + g * 32, s);
+        tmem_ld_wait();
+        if (may_mask && valid - g * 32 < 32) {
 #pragma unroll
           for (int i = 0; i < 32; ++i)
-            if (i >= valid) s[i] = 0xff800000u;  // -inf
+            if (i >= valid - g * 32) s[i] = 0xff800000u;  // -inf
         }
+      };
+      // the first 32 scores are read once for the maximum and once more for the exponentials: 64 held
+      // meanwhile would spill
+      uint32_t s[32];
+      load(0, s);
+      float mx_scaled = max32(s);
+      load(1, s);
+      mx_scaled = fmaxf(mx_scaled, max32(s)) * scale_log2e;
+      bool grow = true;
+      if ((j | c) != 0) {
+        if (!mbar_wait_warp(&refs->ready[c ^ 1][t][quarter], (uint32_t)(c == 1 ? j : j - 1) & 1u, ctl)) return false;
+        m_ref = refs->m_ref[c ^ 1][t][row_in_tile];
+        grow = mx_scaled > m_ref + kFa8Headroom + 0.75f;
       }
-      const float mx_own = max32(s);
-      xchg->row_max[h][t][c][row_in_tile] = mx_own;
-      pair_barrier(barrier_id);
-      ++pair_syncs;
-      const float mx_scaled = fmaxf(mx_own, xchg->row_max[h][t][c ^ 1][row_in_tile]) * scale_log2e;
-      if ((j | h) == 0) {
-        m_ref = mx_scaled - kFa8Headroom;
-      } else {
-        const bool grow = mx_scaled > m_ref + kFa8Headroom + 0.75f;
-        if (__any_sync(0xffffffffu, grow ? 1 : 0)) {
-          const int jp = h == 1 ? j : j - 1;
-          const bool waited = jp + 1 < n_kv
-                                  ? mbar_wait_warp(&bars->s_full[t][h ^ 1], (uint32_t)(jp + 1) & 1u, ctl)
-                                  : mbar_wait_warp(&bars->pv_done[t], 0, ctl);
-          if (!waited) return false;
-          tc_fence_after();
-          const float m_new = grow ? mx_scaled - kFa8Headroom : m_ref;
-          const float alpha = fast_exp2(m_ref - m_new);
-          m_ref = m_new;
-          uint32_t acc[32];
-          tmem_ld32(o_addr, acc);
+      const float m_old = m_ref;
+      if (grow) m_ref = mx_scaled - kFa8Headroom;
+      refs->m_ref[c][t][row_in_tile] = m_ref;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&refs->ready[c][t][quarter]);
+      if ((j | c) != 0 && __any_sync(0xffffffffu, grow ? 1 : 0)) {
+        // O_t may still be the target of the previous step's P V; what follows that tells when it has retired
+        const int jp = c == 1 ? j : j - 1;
+        const bool waited = jp + 1 < n_kv ? mbar_wait_warp(&bars->s_full[t][c ^ 1], (uint32_t)(jp + 1) & 1u, ctl)
+                                          : mbar_wait_warp(&bars->pv_done[t], 0, ctl);
+        if (!waited) return false;
+        tc_fence_after();
+        const float alpha = fast_exp2(m_old - m_ref);
+#pragma unroll 1
+        for (int g = 0; g < 5; ++g) {  // the row's 64 output channels, then its sum and 15 unused columns
+          uint32_t acc[16];
+          tmem_ld16(o_row + g * 16, acc);
           tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 32; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * alpha);
-          tmem_st32(o_addr, acc);
-          if (c == 1) {
-            uint32_t sum[16];
-            tmem_ld16(l_addr, sum);
-            tmem_ld_wait();
-            sum[0] = __float_as_uint(__uint_as_float(sum[0]) * alpha);
-            tmem_st16(l_addr, sum);
-          }
+          for (int i = 0; i < 16; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * alpha);
+          tmem_st16(o_row + g * 16, acc);
         }
       }
       const float2 neg_m2 = make_float2(-m_ref, -m_ref);
-      uint32_t packed[8];  // 32 probabilities as E4M3 bytes
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float2 x0 = __ffma2_rn(make_float2(__uint_as_float(s[4 * i]), __uint_as_float(s[4 * i + 1])), scale2, neg_m2);
-        const float2 x1 = __ffma2_rn(make_float2(__uint_as_float(s[4 * i + 2]), __uint_as_float(s[4 * i + 3])), scale2, neg_m2);
-        packed[i] = pack_e4m3x4(fast_exp2(x0.x), fast_exp2(x0.y), fast_exp2(x1.x), fast_exp2(x1.y));
-      }
-      tmem_st8(s_addr + h * 64 + c * 32, packed);  // over the start of the columns just read
+      uint32_t packed[8];  // 32 probabilities as E4M3 bytes, over the start of their scores' columns
+      exp2_chunk_e4m3(s, scale2, neg_m2, packed);
+      tmem_st8(base + 32, packed);
+      load(0, s);
+      exp2_chunk_e4m3(s, scale2, neg_m2, packed);
+      tmem_st8(base, packed);
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->p_ready[t][h]);
+      if (lane == 0) mbar_arrive_count(&bars->p_ready[t][c], 2);
       return true;
     };
-    for (int j = 0; j + 1 < n_kv && ok; ++j) ok = step(j, 0, false) && step(j, 1, false);
-    if (ok && n_kv > 0) ok = step(n_kv - 1, 0, true) && step(n_kv - 1, 1, true);
-    for (; pair_syncs < n_steps; ++pair_syncs) pair_barrier(barrier_id);
+    for (int j = 0; j + 1 < n_kv && ok; ++j) ok = step(j, false);
+    if (ok && n_kv > 0) ok = step(n_kv - 1, true);
+    if (ok && c == 0 && n_kv > 0) {  // the last step was the partner's
+      ok = mbar_wait_warp(&refs->ready[1][t][quarter], (uint32_t)(n_kv - 1) & 1u, ctl);
+      if (ok) m_ref = refs->m_ref[1][t][row_in_tile];
+    }
     if (ok && mbar_wait_warp(&bars->o_done[t], 0, ctl)) {
       tc_fence_after();
       uint32_t acc[32], sum[16];

@@ -884,3 +884,19 @@ def test_fp8_attention_variant_with_peaked_softmax(lib):
     ref_short = O.attention_core(deq[keep], heads=16, rows=np.arange(200))
     assert rel_err(o[rows], ref_short) > 4 * (bf16_bound(ref_o) + FP8_PEAKED_NOISE)
     ctx.close()
+
+
+@pytest.mark.parametrize("grid", [(1, 1), (1, 59), (4, 15), (3, 41), (4, 31), (4, 47), (14, 18)], ids=lambda g: f"{g[0]}x{g[1]}")
+def test_fp8_attention_at_tile_edges(lib, grid):
+    """6 to 257 rows: one and several key tiles, ragged halves, the reference handed from one warp of a
+    pair to the other after every step.  Rows in groups of near-duplicates, so row maxima sit anywhere
+    in the sequence and the reference keeps growing."""
+    ctx = lib.LiteVGGT(1, grid[0], grid[1], 0.0, qkv_dtype=1)
+    m = ctx.n_merged
+    x, w_qkv, b_qkv, w_o, b_o = make_peaked_attention_inputs(m, 57 + m, groups=max(3, m // 5), sharpness=4.0)
+    ctx.global_attn(x.cuda(), w_qkv.cuda(), b_qkv.cuda(), w_o.cuda(), b_o.cuda())
+    ctx.poll()
+    deq, _, _ = O.quantize_qkv_e4m3(to_f64(ctx.debug_buffer(0)), heads=16)
+    ref_o = O.attention_core(unfold_k(deq), heads=16)
+    check_bf16(f"fp8 edges m={m}: attention core", to_f64(ctx.debug_buffer(1)), ref_o, noise=FP8_PEAKED_NOISE)
+    ctx.close()
