@@ -131,15 +131,11 @@ litevggt_status alloc_plan(litevggt_ctx* ctx, litevggt_plan** out) {
   return LITEVGGT_OK;
 }
 
-// matching -> selection -> index arrays, from the class array in ctx->ws.cls
-litevggt_status plan_from_classes(litevggt_ctx* ctx, const __nv_bfloat16* x, litevggt_plan* plan, cudaStream_t s) {
+// matching -> selection -> index arrays, from the token lists in the workspace
+litevggt_status plan_from_lists(litevggt_ctx* ctx, const __nv_bfloat16* x, litevggt_plan* plan, cudaStream_t s) {
   int n = 0;
   cudaError_t e;
   {
-    StepTimer t(ctx, 2);
-    e = launch_build_lists(ctx, ctx->ws.cls, ctx->ws.src_list, ctx->ws.dst_list, ctx->ws.src_pos, s, &n);
-  }
-  if (e == cudaSuccess) {
     StepTimer t(ctx, 3);
     e = launch_match(ctx, x, s, &n);
   }
@@ -488,7 +484,7 @@ litevggt_status litevggt_merge_plan(litevggt_ctx* ctx, const void* x, const floa
   bump(ctx, n);
   if (e != cudaSuccess) return cuda_status(e);
   plan->has_maps = true;
-  return plan_from_classes(ctx, xb, plan, s);
+  return plan_from_lists(ctx, xb, plan, s);
 }
 
 litevggt_status litevggt_merge_plan_with_partition(litevggt_ctx* ctx, const void* x, const uint8_t* cls,
@@ -504,8 +500,15 @@ litevggt_status litevggt_merge_plan_with_partition(litevggt_ctx* ctx, const void
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = cudaMemcpyAsync(ctx->ws.cls, cls, (size_t)ctx->sz.n_tokens, cudaMemcpyDeviceToDevice, s);
   if (e != cudaSuccess) return cuda_status(e);
+  int n = 0;
+  {
+    StepTimer t(ctx, 2);
+    e = launch_build_lists(ctx, ctx->ws.cls, s, &n);
+  }
+  bump(ctx, n);
+  if (e != cudaSuccess) return cuda_status(e);
   plan->has_maps = false;
-  return plan_from_classes(ctx, static_cast<const __nv_bfloat16*>(x), plan, s);
+  return plan_from_lists(ctx, static_cast<const __nv_bfloat16*>(x), plan, s);
 }
 
 litevggt_status litevggt_merge(litevggt_ctx* ctx, const litevggt_plan* plan, const void* x, void* x_merged,

@@ -17,7 +17,7 @@
 //             segment's tokens.  Which slot a token got depends on scheduling, its rank does not.
 // Ten launches, or - up to kSmallTokens tokens, where a launch costs more than what it does -
 // one launch of one block.  The two bitonic sorts of 64-bit keys that came before took 92 launches at 200
-// frames of 28 x 37 (418 us, 77 now) and 23 at four of 16 x 16 (82 us, 19 now; 50 as ten launches).
+// frames of 28 x 37 (418 us, 77 now) and 23 at four of 16 x 16 (82 us; 19 now, 50 as ten launches, events included).
 // No host synchronisation: all counts follow from the config.
 #include "common.cuh"
 #include "runtime.h"
@@ -170,7 +170,7 @@ __device__ __forceinline__ void phase_select(int block, int blocks, const IndexA
         on = (k >> sel_shift(pass - 1)) == (so_far.prefix >> sel_shift(pass - 1));
       }
     }
-    hist_add(bins, (k >> sel_shift(pass)) & (unsigned)(sel_bins(pass) - 1), on);
+    if (a.n_remove < a.n_src) hist_add(bins, (k >> sel_shift(pass)) & (unsigned)(sel_bins(pass) - 1), on);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < sel_bins(pass); i += kIdxThreads)
@@ -197,7 +197,8 @@ __device__ __forceinline__ unsigned long long token_counts(const IndexArgs& a, u
 // Threshold (from the last histogram) and the counts of every block of tokens.
 __device__ __forceinline__ void phase_count_removed(int block, const IndexArgs& a) {
   __shared__ unsigned long long scratch[32];
-  const Selection s = select_bin<2>(a.hist + 2 * kSelBins, a.sel[1]);
+  // with every src token merged the threshold lies below all keys
+  const Selection s = a.n_remove == a.n_src ? Selection{0u, (unsigned)a.n_src} : select_bin<2>(a.hist + 2 * kSelBins, a.sel[1]);
   if (block == 0 && threadIdx.x == 0) a.sel[2] = s;
   int pos[kScanItems];
   unsigned long long c[kScanItems];
@@ -371,7 +372,7 @@ static __host__ __device__ inline int phase_blocks(int phase, const IndexArgs& a
   if (phase == kNumberTokens) return per(a.n_tokens, kScanChunk);
   if (phase == kRowSums || phase == kSegments) return per(a.n_merged, kScanChunk);
   if (!merges) return 0;
-  if (phase == kSelect1 || phase == kSelect2) return select_blocks;
+  if (phase == kSelect1 || phase == kSelect2) return a.n_remove == a.n_src ? 0 : select_blocks;  // all of them: nothing to select
   if (phase == kCountRemoved) return per(a.n_tokens, kScanChunk);
   return per(a.n_remove, kIdxThreads) + (phase == kOrder && a.n_remove > kLongSegment ? (select_blocks > 1 ? kLongBlocks : 1) : 0);
 }

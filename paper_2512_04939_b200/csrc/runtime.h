@@ -223,8 +223,8 @@ cudaError_t launch_var_map(const litevggt_ctx* ctx, const __nv_bfloat16* x, floa
                            cudaStream_t s, int* launches);
 cudaError_t launch_partition(const litevggt_ctx* ctx, const float* grad, const float* var, float* ga, uint8_t* cls,
                              cudaStream_t s, int* launches);
-cudaError_t launch_build_lists(const litevggt_ctx* ctx, const uint8_t* cls, int* src_list, int* dst_list, int* src_pos,
-                               cudaStream_t s, int* launches);
+// (the partition leaves the token lists behind as well; this is for classes that come from the caller)
+cudaError_t launch_build_lists(const litevggt_ctx* ctx, const uint8_t* cls, cudaStream_t s, int* launches);
 
 // similarity.cu: leaves every src row's best anchor in ctx->ws.match_keys
 cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, cudaStream_t s, int* launches);

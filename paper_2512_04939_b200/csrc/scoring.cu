@@ -10,7 +10,7 @@ namespace lv {
 // ----------------------------------------------------------------------------------------
 // Grad map.  A warp owns a vertical strip of the image - as many whole patches as fit into 30 pixel
 // columns, plus one halo column on either side (lane = pixel column, replicate padding by clamping
-// the coordinate) - over a block of 7 patch rows, and walks down it one image row per step: three
+// the coordinate) - over a block of up to 7 patch rows, and walks down it one image row per step: three
 // coalesced 4-byte loads per lane (R, G, B), the grey value, its left and right neighbours by
 // shuffle, the separable Sobel pair (per row the horizontal difference r - l and the horizontal
 // smoothing l + 2c + r, kept for the last three rows), the magnitude, a running sum per column.  At
@@ -28,7 +28,7 @@ constexpr int kGradThreads = 128;
 #ifndef LV_GRAD_AHEAD14
 #define LV_GRAD_AHEAD14 7
 #endif
-constexpr int kGradPatchRows = LV_GRAD_PATCH_ROWS;  // patch rows per warp
+constexpr int kGradPatchRows = LV_GRAD_PATCH_ROWS;  // patch rows per warp, fewer where that leaves SMs without work
 constexpr int kGradAhead = LV_GRAD_AHEAD;           // image rows in flight
 
 __device__ __forceinline__ float sqrt_approx(float x) {
@@ -38,7 +38,8 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 }
 
 __global__ void __launch_bounds__(kGradThreads)
-grad_map_kernel(const float* __restrict__ images, float* __restrict__ grad, int grid_h, int grid_w, int patch, Stamp stamp) {
+grad_map_kernel(const float* __restrict__ images, float* __restrict__ grad, int grid_h, int grid_w, int patch, int patch_rows,
+                Stamp stamp) {
   const Span span(stamp);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int pps = 30 / patch;  // patches per strip (patch <= 30)
@@ -46,8 +47,8 @@ grad_map_kernel(const float* __restrict__ images, float* __restrict__ grad, int 
   const int strip = blockIdx.x * (kGradThreads / 32) + warp;
   if (strip >= strips) return;  // whole warp; nothing below synchronises across warps
   const int f = blockIdx.z;
-  const int pr0 = blockIdx.y * kGradPatchRows;
-  const int pr1 = min(grid_h, pr0 + kGradPatchRows);
+  const int pr0 = blockIdx.y * patch_rows;
+  const int pr1 = min(grid_h, pr0 + patch_rows);
   const int h = grid_h * patch, w = grid_w * patch;
   const size_t plane = (size_t)h * w;
   int x = strip * pps * patch - 1 + lane;
@@ -114,7 +115,8 @@ grad_map_kernel(const float* __restrict__ images, float* __restrict__ grad, int 
 // per-row bookkeeping (row counters, queue index, end-of-patch test) is gone.  kAhead divides kPatch.
 template <int kPatch, int kAhead>
 __global__ void __launch_bounds__(kGradThreads)
-grad_map_patch_kernel(const float* __restrict__ images, float* __restrict__ grad, int grid_h, int grid_w, Stamp stamp) {
+grad_map_patch_kernel(const float* __restrict__ images, float* __restrict__ grad, int grid_h, int grid_w, int patch_rows,
+                      Stamp stamp) {
   const Span span(stamp);
   static_assert(kPatch % kAhead == 0 && kPatch <= 30 && kAhead >= 2, "queue slots must be static");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -123,8 +125,8 @@ grad_map_patch_kernel(const float* __restrict__ images, float* __restrict__ grad
   const int strip = blockIdx.x * (kGradThreads / 32) + warp;
   if (strip >= strips) return;  // whole warp; nothing below synchronises across warps
   const int f = blockIdx.z;
-  const int pr0 = blockIdx.y * kGradPatchRows;
-  const int pr1 = min(grid_h, pr0 + kGradPatchRows);
+  const int pr0 = blockIdx.y * patch_rows;
+  const int pr1 = min(grid_h, pr0 + patch_rows);
   const int h = grid_h * kPatch, w = grid_w * kPatch;
   const size_t plane = (size_t)h * w;
   int x = strip * pps * kPatch - 1 + lane;
@@ -191,13 +193,18 @@ cudaError_t launch_grad_map(const litevggt_ctx* ctx, const float* images, float*
   const int patch = ctx->cfg.patch_px;
   const int pps = 30 / patch;
   const int strips = (z.grid_w + pps - 1) / pps;
-  const dim3 grid((unsigned)((strips + kGradThreads / 32 - 1) / (kGradThreads / 32)),
-                  (unsigned)((z.grid_h + kGradPatchRows - 1) / kGradPatchRows), (unsigned)z.frames);
+  // A warp's walk is a serial chain of 14 image rows a patch row: below four blocks an SM shorter walks are
+  // quicker although each reads two halo rows (four frames of 224 x 224: 5.7 -> 2.0 us)
+  const unsigned across = (unsigned)((strips + kGradThreads / 32 - 1) / (kGradThreads / 32));
+  int rows = kGradPatchRows;
+  auto down = [&] { return (unsigned)((z.grid_h + rows - 1) / rows); };
+  while (rows > 1 && (long long)across * down() * z.frames < 4ll * ctx->num_sms) rows = (rows + 1) / 2;
+  const dim3 grid(across, down(), (unsigned)z.frames);
   ++*launches;
   if (patch == 14)
-    return launch(grad_map_patch_kernel<14, LV_GRAD_AHEAD14>, grid, kGradThreads, 0, s, images, grad, z.grid_h, z.grid_w,
+    return launch(grad_map_patch_kernel<14, LV_GRAD_AHEAD14>, grid, kGradThreads, 0, s, images, grad, z.grid_h, z.grid_w, rows,
                   next_stamp(ctx));
-  return launch(grad_map_kernel, grid, kGradThreads, 0, s, images, grad, z.grid_h, z.grid_w, patch, next_stamp(ctx));
+  return launch(grad_map_kernel, grid, kGradThreads, 0, s, images, grad, z.grid_h, z.grid_w, patch, rows, next_stamp(ctx));
 }
 
 // ----------------------------------------------------------------------------------------
@@ -308,11 +315,14 @@ __device__ __forceinline__ float var_reduce_rows(const float (&v)[kVarRows], int
 
 __global__ void __launch_bounds__(kVarThreads, LV_VAR_OCC)
 var_map_kernel(const __nv_bfloat16* __restrict__ x, float* __restrict__ var, int grid_h, int grid_w, int n_special,
-               Stamp stamp) {
+               int seg_cols, Stamp stamp) {
   const Span span(stamp);
   __shared__ float part[kVarWarps][kVarRows][kVarMaxW];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int f = blockIdx.y, row_base = blockIdx.x * kVarRows;
+  // this block's columns, and where its walk begins and ends: one column further on either side
+  const int c_lo = blockIdx.z * seg_cols, c_hi = min(grid_w, c_lo + seg_cols);
+  const int c_begin = max(0, c_lo - 1), c_end = min(grid_w, c_hi + 1);
   const int tokens_frame = grid_h * grid_w + n_special;
   // this lane's 8 channels of the frame's first patch token
   const uint4* frame = reinterpret_cast<const uint4*>(x + ((size_t)f * tokens_frame + n_special) * 1024) + warp * 32 + lane;
@@ -335,14 +345,15 @@ var_map_kernel(const __nv_bfloat16* __restrict__ x, float* __restrict__ var, int
   for (int r = 0; r < kVarRows; ++r)
     inv_rows[r] = 1.0f / (float)(1 + (row_ok[r] ? 1 : 0) + (row_ok[r + 2] ? 1 : 0));
   const int row_stride = grid_w * kVarTokenVec;
-  const uint4* col_ptr = frame + (ptrdiff_t)(row_base - 1) * row_stride;  // only dereferenced where row_ok
+  // only dereferenced where row_ok
+  const uint4* col_ptr = frame + (ptrdiff_t)(row_base - 1) * row_stride + (ptrdiff_t)c_begin * kVarTokenVec;
 
   uint4 raw[kVarRows + 2];
 #pragma unroll
   for (int r = 0; r < kVarRows + 2; ++r) raw[r] = row_ok[r] ? __ldg(col_ptr + (ptrdiff_t)r * row_stride) : x0_raw;
   // rows outside the grid keep x0 in their registers for the whole walk
   auto load_next = [&](int c) {
-    if (c < grid_w) {
+    if (c < c_end) {
       col_ptr += kVarTokenVec;
 #pragma unroll
       for (int r = 0; r < kVarRows + 2; ++r)
@@ -350,7 +361,7 @@ var_map_kernel(const __nv_bfloat16* __restrict__ x, float* __restrict__ var, int
     }
     // the registers hold one column ahead; the columns after it are asked into L2 meanwhile, so
     // the loads above find them there instead of waiting for HBM
-    if (c + kVarPrefetch < grid_w) {
+    if (c + kVarPrefetch < c_end) {
 #pragma unroll
       for (int r = 0; r < kVarRows + 2; ++r)
         if (row_ok[r]) prefetch_l2(col_ptr + (ptrdiff_t)r * row_stride + kVarPrefetch * kVarTokenVec);
@@ -390,14 +401,19 @@ var_map_kernel(const __nv_bfloat16* __restrict__ x, float* __restrict__ var, int
   };
 
   VarColumn ca, cb;
-  var_zero(ca);
-  var_column(raw, neg_x0, cb);  // column 0
-  load_next(1);
-  for (int cn = 1; cn < grid_w; cn += 2) {
-    step(ca, cb, cn);
-    if (cn + 1 < grid_w) step(cb, ca, cn + 1);
+  if (c_lo == 0) {
+    var_zero(ca);
+  } else {
+    var_column(raw, neg_x0, ca);  // column c_lo - 1
+    load_next(c_lo);
   }
-  {
+  var_column(raw, neg_x0, cb);  // column c_lo
+  load_next(c_lo + 1);
+  for (int cn = c_lo + 1; cn < c_end; cn += 2) {
+    step(ca, cb, cn);
+    if (cn + 1 < c_end) step(cb, ca, cn + 1);
+  }
+  if (c_hi == grid_w) {
     // last column: nothing to its right
     VarColumn zero;
     var_zero(zero);
@@ -414,9 +430,10 @@ var_map_kernel(const __nv_bfloat16* __restrict__ x, float* __restrict__ var, int
   // the four channel quarters in a fixed order; mean over the 1024 channels
   const int n_rows = min(kVarRows, grid_h - row_base);
   float* out = var + ((size_t)f * grid_h + row_base) * grid_w;
-  for (int i = threadIdx.x; i < n_rows * grid_w; i += kVarThreads) {
-    const int r = i / grid_w, px = i - r * grid_w;
-    out[i] = (((part[0][r][px] + part[1][r][px]) + part[2][r][px]) + part[3][r][px]) / 1024.0f;
+  const int n_cols = c_hi - c_lo;
+  for (int i = threadIdx.x; i < n_rows * n_cols; i += kVarThreads) {
+    const int r = i / n_cols, px = c_lo + i - r * n_cols;
+    out[r * grid_w + px] = (((part[0][r][px] + part[1][r][px]) + part[2][r][px]) + part[3][r][px]) / 1024.0f;
   }
 }
 
@@ -425,9 +442,86 @@ cudaError_t launch_var_map(const litevggt_ctx* ctx, const __nv_bfloat16* x, floa
   const Sizes& z = ctx->sz;
   if (z.grid_w > kVarMaxW) return cudaErrorInvalidValue;
   const unsigned strips = (unsigned)((z.grid_h + kVarRows - 1) / kVarRows);
+  // The walk along a strip is a serial chain; where strips and frames do not fill the chip (three blocks an
+  // SM) it is cut into segments of at least four columns, each of which reads two columns beside its own
+  // (four frames of 16 x 16: 7.4 -> 3.5 us, 32 of 37 x 37: 36.6 -> 32.7).  The sums of a window do not depend on the cut.
+  int cols = z.grid_w;
+  auto segments = [&] { return (unsigned)((z.grid_w + cols - 1) / cols); };
+  while (cols > 4 && (long long)strips * z.frames * segments() < 3ll * ctx->num_sms) cols = cols > 8 ? (cols + 1) / 2 : 4;
   ++*launches;
-  return launch(var_map_kernel, dim3(strips, z.frames), kVarThreads, 0, s, x, var, z.grid_h, z.grid_w, z.n_special,
-                next_stamp(ctx));
+  return launch(var_map_kernel, dim3(strips, z.frames, segments()), kVarThreads, 0, s, x, var, z.grid_h, z.grid_w, z.n_special,
+                cols, next_stamp(ctx));
+}
+
+// ----------------------------------------------------------------------------------------
+// Token lists.  One CTA per frame: src / anchor tokens of the frame in ascending token
+// order, written at the offsets the per-frame class counts imply.  A frame whose counts
+// differ from the expected ones (possible only with a caller-supplied partition) is
+// flagged in the status word; writes never leave the frame's slot.
+struct ListArgs {
+  int *src_list, *dst_list, *src_pos;
+  int p_count, n_special, n_src_frame, n_dst_frame;
+  uint32_t* status;
+};
+
+// Lists of frame blockIdx.x from its classes; a block of kThreads threads.
+template <int kThreads>
+__device__ __forceinline__ void frame_lists(const uint8_t* cls, const ListArgs& a) {
+  int *src_list = a.src_list, *dst_list = a.dst_list, *src_pos = a.src_pos;
+  const int p_count = a.p_count, n_special = a.n_special, n_src_frame = a.n_src_frame, n_dst_frame = a.n_dst_frame;
+  uint32_t* status = a.status;
+  __shared__ int warp_src[kThreads / 32], warp_dst[kThreads / 32];
+  const int f = blockIdx.x;
+  const int tokens_frame = p_count + n_special;
+  const int token0 = f * tokens_frame;
+  const int exp_src = f == 0 ? 0 : n_src_frame;
+  const int exp_dst = f == 0 ? p_count : n_dst_frame;
+  const long long src_base = f == 0 ? 0 : (long long)(f - 1) * n_src_frame;
+  const long long dst_base = f == 0 ? 0 : (long long)p_count + (long long)(f - 1) * n_dst_frame;
+  const int per = (tokens_frame + kThreads - 1) / kThreads;
+  const int t0 = threadIdx.x * per, t1 = min(tokens_frame, t0 + per);
+  int ns = 0, nd = 0;
+  for (int t = t0; t < t1; ++t) {
+    const uint8_t c = cls[token0 + t];
+    ns += c == LITEVGGT_CLS_SRC;
+    nd += c == LITEVGGT_CLS_DST;
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int xs = ns, xd = nd;  // inclusive warp scans
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int a = __shfl_up_sync(0xffffffffu, xs, o), b = __shfl_up_sync(0xffffffffu, xd, o);
+    if (lane >= o) { xs += a; xd += b; }
+  }
+  if (lane == 31) { warp_src[warp] = xs; warp_dst[warp] = xd; }
+  __syncthreads();
+  int off_s = xs - ns, off_d = xd - nd, tot_s = 0, tot_d = 0;
+  for (int i = 0; i < kThreads / 32; ++i) {
+    if (i < warp) { off_s += warp_src[i]; off_d += warp_dst[i]; }
+    tot_s += warp_src[i];
+    tot_d += warp_dst[i];
+  }
+  if (tot_s != exp_src || tot_d != exp_dst) {
+    if (threadIdx.x == 0) atomicOr(status, kStatusBounds);
+  }
+  for (int t = t0; t < t1; ++t) {
+    const uint8_t c = cls[token0 + t];
+    int pos = -1;
+    if (c == LITEVGGT_CLS_SRC) {
+      if (off_s < exp_src) {
+        src_list[src_base + off_s] = token0 + t;
+        pos = (int)src_base + off_s;
+      }
+      ++off_s;
+    } else if (c == LITEVGGT_CLS_DST) {
+      if (off_d < exp_dst) dst_list[dst_base + off_d] = token0 + t;
+      ++off_d;
+    }
+    src_pos[token0 + t] = pos;
+  }
+  // a short frame (flagged above) still gets valid token indices in its unused slots
+  for (int i = tot_s + (int)threadIdx.x; i < exp_src; i += kThreads) src_list[src_base + i] = token0;
+  for (int i = tot_d + (int)threadIdx.x; i < exp_dst; i += kThreads) dst_list[dst_base + i] = token0;
 }
 
 // ----------------------------------------------------------------------------------------
@@ -460,8 +554,8 @@ __device__ __forceinline__ unsigned score_key(float v) {
 
 __global__ void __launch_bounds__(kPartThreads)
 partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, float* __restrict__ ga,
-                 uint8_t* __restrict__ cls, int grid_h, int grid_w, int n_special, int n_ga, int cell_h, int cell_w,
-                 float alpha, float beta, Stamp stamp) {
+                 uint8_t* cls, int grid_h, int grid_w, int n_special, int n_ga, int cell_h, int cell_w,
+                 float alpha, float beta, const ListArgs lists, Stamp stamp) {
   const Span span(stamp);
   extern __shared__ float part_smem[];
   const int p_count = grid_h * grid_w;
@@ -493,6 +587,8 @@ partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, 
   out += n_special;
   if (f == 0) {  // the first frame's patches are all anchors
     for (int p = threadIdx.x; p < p_count; p += kPartThreads) out[p] = LITEVGGT_CLS_DST;
+    __syncthreads();
+    frame_lists<kPartThreads>(cls, lists);
     return;
   }
   __syncthreads();
@@ -587,6 +683,14 @@ partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, 
     }
     out[p] = c;
   }
+  __syncthreads();
+  frame_lists<kPartThreads>(cls, lists);
+}
+
+static ListArgs list_args(const litevggt_ctx* ctx) {
+  const Sizes& z = ctx->sz;
+  return ListArgs{ctx->ws.src_list, ctx->ws.dst_list, ctx->ws.src_pos, z.patches, z.n_special,
+                  z.n_src_frame,    z.n_dst_frame,    ctx->ws.status};
 }
 
 cudaError_t launch_partition(const litevggt_ctx* ctx, const float* grad, const float* var, float* ga, uint8_t* cls,
@@ -595,80 +699,20 @@ cudaError_t launch_partition(const litevggt_ctx* ctx, const float* grad, const f
   const size_t smem = (size_t)z.patches * (sizeof(float) + 1) + 16;  // at most 41 KB (8192 patches)
   ++*launches;
   return launch(partition_kernel, dim3(z.frames), kPartThreads, smem, s, grad, var, ga, cls, z.grid_h, z.grid_w, z.n_special,
-                z.n_ga_frame, (int)ctx->cfg.cell_h, (int)ctx->cfg.cell_w, ctx->cfg.alpha, ctx->cfg.beta, next_stamp(ctx));
+                z.n_ga_frame, (int)ctx->cfg.cell_h, (int)ctx->cfg.cell_w, ctx->cfg.alpha, ctx->cfg.beta, list_args(ctx), next_stamp(ctx));
 }
 
-// ----------------------------------------------------------------------------------------
-// Token lists.  One CTA per frame: src / anchor tokens of the frame in ascending token
-// order, written at the offsets the per-frame class counts imply.  A frame whose counts
-// differ from the expected ones (possible only with a caller-supplied partition) is
-// flagged in the status word; writes never leave the frame's slot.
 constexpr int kListThreads = 256;
-
 __global__ void __launch_bounds__(kListThreads)
-build_lists_kernel(const uint8_t* __restrict__ cls, int* __restrict__ src_list, int* __restrict__ dst_list,
-                   int* __restrict__ src_pos, int p_count, int n_special, int n_src_frame, int n_dst_frame, uint32_t* status, Stamp stamp) {
+build_lists_kernel(const uint8_t* __restrict__ cls, const ListArgs lists, Stamp stamp) {
   const Span span(stamp);
-  __shared__ int warp_src[kListThreads / 32], warp_dst[kListThreads / 32];
-  const int f = blockIdx.x;
-  const int tokens_frame = p_count + n_special;
-  const int token0 = f * tokens_frame;
-  const int exp_src = f == 0 ? 0 : n_src_frame;
-  const int exp_dst = f == 0 ? p_count : n_dst_frame;
-  const long long src_base = f == 0 ? 0 : (long long)(f - 1) * n_src_frame;
-  const long long dst_base = f == 0 ? 0 : (long long)p_count + (long long)(f - 1) * n_dst_frame;
-  const int per = (tokens_frame + kListThreads - 1) / kListThreads;
-  const int t0 = threadIdx.x * per, t1 = min(tokens_frame, t0 + per);
-  int ns = 0, nd = 0;
-  for (int t = t0; t < t1; ++t) {
-    const uint8_t c = cls[token0 + t];
-    ns += c == LITEVGGT_CLS_SRC;
-    nd += c == LITEVGGT_CLS_DST;
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int xs = ns, xd = nd;  // inclusive warp scans
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int a = __shfl_up_sync(0xffffffffu, xs, o), b = __shfl_up_sync(0xffffffffu, xd, o);
-    if (lane >= o) { xs += a; xd += b; }
-  }
-  if (lane == 31) { warp_src[warp] = xs; warp_dst[warp] = xd; }
-  __syncthreads();
-  int off_s = xs - ns, off_d = xd - nd, tot_s = 0, tot_d = 0;
-  for (int i = 0; i < kListThreads / 32; ++i) {
-    if (i < warp) { off_s += warp_src[i]; off_d += warp_dst[i]; }
-    tot_s += warp_src[i];
-    tot_d += warp_dst[i];
-  }
-  if (tot_s != exp_src || tot_d != exp_dst) {
-    if (threadIdx.x == 0) atomicOr(status, kStatusBounds);
-  }
-  for (int t = t0; t < t1; ++t) {
-    const uint8_t c = cls[token0 + t];
-    int pos = -1;
-    if (c == LITEVGGT_CLS_SRC) {
-      if (off_s < exp_src) {
-        src_list[src_base + off_s] = token0 + t;
-        pos = (int)src_base + off_s;
-      }
-      ++off_s;
-    } else if (c == LITEVGGT_CLS_DST) {
-      if (off_d < exp_dst) dst_list[dst_base + off_d] = token0 + t;
-      ++off_d;
-    }
-    src_pos[token0 + t] = pos;
-  }
-  // a short frame (flagged above) still gets valid token indices in its unused slots
-  for (int i = tot_s + (int)threadIdx.x; i < exp_src; i += kListThreads) src_list[src_base + i] = token0;
-  for (int i = tot_d + (int)threadIdx.x; i < exp_dst; i += kListThreads) dst_list[dst_base + i] = token0;
+  frame_lists<kListThreads>(cls, lists);
 }
 
-cudaError_t launch_build_lists(const litevggt_ctx* ctx, const uint8_t* cls, int* src_list, int* dst_list, int* src_pos,
-                               cudaStream_t s, int* launches) {
+cudaError_t launch_build_lists(const litevggt_ctx* ctx, const uint8_t* cls, cudaStream_t s, int* launches) {
   const Sizes& z = ctx->sz;
   ++*launches;
-  return launch(build_lists_kernel, dim3(z.frames), kListThreads, 0, s, cls, src_list, dst_list, src_pos, z.patches, z.n_special,
-                z.n_src_frame, z.n_dst_frame, ctx->ws.status, next_stamp(ctx));
+  return launch(build_lists_kernel, dim3(z.frames), kListThreads, 0, s, cls, list_args(ctx), next_stamp(ctx));
 }
 
 }  // namespace lv
