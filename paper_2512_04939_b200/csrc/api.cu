@@ -301,7 +301,7 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
   const size_t o_pos = c.take<int>(z.n_tokens), o_idx = c.take<int>(index_scratch_words(z));
   const size_t o_qkv = c.take<__nv_bfloat16>(z.n_merged * 3 * z.dim), o_o = c.take<__nv_bfloat16>(z.n_merged * z.dim);
   size_t ml_off = 0;
-  const size_t state_bytes = attention_state_bytes(z.n_merged, z.dim, z.heads, &ml_off);
+  const size_t state_bytes = attention_state_bytes(z.n_merged, z.dim, z.heads, ctx->num_sms, &ml_off);
   const size_t o_state = c.take<uint8_t>((long long)state_bytes);
   const size_t o_kmax = c.take<float>((long long)z.frames * z.heads);
   const bool fp8 = cfg->qkv_dtype == 1;

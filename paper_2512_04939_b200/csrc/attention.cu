@@ -141,6 +141,40 @@ constexpr float kFaShiftUp = 84.0f, kFaShiftDown = 92.0f;
 #endif
 constexpr long long kFaOneTileRows = LV_FA_ONE_TILE_ROWS;
 
+// The CTAs of a launch that its last wave would leave alone on the chip, split along the keys: linear block
+// ids from `full` on are (job, part) with `parts` parts to a job (one query block of one head), and leave
+// partial rows for combine_parts_kernel.  parts = 0: a grid of (query blocks, heads, sequences), nothing split.
+struct FaSplit {
+  int q_blocks, full, parts;
+  float* o;   // [slot][256][64] partial output rows, slot = block id - full
+  float* ml;  // [slot][256]{reference, row sum}
+};
+struct FaJob {
+  int q_block, head, seq, slot;  // slot < 0: a whole job
+};
+__device__ __forceinline__ FaJob fa_job(const FaSplit& split, int& tile_begin, int& tile_end) {
+  if (split.parts == 0) return FaJob{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, -1};
+  const int id = blockIdx.x, slot = id - split.full;
+  int job = id;
+  if (slot >= 0) {
+    const int part = slot % split.parts, tiles = tile_end;
+    job = split.full + slot / split.parts;
+    tile_begin = (int)((long long)tiles * part / split.parts);
+    tile_end = (int)((long long)tiles * (part + 1) / split.parts);
+  }
+  return FaJob{job % split.q_blocks, job / split.q_blocks, 0, slot};
+}
+// This thread's 32 channels of row r (0..255) of the job.
+__device__ __forceinline__ void fa_store_part(const FaSplit& split, int slot, int r, int c, const uint32_t (&acc)[32], float scale,
+                                              float m_ref, float row_sum) {
+  float4* dst = reinterpret_cast<float4*>(split.o + ((size_t)slot * 256 + r) * 64 + c * 32);
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    dst[i] = make_float4(__uint_as_float(acc[4 * i]) * scale, __uint_as_float(acc[4 * i + 1]) * scale,
+                         __uint_as_float(acc[4 * i + 2]) * scale, __uint_as_float(acc[4 * i + 3]) * scale);
+  if (c == 0) *reinterpret_cast<float2*>(split.ml + ((size_t)slot * 256 + r) * 2) = make_float2(m_ref, row_sum);
+}
+
 template <int kStages>
 struct FaBarriers {
   uint64_t q_ready;
@@ -296,7 +330,7 @@ __global__ void __launch_bounds__(FaShape<kTiles>::kThreads, kTiles == 2 ? 1 : 2
 flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_bfloat16* __restrict__ qkv,
                        __nv_bfloat16* __restrict__ o, float* __restrict__ o_state, float* __restrict__ ml_state,
                        const float* __restrict__ k_norm2_max, int seq_len, int dim, int tile_begin, int tile_end,
-                       uint32_t* status, Stamp stamp) {
+                       FaSplit split, uint32_t* status, Stamp stamp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* smem_k = smem;
@@ -308,11 +342,14 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
   FaBarriers<kStages>* bars = reinterpret_cast<FaBarriers<kStages>*>(xchg + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // blockIdx.z selects one of the independent sequences of seq_len rows laid back to back (the
+  constexpr bool kSplit = kTiles == 2 && kFirst && kLast;
+  FaJob job{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, -1};
+  if constexpr (kSplit) job = fa_job(split, tile_begin, tile_end);
+  // job.seq selects one of the independent sequences of seq_len rows laid back to back (the
   // global layer has one; a frame-local layer has one per frame)
-  const int row_base = blockIdx.z * seq_len;
-  const int q0 = blockIdx.x * (128 * kTiles);  // within the sequence
-  const int head = blockIdx.y;
+  const int row_base = job.seq * seq_len;
+  const int q0 = job.q_block * (128 * kTiles);  // within the sequence
+  const int head = job.head;
   // this launch covers key tiles [tile_begin, tile_end) of ceil(seq_len / 128); local tile j is
   // key tile tile_begin + j, step n = local tile n/2, half n%2
   const int n_kv = tile_end - tile_begin;
@@ -509,7 +546,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       // Cauchy-Schwarz bound on this row's scores (K carries the softmax scale, so the scores are in
       // base-2 units already); both threads of a row hold the same value, and both warps of a pair
       // vote over the same 32 rows, so they agree on the form they run
-      score_bound = sqrtf(q_norm2 * k_norm2_max[blockIdx.z * gridDim.y + head]);
+      score_bound = sqrtf(q_norm2 * k_norm2_max[job.seq * (dim / 64) + head]);
       fixed_ref = __all_sync(0xffffffffu, score_bound <= kFaFixedRefLimit ? 1 : 0) != 0;
       tmem_st16(tmem_base + lane_base + Shape::kColQ + t * 32 + c * 16, qreg);
       tmem_st_wait();
@@ -696,7 +733,9 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       tmem_ld32(o_addr, acc);
       tmem_ld16(l_addr, sum);
       tmem_ld_wait();
-      if (row_live) {
+      if (kSplit && job.slot >= 0) {
+        if (row_live) fa_store_part(split, job.slot, t * 128 + row_in_tile, c, acc, 1.0f, m_ref, __uint_as_float(sum[0]));
+      } else if (row_live) {
         float row_sum = __uint_as_float(sum[0]);
         // each of the row's two threads keeps its own copy of {reference, row sum} in the state
         float* ml_mine = ml_state + ((size_t)row * (dim / 64) + head) * 4 + 2 * c;
@@ -819,7 +858,7 @@ __global__ void __launch_bounds__(kFaThreads, 1)
 flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __grid_constant__ CUtensorMap tmap_v8t,
                            const uint8_t* __restrict__ q8, const float* __restrict__ amax, __nv_bfloat16* __restrict__ o,
                            float* __restrict__ o_state, float* __restrict__ ml_state, int seq_len, int dim, int tile_begin,
-                           int tile_end, uint32_t* status, Stamp stamp) {
+                           int tile_end, FaSplit split, uint32_t* status, Stamp stamp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* smem_k = smem;
@@ -828,8 +867,11 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
   FaBarriers<kFaStages>* bars = reinterpret_cast<FaBarriers<kFaStages>*>(refs + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int q0 = blockIdx.x * 256;
-  const int head = blockIdx.y;
+  constexpr bool kSplit = kFirst && kLast;
+  FaJob job{(int)blockIdx.x, (int)blockIdx.y, 0, -1};
+  if constexpr (kSplit) job = fa_job(split, tile_begin, tile_end);
+  const int q0 = job.q_block * 256;
+  const int head = job.head;
   const int n_kv = tile_end - tile_begin;
   constexpr bool first_chunk = kFirst;
   constexpr bool last_chunk = kLast;
@@ -1077,7 +1119,9 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
       tmem_ld32(o_addr, acc);
       tmem_ld16(l_addr, sum);
       tmem_ld_wait();
-      if (row_live) {
+      if (kSplit && job.slot >= 0) {
+        if (row_live) fa_store_part(split, job.slot, t * 128 + row_in_tile, c, acc, scale_v, m_ref, __uint_as_float(sum[0]));
+      } else if (row_live) {
         float row_sum = __uint_as_float(sum[0]);
         float* ml_mine = ml_state + ((size_t)row * (dim / 64) + head) * 4 + 2 * c;
         if (!first_chunk) {
@@ -1131,6 +1175,81 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
   }
 }
 
+// Rows of the split jobs: the parts brought to a common reference and added in the order of their keys.
+constexpr int kCombineRows = 32;  // a block's rows; a thread has 8 channels of one
+__global__ void __launch_bounds__(kCombineRows * 8)
+combine_parts_kernel(FaSplit split, __nv_bfloat16* __restrict__ o, int seq_len, int dim, Stamp stamp) {
+  const Span span(stamp);
+  const int job = split.full + blockIdx.x, q_block = job % split.q_blocks, head = job / split.q_blocks;
+  const int r = blockIdx.y * kCombineRows + (threadIdx.x >> 3), ch = (threadIdx.x & 7) * 8;
+  const int row = q_block * 256 + r;
+  if (row >= seq_len) return;
+  const size_t slot0 = (size_t)blockIdx.x * split.parts;
+  float m = -INFINITY;
+  for (int p = 0; p < split.parts; ++p) m = fmaxf(m, split.ml[((slot0 + p) * 256 + r) * 2]);
+  float acc[8], sum = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
+  for (int p = 0; p < split.parts; ++p) {
+    const float2 ml = *reinterpret_cast<const float2*>(split.ml + ((slot0 + p) * 256 + r) * 2);
+    const float w = ml.x == m ? 1.0f : fast_exp2(ml.x - m);
+    sum = fmaf(ml.y, w, sum);
+    const float4* src = reinterpret_cast<const float4*>(split.o + ((slot0 + p) * 256 + r) * 64 + ch);
+    const float4 a = src[0], b = src[1];
+    acc[0] = fmaf(a.x, w, acc[0]);
+    acc[1] = fmaf(a.y, w, acc[1]);
+    acc[2] = fmaf(a.z, w, acc[2]);
+    acc[3] = fmaf(a.w, w, acc[3]);
+    acc[4] = fmaf(b.x, w, acc[4]);
+    acc[5] = fmaf(b.y, w, acc[5]);
+    acc[6] = fmaf(b.z, w, acc[6]);
+    acc[7] = fmaf(b.w, w, acc[7]);
+  }
+  const float inv = 1.0f / sum;
+  *reinterpret_cast<uint4*>(o + (size_t)row * dim + head * 64 + ch) =
+      make_uint4(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv), pack_bf16(acc[4] * inv, acc[5] * inv),
+                 pack_bf16(acc[6] * inv, acc[7] * inv));
+}
+
+// How the jobs that do not fill a wave of one CTA an SM are split: into so many parts that their waves end
+// soonest.  A key tile of two query tiles takes about 1.05 us, a CTA 8 us besides, adding the parts up 8.
+// (21,984 rows: 1376 jobs = 9 waves and 44 jobs, three parts each, 1.776 -> 1.718 ms; in the E4M3 form 2.14 ->
+// 2.07; 31,751 rows, shifted reference, 4.36 -> 4.17.)  Sequences of several key chunks have hundreds of waves and are left alone.
+static FaSplit split_plan(long long seq_len, int n_seq, int heads, int num_sms) {
+  const long long n_tiles = (seq_len + 127) / 128, q_blocks = (seq_len + 255) / 256, jobs = q_blocks * heads;
+  FaSplit best{(int)q_blocks, 0, 0, nullptr, nullptr};
+  if (n_seq != 1 || seq_len <= kFaOneTileRows || n_tiles > kFaChunkTiles) return best;
+  const long long rest = jobs % num_sms;
+  if (rest == 0) return best;
+  float best_us = 8.0f + 1.05f * (float)n_tiles;
+  for (int parts = 2; parts <= 16 && n_tiles / parts >= 4; ++parts) {
+    const float us = 8.0f + (float)((rest * parts + num_sms - 1) / num_sms) * (8.0f + 1.05f * (float)n_tiles / (float)parts);
+    if (us < best_us) {
+      best_us = us;
+      best.parts = parts;
+      best.full = (int)(jobs - rest);
+    }
+  }
+  return best;
+}
+static long long split_slots(const FaSplit& split, int heads) {
+  return split.parts == 0 ? 0 : ((long long)split.q_blocks * heads - split.full) * split.parts;
+}
+// Points the plan at the context's state buffers; a context without them (or of another size) splits nothing.
+static FaSplit split_for(const litevggt_ctx* ctx, long long seq_len, int n_seq) {
+  FaSplit split = split_plan(seq_len, n_seq, ctx->sz.heads, ctx->num_sms);
+  if (ctx->ws.attn_o_state == nullptr || seq_len != ctx->sz.n_merged) split.parts = 0;
+  split.o = ctx->ws.attn_o_state;
+  split.ml = ctx->ws.attn_ml_state;
+  return split;
+}
+static cudaError_t launch_combine(const litevggt_ctx* ctx, const FaSplit& split, __nv_bfloat16* o, long long seq_len, cudaStream_t s,
+                                  int* launches) {
+  ++*launches;
+  return launch(combine_parts_kernel, dim3((unsigned)(split.q_blocks * ctx->sz.heads - split.full), 256 / kCombineRows),
+                kCombineRows * 8, 0, s, split, o, (int)seq_len, ctx->sz.dim, next_stamp(ctx));
+}
+
 cudaError_t launch_flash_attention_fp8(litevggt_ctx* ctx, long long m, __nv_bfloat16* o, cudaStream_t s, int* launches) {
   if (m == 0) return cudaSuccess;
   const int dim = ctx->sz.dim;
@@ -1142,7 +1261,7 @@ cudaError_t launch_flash_attention_fp8(litevggt_ctx* ctx, long long m, __nv_bflo
       !make_tmap_u8_2d(ctx->encode_tiled, &tmap_v, ws.v8t, (uint64_t)m_pad, (uint64_t)dim, (uint64_t)m_pad, 128, 64))
     return cudaErrorInvalidValue;
   using Kernel = void (*)(const CUtensorMap, const CUtensorMap, const uint8_t*, const float*, __nv_bfloat16*, float*,
-                          float*, int, int, int, int, uint32_t*, Stamp);
+                          float*, int, int, int, int, FaSplit, uint32_t*, Stamp);
   const Kernel kernels[2][2] = {{flash_attention_fp8_kernel<false, false>, flash_attention_fp8_kernel<false, true>},
                                 {flash_attention_fp8_kernel<true, false>, flash_attention_fp8_kernel<true, true>}};
   static std::atomic<unsigned long long> smem_set[2][2];
@@ -1151,7 +1270,9 @@ cudaError_t launch_flash_attention_fp8(litevggt_ctx* ctx, long long m, __nv_bflo
       cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(kernels[a][b]), kFa8SmemBytes, smem_set[a][b]);
       if (e != cudaSuccess) return e;
     }
-  const dim3 grid((unsigned)((m + 255) / 256), (unsigned)ctx->sz.heads, 1);
+  const FaSplit split = split_for(ctx, m, 1);
+  const dim3 grid = split.parts > 0 ? dim3((unsigned)(split.full + split_slots(split, ctx->sz.heads)))
+                                    : dim3((unsigned)((m + 255) / 256), (unsigned)ctx->sz.heads, 1);
   const int n_tiles = (int)((m + 127) / 128);
   const int n_chunks = (n_tiles + kFaChunkTiles - 1) / kFaChunkTiles;
   const int per_chunk = (n_tiles + n_chunks - 1) / n_chunks;
@@ -1159,12 +1280,12 @@ cudaError_t launch_flash_attention_fp8(litevggt_ctx* ctx, long long m, __nv_bflo
   for (int begin = 0; begin < n_tiles; begin += per_chunk) {
     const int end = begin + per_chunk < n_tiles ? begin + per_chunk : n_tiles;
     cudaError_t e = launch_clusters(1, false, kernels[begin == 0][end == n_tiles], grid, kFaThreads, kFa8SmemBytes, s, tmap_k, tmap_v, ws.q8,
-                           ws.qkv_amax, o, ws.attn_o_state, ws.attn_ml_state, (int)m, dim, begin, end, ws.status,
-                           next_stamp(ctx));
+                           ws.qkv_amax, o, ws.attn_o_state, ws.attn_ml_state, (int)m, dim, begin, end, split,
+                           ws.status, next_stamp(ctx));
     if (e != cudaSuccess) return e;
     ++*launches;
   }
-  return cudaGetLastError();
+  return split.parts > 0 ? launch_combine(ctx, split, o, m, s, launches) : cudaSuccess;
 }
 
 cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long seq_len, int n_seq,
@@ -1177,7 +1298,7 @@ cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, 
   if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap, qkv, (uint64_t)3 * dim, (uint64_t)rows, (uint64_t)3 * dim, 64, 128))
     return cudaErrorInvalidValue;
   using Kernel = void (*)(const CUtensorMap, const __nv_bfloat16*, __nv_bfloat16*, float*, float*, const float*, int,
-                          int, int, int, uint32_t*, Stamp);
+                          int, int, int, FaSplit, uint32_t*, Stamp);
   // [query tiles of a CTA - 1][first chunk][last chunk]
   const Kernel kernels[2][2][2] = {
       {{flash_attention_kernel<1, false, false>, flash_attention_kernel<1, false, true>},
@@ -1194,7 +1315,9 @@ cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, 
   const int per_chunk = (n_tiles + n_chunks - 1) / n_chunks;
   if (n_chunks > 1 && (n_seq != 1 || ctx->ws.attn_o_state == nullptr || ctx->ws.attn_ml_state == nullptr))
     return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)((n_tiles + tiles - 1) / tiles), (unsigned)ctx->sz.heads, (unsigned)n_seq);
+  const FaSplit split = split_for(ctx, seq_len, n_seq);
+  const dim3 grid = split.parts > 0 ? dim3((unsigned)(split.full + split_slots(split, ctx->sz.heads)))
+                                    : dim3((unsigned)((n_tiles + tiles - 1) / tiles), (unsigned)ctx->sz.heads, (unsigned)n_seq);
   const int threads = tiles == 2 ? FaShape<2>::kThreads : FaShape<1>::kThreads;
   for (int begin = 0; begin < n_tiles; begin += per_chunk) {
     const int end = begin + per_chunk < n_tiles ? begin + per_chunk : n_tiles;
@@ -1204,24 +1327,29 @@ cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, 
     // not before the projection has ended: CTAs that came early would sit two to an SM on the first SMs to
     // become free (four small frames: 9.9 us against 6.2)
     e = launch_clusters(1, false, kernels[a][b][c], grid, threads, smem_bytes[a], s, tmap, qkv, o, ctx->ws.attn_o_state, ctx->ws.attn_ml_state,
-               ctx->ws.attn_kmax, (int)seq_len, dim, begin, end, ctx->ws.status, next_stamp(ctx));
+               ctx->ws.attn_kmax, (int)seq_len, dim, begin, end, split, ctx->ws.status, next_stamp(ctx));
     if (e != cudaSuccess) return e;
     ++*launches;
   }
-  return cudaGetLastError();
+  return split.parts > 0 ? launch_combine(ctx, split, o, seq_len, s, launches) : cudaSuccess;
 }
 
-// Rows of fp32 partial output and of {reference, row sum} x 2 per head (one copy per thread of a row)
-// that the chunked sweep sums up between launches; zero when m fits one chunk.
-size_t attention_state_bytes(long long m, int dim, int heads, size_t* ml_offset) {
+// What passes between launches: for several key chunks rows of fp32 partial output and of {reference, row
+// sum} x 2 per head (one copy per thread of a row), for a split last wave the parts' rows; zero where
+// neither happens.
+size_t attention_state_bytes(long long m, int dim, int heads, int num_sms, size_t* ml_offset) {
   const long long n_tiles = (m + 127) / 128;
-  if (n_tiles <= kFaChunkTiles) {
-    if (ml_offset) *ml_offset = 0;
-    return 0;
+  size_t o_bytes = 0, ml_bytes = 0;
+  if (n_tiles > kFaChunkTiles) {
+    o_bytes = (size_t)round_up(m * dim * 4, 256);
+    ml_bytes = (size_t)round_up(m * heads * 16, 256);
+  } else {
+    const long long slots = split_slots(split_plan(m, 1, heads, num_sms), heads);
+    o_bytes = (size_t)slots * 256 * 64 * 4;
+    ml_bytes = (size_t)slots * 256 * 2 * 4;
   }
-  const size_t o_bytes = (size_t)round_up(m * dim * 4, 256);
-  if (ml_offset) *ml_offset = o_bytes;
-  return o_bytes + (size_t)round_up(m * heads * 16, 256);
+  *ml_offset = o_bytes;
+  return o_bytes + ml_bytes;
 }
 
 }  // namespace lv

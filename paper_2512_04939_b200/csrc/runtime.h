@@ -70,8 +70,8 @@ struct Workspace {
   // attention
   __nv_bfloat16* qkv = nullptr;    // [M, 3D]
   __nv_bfloat16* attn_o = nullptr; // [M, D]
-  float* attn_o_state = nullptr;   // [M, D] running output between key chunks (long sequences only)
-  float* attn_ml_state = nullptr;  // [M, heads, 4] reference maximum and partial row sums
+  float* attn_o_state = nullptr;   // [M, D] running output between key chunks (long sequences), or split parts
+  float* attn_ml_state = nullptr;  // [M, heads, 4] references and partial row sums, or those of the parts
   float* attn_kmax = nullptr;      // [max(frames, 1), heads] largest |k|^2 per sequence and head
   // E4M3 variant of the attention operands (qkv_dtype = 1)
   uint8_t* q8 = nullptr;           // [M, D] bytes
@@ -283,7 +283,7 @@ cudaError_t launch_qk_embed(const litevggt_ctx* ctx, __nv_bfloat16* qkv, const i
 // K last: the projection or qk_embed)
 cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long seq_len, int n_seq,
                                    __nv_bfloat16* o, cudaStream_t s, int* launches);
-size_t attention_state_bytes(long long m, int dim, int heads, size_t* ml_offset);
+size_t attention_state_bytes(long long m, int dim, int heads, int num_sms, size_t* ml_offset);
 // E4M3 variant: quantised copies of Q, K, V by the per-head magnitudes in ctx->ws.qkv_amax - taken from
 // qkv here first unless the projection has left them there - (fp8_quant.cu), then the attention core on
 // those (attention.cu); one sequence of m rows
