@@ -610,7 +610,8 @@ litevggt_status litevggt_global_attn_ext(litevggt_ctx* ctx, const litevggt_plan*
     StepTimer t(ctx, 6);
     e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x_merged), m, d,
                              static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
-                             2 * d, 1.0f, embeds ? LinearStat{} : core_stat(ctx, m), ctx->ws.qkv, s, &n);
+                             2 * d, embeds ? 1.0f : kKeyScaleLog2e,  // (the Q/K pass scales K itself, when there is one)
+                             embeds ? LinearStat{} : core_stat(ctx, m), ctx->ws.qkv, s, &n);
   }
   if (e == cudaSuccess) {
     StepTimer t(ctx, 13);

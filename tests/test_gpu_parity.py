@@ -585,6 +585,21 @@ def test_global_attention_with_qk_norm_and_rope(lib, wl, mode):
     ctx.close()
 
 
+@pytest.mark.parametrize("qkv_dtype", [0, 1])
+def test_ext_entry_without_options_is_the_plain_layer(lib, qkv_dtype):
+    """Neither normalisation nor rotation (and no plan): bit for bit what global_attn returns."""
+    wl = WORKLOADS["C1"]
+    ctx = _ctx(lib, wl, qkv_dtype=qkv_dtype)
+    g = torch.Generator().manual_seed(11)
+    xm = torch.randn(ctx.n_merged, 1024, generator=g).to(torch.bfloat16).cuda()
+    w = [t.cuda() for t in make_attention_weights(wl, 0)]
+    plain, plain_qkv = ctx.global_attn(xm, *w), ctx.debug_buffer(0)
+    ext, ext_qkv = ctx.global_attn_ext(None, xm, *w), ctx.debug_buffer(0)
+    ctx.poll()
+    assert torch.equal(ext_qkv, plain_qkv) and torch.equal(ext, plain)
+    ctx.close()
+
+
 # ------------------------------------------------------------------ other sub-layers of a block
 @pytest.mark.parametrize("wl", [WORKLOADS["C1"], ODD], ids=lambda w: w.name)
 def test_layernorm_frame_attention_and_mlp(lib, wl):
