@@ -306,7 +306,9 @@ litevggt_status litevggt_selftest_bounded_wait(litevggt_ctx* ctx, int64_t limit_
                                                void* stream);
 
 /* Device-time stopwatches.  The kernels of each step of the path note on the device's clock when the
- * first of them started and the last one ended: which = 0 grad map, 1 var map, 2 partition + token lists, 3 cosine
+ * first of them began its work - after its own set-up (barriers, tensor memory), which small kernels do
+ * while the one before is still running - and the last one ended; a step that launched nothing
+ * took no time: which = 0 grad map, 1 var map, 2 partition + token lists, 3 cosine
  * matching (pack + GEMM/argmax), 4 selection + index build, 5 merge, 6 qkv projection,
  * 7 attention core, 8 output projection, 9 unmerge, 10 LayerNorm, 11 frame-local attention layer,
  * 12 MLP, 13 Q/K normalisation + rotary embedding, 14 E4M3 quantisation of Q/K/V.

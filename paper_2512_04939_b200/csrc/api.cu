@@ -78,17 +78,23 @@ struct Carver {
 
 void bump(litevggt_ctx* ctx, int n) { ctx->launches += n; }
 
-// Hands the launches of one step the stopwatch slot that their kernels write.
+// Hands the launches of one step the stopwatch slot that their kernels write; `launches` and `e` are what
+// the step counts its launches in and ends with.
 struct StepTimer {
   litevggt_ctx* ctx;
-  int which;
-  StepTimer(litevggt_ctx* c, int w) : ctx(c), which(w) {
-    unsigned long long* slot = c->timers.stamps + 2 * (w * kTimerSlots + c->timers.used[w] % kTimerSlots);
-    c->step.start = slot;
-    c->step.stop = slot + 1;
+  int which, slot;
+  const int& launches;
+  const int before;
+  const cudaError_t& e;
+  StepTimer(litevggt_ctx* c, int w, const int& n, const cudaError_t& err)
+      : ctx(c), which(w), slot(c->timers.used[w] % kTimerSlots), launches(n), before(n), e(err) {
+    unsigned long long* stamps = c->timers.stamps + 2 * (w * kTimerSlots + slot);
+    c->step.start = stamps;
+    c->step.stop = stamps + 1;
   }
   ~StepTimer() {
     ctx->step = Stamp{};
+    ctx->timers.empty[which][slot] = launches == before || e != cudaSuccess;
     ++ctx->timers.used[which];
   }
 };
@@ -134,13 +140,13 @@ litevggt_status alloc_plan(litevggt_ctx* ctx, litevggt_plan** out) {
 // matching -> selection -> index arrays, from the token lists in the workspace
 litevggt_status plan_from_lists(litevggt_ctx* ctx, const __nv_bfloat16* x, litevggt_plan* plan, cudaStream_t s) {
   int n = 0;
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   {
-    StepTimer t(ctx, 3);
+    StepTimer t(ctx, 3, n, e);
     e = launch_match(ctx, x, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 4);
+    StepTimer t(ctx, 4, n, e);
     e = launch_index_build(ctx, plan, s, &n);
   }
   bump(ctx, n);
@@ -376,8 +382,10 @@ static litevggt_status read_stamps(litevggt_ctx* ctx, int which, float (&ms)[kTi
     e = cudaMemcpy(t, ctx->timers.stamps + 2 * kTimerSlots * which, sizeof(t), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_status(e);
   for (int i = 0; i < *kept; ++i) {
-    const unsigned long long* r = t[(used - *kept + i) % kTimerSlots];
-    ms[i] = r[1] > r[0] ? (float)((double)(r[1] - r[0]) * 1e-6) : 0.0f;  // a step without kernels took no time
+    const int slot = (used - *kept + i) % kTimerSlots;
+    const unsigned long long* r = t[slot];
+    // a step without kernels took no time
+    ms[i] = !ctx->timers.empty[which][slot] && r[1] > r[0] ? (float)((double)(r[1] - r[0]) * 1e-6) : 0.0f;
   }
   return LITEVGGT_OK;
 }
@@ -450,9 +458,9 @@ litevggt_status litevggt_grad_map(litevggt_ctx* ctx, const float* images, float*
   if (!ctx_ok(ctx) || images == nullptr || grad == nullptr) return LITEVGGT_ERR_NULL;
   if (!aligned16(images) || !aligned16(grad)) return LITEVGGT_ERR_ALIGN;
   int n = 0;
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   {
-    StepTimer t(ctx, 0);
+    StepTimer t(ctx, 0, n, e);
     e = launch_grad_map(ctx, images, grad, (cudaStream_t)stream, &n);
   }
   bump(ctx, n);
@@ -472,13 +480,13 @@ litevggt_status litevggt_merge_plan(litevggt_ctx* ctx, const void* x, const floa
   cudaStream_t s = (cudaStream_t)stream;
   const __nv_bfloat16* xb = static_cast<const __nv_bfloat16*>(x);
   int n = 0;
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   {
-    StepTimer t(ctx, 1);
+    StepTimer t(ctx, 1, n, e);
     e = launch_var_map(ctx, xb, ctx->ws.var_map, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 2);
+    StepTimer t(ctx, 2, n, e);
     e = launch_partition(ctx, grad, ctx->ws.var_map, ctx->ws.ga_score, ctx->ws.cls, s, &n);
   }
   bump(ctx, n);
@@ -502,7 +510,7 @@ litevggt_status litevggt_merge_plan_with_partition(litevggt_ctx* ctx, const void
   if (e != cudaSuccess) return cuda_status(e);
   int n = 0;
   {
-    StepTimer t(ctx, 2);
+    StepTimer t(ctx, 2, n, e);
     e = launch_build_lists(ctx, ctx->ws.cls, s, &n);
   }
   bump(ctx, n);
@@ -517,9 +525,9 @@ litevggt_status litevggt_merge(litevggt_ctx* ctx, const litevggt_plan* plan, con
   if (!plan_ok(plan) || plan->owner != ctx || !plan->built) return LITEVGGT_ERR_STALE_PLAN;
   if (!aligned16(x) || !aligned16(x_merged)) return LITEVGGT_ERR_ALIGN;
   int n = 0;
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   {
-    StepTimer t(ctx, 5);
+    StepTimer t(ctx, 5, n, e);
     e = launch_merge(ctx, plan, static_cast<const __nv_bfloat16*>(x), static_cast<__nv_bfloat16*>(x_merged),
                      (cudaStream_t)stream, &n);
   }
@@ -554,24 +562,24 @@ litevggt_status litevggt_global_attn(litevggt_ctx* ctx, const void* x_merged, in
   const int d = ctx->sz.dim;
   cudaStream_t s = (cudaStream_t)stream;
   int n = 0;
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   {
-    StepTimer t(ctx, 6);
+    StepTimer t(ctx, 6, n, e);
     e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x_merged), m, d,
                              static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
                              2 * d, kKeyScaleLog2e, core_stat(ctx, m), ctx->ws.qkv, s, &n);
   }
   if (e == cudaSuccess && ctx->cfg.qkv_dtype == 1) {
-    StepTimer t(ctx, 14);
+    StepTimer t(ctx, 14, n, e);
     e = launch_qkv_quantize(ctx, ctx->ws.qkv, m, true, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 7);
+    StepTimer t(ctx, 7, n, e);
     e = ctx->cfg.qkv_dtype == 1 ? launch_flash_attention_fp8(ctx, m, ctx->ws.attn_o, s, &n)
                                 : launch_flash_attention(ctx, ctx->ws.qkv, m, 1, ctx->ws.attn_o, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 8);
+    StepTimer t(ctx, 8, n, e);
     e = launch_linear(ctx, ctx->ws.attn_o, m, d, static_cast<const __nv_bfloat16*>(w_o), d,
                       static_cast<const __nv_bfloat16*>(b_o), kmax_words(ctx, 1), static_cast<__nv_bfloat16*>(y_merged), s, &n);
   }
@@ -605,16 +613,16 @@ litevggt_status litevggt_global_attn_ext(litevggt_ctx* ctx, const litevggt_plan*
   const int d = ctx->sz.dim;
   cudaStream_t s = (cudaStream_t)stream;
   int n = 0;
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   {
-    StepTimer t(ctx, 6);
+    StepTimer t(ctx, 6, n, e);
     e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x_merged), m, d,
                              static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
                              2 * d, embeds ? 1.0f : kKeyScaleLog2e,  // (the Q/K pass scales K itself, when there is one)
                              embeds ? LinearStat{} : core_stat(ctx, m), ctx->ws.qkv, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 13);
+    StepTimer t(ctx, 13, n, e);
     e = launch_qk_embed(ctx, ctx->ws.qkv, ext->rope != 0 ? plan->kept_idx : nullptr, m,
                         static_cast<const __nv_bfloat16*>(ext->q_norm_gamma),
                         static_cast<const __nv_bfloat16*>(ext->q_norm_beta),
@@ -623,16 +631,16 @@ litevggt_status litevggt_global_attn_ext(litevggt_ctx* ctx, const litevggt_plan*
                         ext->rope_base, fp8 ? nullptr : ctx->ws.attn_kmax, s, &n);
   }
   if (e == cudaSuccess && ctx->cfg.qkv_dtype == 1) {
-    StepTimer t(ctx, 14);
+    StepTimer t(ctx, 14, n, e);
     e = launch_qkv_quantize(ctx, ctx->ws.qkv, m, !embeds, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 7);
+    StepTimer t(ctx, 7, n, e);
     e = ctx->cfg.qkv_dtype == 1 ? launch_flash_attention_fp8(ctx, m, ctx->ws.attn_o, s, &n)
                                 : launch_flash_attention(ctx, ctx->ws.qkv, m, 1, ctx->ws.attn_o, s, &n);
   }
   if (e == cudaSuccess) {
-    StepTimer t(ctx, 8);
+    StepTimer t(ctx, 8, n, e);
     e = launch_linear(ctx, ctx->ws.attn_o, m, d, static_cast<const __nv_bfloat16*>(w_o), d,
                       static_cast<const __nv_bfloat16*>(b_o), kmax_words(ctx, 1), static_cast<__nv_bfloat16*>(y_merged), s, &n);
   }
@@ -646,9 +654,9 @@ litevggt_status litevggt_layernorm(litevggt_ctx* ctx, const void* x, int64_t row
   if (rows < 0 || !(eps > 0.0f)) return LITEVGGT_ERR_SHAPE;
   if (!aligned16(x) || !aligned16(gamma) || !aligned16(beta) || !aligned16(out)) return LITEVGGT_ERR_ALIGN;
   int n = 0;
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   {
-    StepTimer t(ctx, 10);
+    StepTimer t(ctx, 10, n, e);
     e = launch_layernorm(static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(gamma),
                          static_cast<const __nv_bfloat16*>(beta), static_cast<__nv_bfloat16*>(out), rows, eps,
                          next_stamp(ctx), (cudaStream_t)stream, &n);
@@ -670,9 +678,9 @@ litevggt_status litevggt_frame_attn(litevggt_ctx* ctx, const void* x, const void
   const int d = z.dim;
   cudaStream_t s = (cudaStream_t)stream;
   int n = 0;
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   {
-    StepTimer t(ctx, 11);
+    StepTimer t(ctx, 11, n, e);
     e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x), z.n_tokens, d,
                              static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
                              2 * d, kKeyScaleLog2e, LinearStat{ctx->ws.attn_kmax, z.tokens_frame, nullptr},
@@ -704,7 +712,7 @@ litevggt_status litevggt_mlp(litevggt_ctx* ctx, const void* x, int64_t rows, con
   int n = 0;
   cudaError_t e = cudaSuccess;
   {
-    StepTimer t(ctx, 12);
+    StepTimer t(ctx, 12, n, e);
     for (long long r0 = 0; r0 < rows && e == cudaSuccess; r0 += kMlpChunkRows) {
       const long long nr = rows - r0 < kMlpChunkRows ? rows - r0 : kMlpChunkRows;
       e = launch_linear_mlp(ctx, xb + r0 * d, nr, d, static_cast<const __nv_bfloat16*>(w1), 4 * d,
@@ -726,9 +734,9 @@ litevggt_status litevggt_unmerge(litevggt_ctx* ctx, const litevggt_plan* plan, c
   if (!aligned16(y_merged) || !aligned16(out) || (residual != nullptr && !aligned16(residual)))
     return LITEVGGT_ERR_ALIGN;
   int n = 0;
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   {
-    StepTimer t(ctx, 9);
+    StepTimer t(ctx, 9, n, e);
     e = launch_unmerge(ctx, plan, static_cast<const __nv_bfloat16*>(y_merged),
                        static_cast<const __nv_bfloat16*>(residual), static_cast<__nv_bfloat16*>(out),
                        (cudaStream_t)stream, &n);

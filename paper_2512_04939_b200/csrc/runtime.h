@@ -105,6 +105,7 @@ constexpr int kTimerSlots = 64;
 struct Timers {
   unsigned long long* stamps = nullptr;  // device [kNumTimers][kTimerSlots]{start, stop}, in the workspace
   int used[kNumTimers] = {};             // launches recorded since the last reset
+  bool empty[kNumTimers][kTimerSlots] = {};  // the record's step launched nothing (or failed): its stamps are an older one's
 };
 }  // namespace lv
 

@@ -1,0 +1,90 @@
+"""The host side of the library (api.cu, attn_static.cu) linked against stand-ins for the CUDA runtime and
+the kernel launchers (host_fakes.cpp): what it hands from call to call, without a GPU."""
+import ctypes as C
+import os
+import subprocess
+
+import pytest
+
+from paper_2512_04939_b200.binding import AttnExt, Config
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2512_04939_b200", "csrc")
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("host") / "libhost.so")
+    # (-Bsymbolic: its own stand-ins, not the runtime that torch has loaded into the process)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-w", "-Wl,-Bsymbolic", "-I/usr/local/cuda/include", "-x", "c++",
+                    os.path.join(CSRC, "api.cu"), os.path.join(CSRC, "attn_static.cu"), os.path.join(HERE, "host_fakes.cpp"),
+                    "-o", so], check=True)
+    lib = C.CDLL(so)
+    lib.fake_norm_seen.restype = lib.fake_norm_last_seen.restype = C.c_float
+    return lib
+
+
+class Ctx:
+    def __init__(self, lib, qkv_dtype=0):
+        cfg = Config()
+        assert lib.litevggt_default_config(3, 4, 5, C.c_float(0.5), C.byref(cfg)) == 0
+        cfg.qkv_dtype = qkv_dtype
+        self.lib, self.h = lib, C.c_void_p()
+        assert lib.litevggt_create(C.byref(cfg), 0, C.byref(self.h)) == 0
+        n, m = C.c_int64(), C.c_int64()
+        lib.litevggt_sizes(self.h, C.byref(n), C.byref(m), None, None, None)
+        self.n, self.m = n.value, m.value
+        self.buf = C.create_string_buffer(1 << 12)
+        self.p = C.c_void_p((C.addressof(self.buf) + 255) & ~255)  # the stand-ins read none of it
+
+    def layernorm(self, rows):
+        return self.lib.litevggt_layernorm(self.h, self.p, C.c_int64(rows), self.p, self.p, C.c_float(1e-6), self.p, None)
+
+    def mlp(self, rows):
+        p = self.p
+        return self.lib.litevggt_mlp(self.h, p, C.c_int64(rows), p, p, p, p, None, p, None)
+
+    def global_attn(self):
+        p = self.p
+        return self.lib.litevggt_global_attn(self.h, p, C.c_int64(self.m), p, p, p, p, p, None)
+
+    def global_attn_ext(self, normed):
+        p, ext = self.p, AttnExt()
+        if normed:
+            ext.q_norm_gamma = ext.q_norm_beta = ext.k_norm_gamma = ext.k_norm_beta = p
+        ext.norm_eps = 1e-5
+        return self.lib.litevggt_global_attn_ext(self.h, None, p, C.c_int64(self.m), p, p, p, p, C.byref(ext), p, None)
+
+    def frame_attn(self):
+        p = self.p
+        return self.lib.litevggt_frame_attn(self.h, p, p, p, p, p, None, p, None)
+
+    def timer(self, which):
+        ms, count, one = C.c_float(), C.c_int32(), (C.c_float * 64)()
+        assert self.lib.litevggt_timer_samples(self.h, which, one, 64, C.byref(count)) == 0
+        samples = [round(v * 1e6) for v in one[:count.value]]
+        assert self.lib.litevggt_timer_read(self.h, which, C.byref(ms), C.byref(count)) == 0
+        assert count.value == len(samples) and round(ms.value * 1e6) == sum(samples)
+        return samples  # nanoseconds
+
+
+@pytest.mark.parametrize("which", [10, 12, 13, 8])
+def test_a_step_that_launched_nothing_took_no_time(host, which):
+    """LayerNorm and MLP of no rows, the Q/K pass with neither option, an output projection that is refused:
+    their records are zero, also where the ring slot held an earlier step's times."""
+    c = Ctx(host)
+    busy = {10: lambda: c.layernorm(7), 12: lambda: c.mlp(7), 13: lambda: c.global_attn_ext(True), 8: c.global_attn}[which]
+    each = 1000 if which == 12 else 500  # the stand-in kernels take 500 ns, the MLP has two
+    for _ in range(64):
+        assert busy() == 0
+    assert c.timer(which) == [each] * 64
+    if which == 8:
+        host.fake_fail_linear(1)
+        assert c.global_attn() != 0
+    else:
+        assert {10: lambda: c.layernorm(0), 12: lambda: c.mlp(0), 13: lambda: c.global_attn_ext(False)}[which]() == 0
+    assert c.timer(which) == [each] * 63 + [0]
+    host.litevggt_timers_reset(c.h)
+    assert busy() == 0
+    assert c.timer(which) == [each]
+    host.litevggt_destroy(c.h)
