@@ -240,6 +240,16 @@ ZeroWords kmax_words(const litevggt_ctx* ctx, long long sequences) {
   return ZeroWords{reinterpret_cast<uint32_t*>(ctx->ws.attn_kmax), sequences * ctx->sz.heads};
 }
 
+// Before a call raises the key norms: they are zero unless an earlier call failed half-way.
+cudaError_t begin_norms(litevggt_ctx* ctx, cudaStream_t s) {
+  if (ctx->norms_left) {
+    const cudaError_t e = cudaMemsetAsync(ctx->ws.attn_kmax, 0, sizeof(float) * (size_t)ctx->sz.frames * ctx->sz.heads, s);
+    if (e != cudaSuccess) return e;
+  }
+  ctx->norms_left = true;  // until the output projection is enqueued
+  return cudaSuccess;
+}
+
 // What the global layer's attention core needs to know about Q, K and V before it starts.
 LinearStat core_stat(const litevggt_ctx* ctx, long long m) {
   LinearStat st;
@@ -562,8 +572,8 @@ litevggt_status litevggt_global_attn(litevggt_ctx* ctx, const void* x_merged, in
   const int d = ctx->sz.dim;
   cudaStream_t s = (cudaStream_t)stream;
   int n = 0;
-  cudaError_t e = cudaSuccess;
-  {
+  cudaError_t e = begin_norms(ctx, s);
+  if (e == cudaSuccess) {
     StepTimer t(ctx, 6, n, e);
     e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x_merged), m, d,
                              static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
@@ -583,6 +593,7 @@ litevggt_status litevggt_global_attn(litevggt_ctx* ctx, const void* x_merged, in
     e = launch_linear(ctx, ctx->ws.attn_o, m, d, static_cast<const __nv_bfloat16*>(w_o), d,
                       static_cast<const __nv_bfloat16*>(b_o), kmax_words(ctx, 1), static_cast<__nv_bfloat16*>(y_merged), s, &n);
   }
+  if (e == cudaSuccess) ctx->norms_left = false;
   bump(ctx, n);
   return cuda_status(e);
 }
@@ -613,8 +624,8 @@ litevggt_status litevggt_global_attn_ext(litevggt_ctx* ctx, const litevggt_plan*
   const int d = ctx->sz.dim;
   cudaStream_t s = (cudaStream_t)stream;
   int n = 0;
-  cudaError_t e = cudaSuccess;
-  {
+  cudaError_t e = begin_norms(ctx, s);
+  if (e == cudaSuccess) {
     StepTimer t(ctx, 6, n, e);
     e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x_merged), m, d,
                              static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
@@ -644,6 +655,7 @@ litevggt_status litevggt_global_attn_ext(litevggt_ctx* ctx, const litevggt_plan*
     e = launch_linear(ctx, ctx->ws.attn_o, m, d, static_cast<const __nv_bfloat16*>(w_o), d,
                       static_cast<const __nv_bfloat16*>(b_o), kmax_words(ctx, 1), static_cast<__nv_bfloat16*>(y_merged), s, &n);
   }
+  if (e == cudaSuccess) ctx->norms_left = false;
   bump(ctx, n);
   return cuda_status(e);
 }
@@ -678,8 +690,8 @@ litevggt_status litevggt_frame_attn(litevggt_ctx* ctx, const void* x, const void
   const int d = z.dim;
   cudaStream_t s = (cudaStream_t)stream;
   int n = 0;
-  cudaError_t e = cudaSuccess;
-  {
+  cudaError_t e = begin_norms(ctx, s);
+  if (e == cudaSuccess) {
     StepTimer t(ctx, 11, n, e);
     e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x), z.n_tokens, d,
                              static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
@@ -691,6 +703,7 @@ litevggt_status litevggt_frame_attn(litevggt_ctx* ctx, const void* x, const void
                             static_cast<const __nv_bfloat16*>(b_o), 0, static_cast<const __nv_bfloat16*>(residual),
                             kmax_words(ctx, z.frames), static_cast<__nv_bfloat16*>(y), s, &n);
   }
+  if (e == cudaSuccess) ctx->norms_left = false;
   bump(ctx, n);
   return cuda_status(e);
 }

@@ -8,6 +8,7 @@
 // an allocation implies.  For them the two intermediates live in the array below, which is
 // part of the library image: every GPU that loads the library reserves it once and keeps
 // it until the process exits.
+#include <atomic>
 #include <mutex>
 
 #include "runtime.h"
@@ -31,6 +32,7 @@ struct DeviceSetup {
   unsigned char* scratch = nullptr;  // device address of g_attn_scratch on this device
   void* encode_tiled = nullptr;
   int num_sms = 0;
+  std::atomic<bool> norms_left{false};  // a call that raised the key norms did not get as far as zeroing them
 };
 DeviceSetup g_setup[kMaxDevices];
 std::mutex g_setup_mutex;
@@ -97,6 +99,11 @@ extern "C" litevggt_status litevggt_global_attn_static(const void* x_merged, int
     (void)cudaGetLastError();
     return LITEVGGT_ERR_CUDA;
   }
+  if (dev->norms_left.load() && cudaMemsetAsync(dev->scratch + 64, 0, kStaticHeads * sizeof(float), s) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return LITEVGGT_ERR_CUDA;
+  }
+  dev->norms_left.store(true);
   // the launchers only read these fields of a context; this one lives on the stack
   litevggt_ctx local{};
   local.device = device;
@@ -121,5 +128,6 @@ extern "C" litevggt_status litevggt_global_attn_static(const void* x_merged, int
     (void)cudaGetLastError();
     return LITEVGGT_ERR_CUDA;
   }
+  dev->norms_left.store(false);
   return LITEVGGT_OK;
 }

@@ -132,6 +132,7 @@ struct litevggt_ctx {
   void* encode_tiled;  // cuTensorMapEncodeTiled, resolved at run time
   lv::Timers timers;
   mutable lv::Stamp step;  // of the step whose kernels are being launched
+  bool norms_left = false;  // a call that raised the key norms did not get as far as zeroing them
   HostPipe pipe;
 };
 

@@ -88,3 +88,25 @@ def test_a_step_that_launched_nothing_took_no_time(host, which):
     assert busy() == 0
     assert c.timer(which) == [each]
     host.litevggt_destroy(c.h)
+
+
+@pytest.mark.parametrize("entry", ["global_attn", "frame_attn", "static"])
+def test_key_norms_are_zero_after_a_call_that_failed_half_way(host, entry):
+    """The projection raises the key norms, the output projection zeroes them; where that one is refused, the
+    next call - also of the other layer, with more or fewer sequences - must not start from what is left."""
+    c = Ctx(host)
+    buf = C.create_string_buffer(1 << 12)
+    p = C.c_void_p((C.addressof(buf) + 255) & ~255)
+
+    def static():
+        return host.litevggt_global_attn_static(p, C.c_int64(100), p, p, p, p, p, p, None)
+
+    call = static if entry == "static" else getattr(c, entry)
+    for follow in (call, c.frame_attn if entry != "static" else call):
+        assert call() == 0 and call() == 0
+        assert host.fake_norm_seen() == 0.0 and host.fake_norm_last_seen() == 0.0
+        host.fake_fail_linear(1)
+        assert call() != 0
+        assert follow() == 0
+        assert host.fake_norm_seen() == 0.0 and host.fake_norm_last_seen() == 0.0
+    host.litevggt_destroy(c.h)
