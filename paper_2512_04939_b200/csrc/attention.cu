@@ -124,10 +124,11 @@ constexpr int kFaChunkTiles = LV_FA_CHUNK_TILES;  // 65536 keys: K and V of one 
 #endif
 constexpr int kFaPolyPairs = LV_FA_POLY_PAIRS;
 // The same in the shifted-reference form, whose polynomial pairs also need a clamp and whose other
-// pairs a subtraction.  At 31,751 rows, time over that of the QKV projection in the same run (the
-// clock moves under the power cap): 0 pairs 30.3, 3: 29.9, 4: 28.5, 5: 28.3, 7: 28.0.
+// pairs a subtraction, and which takes the polynomial of degree 6 (the running maximum that served these
+// rows before is as good as the special-function unit).  Core at 31,751 rows: 0 pairs 4.52 ms, 1: 4.47, 2: 4.47,
+// 3: 4.45, 4: 4.45, 5: 4.50; with a cubic, which moves probabilities by 7.5e-5, 4.22.
 #ifndef LV_FA_SHIFT_POLY_PAIRS
-#define LV_FA_SHIFT_POLY_PAIRS 5
+#define LV_FA_SHIFT_POLY_PAIRS 3
 #endif
 constexpr int kFaShiftPolyPairs = LV_FA_SHIFT_POLY_PAIRS;
 // Shifted reference m of a row with score bound B and a known score s0: B - m <= kFaShiftUp keeps row sums
@@ -210,22 +211,36 @@ __device__ __forceinline__ float fast_exp2(float x) {
 
 // 2^(x - m) for a pair of arguments on the FMA pipes, `magic` = 1.5 * 2^23 - m with m a whole number.
 // Adding it rounds x to the nearest integer and leaves n = that integer - m in the low mantissa
-// bits; the fraction's power comes from a cubic fitted on [-1/2, 1/2] and n is added to the exponent
-// field.  Valid for x - m in [-120, 120].
+// bits; the fraction's power comes from a polynomial fitted on [-1/2, 1/2] and n is added to the exponent
+// field.  Valid for x - m in [-120, 120].  The cubic is good to 7.5e-5 relative.  With kFull the degree is 6 and
+// the result, rounding included, within 6.6e-8 of 2^(x - m): closer than the special-function unit,
+// whose ex2.approx was measured at up to 1.45e-7 (5.4e-8 against 2.6e-8 in the mean square).
+template <bool kFull>
 __device__ __forceinline__ float2 poly_exp2_pair(float2 x, float2 magic, float2 neg_magic) {
   const float2 t = __fadd2_rn(x, magic);
   const float2 n = __fadd2_rn(t, neg_magic);
   const float2 f = __ffma2_rn(n, make_float2(-1.0f, -1.0f), x);
-  float2 p = __ffma2_rn(make_float2(0.0551716648f, 0.0551716648f), f, make_float2(0.2426111251f, 0.2426111251f));
-  p = __ffma2_rn(p, f, make_float2(0.6932609677f, 0.6932609677f));
-  p = __ffma2_rn(p, f, make_float2(0.9999280572f, 0.9999280572f));
+  auto horner = [&](float2 p, float c) { return __ffma2_rn(p, f, make_float2(c, c)); };
+  float2 p;
+  if constexpr (kFull) {
+    p = horner(make_float2(1.5820509e-4f, 1.5820509e-4f), 1.341820345e-3f);
+    p = horner(p, 9.617063217e-3f);
+    p = horner(p, 5.55027239e-2f);
+    p = horner(p, 0.2402265519f);
+    p = horner(p, 0.6931472421f);
+    p = horner(p, 1.0f);
+  } else {
+    p = horner(make_float2(0.0551716648f, 0.0551716648f), 0.2426111251f);
+    p = horner(p, 0.6932609677f);
+    p = horner(p, 0.9999280572f);
+  }
   float2 r;
   r.x = __uint_as_float(__float_as_uint(p.x) + (__float_as_uint(t.x) << 23));
   r.y = __uint_as_float(__float_as_uint(p.y) + (__float_as_uint(t.y) << 23));
   return r;
 }
 __device__ __forceinline__ float2 poly_exp2_pair(float2 x) {
-  return poly_exp2_pair(x, make_float2(12582912.0f, 12582912.0f), make_float2(-12582912.0f, -12582912.0f));
+  return poly_exp2_pair<false>(x, make_float2(12582912.0f, 12582912.0f), make_float2(-12582912.0f, -12582912.0f));
 }
 
 // Wait until the most recent loads into a ring (up to one per stage) have landed.
@@ -295,7 +310,7 @@ __device__ __forceinline__ void exp2_chunk_shifted(const uint32_t (&s)[32], floa
     float2 p;
     if (i < kPoly) {
       const float2 x = make_float2(fmaxf(__uint_as_float(s[2 * i]), floor_s), fmaxf(__uint_as_float(s[2 * i + 1]), floor_s));
-      p = poly_exp2_pair(x, magic2, neg_magic2);
+      p = poly_exp2_pair<true>(x, magic2, neg_magic2);
     } else {
       const float2 x = __fadd2_rn(make_float2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), neg_m);
       p.x = fast_exp2(x.x);

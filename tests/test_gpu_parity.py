@@ -515,6 +515,40 @@ def test_attention_core_at_tile_edges_in_every_softmax_form(lib, frames, grid, s
     ctx.close()
 
 
+def uniform_rows_ctx(lib, rows, qkv_dtype=0):
+    """A context whose merged sequence is `rows` tokens without special ones, and zeroed weights for it."""
+    ctx = lib.LiteVGGT(-(-rows // 4096), 64, min(64, rows // 64), 0.0, n_special=0, qkv_dtype=qkv_dtype)
+    assert ctx.n_merged == rows
+    zeros = [torch.zeros(*s, dtype=torch.bfloat16) for s in ((rows, 1024), (3072, 1024), (3072,), (1024, 1024), (1024,))]
+    return ctx, zeros
+
+
+@pytest.mark.parametrize("rows,qkv_dtype", [(4096, 0), (8192, 0)])
+def test_exponentials_are_equally_good_at_every_key_position(lib, rows, qkv_dtype):
+    """Some positions of a key tile take their exponential from the special-function unit (within 1.45e-7), others
+    from a polynomial (within 6.6e-8, where the fixed reference does not serve).  All keys of a row score the same
+    here and V is +1 at the positions 0 and -1 at the positions 31 of every 32, so an output is exactly zero
+    unless the two round to different probabilities.  That takes a rounding boundary between them, within
+    2.2e-7 relative where neighbours lie 2^-8 apart (bf16): 5.5e-5 of the rows, 4 or 8 of
+    65,536 or 131,072, and 30 with a chance below 1e-8; a cubic (7.5e-5) splits hundreds."""
+    ctx, (x, w_qkv, b_qkv, w_o, b_o) = uniform_rows_ctx(lib, rows, qkv_dtype)
+    g = torch.Generator().manual_seed(rows)
+    x[:, :16] = 100 + 100 * torch.rand(rows, 16, generator=g).to(torch.bfloat16)
+    x[:, 16:32] = torch.randn(rows, 16, generator=g).to(torch.bfloat16)
+    x[::32, 32], x[31::32, 32] = 1.0, -1.0
+    for h in range(16):  # q = (x_h, x_16+h), k = (1, 1/64) before the softmax scale, v = x_32
+        w_qkv[64 * h, h] = w_qkv[64 * h + 1, 16 + h] = w_qkv[2048 + 64 * h, 32] = 1.0
+        b_qkv[1024 + 64 * h], b_qkv[1024 + 64 * h + 1] = 8.0, 0.125
+    ctx.global_attn(x.cuda(), w_qkv.cuda(), b_qkv.cuda(), w_o.cuda(), b_o.cuda())
+    ctx.poll()
+    assert set(softmax_forms(to_f64(ctx.debug_buffer(0)))) == {"shifted"}
+    o = to_f64(ctx.debug_buffer(1))[:, ::64]
+    split = int((o != 0).sum())
+    report(f"probabilities that differ by position, {rows} rows, qkv_dtype {qkv_dtype}", rows=o.size, split=split)
+    assert np.abs(o).max() < 2.0 ** -7 and split <= 30
+    ctx.close()
+
+
 @pytest.mark.parametrize("grid", [(1, 1), (1, 59), (4, 15), (3, 41), (4, 31)], ids=lambda g: f"{g[0]}x{g[1]}")
 def test_frame_attention_at_tile_edges(lib, grid):
     """6, 64, 65, 128 and 129 tokens a frame.  The rows share a common part, as a frame's tokens do:
