@@ -839,15 +839,9 @@ struct Fa8Refs {
 };
 constexpr int kFa8SmemBytes = kFaStages * (kFa8KTileBytes + kFa8VStageBytes) + (int)sizeof(Fa8Refs) + 512 + 1024;
 
-// Of the 16 pairs of 32 scores, this many take the polynomial exponential.  Core at 21,984 rows: 4 pairs
-// 2.20 ms, 5: 2.14, 6: 2.14, 7: 2.16 (0, with both halves read twice: 2.32); 2.22 when the two warps of a
-// pair shared every step and swapped row maxima in it.
-#ifndef LV_FA8_POLY_PAIRS
-#define LV_FA8_POLY_PAIRS 6
-#endif
-constexpr int kFa8PolyPairs = LV_FA8_POLY_PAIRS;
-
-// 32 scores -> 32 E4M3 probabilities 2^(s * scale - m)
+// 32 scores -> 32 E4M3 probabilities 2^(s * scale - m), all from the special-function unit.  A polynomial good enough
+// to stand beside it (poly_exp2_pair<true>) saves nothing here: core at 21,984 rows 2.13 ms as it is, 2.12
+// with one pair of 16 on the FMA pipes, 2.17 with two, 2.18 with three.
 __device__ __forceinline__ void exp2_chunk_e4m3(const uint32_t (&s)[32], float2 scale2, float2 neg_m2, uint32_t (&packed)[8]) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -855,14 +849,9 @@ __device__ __forceinline__ void exp2_chunk_e4m3(const uint32_t (&s)[32], float2 
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const int pair = 2 * i + k;
-      float2 x = __ffma2_rn(make_float2(__uint_as_float(s[2 * pair]), __uint_as_float(s[2 * pair + 1])), scale2, neg_m2);
-      if (pair < kFa8PolyPairs) {
-        // (below 2^-10 an E4M3 probability is zero; the polynomial takes arguments down to -120)
-        p[k] = poly_exp2_pair(make_float2(fmaxf(x.x, -64.0f), fmaxf(x.y, -64.0f)));
-      } else {
-        p[k].x = fast_exp2(x.x);
-        p[k].y = fast_exp2(x.y);
-      }
+      const float2 x = __ffma2_rn(make_float2(__uint_as_float(s[2 * pair]), __uint_as_float(s[2 * pair + 1])), scale2, neg_m2);
+      p[k].x = fast_exp2(x.x);
+      p[k].y = fast_exp2(x.y);
     }
     packed[i] = pack_e4m3x4(p[0].x, p[0].y, p[1].x, p[1].y);
   }

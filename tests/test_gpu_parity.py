@@ -549,6 +549,51 @@ def test_exponentials_are_equally_good_at_every_key_position(lib, rows, qkv_dtyp
     ctx.close()
 
 
+def test_e4m3_probabilities_do_not_depend_on_the_key_position(lib):
+    """Key 0 holds every row's maximum, all other keys score zero; V is +1 at the positions 0 and -1 at the
+    positions 31 of every 32 of them, so an output is exactly zero where equal scores give equal
+    probabilities.  (A cubic at some positions, 7.5e-5 off, split dozens of the 131,072 rows.)"""
+    rows = 8192
+    ctx, (x, w_qkv, b_qkv, w_o, b_o) = uniform_rows_ctx(lib, rows, qkv_dtype=1)
+    g = torch.Generator().manual_seed(rows)
+    x[:, :16] = 0.25 + 3 * torch.rand(rows, 16, generator=g).to(torch.bfloat16)
+    x[:, 16:32] = torch.rand(rows, 16, generator=g).to(torch.bfloat16)
+    x[32::32, 32], x[63::32, 32], x[0, 33] = 1.0, -1.0, 1.0
+    for h in range(16):
+        w_qkv[64 * h, h] = w_qkv[64 * h + 1, 16 + h] = w_qkv[2048 + 64 * h, 32] = 1.0
+        w_qkv[1024 + 64 * h, 33], w_qkv[1024 + 64 * h + 1, 33] = 12 + h / 2, 9 - h / 4
+    ctx.global_attn(x.cuda(), w_qkv.cuda(), b_qkv.cuda(), w_o.cuda(), b_o.cuda())
+    ctx.poll()
+    o = to_f64(ctx.debug_buffer(1))[:, ::64]
+    report("E4M3 probabilities that differ by position", rows=o.size, split=int((o != 0).sum()))
+    assert not o.any()
+    ctx.close()
+
+
+@pytest.mark.parametrize("key", [128, 159])  # first and last of the 32 keys that a thread takes at a time
+@pytest.mark.parametrize("rows,qkv_dtype", [(4096, 1)])
+def test_a_key_that_is_not_a_number_shows_in_every_output(lib, rows, qkv_dtype, key):
+    """One token's K of one head overflows before its normalisation and is NaN after it, with a finite V: every
+    row attends to it, so that head's outputs are NaN throughout, and no other head's."""
+    ctx, (x, w_qkv, b_qkv, w_o, b_o) = uniform_rows_ctx(lib, rows, qkv_dtype)
+    g = torch.Generator().manual_seed(rows + key)
+    x[:] = torch.randn(rows, 1024, generator=g).to(torch.bfloat16)
+    w_qkv, b_qkv, w_o, b_o = make_attention_weights(WORKLOADS["C1"], 0)
+    x[:, 7], w_qkv[:, 7] = 0.0, 0.0
+    x[key, 7], w_qkv[1024 + 3 * 64:1024 + 4 * 64, 7] = 2.0 ** 100, 2.0 ** 100
+    one, zero = torch.ones(64, dtype=torch.bfloat16).cuda(), torch.zeros(64, dtype=torch.bfloat16).cuda()
+    ctx.global_attn_ext(None, x.cuda(), w_qkv.cuda(), b_qkv.cuda(), w_o.cuda(), b_o.cuda(), q_norm=(10 * one, zero), k_norm=(one, zero))
+    ctx.poll()
+    qkv, o = ctx.debug_buffer(0).float().cpu().numpy(), ctx.debug_buffer(1).float().cpu().numpy()
+    bad = np.isnan(qkv)
+    assert bad[key, 1024 + 192:1024 + 256].all() and bad.sum() == 64
+    if qkv_dtype == 0:
+        assert set(softmax_forms(np.nan_to_num(qkv).astype(np.float64))) == {"shifted"}
+    nan = np.isnan(o)
+    assert nan[:, 192:256].all() and not nan[:, :192].any() and not nan[:, 256:].any()
+    ctx.close()
+
+
 @pytest.mark.parametrize("grid", [(1, 1), (1, 59), (4, 15), (3, 41), (4, 31)], ids=lambda g: f"{g[0]}x{g[1]}")
 def test_frame_attention_at_tile_edges(lib, grid):
     """6, 64, 65, 128 and 129 tokens a frame.  The rows share a common part, as a frame's tokens do:
