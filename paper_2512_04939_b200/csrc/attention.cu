@@ -81,7 +81,7 @@
 // between the tensor core's scores and the exponential.
 // Rows with larger B need a reference other than zero, but seldom a running one: the largest score s0
 // among the first 64 keys bounds the row maximum from below as B does from above, and wherever a
-// whole number m lies close enough to both (kFaShiftUp, kFaShiftDown) it serves the whole sweep - the
+// whole number m lies close enough to both (kFaShiftUp, fa_shift_down) it serves the whole sweep - the
 // shifted form, at the cost of a subtraction or a clamp per score, both of which the bound spares the
 // fixed form.  Trained projections attend that sharply (query weights x 16 on the generator's tokens:
 // B up to 213, 98.6 % of the warps): 31,751 rows went from 4.69 to 4.36 ms there, and from 5.35
@@ -131,11 +131,17 @@ constexpr int kFaPolyPairs = LV_FA_POLY_PAIRS;
 #define LV_FA_SHIFT_POLY_PAIRS 3
 #endif
 constexpr int kFaShiftPolyPairs = LV_FA_SHIFT_POLY_PAIRS;
-// Shifted reference m of a row with score bound B and a known score s0: B - m <= kFaShiftUp keeps row sums
-// over 2^20 keys and |v| <= 2^20 below 2^124; m - s0 <= kFaShiftDown leaves 34 binades between the row's
-// largest probability and the smallest normal number, so that even 2^20 keys that are rounded to
-// zero hold less than 2^-14 of the row's mass (the probabilities' own rounding is 2^-9).
-constexpr float kFaShiftUp = 84.0f, kFaShiftDown = 92.0f;
+// Shifted reference m of a row with score bound B and a known score s0.  B - m <= kFaShiftUp: row sums over the 2^22
+// keys that a sequence may have, times |v| <= 2^20, stay below 2^126.  m - s0 <= fa_shift_down(keys): what lies more
+// than 126 under m is off by up to 2^-126 a key (flushed to zero by the special-function unit, held up at
+// 2^-126 by the polynomial's clamp), the row's largest probability is at least 2^-fa_shift_down, so all such keys
+// together are off by 2^-24 of the row's mass at most - no more than one fp32 rounding of the row sum.
+constexpr float kFaShiftUp = 84.0f;
+static float fa_shift_down(long long keys) {
+  int bits = 0;
+  while ((1ll << bits) < keys) ++bits;
+  return (float)(126 - 24 - bits);
+}
 // Sequences of at most this many rows take CTAs of one query tile, two to an SM (figures at the top).
 #ifndef LV_FA_ONE_TILE_ROWS
 #define LV_FA_ONE_TILE_ROWS 4096
@@ -212,7 +218,7 @@ __device__ __forceinline__ float fast_exp2(float x) {
 // 2^(x - m) for a pair of arguments on the FMA pipes, `magic` = 1.5 * 2^23 - m with m a whole number.
 // Adding it rounds x to the nearest integer and leaves n = that integer - m in the low mantissa
 // bits; the fraction's power comes from a polynomial fitted on [-1/2, 1/2] and n is added to the exponent
-// field.  Valid for x - m in [-120, 120].  The cubic is good to 7.5e-5 relative.  With kFull the degree is 6 and
+// field.  Valid for x - m in [-126, 126].  The cubic is good to 7.5e-5 relative.  With kFull the degree is 6 and
 // the result, rounding included, within 6.6e-8 of 2^(x - m): closer than the special-function unit,
 // whose ex2.approx was measured at up to 1.45e-7 (5.4e-8 against 2.6e-8 in the mean square).
 template <bool kFull>
@@ -299,11 +305,11 @@ __device__ __forceinline__ void exp2_chunk(const uint32_t (&s)[32], uint32_t (&p
 
 // The same for a reference m that is a whole number, |m| <= 2^20: p = 2^(s - m).  For the polynomial
 // pairs the subtraction is free, m being part of the constant that rounds to the nearest integer; they
-// clamp at m - 120, below which the exponent field would wrap.
+// clamp at m - 126, below which the exponent field would wrap.
 template <int kPoly>
 __device__ __forceinline__ void exp2_chunk_shifted(const uint32_t (&s)[32], float m, uint32_t (&packed)[16]) {
   const float2 neg_m = make_float2(-m, -m);
-  const float floor_s = m - 120.0f, magic = 12582912.0f - m;  // exact: 1.5 * 2^23 -+ 2^20 keeps its exponent
+  const float floor_s = m - 126.0f, magic = 12582912.0f - m;  // exact: 1.5 * 2^23 -+ 2^20 keeps its exponent
   const float2 magic2 = make_float2(magic, magic), neg_magic2 = make_float2(-magic, -magic);
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
@@ -344,8 +350,8 @@ template <int kTiles, bool kFirst, bool kLast>
 __global__ void __launch_bounds__(FaShape<kTiles>::kThreads, kTiles == 2 ? 1 : 2)
 flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_bfloat16* __restrict__ qkv,
                        __nv_bfloat16* __restrict__ o, float* __restrict__ o_state, float* __restrict__ ml_state,
-                       const float* __restrict__ k_norm2_max, int seq_len, int dim, int tile_begin, int tile_end,
-                       FaSplit split, uint32_t* status, Stamp stamp) {
+                       const float* __restrict__ k_norm2_max, float shift_down, int seq_len, int dim, int tile_begin,
+                       int tile_end, FaSplit split, uint32_t* status, Stamp stamp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* smem_k = smem;
@@ -656,7 +662,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       pair_barrier(barrier_id);
       const float mx_first = fmaxf(mx_own, xchg->row_max[1][t][c ^ 1][row_in_tile]);
       const float m = ceilf(fmaxf(score_bound - kFaShiftUp, mx_first));
-      shifted = __all_sync(0xffffffffu, m - mx_first <= kFaShiftDown && fabsf(m) <= 1048576.0f ? 1 : 0) != 0;
+      shifted = __all_sync(0xffffffffu, m - mx_first <= shift_down && fabsf(m) <= 1048576.0f ? 1 : 0) != 0;
       if (shifted) m_ref = m;
     } else {
       xchg->row_max[1][t][c][row_in_tile] = INFINITY;  // sends the partner to the form that keeps meeting this warp
@@ -1301,7 +1307,7 @@ cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, 
   CUtensorMap tmap;
   if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap, qkv, (uint64_t)3 * dim, (uint64_t)rows, (uint64_t)3 * dim, 64, 128))
     return cudaErrorInvalidValue;
-  using Kernel = void (*)(const CUtensorMap, const __nv_bfloat16*, __nv_bfloat16*, float*, float*, const float*, int,
+  using Kernel = void (*)(const CUtensorMap, const __nv_bfloat16*, __nv_bfloat16*, float*, float*, const float*, float, int,
                           int, int, int, FaSplit, uint32_t*, Stamp);
   // [query tiles of a CTA - 1][first chunk][last chunk]
   const Kernel kernels[2][2][2] = {
@@ -1331,7 +1337,7 @@ cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, 
     // not before the projection has ended: CTAs that came early would sit two to an SM on the first SMs to
     // become free (four small frames: 9.9 us against 6.2)
     e = launch_clusters(1, false, kernels[a][b][c], grid, threads, smem_bytes[a], s, tmap, qkv, o, ctx->ws.attn_o_state, ctx->ws.attn_ml_state,
-               ctx->ws.attn_kmax, (int)seq_len, dim, begin, end, split, ctx->ws.status, next_stamp(ctx));
+               ctx->ws.attn_kmax, fa_shift_down(seq_len), (int)seq_len, dim, begin, end, split, ctx->ws.status, next_stamp(ctx));
     if (e != cudaSuccess) return e;
     ++*launches;
   }
