@@ -218,7 +218,7 @@ __device__ __forceinline__ float fast_exp2(float x) {
 // 2^(x - m) for a pair of arguments on the FMA pipes, `magic` = 1.5 * 2^23 - m with m a whole number.
 // Adding it rounds x to the nearest integer and leaves n = that integer - m in the low mantissa
 // bits; the fraction's power comes from a polynomial fitted on [-1/2, 1/2] and n is added to the exponent
-// field.  Valid for x - m in [-126, 126].  The cubic is good to 7.5e-5 relative.  With kFull the degree is 6 and
+// field; of a NaN that makes a number beyond the largest bf16, so its row still ends up not finite.  Valid for x - m in [-126, 126].  The cubic is good to 7.5e-5 relative.  With kFull the degree is 6 and
 // the result, rounding included, within 6.6e-8 of 2^(x - m): closer than the special-function unit,
 // whose ex2.approx was measured at up to 1.45e-7 (5.4e-8 against 2.6e-8 in the mean square).
 template <bool kFull>
@@ -247,6 +247,13 @@ __device__ __forceinline__ float2 poly_exp2_pair(float2 x, float2 magic, float2 
 }
 __device__ __forceinline__ float2 poly_exp2_pair(float2 x) {
   return poly_exp2_pair<false>(x, make_float2(12582912.0f, 12582912.0f), make_float2(-12582912.0f, -12582912.0f));
+}
+
+// The larger of the two, NaN if either is.
+__device__ __forceinline__ float fmax_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
 }
 
 // Wait until the most recent loads into a ring (up to one per stage) have landed.
@@ -315,7 +322,7 @@ __device__ __forceinline__ void exp2_chunk_shifted(const uint32_t (&s)[32], floa
   for (int i = 0; i < 16; ++i) {
     float2 p;
     if (i < kPoly) {
-      const float2 x = make_float2(fmaxf(__uint_as_float(s[2 * i]), floor_s), fmaxf(__uint_as_float(s[2 * i + 1]), floor_s));
+      const float2 x = make_float2(fmax_nan(__uint_as_float(s[2 * i]), floor_s), fmax_nan(__uint_as_float(s[2 * i + 1]), floor_s));
       p = poly_exp2_pair<true>(x, magic2, neg_magic2);
     } else {
       const float2 x = __fadd2_rn(make_float2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), neg_m);

@@ -575,7 +575,7 @@ def test_e4m3_probabilities_do_not_depend_on_the_key_position(lib):
 
 
 @pytest.mark.parametrize("key", [128, 159])  # first and last of the 32 keys that a thread takes at a time
-@pytest.mark.parametrize("rows,qkv_dtype", [(4096, 1)])
+@pytest.mark.parametrize("rows,qkv_dtype", [(4096, 0), (8192, 0), (4096, 1)])
 def test_a_key_that_is_not_a_number_shows_in_every_output(lib, rows, qkv_dtype, key):
     """One token's K of one head overflows before its normalisation and is NaN after it, with a finite V: every
     row attends to it, so that head's outputs are NaN throughout, and no other head's."""
