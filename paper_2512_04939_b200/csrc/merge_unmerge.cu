@@ -94,11 +94,12 @@ merge_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ kept_i
   }
 }
 
+template <bool kSmall>  // a grid of at most kOverlapBlocks blocks (common.cuh: SpanOf)
 __global__ void __launch_bounds__(kRowThreads)
 unmerge_kernel(const __nv_bfloat16* __restrict__ ym, const int* __restrict__ dst_of,
                const __nv_bfloat16* __restrict__ residual, __nv_bfloat16* __restrict__ out, long long n_tokens,
                long long n_merged, uint32_t* status, Stamp stamp) {
-  const Span span(stamp);
+  const SpanOf<kSmall> span(stamp);
   const int lane = threadIdx.x & 31;
   const long long i = (long long)blockIdx.x * kRowsPerCta + (threadIdx.x >> 5);
   if (i >= n_tokens) return;
@@ -205,7 +206,7 @@ cudaError_t launch_unmerge(const litevggt_ctx* ctx, const litevggt_plan* plan, c
   const Sizes& z = ctx->sz;
   const unsigned blocks = (unsigned)((z.n_tokens + kRowsPerCta - 1) / kRowsPerCta);
   ++*launches;
-  return launch(unmerge_kernel, dim3(blocks), kRowThreads, 0, s, ym, plan->dst_of, residual, out, z.n_tokens, z.n_merged,
+  return launch(blocks <= kOverlapBlocks ? unmerge_kernel<true> : unmerge_kernel<false>, dim3(blocks), kRowThreads, 0, s, ym, plan->dst_of, residual, out, z.n_tokens, z.n_merged,
                 ctx->ws.status, next_stamp(ctx));
 }
 
