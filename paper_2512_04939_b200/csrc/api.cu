@@ -360,9 +360,19 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
   }
   ctx->timers.stamps = reinterpret_cast<unsigned long long*>(ws.base + o_stamps);
   ws.status = reinterpret_cast<uint32_t*>(ws.base + o_status);
-  if (cudaMemset(ws.base + o_var, 0, o_src - o_var) != cudaSuccess ||
-      cudaMemset(ws.attn_kmax, 0, sizeof(float) * (size_t)z.frames * z.heads) != cudaSuccess ||
-      cudaMemset(ctx->timers.stamps, 0, o_status - o_stamps) != cudaSuccess || cudaMemset(ws.status, 0, 16) != cudaSuccess) {
+  // on a stream of their own and finished before the context is handed out: the caller's stream need not wait
+  // for the default stream, which may be busy with something else
+  cudaStream_t clear = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&clear, cudaStreamNonBlocking);
+  if (e == cudaSuccess) {
+    e = cudaMemsetAsync(ws.base + o_var, 0, o_src - o_var, clear);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws.attn_kmax, 0, sizeof(float) * (size_t)z.frames * z.heads, clear);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->timers.stamps, 0, o_status - o_stamps, clear);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws.status, 0, 16, clear);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(clear);
+    cudaStreamDestroy(clear);
+  }
+  if (e != cudaSuccess) {
     (void)cudaGetLastError();
     cudaFree(ws.base);
     delete ctx;

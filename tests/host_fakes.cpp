@@ -4,6 +4,9 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <functional>
+#include <vector>
+
 #include "../paper_2512_04939_b200/csrc/runtime.h"
 
 using namespace lv;
@@ -14,6 +17,14 @@ static float g_norm_last_seen = 0.0f; // and of the last sequence
 extern "C" void fake_fail_linear(int n) { g_fail_linear = n; }
 extern "C" float fake_norm_seen() { return g_norm_seen; }
 extern "C" float fake_norm_last_seen() { return g_norm_last_seen; }
+// cudaMemset goes to the default stream and returns before it has run; nothing but a synchronisation orders it
+// before work on a non-blocking stream.
+static std::vector<std::function<void()>> g_default_stream;
+static void finish_default_stream() {
+  for (auto& f : g_default_stream) f();
+  g_default_stream.clear();
+}
+extern "C" int fake_default_stream_pending() { return (int)g_default_stream.size(); }
 
 // ---- CUDA runtime
 extern "C" {
@@ -33,13 +44,20 @@ cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaMalloc(void** p, size_t n) { return (*p = calloc(n, 1)) != nullptr ? cudaSuccess : cudaErrorMemoryAllocation; }
 cudaError_t cudaFree(void* p) { free(p); return cudaSuccess; }
-cudaError_t cudaMemset(void* p, int v, size_t n) { memset(p, v, n); return cudaSuccess; }
+cudaError_t cudaMemset(void* p, int v, size_t n) { g_default_stream.push_back([=] { memset(p, v, n); }); return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) { memset(p, v, n); return cudaSuccess; }
-cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { memcpy(d, s, n); return cudaSuccess; }
+cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
+  finish_default_stream();
+  memcpy(d, s, n);
+  return cudaSuccess;
+}
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) { memcpy(d, s, n); return cudaSuccess; }
-cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = nullptr; return cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() { finish_default_stream(); return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+  if (s == nullptr) finish_default_stream();
+  return cudaSuccess;
+}
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = reinterpret_cast<cudaStream_t>(64); return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { *e = nullptr; return cudaSuccess; }

@@ -110,3 +110,12 @@ def test_key_norms_are_zero_after_a_call_that_failed_half_way(host, entry):
         assert follow() == 0
         assert host.fake_norm_seen() == 0.0 and host.fake_norm_last_seen() == 0.0
     host.litevggt_destroy(c.h)
+
+
+def test_a_new_context_has_nothing_pending_on_the_default_stream(host):
+    """The key norms and stopwatch stamps start at zero.  A caller's stream that does not wait for the default
+    stream may use the context at once: a late clearing would wipe norms between projection and attention."""
+    for _ in range(2):
+        c = Ctx(host)
+        assert host.fake_default_stream_pending() == 0
+        host.litevggt_destroy(c.h)
