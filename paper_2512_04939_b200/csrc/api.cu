@@ -105,7 +105,8 @@ litevggt_status cuda_status(cudaError_t e) {
   return e == cudaErrorMemoryAllocation ? LITEVGGT_ERR_ALLOC : LITEVGGT_ERR_CUDA;
 }
 
-litevggt_status alloc_plan(litevggt_ctx* ctx, litevggt_plan** out) {
+// A plan whose memory is cleared on `s`, ahead of whatever fills it there.
+litevggt_status alloc_plan(litevggt_ctx* ctx, cudaStream_t s, litevggt_plan** out) {
   const Sizes& z = ctx->sz;
   DeviceGuard g(ctx->device);
   if (!g.ok) return LITEVGGT_ERR_CUDA;
@@ -120,7 +121,12 @@ litevggt_status alloc_plan(litevggt_ctx* ctx, litevggt_plan** out) {
     delete p;
     return LITEVGGT_ERR_ALLOC;
   }
-  cudaMemset(p->base, 0, c.off);
+  const cudaError_t e = cudaMemsetAsync(p->base, 0, c.off, s);
+  if (e != cudaSuccess) {
+    cudaFree(p->base);
+    delete p;
+    return cuda_status(e);
+  }
   p->magic = kPlanMagic;
   p->owner = ctx;
   p->built = 0;
@@ -493,7 +499,7 @@ litevggt_status litevggt_merge_plan(litevggt_ctx* ctx, const void* x, const floa
   if (!aligned16(x) || !aligned16(grad)) return LITEVGGT_ERR_ALIGN;
   if (*plan_inout != nullptr && (!plan_ok(*plan_inout) || (*plan_inout)->owner != ctx)) return LITEVGGT_ERR_STALE_PLAN;
   if (*plan_inout == nullptr) {
-    litevggt_status st = alloc_plan(ctx, plan_inout);
+    litevggt_status st = alloc_plan(ctx, (cudaStream_t)stream, plan_inout);
     if (st != LITEVGGT_OK) return st;
   }
   litevggt_plan* plan = *plan_inout;
@@ -521,7 +527,7 @@ litevggt_status litevggt_merge_plan_with_partition(litevggt_ctx* ctx, const void
   if (!aligned16(x)) return LITEVGGT_ERR_ALIGN;
   if (*plan_inout != nullptr && (!plan_ok(*plan_inout) || (*plan_inout)->owner != ctx)) return LITEVGGT_ERR_STALE_PLAN;
   if (*plan_inout == nullptr) {
-    litevggt_status st = alloc_plan(ctx, plan_inout);
+    litevggt_status st = alloc_plan(ctx, (cudaStream_t)stream, plan_inout);
     if (st != LITEVGGT_OK) return st;
   }
   litevggt_plan* plan = *plan_inout;
@@ -932,13 +938,14 @@ litevggt_status litevggt_plan_import(litevggt_ctx* ctx, const int32_t* dst_of, l
       }
   }
   litevggt_plan* p = nullptr;
-  litevggt_status st = alloc_plan(ctx, &p);
+  litevggt_status st = alloc_plan(ctx, nullptr, &p);
   if (st != LITEVGGT_OK) return st;
   cudaError_t e = cudaMemcpy(p->dst_of, dst_of, (size_t)n * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(p->size, size.data(), (size_t)m * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(p->kept_idx, kept_idx.data(), (size_t)m * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(p->seg_off, seg_off.data(), (size_t)(m + 1) * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess && r > 0) e = cudaMemcpy(p->seg_src, seg_src.data(), (size_t)r * 4, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // the last copy may still be on its way from the staging buffer
   if (e != cudaSuccess) {
     litevggt_plan_destroy(p);
     return cuda_status(e);

@@ -59,6 +59,11 @@ class Ctx:
         p = self.p
         return self.lib.litevggt_frame_attn(self.h, p, p, p, p, p, None, p, None)
 
+    def merge_plan(self):
+        plan = C.c_void_p()
+        assert self.lib.litevggt_merge_plan(self.h, self.p, self.p, C.byref(plan), None) == 0
+        return plan
+
     def timer(self, which):
         ms, count, one = C.c_float(), C.c_int32(), (C.c_float * 64)()
         assert self.lib.litevggt_timer_samples(self.h, which, one, 64, C.byref(count)) == 0
@@ -119,3 +124,11 @@ def test_a_new_context_has_nothing_pending_on_the_default_stream(host):
         c = Ctx(host)
         assert host.fake_default_stream_pending() == 0
         host.litevggt_destroy(c.h)
+
+
+def test_a_new_plan_is_cleared_on_the_stream_that_fills_it(host):
+    c = Ctx(host)
+    plan = c.merge_plan()
+    assert host.fake_default_stream_pending() == 0
+    assert host.litevggt_plan_destroy(plan) == 0
+    host.litevggt_destroy(c.h)
