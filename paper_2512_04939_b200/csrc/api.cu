@@ -50,7 +50,7 @@ litevggt_status compute_sizes(const litevggt_config& c, Sizes* out) {
   z.patches = (int)p;
   z.tokens_frame = (int)p + c.n_special;
   z.n_tokens = (long long)c.frames * z.tokens_frame;
-  if (z.n_tokens > (1ll << 22)) return LITEVGGT_ERR_BAD_CONFIG;  // scans and sorts are sized for <= 4 Mi tokens
+  if (z.n_tokens > (1ll << 22)) return LITEVGGT_ERR_BAD_CONFIG;  // the index build's scans are sized for <= 4 Mi tokens
   z.n_dst_frame = ((c.grid_h + c.cell_h - 1) / c.cell_h) * ((c.grid_w + c.cell_w - 1) / c.cell_w);
   long long n_ga = (long long)floor(snap(c.ga_keep_frac) * (double)p + 1e-9);
   if (n_ga > p - z.n_dst_frame) n_ga = p - z.n_dst_frame;

@@ -84,8 +84,7 @@
 // whole number m lies close enough to both (kFaShiftUp, fa_shift_down) it serves the whole sweep - the
 // shifted form, at the cost of a subtraction or a clamp per score, both of which the bound spares the
 // fixed form.  Trained projections attend that sharply (query weights x 16 on the generator's tokens:
-// B up to 213, 98.6 % of the warps): 31,751 rows went from 4.69 to 4.36 ms there, and from 5.35
-// to 4.0 ms on Gaussian rows, where the online form rescales more.
+// B up to 213): 31,751 rows went from 4.81 to 4.41 ms there.
 // What remains takes the online form: base-2 softmax with a lazily updated reference
 // maximum, the running output rescaled only when a row maximum grows by more than 2^8 over the
 // reference (the threads then first wait until the tile's last P V has retired).  All three equal
@@ -102,7 +101,7 @@ constexpr int kFaSoftmaxWarps = 16;
 constexpr int kFaThreads = (kFaSoftmaxWarps + 4) * 32;
 constexpr int kFaTileBytes = 128 * 64 * 2;
 constexpr int kFaOnesBytes = 16 * 128;  // 16 key rows of the ones column block
-constexpr uint32_t kFaColS = 0, kFaColO = 256, kFaColQ = 416;
+constexpr uint32_t kFaColS = 0, kFaColO = 256;
 constexpr uint32_t kFaOCols = 80;  // 64 output channels, the row sum, 15 unused columns
 constexpr float kFaRescaleThreshold = 8.0f;
 // Largest Cauchy-Schwarz bound B on the base-2 scores of a row for which the fixed reference is
@@ -125,8 +124,8 @@ constexpr int kFaChunkTiles = LV_FA_CHUNK_TILES;  // 65536 keys: K and V of one 
 constexpr int kFaPolyPairs = LV_FA_POLY_PAIRS;
 // The same in the shifted-reference form, whose polynomial pairs also need a clamp and whose other
 // pairs a subtraction, and which takes the polynomial of degree 6 (the running maximum that served these
-// rows before is as good as the special-function unit).  Core at 31,751 rows: 0 pairs 4.52 ms, 1: 4.47, 2: 4.47,
-// 3: 4.45, 4: 4.45, 5: 4.50; with a cubic, which moves probabilities by 7.5e-5, 4.22.
+// rows before is as good as the special-function unit).  Core at 31,751 rows: 0 pairs 4.53 ms, 2: 4.46, 3: 4.41,
+// 4: 4.39 (level with 3 on another box), 5: 1 % more; with a cubic, which moves probabilities by 7.5e-5, 4.22.
 #ifndef LV_FA_SHIFT_POLY_PAIRS
 #define LV_FA_SHIFT_POLY_PAIRS 3
 #endif
@@ -1230,8 +1229,8 @@ combine_parts_kernel(FaSplit split, __nv_bfloat16* __restrict__ o, int seq_len, 
 
 // How the jobs that do not fill a wave of one CTA an SM are split: into so many parts that their waves end
 // soonest.  A key tile of two query tiles takes about 1.05 us, a CTA 8 us besides, adding the parts up 8.
-// (21,984 rows: 1376 jobs = 9 waves and 44 jobs, three parts each, 1.776 -> 1.718 ms; in the E4M3 form 2.14 ->
-// 2.07; 31,751 rows, shifted reference, 4.36 -> 4.17.)  Sequences of several key chunks have hundreds of waves and are left alone.
+// (21,984 rows: 1376 jobs = 9 waves and 44 jobs, three parts each, 1.776 -> 1.718 ms; in the E4M3 form, when it took part of
+// its exponentials from a polynomial, 2.14 -> 2.07; 31,751 rows, shifted, 4.36 -> 4.17 with its then exponentials.)  Sequences of several key chunks have hundreds of waves and are left alone.
 static FaSplit split_plan(long long seq_len, int n_seq, int heads, int num_sms) {
   const long long n_tiles = (seq_len + 127) / 128, q_blocks = (seq_len + 255) / 256, jobs = q_blocks * heads;
   FaSplit best{(int)q_blocks, 0, 0, nullptr, nullptr};

@@ -35,7 +35,7 @@ __device__ __forceinline__ void wait_for_previous_kernel() {
 
 // A kernel's presence on the device, written into its step's stopwatch: the first block's arrival, and the
 // latest departure of the blocks that can be among the last to leave (blocks start in order, and no more
-// than kSpanBlocks are resident at a time).  Two stores to memory in place of two events between
+// than kSpanBlocks, 32 on each of 148 SMs, are resident at a time).  Two stores to memory in place of two events between
 // kernels, which held the stream for about 2.7 us each: 72 -> 45 us for the layer of four small frames.
 // kMaySmall = false: an instance that is only launched on grids of more than kOverlapBlocks blocks, which have
 // nothing to wait for; without that question in front of its first load, unmerge takes 901 us instead of 991 at

@@ -159,7 +159,7 @@ namespace lv {
 // wait_for_previous_kernel (common.cuh) before it touches memory, so what overlaps is launch latency and
 // set-up: 288 -> 255 us for a block over seven frames, 116 -> 94 us for the first layer of four small
 // ones.  Larger grids gain nothing by it, and asking costs their short blocks time (LayerNorm of 208 K
-// rows: 145 -> 181 us).
+// rows: 145 -> 181 us).  The line, eight blocks on each of 148 SMs, is known to both sides of a launch.
 constexpr long long kOverlapBlocks = 148 * 8;
 template <class... P, class... A>
 inline cudaError_t launch_clusters(int cluster, bool overlap, void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem,

@@ -5,7 +5,7 @@ import os
 import numpy as np
 import torch
 
-_REPORT = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "gpurun_out", "parity_report.jsonl")
+_REPORT = os.environ.get("PARITY_REPORT")  # a file that collects the measured figures
 
 
 # What the bf16 intermediates that the GPU stores inside a layer (qkv and o of an attention layer, the
@@ -80,17 +80,14 @@ def half_ulp_bf16(ref: np.ndarray) -> np.ndarray:
 
 
 def report(name: str, **values):
-    """Print one measured figure of a parity check and append it to the report file (_REPORT)
-    (the tables of measured error against bound are made from that file)."""
+    """Print one measured figure of a parity check and append it to the report file, if one is named
+    (the tables of measured error against bound are made from it)."""
     rec = {"check": name}
     rec.update({k: (float(v) if isinstance(v, (float, np.floating)) else v) for k, v in values.items()})
     print("PARITY " + json.dumps(rec))
-    try:
-        os.makedirs(os.path.dirname(_REPORT), exist_ok=True)
+    if _REPORT:
         with open(_REPORT, "a") as fh:
             fh.write(json.dumps(rec) + "\n")
-    except OSError:
-        pass
 
 
 def check_bf16(name: str, got: np.ndarray, ref: np.ndarray, noise: float = 0.0, elem_noise=None, sampled: bool = False):
