@@ -217,7 +217,8 @@ __device__ __forceinline__ float fast_exp2(float x) {
 // 2^(x - m) for a pair of arguments on the FMA pipes, `magic` = 1.5 * 2^23 - m with m a whole number.
 // Adding it rounds x to the nearest integer and leaves n = that integer - m in the low mantissa
 // bits; the fraction's power comes from a polynomial fitted on [-1/2, 1/2] and n is added to the exponent
-// field; of a NaN that makes a number beyond the largest bf16, so its row still ends up not finite.  Valid for x - m in [-126, 126].  The cubic is good to 7.5e-5 relative.  With kFull the degree is 6 and
+// field; of a NaN that makes a number beyond the largest bf16, so its row still ends up not finite.
+// Valid for x - m in [-126, 120].  The cubic is good to 7.5e-5 relative.  With kFull the degree is 6 and
 // the result, rounding included, within 6.6e-8 of 2^(x - m): closer than the special-function unit,
 // whose ex2.approx was measured at up to 1.45e-7 (5.4e-8 against 2.6e-8 in the mean square).
 template <bool kFull>
@@ -1229,8 +1230,9 @@ combine_parts_kernel(FaSplit split, __nv_bfloat16* __restrict__ o, int seq_len, 
 
 // How the jobs that do not fill a wave of one CTA an SM are split: into so many parts that their waves end
 // soonest.  A key tile of two query tiles takes about 1.05 us, a CTA 8 us besides, adding the parts up 8.
-// (21,984 rows: 1376 jobs = 9 waves and 44 jobs, three parts each, 1.776 -> 1.718 ms; in the E4M3 form, when it took part of
-// its exponentials from a polynomial, 2.14 -> 2.07; 31,751 rows, shifted, 4.36 -> 4.17 with its then exponentials.)  Sequences of several key chunks have hundreds of waves and are left alone.
+// (21,984 rows: 1376 jobs = 9 waves and 44 jobs, three parts each, 1.776 -> 1.718 ms; in the E4M3 form, when it
+// took part of its exponentials from a polynomial, 2.14 -> 2.07; 31,751 rows, shifted, 4.36 -> 4.17 with its
+// exponentials of that time.)  Sequences of several key chunks have hundreds of waves and are left alone.
 static FaSplit split_plan(long long seq_len, int n_seq, int heads, int num_sms) {
   const long long n_tiles = (seq_len + 127) / 128, q_blocks = (seq_len + 255) / 256, jobs = q_blocks * heads;
   FaSplit best{(int)q_blocks, 0, 0, nullptr, nullptr};
