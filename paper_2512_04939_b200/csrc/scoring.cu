@@ -469,9 +469,9 @@ struct ListArgs {
   uint32_t* status;
 };
 
-// Lists of frame blockIdx.x from its classes; a block of kThreads threads.
-template <int kThreads>
-__device__ __forceinline__ void frame_lists(const uint8_t* cls, const ListArgs& a) {
+// Lists of frame blockIdx.x; a block of kThreads threads.  class_of(t) is the class of the frame's token t.
+template <int kThreads, class Classes>
+__device__ __forceinline__ void frame_lists(const Classes& class_of, const ListArgs& a) {
   int *src_list = a.src_list, *dst_list = a.dst_list, *src_pos = a.src_pos;
   const int p_count = a.p_count, n_special = a.n_special, n_src_frame = a.n_src_frame, n_dst_frame = a.n_dst_frame;
   uint32_t* status = a.status;
@@ -487,7 +487,7 @@ __device__ __forceinline__ void frame_lists(const uint8_t* cls, const ListArgs& 
   const int t0 = threadIdx.x * per, t1 = min(tokens_frame, t0 + per);
   int ns = 0, nd = 0;
   for (int t = t0; t < t1; ++t) {
-    const uint8_t c = cls[token0 + t];
+    const uint8_t c = class_of(t);
     ns += c == LITEVGGT_CLS_SRC;
     nd += c == LITEVGGT_CLS_DST;
   }
@@ -510,7 +510,7 @@ __device__ __forceinline__ void frame_lists(const uint8_t* cls, const ListArgs& 
     if (threadIdx.x == 0) atomicOr(status, kStatusBounds);
   }
   for (int t = t0; t < t1; ++t) {
-    const uint8_t c = cls[token0 + t];
+    const uint8_t c = class_of(t);
     int pos = -1;
     if (c == LITEVGGT_CLS_SRC) {
       if (off_s < exp_src) {
@@ -535,20 +535,24 @@ __device__ __forceinline__ void frame_lists(const uint8_t* cls, const ListArgs& 
 // remaining patches by rank counting (rank = number of candidates that beat this one,
 // ties towards the lower index); P <= a few thousand, so all of it lives in shared memory.
 constexpr int kPartThreads = 512;
+constexpr int kRankPatches = kPartThreads / 2;
 
-__device__ __forceinline__ float block_reduce_minmax(float v, bool is_max, float* scratch) {
+// Smallest and largest of two values over the block: v = {min a, max a, min b, max b}, the minima negated.
+__device__ __forceinline__ void block_maxima(float (&v)[4], float (*scratch)[kPartThreads / 32]) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float other = __shfl_xor_sync(0xffffffffu, v, o);
-    v = is_max ? fmaxf(v, other) : fminf(v, other);
+  for (int k = 0; k < 4; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[k] = fmaxf(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
+    if (lane == 0) scratch[k][warp] = v[k];
   }
   __syncthreads();
-  if (lane == 0) scratch[warp] = v;
-  __syncthreads();
-  float r = scratch[0];
-  for (int i = 1; i < kPartThreads / 32; ++i) r = is_max ? fmaxf(r, scratch[i]) : fminf(r, scratch[i]);
-  return r;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[k] = scratch[k][lane % (kPartThreads / 32)];
+#pragma unroll
+    for (int o = kPartThreads / 64; o > 0; o >>= 1) v[k] = fmaxf(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
+  }
 }
 
 // Scores as unsigned words of the same order; -0 and +0 are the same score.
@@ -565,21 +569,20 @@ partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, 
   extern __shared__ float part_smem[];
   const int p_count = grid_h * grid_w;
   float* score = part_smem;                                        // [P]
-  uint8_t* is_dst = reinterpret_cast<uint8_t*>(score + p_count);   // [P]
-  __shared__ float scratch[kPartThreads / 32];
+  uint8_t* is_dst = reinterpret_cast<uint8_t*>(score + p_count);   // [P], the classes in the end
+  __shared__ float scratch[4][kPartThreads / 32];
   __shared__ int hist[256], found_bin, found_need;
   const int f = blockIdx.x;
   const float* g = grad + (size_t)f * p_count;
   const float* v = var + (size_t)f * p_count;
-  float gmin = INFINITY, gmax = -INFINITY, vmin = INFINITY, vmax = -INFINITY;
+  float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
   for (int p = threadIdx.x; p < p_count; p += kPartThreads) {
-    gmin = fminf(gmin, g[p]); gmax = fmaxf(gmax, g[p]);
-    vmin = fminf(vmin, v[p]); vmax = fmaxf(vmax, v[p]);
+    const float a = g[p], b = v[p];
+    m[0] = fmaxf(m[0], -a); m[1] = fmaxf(m[1], a);
+    m[2] = fmaxf(m[2], -b); m[3] = fmaxf(m[3], b);
   }
-  gmin = block_reduce_minmax(gmin, false, scratch);
-  gmax = block_reduce_minmax(gmax, true, scratch);
-  vmin = block_reduce_minmax(vmin, false, scratch);
-  vmax = block_reduce_minmax(vmax, true, scratch);
+  block_maxima(m, scratch);
+  const float gmin = -m[0], gmax = m[1], vmin = -m[2], vmax = m[3];
   const float gden = gmax - gmin + 1e-6f, vden = vmax - vmin + 1e-6f;
   for (int p = threadIdx.x; p < p_count; p += kPartThreads) {
     const float sc = alpha * ((g[p] - gmin) / gden) + beta * ((v[p] - vmin) / vden);
@@ -592,8 +595,7 @@ partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, 
   out += n_special;
   if (f == 0) {  // the first frame's patches are all anchors
     for (int p = threadIdx.x; p < p_count; p += kPartThreads) out[p] = LITEVGGT_CLS_DST;
-    __syncthreads();
-    frame_lists<kPartThreads>(cls, lists);
+    frame_lists<kPartThreads>([&](int t) { return (uint8_t)(t < n_special ? LITEVGGT_CLS_PROTECTED : LITEVGGT_CLS_DST); }, lists);
     return;
   }
   __syncthreads();
@@ -610,6 +612,37 @@ partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, 
     is_dst[best] = 1;
   }
   __syncthreads();
+  auto set_class = [&](int p, uint8_t c) { out[p] = is_dst[p] = c; };
+  auto lists_from_classes = [&] {
+    __syncthreads();
+    frame_lists<kPartThreads>([&](int t) { return t < n_special ? (uint8_t)LITEVGGT_CLS_PROTECTED : is_dst[t - n_special]; }, lists);
+  };
+  // Up to kRankPatches patches: two threads count how many of the others beat one, three barriers where the search below
+  // takes sixteen (four frames of 16 x 16: 6.1 us for the whole kernel, 7.1 with the search and a reduction each
+  // for the two minima and maxima).
+  if (p_count <= kRankPatches) {
+    unsigned* key = reinterpret_cast<unsigned*>(score);  // in their scores' place; 0, below every key, for who takes no part
+    const int p = threadIdx.x >> 1, part = threadIdx.x & 1;
+    float sp = 0.0f;
+    bool dst = true;
+    if (p < p_count) {
+      sp = score[p];
+      dst = is_dst[p] != 0;
+    }
+    __syncthreads();
+    if (p < p_count && part == 0) key[p] = dst || sp != sp ? 0u : score_key(sp);
+    __syncthreads();
+    int rank = 0;
+    if (p < p_count) {
+      const unsigned own = key[p];
+      for (int q = part; q < p_count; q += 2) rank += key[q] > own || (key[q] == own && q < p) ? 1 : 0;
+    }
+    rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+    if (p < p_count && part == 0)
+      set_class(p, dst ? LITEVGGT_CLS_DST : n_ga > 0 && (sp != sp || rank < n_ga) ? LITEVGGT_CLS_GA : LITEVGGT_CLS_SRC);
+    lists_from_classes();
+    return;
+  }
   // The n_ga highest of the other scores, ties towards the lower index: the threshold is found eight
   // bits at a time from the highest (a histogram of the scores that share the bits fixed so far), the
   // scores equal to it are numbered in index order.  (Ranking every patch against every other was 131 of the
@@ -686,10 +719,9 @@ partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, 
       }
       c = ga_token ? LITEVGGT_CLS_GA : LITEVGGT_CLS_SRC;
     }
-    out[p] = c;
+    set_class(p, c);
   }
-  __syncthreads();
-  frame_lists<kPartThreads>(cls, lists);
+  lists_from_classes();
 }
 
 static ListArgs list_args(const litevggt_ctx* ctx) {
@@ -711,7 +743,8 @@ constexpr int kListThreads = 256;
 __global__ void __launch_bounds__(kListThreads)
 build_lists_kernel(const uint8_t* __restrict__ cls, const ListArgs lists, Stamp stamp) {
   const Span span(stamp);
-  frame_lists<kListThreads>(cls, lists);
+  const uint8_t* frame_cls = cls + (long long)blockIdx.x * (lists.p_count + lists.n_special);
+  frame_lists<kListThreads>([&](int t) { return frame_cls[t]; }, lists);
 }
 
 cudaError_t launch_build_lists(const litevggt_ctx* ctx, const uint8_t* cls, cudaStream_t s, int* launches) {
