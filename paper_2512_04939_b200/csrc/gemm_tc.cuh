@@ -460,21 +460,28 @@ struct LinearEpilogue {
 // GELU with the error function, x Phi(x) = 0.5 x (1 + erf(x / sqrt 2)).  erf comes from the five-term
 // rational approximation of Abramowitz & Stegun (7.1.26): for z >= 0, 1 - erf(z) = P(t) exp(-z^2) with
 // t = 1 / (1 + p z), absolute error below 1.5e-7 - three orders of magnitude under the bf16 rounding
-// of the result.  With e = P(t) exp(-z^2), z = |x| / sqrt 2: the result is x (1 - e/2) for x >= 0 and
-// x e/2 for x < 0, so the negative side has no cancellation.
-__device__ __forceinline__ float gelu_erf(float x) {
-  const float z = fabsf(x) * 0.70710678118654752f;
-  float t;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.3275911f, z, 1.0f)));
-  float p = fmaf(1.061405429f, t, -1.453152027f);
-  p = fmaf(p, t, 1.421413741f);
-  p = fmaf(p, t, -0.284496736f);
-  p = fmaf(p, t, 0.254829592f);
-  p *= t;
-  float ex;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(z * z * -1.4426950408889634f));
-  const float h = 0.5f * p * ex;
-  return x * (x >= 0.0f ? 1.0f - h : h);
+// of the result.  With h = P(t) exp(-z^2) / 2, z = |x| / sqrt 2, the result is max(x, 0) - |x| h, so the
+// negative side has no cancellation and neither side a branch.  Two values at a time, in packed arithmetic, 1 / sqrt 2
+// and the 1/2 in the constants: about 9 issue slots a value where the scalar form took 16, in an epilogue that shares
+// them with nobody but draws on the same power (MLP of 208,200 rows 2.75 -> 2.68 ms, of 3,360 rows 55.6 -> 54.8 us;
+// largest error against 64 bits over [-12, 12] 3.3e-7, scalar 4.2e-7).
+__device__ __forceinline__ float2 gelu_erf(float2 x) {
+  auto both = [](float c) { return make_float2(c, c); };
+  const float2 m = make_float2(-fabsf(x.x), -fabsf(x.y));  // -|x|
+  const float2 d = __ffma2_rn(m, both(-0.3275911f * 0.70710678118654752f), both(1.0f));
+  float2 t, ex;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t.x) : "f"(d.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t.y) : "f"(d.y));
+  float2 p = __ffma2_rn(both(0.5f * 1.061405429f), t, both(0.5f * -1.453152027f));
+  p = __ffma2_rn(p, t, both(0.5f * 1.421413741f));
+  p = __ffma2_rn(p, t, both(0.5f * -0.284496736f));
+  p = __ffma2_rn(p, t, both(0.5f * 0.254829592f));
+  p = __fmul2_rn(p, t);
+  const float2 y = __fmul2_rn(m, both(0.84932180028801907f));  // sqrt(log2(e) / 2): 2^(-y^2) = exp(-z^2)
+  const float2 y2 = __fmul2_rn(y, y);
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex.x) : "f"(-y2.x));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex.y) : "f"(-y2.y));
+  return __ffma2_rn(m, __fmul2_rn(p, ex), make_float2(fmaxf(x.x, 0.0f), fmaxf(x.y, 0.0f)));
 }
 
 // Epilogue of the MLP layers: out[row, col] = bf16(act(acc + bias[col]) + residual[row, col]) with
@@ -510,7 +517,11 @@ struct MlpEpilogue {
       }
       if (gelu) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = gelu_erf(v[i]);
+        for (int i = 0; i < 4; ++i) {
+          const float2 g = gelu_erf(make_float2(v[2 * i], v[2 * i + 1]));
+          v[2 * i] = g.x;
+          v[2 * i + 1] = g.y;
+        }
       }
       if (has_res) {
         const uint4 r = rp[q];
