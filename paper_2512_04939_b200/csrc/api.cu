@@ -331,6 +331,7 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
   const size_t o_q8 = c.take<uint8_t>(fp8 ? z.n_merged * z.dim : 0), o_k8 = c.take<uint8_t>(fp8 ? z.n_merged * z.dim : 0);
   const size_t o_v8 = c.take<uint8_t>(fp8 ? m_pad * z.dim : 0), o_amax = c.take<float>(48);
   const size_t o_stamps = c.take<unsigned long long>(2 * kNumTimers * kTimerSlots);
+  const size_t o_taken = c.take<int>(kAttnCounters);
   const size_t o_status = c.take<uint32_t>(4);
   Workspace& ws = ctx->ws;
   if (cudaMalloc(&ws.base, c.off) != cudaSuccess) {
@@ -364,6 +365,7 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
     ws.v8t = ws.base + o_v8;
     ws.qkv_amax = reinterpret_cast<float*>(ws.base + o_amax);
   }
+  ws.attn_taken = reinterpret_cast<int*>(ws.base + o_taken);
   ctx->timers.stamps = reinterpret_cast<unsigned long long*>(ws.base + o_stamps);
   ws.status = reinterpret_cast<uint32_t*>(ws.base + o_status);
   // on a stream of their own and finished before the context is handed out: the caller's stream need not wait
@@ -373,7 +375,7 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
   if (e == cudaSuccess) {
     e = cudaMemsetAsync(ws.base + o_var, 0, o_src - o_var, clear);
     if (e == cudaSuccess) e = cudaMemsetAsync(ws.attn_kmax, 0, sizeof(float) * (size_t)z.frames * z.heads, clear);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->timers.stamps, 0, o_status - o_stamps, clear);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->timers.stamps, 0, o_taken - o_stamps, clear);
     if (e == cudaSuccess) e = cudaMemsetAsync(ws.status, 0, 16, clear);
     if (e == cudaSuccess) e = cudaStreamSynchronize(clear);
     cudaStreamDestroy(clear);

@@ -11,18 +11,27 @@
 // outside its nine key tiles bounded it; the frame-local layer of 200 such frames, projections
 // included, went from 3.09 to 2.58 ms.  The pair of tiles reads every K/V tile once for 256 rows and
 // is the faster one when the sweep is longer: 286 us (one tile) against 279 at 8.3 K rows, 80 each at
-// 4.2 K.  Warp roles of the pair (20 warps):
+// 4.2 K.  Warp roles of the pair (19 warps):
 //   warps 0-15  softmax.  Warp w works on query tile t = w / 8 and TMEM lane quarter w % 4 (one
 //               thread = one query row); the two warps of a (tile, quarter), c = (w / 4) % 2, either
 //               take every other step whole or share each, 32 of its 64 scores per row and warp
 //               (see the sweep in the kernel).  In the online form, which shares, the two threads of
 //               a row swap their partial row maxima through shared memory once per step.  Four
 //               softmax warps per scheduler keep the special-function unit busy while others wait.
+//               (Steps of 48 keys in three score buffers, so that no warp waits for the scores to be
+//               refilled, measured 7 % slower: what a step costs besides its scores counts more.)
 //   warp  16    MMA issuer of tile 0 (one elected lane):  S_h = Q K_jh^T  and  O += P_h V_jh
 //   warp  17    TMA producer (one elected lane): K_j / V_j through two 4-stage shared-memory rings
 //   warp  18    MMA issuer of tile 1 (issuing costs tens of cycles per instruction, so one
 //               thread cannot feed both tiles)
-//   warp  19    idle
+// One CTA of two tiles sits on an SM, so nothing would run under the set-up, the first loads and the write-back of the
+// next: a launch is one such CTA per SM, and each works off jobs (256 rows of one head) until they run out.  The
+// K/V ring goes on from job to job; the next job's queries are fetched while the tensor cores finish this one's last
+// step, take the old ones' place as soon as they have, and the next scores are under way before this job's rows are
+// written.  52,050 rows 10.8 -> 10.5 ms, 251,872 rows 241 -> 237 (of which the power cap takes part back); 31,751 rows
+// at fixed reference 3.85 -> 3.78.  Jobs come off a counter, late in the job before: with a fixed stride, or taken a whole
+// job ahead, rows in the online form left 3 % of 31,751 rows' time to a few CTAs at the end.  With one tile, two
+// CTAs an SM run under each other anyway, and jobs measured 3 % slower.
 // Tensor memory (512 columns allocated, 480 used):
 //   [0,256)    S/P: tile t, half h at column t*128 + h*64.  S_th is 128 x 64 fp32.  A softmax
 //              thread reads its 32 columns and writes its 32 probabilities (16 columns of bf16
@@ -96,12 +105,11 @@
 
 namespace lv {
 
-constexpr int kFaStages = 4;
+constexpr int kFaTileKeys = 128;  // keys of a K/V tile, two steps
 constexpr int kFaSoftmaxWarps = 16;
-constexpr int kFaThreads = (kFaSoftmaxWarps + 4) * 32;
-constexpr int kFaTileBytes = 128 * 64 * 2;
+constexpr int kFaThreads = (kFaSoftmaxWarps + 3) * 32;
+constexpr int kFaTileBytes = kFaTileKeys * 64 * 2;
 constexpr int kFaOnesBytes = 16 * 128;  // 16 key rows of the ones column block
-constexpr uint32_t kFaColS = 0, kFaColO = 256;
 constexpr uint32_t kFaOCols = 80;  // 64 output channels, the row sum, 15 unused columns
 constexpr float kFaRescaleThreshold = 8.0f;
 // Largest Cauchy-Schwarz bound B on the base-2 scores of a row for which the fixed reference is
@@ -124,10 +132,10 @@ constexpr int kFaChunkTiles = LV_FA_CHUNK_TILES;  // 65536 keys: K and V of one 
 constexpr int kFaPolyPairs = LV_FA_POLY_PAIRS;
 // The same in the shifted-reference form, whose polynomial pairs also need a clamp and whose other
 // pairs a subtraction, and which takes the polynomial of degree 6 (the running maximum that served these
-// rows before is as good as the special-function unit).  Core at 31,751 rows: 0 pairs 4.53 ms, 2: 4.46, 3: 4.41,
-// 4: 4.39 (level with 3 on another box), 5: 1 % more; with a cubic, which moves probabilities by 7.5e-5, 4.22.
+// rows before is as good as the special-function unit).  Core at 31,751 rows, query weights x 16: 0 pairs 4.61 ms, 2: 4.52,
+// 3: 4.57, 4: 4.58; x 8: 4.21, 4.13, 4.14, 4.12; with a cubic, which moves probabilities by 7.5e-5, less still.
 #ifndef LV_FA_SHIFT_POLY_PAIRS
-#define LV_FA_SHIFT_POLY_PAIRS 3
+#define LV_FA_SHIFT_POLY_PAIRS 2
 #endif
 constexpr int kFaShiftPolyPairs = LV_FA_SHIFT_POLY_PAIRS;
 // Shifted reference m of a row with score bound B and a known score s0.  B - m <= kFaShiftUp: row sums over the 2^22
@@ -147,31 +155,34 @@ static float fa_shift_down(long long keys) {
 #endif
 constexpr long long kFaOneTileRows = LV_FA_ONE_TILE_ROWS;
 
-// The CTAs of a launch that its last wave would leave alone on the chip, split along the keys: linear block
-// ids from `full` on are (job, part) with `parts` parts to a job (one query block of one head), and leave
-// partial rows for combine_parts_kernel.  parts = 0: a grid of (query blocks, heads, sequences), nothing split.
-struct FaSplit {
-  int q_blocks, full, parts;
-  float* o;   // [slot][256][64] partial output rows, slot = block id - full
+// The jobs of a launch, one query block of one head of one sequence each, query blocks fastest.  Those that the last
+// round would leave alone on the chip are split along the keys: ids from `full` on are (job, part) with
+// `parts` parts to a job, and leave partial rows for combine_parts_kernel.
+struct FaJobs {
+  int q_first, q_blocks, heads, count, full, parts;
+  float* o;   // [slot][256][64] partial output rows, slot = id - full
   float* ml;  // [slot][256]{reference, row sum}
+  int* taken; // how many jobs beyond the CTAs' first ones have been taken; zero when the launch starts
 };
+struct FaTiles {
+  int begin, end;  // a job's key tiles
+};
+__device__ __forceinline__ FaTiles fa_tiles(const FaJobs& jobs, int id, int tile_begin, int tile_end) {
+  const int slot = id - jobs.full;
+  if (slot < 0) return FaTiles{tile_begin, tile_end};
+  const int part = slot % jobs.parts;
+  return FaTiles{(int)((long long)tile_end * part / jobs.parts), (int)((long long)tile_end * (part + 1) / jobs.parts)};
+}
 struct FaJob {
   int q_block, head, seq, slot;  // slot < 0: a whole job
 };
-__device__ __forceinline__ FaJob fa_job(const FaSplit& split, int& tile_begin, int& tile_end) {
-  if (split.parts == 0) return FaJob{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, -1};
-  const int id = blockIdx.x, slot = id - split.full;
-  int job = id;
-  if (slot >= 0) {
-    const int part = slot % split.parts, tiles = tile_end;
-    job = split.full + slot / split.parts;
-    tile_begin = (int)((long long)tiles * part / split.parts);
-    tile_end = (int)((long long)tiles * (part + 1) / split.parts);
-  }
-  return FaJob{job % split.q_blocks, job / split.q_blocks, 0, slot};
+__device__ __forceinline__ FaJob fa_job(const FaJobs& jobs, int id) {
+  const int slot = id - jobs.full, job = slot < 0 ? id : jobs.full + slot / jobs.parts;
+  const int rest = job / jobs.q_blocks;
+  return FaJob{jobs.q_first + job % jobs.q_blocks, rest % jobs.heads, rest / jobs.heads, slot};
 }
 // This thread's 32 channels of row r (0..255) of the job.
-__device__ __forceinline__ void fa_store_part(const FaSplit& split, int slot, int r, int c, const uint32_t (&acc)[32], float scale,
+__device__ __forceinline__ void fa_store_part(const FaJobs& split, int slot, int r, int c, const uint32_t (&acc)[32], float scale,
                                               float m_ref, float row_sum) {
   float4* dst = reinterpret_cast<float4*>(split.o + ((size_t)slot * 256 + r) * 64 + c * 32);
 #pragma unroll
@@ -181,32 +192,37 @@ __device__ __forceinline__ void fa_store_part(const FaSplit& split, int slot, in
   if (c == 0) *reinterpret_cast<float2*>(split.ml + ((size_t)slot * 256 + r) * 2) = make_float2(m_ref, row_sum);
 }
 
-template <int kStages>
+template <int kTiles, int kStages>
 struct FaBarriers {
-  uint64_t q_ready;
   uint64_t k_full[kStages], k_empty[kStages];
   uint64_t v_full[kStages], v_empty[kStages];
-  uint64_t s_full[2][2], p_ready[2][2], pv_done[2], o_done[2];
-  uint64_t teardown[2];
+  uint64_t q_ready[kTiles], s_full[kTiles][2], p_ready[kTiles][2], pv_done[kTiles], o_done[kTiles], o_free[kTiles];
+  uint64_t teardown[kTiles];
+  uint64_t job_full[2], job_empty[2];
+  int job[2];  // the CTA's next jobs
   uint32_t tmem_base;
   uint32_t abort_flag;
 };
-// partial row maxima swapped between the two threads of a row: [step parity][tile][column half][row]
+// what the two warps of a pair tell each other about their 32 rows: [tile][warp of the pair][row]
 template <int kTiles>
-struct FaExchange {
-  float row_max[2][kTiles][2][128];
+struct FaPairs {
+  float first_max[kTiles][2][128];
+  float row_max[2][kTiles][2][128];  // of either half of a key tile
 };
 // What differs between the CTA of two query tiles (one CTA per SM) and that of one (two per SM).
 template <int kTiles>
 struct FaShape {
   static constexpr int kSoftmaxWarps = 8 * kTiles;
-  static constexpr int kThreads = (kSoftmaxWarps + (kTiles == 2 ? 4 : 2)) * 32;
+  static constexpr int kThreads = (kSoftmaxWarps + 1 + kTiles) * 32;
   static constexpr int kStages = kTiles == 2 ? 4 : 3;
   static constexpr uint32_t kTmemCols = 256 * kTiles;
   static constexpr uint32_t kColS = 0, kColO = 128 * kTiles, kColQ = (128 + 80) * kTiles;
   static constexpr int kSmemBytes =
-      2 * kStages * kFaTileBytes + kFaOnesBytes + (int)sizeof(FaExchange<kTiles>) + 512 + 1024;
+      2 * kStages * kFaTileBytes + kFaOnesBytes + (int)sizeof(FaPairs<kTiles>) + 512 + 1024;
 };
+
+constexpr int kFaAloneBytes = 120 * 1024;  // shared memory that keeps a second CTA off the SM
+static_assert(kFaAloneBytes >= FaShape<1>::kSmemBytes, "");
 
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;
@@ -272,28 +288,10 @@ __device__ __forceinline__ void drain_ring(uint64_t* full, uint32_t issued, uint
   }
 }
 
-// Exponentials of 32 scores of a row: p = 2^(s * scale - m_ref), packed to bf16 pairs (the row sum
-// is formed by the tensor core from these rounded values).  The first kPoly of the 16 pairs take the
+// Exponentials of 32 scores of a row, which arrive scaled, with no reference to subtract: p = 2^s, packed to bf16 pairs (the
+// row sum is formed by the tensor core from these rounded values).  The first kPoly of the 16 pairs take the
 // polynomial on the FMA pipes (callers guarantee arguments above -120 for them), the others the
 // special-function unit.
-template <int kPoly>
-__device__ __forceinline__ void softmax_chunk(const uint32_t (&s)[32], float2 scale2, float2 neg_m2,
-                                              uint32_t (&packed)[16]) {
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const float2 x = __ffma2_rn(make_float2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), scale2, neg_m2);
-    float2 p;
-    if (i < kPoly) {
-      p = poly_exp2_pair(x);
-    } else {
-      p.x = fast_exp2(x.x);
-      p.y = fast_exp2(x.y);
-    }
-    packed[i] = pack_bf16(p.x, p.y);
-  }
-}
-
-// The same for scores that arrive already scaled, with no reference to subtract: p = 2^s.
 template <int kPoly>
 __device__ __forceinline__ void exp2_chunk(const uint32_t (&s)[32], uint32_t (&packed)[16]) {
 #pragma unroll
@@ -347,9 +345,10 @@ __device__ __forceinline__ float max32(const uint32_t (&s)[32]) {
   return fmaxf(fmax3(mx[0], mx[1], mx[2]), mx[3]);
 }
 
-__device__ __forceinline__ void pair_barrier(int id) {  // the two warps of one (tile, lane quarter)
-  asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory");
-}
+// The two warps of one (tile, lane quarter).  A warp that gives up arrives once more without waiting, so a partner who comes to
+// the barrier passes it - and then finds the abort flag up and gives up too.
+__device__ __forceinline__ void pair_barrier(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void pair_barrier_leave(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
 
 // kFirst / kLast: this launch holds the first / the last key chunk of the sweep.
 // kTiles: query tiles of the CTA.
@@ -358,7 +357,7 @@ __global__ void __launch_bounds__(FaShape<kTiles>::kThreads, kTiles == 2 ? 1 : 2
 flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_bfloat16* __restrict__ qkv,
                        __nv_bfloat16* __restrict__ o, float* __restrict__ o_state, float* __restrict__ ml_state,
                        const float* __restrict__ k_norm2_max, float shift_down, int seq_len, int dim, int tile_begin,
-                       int tile_end, FaSplit split, uint32_t* status, Stamp stamp) {
+                       int tile_end, FaJobs jobs, uint32_t* status, Stamp stamp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* smem_k = smem;
@@ -366,48 +365,59 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
   constexpr int kStages = Shape::kStages;
   uint8_t* smem_v = smem_k + kStages * kFaTileBytes;
   uint8_t* smem_ones = smem_v + kStages * kFaTileBytes;  // see below
-  FaExchange<kTiles>* xchg = reinterpret_cast<FaExchange<kTiles>*>(smem_ones + kFaOnesBytes);
-  FaBarriers<kStages>* bars = reinterpret_cast<FaBarriers<kStages>*>(xchg + 1);
+  FaPairs<kTiles>* pairs = reinterpret_cast<FaPairs<kTiles>*>(smem_ones + kFaOnesBytes);
+  FaBarriers<kTiles, kStages>* bars = reinterpret_cast<FaBarriers<kTiles, kStages>*>(pairs + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr bool kSplit = kTiles == 2 && kFirst && kLast;
-  FaJob job{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, -1};
-  if constexpr (kSplit) job = fa_job(split, tile_begin, tile_end);
-  // job.seq selects one of the independent sequences of seq_len rows laid back to back (the
-  // global layer has one; a frame-local layer has one per frame)
-  const int row_base = job.seq * seq_len;
-  const int q0 = job.q_block * (128 * kTiles);  // within the sequence
-  const int head = job.head;
-  // this launch covers key tiles [tile_begin, tile_end) of ceil(seq_len / 128); local tile j is
-  // key tile tile_begin + j, step n = local tile n/2, half n%2
-  const int n_kv = tile_end - tile_begin;
-  // a last key tile with at most 64 keys has no second half
-  const bool half_tail = kLast && seq_len - (tile_end - 1) * 128 <= 64;
-  const int n_steps = 2 * n_kv - (half_tail ? 1 : 0);
-  const int n_tiles_live = kTiles == 2 && q0 + 128 < seq_len ? 2 : 1;  // a tile without rows takes no part
   constexpr bool first_chunk = kFirst;
   constexpr bool last_chunk = kLast;
+  // Every role walks over the CTA's jobs by itself; where a CTA has only one it is the block's own.
+  constexpr bool kJobs = kTiles == 2;
+  // The first is the block's own too, the others come off a counter, so that CTAs whose rows need a slower form
+  // of the softmax take fewer.
+  const int id0 = kJobs ? (int)blockIdx.x : 0, id_end = kJobs ? jobs.count : 1;
+  auto job_at = [&](int id) {
+    if constexpr (kJobs) return fa_job(jobs, id);
+    else return FaJob{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, -1};
+  };
+  // A job covers key tiles [begin, end) of ceil(seq_len / 128); its step n is half n % 2 of its tile n / 2.
+  auto tiles_at = [&](int id) {
+    if constexpr (kJobs) return fa_tiles(jobs, id, tile_begin, tile_end);
+    else return FaTiles{tile_begin, tile_end};
+  };
+  auto keys_of = [&](const FaTiles& kv) { return (kLast ? seq_len : kv.end * kFaTileKeys) - kv.begin * kFaTileKeys; };  // at least one
+  // a last key tile with at most 64 keys has no second half
+  auto steps_of = [&](const FaTiles& kv) { return min(2 * (kv.end - kv.begin), (keys_of(kv) + 63) / 64); };
+  // a tile without rows takes no part
+  auto tile_live = [&](int id, int t) { return t == 0 || job_at(id).q_block * (128 * kTiles) + 128 < seq_len; };
 
-  if (threadIdx.x == 0) {
-    mbar_init(&bars->q_ready, 8 * n_tiles_live);
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(&bars->k_full[s], 1);
-      mbar_init(&bars->k_empty[s], n_tiles_live);  // every live tile's MMA issuer releases a stage
-      mbar_init(&bars->v_full[s], 1);
-      mbar_init(&bars->v_empty[s], n_tiles_live);
-    }
-    for (int t = 0; t < 2; ++t) {
-      for (int h = 0; h < 2; ++h) {
-        mbar_init(&bars->s_full[t][h], 1);
-        mbar_init(&bars->p_ready[t][h], 8);
-      }
-      mbar_init(&bars->pv_done[t], 1);
-      mbar_init(&bars->o_done[t], 1);
-    }
-    mbar_init(&bars->teardown[0], 1);
-    mbar_init(&bars->teardown[1], 1);
-    bars->abort_flag = 0;
+  // (by many threads at once: a CTA of a short sequence lives for few microseconds)
+  if (threadIdx.x < kStages) {
+    mbar_init(&bars->k_full[threadIdx.x], 1);
+    mbar_init(&bars->k_empty[threadIdx.x], kTiles);  // every tile's MMA issuer releases a stage
+    mbar_init(&bars->v_full[threadIdx.x], 1);
+    mbar_init(&bars->v_empty[threadIdx.x], kTiles);
     mbar_fence_init();
+  } else if (threadIdx.x >= 32 && threadIdx.x < 32 + 2 * kTiles) {
+    const int t = (threadIdx.x - 32) >> 1, h = threadIdx.x & 1;
+    mbar_init(&bars->s_full[t][h], 1);
+    mbar_init(&bars->p_ready[t][h], 8);
+    if (h == 0) {
+      mbar_init(&bars->q_ready[t], 8);
+      mbar_init(&bars->o_done[t], 1);
+      mbar_init(&bars->teardown[t], 1);
+    } else {
+      mbar_init(&bars->o_free[t], 8);
+      mbar_init(&bars->pv_done[t], 1);
+    }
+    mbar_fence_init();
+  } else if (threadIdx.x == 96) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&bars->job_full[i], 1);
+      mbar_init(&bars->job_empty[i], Shape::kSoftmaxWarps + kTiles);
+    }
+    mbar_fence_init();
+    bars->abort_flag = 0;
     tma_prefetch_desc(&tmap_qkv);
   }
   // The row sums come out of the second MMA: its B operand is 80 columns wide, V's 64 channels and,
@@ -434,29 +444,58 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
   const WaitCtl ctl{&bars->abort_flag, status};
   const Span span(stamp);
 
+  // `turn` (0..3, in the low bits): the CTA's jobs so far; id_end or more where there is no further one, or on a wait given up
+  auto job_after = [&](uint32_t turn, bool one_lane, bool& ok) -> int {
+    if constexpr (kJobs) {
+      ok = one_lane ? mbar_wait(&bars->job_full[turn & 1u], turn >> 1 & 1u, ctl) : mbar_wait_warp(&bars->job_full[turn & 1u], turn >> 1 & 1u, ctl);
+      if (!ok) return id_end;
+      const int id = *reinterpret_cast<volatile int*>(&bars->job[turn & 1u]);
+      if (!one_lane) __syncwarp();
+      if (one_lane || lane == 0) mbar_arrive(&bars->job_empty[turn & 1u]);
+      return id;
+    } else {
+      return id_end;
+    }
+  };
   if (warp == kIssuerWarp + 1) {
     // ------------------------------------------------------------------ TMA producer
     if (elect_one()) {
-      uint32_t k_issued = 0, v_issued = 0;
-      for (int j = 0; j < n_kv; ++j) {
-        const int stage = j % kStages;
-        const uint32_t phase = (uint32_t)(j / kStages) & 1u;
-        if (!mbar_wait(&bars->k_empty[stage], phase ^ 1u, ctl)) break;
-        mbar_expect_tx(&bars->k_full[stage], kFaTileBytes);
-        tma_load_2d(smem_k + stage * kFaTileBytes, &tmap_qkv, &bars->k_full[stage], dim + head * 64,
-                    row_base + (tile_begin + j) * 128);
-        ++k_issued;
-        if (!mbar_wait(&bars->v_empty[stage], phase ^ 1u, ctl)) break;
-        mbar_expect_tx(&bars->v_full[stage], kFaTileBytes);
-        tma_load_2d(smem_v + stage * kFaTileBytes, &tmap_qkv, &bars->v_full[stage], 2 * dim + head * 64,
-                    row_base + (tile_begin + j) * 128);
-        ++v_issued;
+      uint32_t k_issued = 0, v_issued = 0, phase = 0;
+      int stage = 0;
+      bool ok = true;
+      uint32_t turn = 0;
+      for (int id = id0; id < id_end && ok;) {
+        const FaJob job = job_at(id);
+        const FaTiles kv = tiles_at(id);
+        int next_id = id_end;
+        const int row0 = job.seq * seq_len, col = job.head * 64;
+        for (int j = kv.begin; j < kv.end; ++j) {
+          if (kJobs && j == max(kv.begin, kv.end - 2)) {
+            // The next job, to everybody; late, so that it is not kept waiting here while another CTA has nothing to do, and
+            // early enough for the counter's answer to come before these tiles are through.
+            if (turn >= 2 && !mbar_wait(&bars->job_empty[turn & 1u], (turn >> 1 & 1u) ^ 1u, ctl)) { ok = false; break; }
+            next_id = (int)gridDim.x + atomicAdd(jobs.taken, 1);
+            bars->job[turn & 1u] = next_id;
+            mbar_arrive(&bars->job_full[turn & 1u]);
+            ++turn;
+          }
+          if (!mbar_wait(&bars->k_empty[stage], phase ^ 1u, ctl)) { ok = false; break; }
+          mbar_expect_tx(&bars->k_full[stage], kFaTileBytes);
+          tma_load_2d(smem_k + stage * kFaTileBytes, &tmap_qkv, &bars->k_full[stage], dim + col, row0 + j * kFaTileKeys);
+          ++k_issued;
+          if (!mbar_wait(&bars->v_empty[stage], phase ^ 1u, ctl)) { ok = false; break; }
+          mbar_expect_tx(&bars->v_full[stage], kFaTileBytes);
+          tma_load_2d(smem_v + stage * kFaTileBytes, &tmap_qkv, &bars->v_full[stage], 2 * dim + col, row0 + j * kFaTileKeys);
+          ++v_issued;
+          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+        }
+        id = next_id;
       }
       // every load issued by this thread must have landed before the CTA may exit
       drain_ring<kStages>(bars->k_full, k_issued, status);
       drain_ring<kStages>(bars->v_full, v_issued, status);
     }
-  } else if (warp == kIssuerWarp || (n_tiles_live == 2 && warp == kIssuerWarp + 2)) {
+  } else if (warp == kIssuerWarp || (kTiles == 2 && warp == kIssuerWarp + 2)) {
     // ------------------------------------------------------------------ MMA issuer of tile t
     if (elect_one()) {
       const int t = warp == kIssuerWarp ? 0 : 1;
@@ -479,51 +518,72 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         for (int k = 0; k < 4; ++k) umma_ts(s_col + h * 64, q_col + k * 8, b_desc + 2 * k, idesc_qk, k != 0 ? 1u : 0u);
         umma_commit(&bars->s_full[t][h]);
       };
-      bool ok = mbar_wait(&bars->q_ready, 0, ctl);
-      if (ok) ok = mbar_wait(&bars->k_full[0], 0, ctl);
-      if (ok) {
-        tc_fence_after();
-        issue_qk(0, 0);
-        if (n_steps > 1) issue_qk(1, 0);
-        umma_commit(&bars->k_empty[0]);
-      }
+      // the rings and the barriers' phases go on from job to job
       int stage = 0;
-      uint32_t phase = 0;
-      for (int j = 0; j < n_kv && ok; ++j) {
-        int next_stage = stage + 1;
-        uint32_t next_phase = phase;
-        if (next_stage == kStages) { next_stage = 0; next_phase ^= 1u; }
-        const bool last = j + 1 == n_kv;
-        if (!mbar_wait(&bars->v_full[stage], phase, ctl)) { ok = false; break; }
-        if (!last && !mbar_wait(&bars->k_full[next_stage], next_phase, ctl)) { ok = false; break; }
-        for (int h = 0; h < 2; ++h) {
-          if (last && h == 1 && half_tail) break;
-          if (!mbar_wait(&bars->p_ready[t][h], j & 1, ctl)) { ok = false; break; }
-          tc_fence_after();
-          // 64 keys of V_j (64 rows of 128 bytes = 8192 bytes per half), 16 keys per instruction:
-          // 8 TMEM columns of P (keys 0-31 in columns [0,16) of the half, keys 32-63 in [32,48)),
-          // 2048 bytes of V; second 64-column block of B = the ones block
-          const uint32_t v_at = (uint32_t)((stage * kFaTileBytes + h * 8192) >> 4);
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            umma_ts(o_col, s_col + h * 64 + (k >> 1) * 32 + (k & 1) * 8, v_desc_at(v_at + 128 * k), idesc_pv,
-                    (j | h | k) != 0 ? 1u : 0u);  // every launch starts its accumulators from zero
-          if (last) {
-            // no further Q K^T follows whose completion would tell the softmax threads that this
-            // P V has retired
-            umma_commit(&bars->pv_done[t]);
-            if (h == 1 || half_tail) umma_commit(&bars->o_done[t]);
-          } else if (h == 1 && half_tail && j + 2 == n_kv) {
-            umma_commit(&bars->pv_done[t]);  // the half that would follow does not exist
-          } else {
-            issue_qk(h, next_stage);
+      uint32_t phase = 0, round = 0;              // round: jobs of this tile so far
+      uint32_t turn = 0;                          // parities of the two halves' barriers when a job starts, a bit each
+      bool ok = true;
+      uint32_t jobs_done = 0;
+      for (int id = id0; id < id_end && ok; id = ok ? job_after(jobs_done++, true, ok) : id_end) {
+        const FaTiles kv = tiles_at(id);
+        const int n_kv = kv.end - kv.begin, n_steps = steps_of(kv);
+        if (!tile_live(id, t)) {
+          for (int j = 0; j < n_kv && ok; ++j) {  // the stages go by
+            ok = mbar_wait(&bars->k_full[stage], phase, ctl);
+            if (ok) mbar_arrive(&bars->k_empty[stage]);
+            if (ok) ok = mbar_wait(&bars->v_full[stage], phase, ctl);
+            if (ok) mbar_arrive(&bars->v_empty[stage]);
+            if (++stage == kStages) { stage = 0; phase ^= 1u; }
           }
+          continue;
         }
-        if (!ok) break;
-        umma_commit(&bars->v_empty[stage]);
-        if (!last) umma_commit(&bars->k_empty[next_stage]);
-        stage = next_stage;
-        phase = next_phase;
+        ok = mbar_wait(&bars->q_ready[t], round & 1u, ctl);
+        if (ok) ok = mbar_wait(&bars->k_full[stage], phase, ctl);
+        if (ok) {
+          tc_fence_after();
+          issue_qk(0, stage);
+          if (n_steps > 1) issue_qk(1, stage);
+          umma_commit(&bars->k_empty[stage]);
+        }
+        for (int j = 0; j < n_kv && ok; ++j) {
+          int next_stage = stage + 1;
+          uint32_t next_phase = phase;
+          if (next_stage == kStages) { next_stage = 0; next_phase ^= 1u; }
+          const bool last = j + 1 == n_kv;
+          if (!mbar_wait(&bars->v_full[stage], phase, ctl)) { ok = false; break; }
+          if (!last && !mbar_wait(&bars->k_full[next_stage], next_phase, ctl)) { ok = false; break; }
+          // the previous job's output has been read
+          if (j == 0 && round != 0 && !mbar_wait(&bars->o_free[t], (round - 1) & 1u, ctl)) { ok = false; break; }
+          for (int h = 0; h < 2; ++h) {
+            const int n = 2 * j + h;
+            if (n == n_steps) break;
+            if (!mbar_wait(&bars->p_ready[t][h], ((turn >> h) ^ (uint32_t)j) & 1u, ctl)) { ok = false; break; }
+            tc_fence_after();
+            // 64 keys of V_j (64 rows of 128 bytes = 8192 bytes per half), 16 keys per instruction:
+            // 8 TMEM columns of P (keys 0-31 in columns [0,16) of the half, keys 32-63 in [32,48)),
+            // 2048 bytes of V; second 64-column block of B = the ones block
+            const uint32_t v_at = (uint32_t)((stage * kFaTileBytes + h * 8192) >> 4);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              umma_ts(o_col, s_col + h * 64 + (k >> 1) * 32 + (k & 1) * 8, v_desc_at(v_at + 128 * k), idesc_pv,
+                      (j | h | k) != 0 ? 1u : 0u);  // every job starts its accumulators from zero
+            if (n + 2 < n_steps) {
+              issue_qk(h, next_stage);  // where these probabilities were
+            } else {
+              // no Q K^T follows whose completion would tell the softmax threads that this P V has retired; they
+              // ask for the last but one (a job of one step counts too)
+              if (n + 2 == n_steps || n_steps == 1) umma_commit(&bars->pv_done[t]);
+              if (n + 1 == n_steps) umma_commit(&bars->o_done[t]);
+            }
+          }
+          if (!ok) break;
+          umma_commit(&bars->v_empty[stage]);
+          if (!last) umma_commit(&bars->k_empty[next_stage]);
+          stage = next_stage;
+          phase = next_phase;
+        }
+        turn ^= ((uint32_t)(n_steps + 1) >> 1 & 1u) | ((uint32_t)n_steps & 2u);
+        ++round;
       }
       if (!ok) {
         umma_commit(&bars->teardown[t]);
@@ -533,285 +593,319 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         }
       }
     }
-  } else if (warp < 8 * n_tiles_live) {
+  } else if (warp < Shape::kSoftmaxWarps) {
     // ------------------------------------------------------------------ softmax warps
     const int t = warp >> 3;
     const int c = (warp >> 2) & 1;
     const uint32_t quarter = warp & 3u;
-    const int barrier_id = 1 + t * 4 + (int)quarter;
     const int row_in_tile = (int)quarter * 32 + lane;
     const uint32_t lane_base = (quarter * 32u) << 16;
-    const int row_local = q0 + t * 128 + row_in_tile;
-    const bool row_live = row_local < seq_len;
-    const int row = row_base + row_local;  // global row of qkv / o
     const uint32_t s_addr = tmem_base + lane_base + Shape::kColS + t * 128;
-    const uint32_t o_addr = tmem_base + lane_base + Shape::kColO + t * kFaOCols + c * 32;
-    const uint32_t l_addr = tmem_base + lane_base + Shape::kColO + t * kFaOCols + 64;  // row sum column (+15 unused)
-    float q_norm2 = 0.0f;  // |q|^2 of the whole row, summed in the same order by both of its threads
-    bool fixed_ref;
-    float score_bound;
-    {
-      // this thread's half (32 channels) of its query row goes to tensor memory
-      uint32_t qreg[16];
+    const uint32_t o_row = tmem_base + lane_base + Shape::kColO + t * kFaOCols, o_addr = o_row + c * 32;
+
+    auto row_of = [&](const FaJob& job) { return job.q_block * (128 * kTiles) + t * 128 + row_in_tile; };  // within the sequence
+    // This thread's half (32 channels) of its query row, and the Cauchy-Schwarz bound on the whole row's scores (K
+    // carries the softmax scale, so they are in base-2 units already); both threads of the row find the same |q|^2.
+    auto load_q = [&](const FaJob& job, uint32_t (&qreg)[16]) -> float {
+      float own = 0.0f, other = 0.0f;
 #pragma unroll
       for (int i = 0; i < 16; ++i) qreg[i] = 0u;
-      if (row_live) {
-        const uint4* src = reinterpret_cast<const uint4*>(qkv + (size_t)row * 3 * dim + head * 64);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const uint4 v = __ldg(src + i);
+      if (row_of(job) < seq_len) {
+        const uint4* src = reinterpret_cast<const uint4*>(qkv + (size_t)(job.seq * seq_len + row_of(job)) * 3 * dim + job.head * 64);
+        auto square = [](const uint4& v, float sum) {
           const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            q_norm2 = fmaf(bf16_lo(w[e]), bf16_lo(w[e]), q_norm2);
-            q_norm2 = fmaf(bf16_hi(w[e]), bf16_hi(w[e]), q_norm2);
-          }
-          if ((i >> 2) == c) {
-            qreg[4 * (i & 3)] = v.x; qreg[4 * (i & 3) + 1] = v.y; qreg[4 * (i & 3) + 2] = v.z; qreg[4 * (i & 3) + 3] = v.w;
-          }
+          for (int e = 0; e < 4; ++e) sum = fmaf(bf16_hi(w[e]), bf16_hi(w[e]), fmaf(bf16_lo(w[e]), bf16_lo(w[e]), sum));
+          return sum;
+        };
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint4 v = __ldg(src + 4 * c + i);
+          own = square(v, own);
+          qreg[4 * i] = v.x; qreg[4 * i + 1] = v.y; qreg[4 * i + 2] = v.z; qreg[4 * i + 3] = v.w;
         }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) other = square(__ldg(src + 4 * (c ^ 1) + i), other);
       }
-      // Cauchy-Schwarz bound on this row's scores (K carries the softmax scale, so the scores are in
-      // base-2 units already); both threads of a row hold the same value, and both warps of a pair
-      // vote over the same 32 rows, so they agree on the form they run
-      score_bound = sqrtf(q_norm2 * k_norm2_max[job.seq * (dim / 64) + head]);
-      fixed_ref = __all_sync(0xffffffffu, score_bound <= kFaFixedRefLimit ? 1 : 0) != 0;
+      const float q_norm2 = own + other;
+      return sqrtf(q_norm2 * k_norm2_max[job.seq * (dim / 64) + job.head]);
+    };
+    auto hand_q = [&](const uint32_t (&qreg)[16]) {
       tmem_st16(tmem_base + lane_base + Shape::kColQ + t * 32 + c * 16, qreg);
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->q_ready);
-    }
-    float m_ref = -INFINITY;  // reference, in the scores' own (base-2) units
+      if (lane == 0) mbar_arrive(&bars->q_ready[t]);
+    };
     bool ok = true;
-    int pair_syncs = 0;  // both warps of a pair must pass the same number of pair barriers
-    // The sweep of a row whose reference stays what it is: `exps` turns 32 scores into 16 bf16 pairs.  The two
-    // warps of a pair need nothing from each other here, so in the CTA of two tiles (kWide) each takes every
-    // other step whole - one wait and one hand-over for 64 scores a thread where sharing a step pays for
-    // both twice: 1.85 -> 1.79 ms at 22 K rows, 3.73 -> 3.62 at 32 K, 11.2 -> 10.7 at 52 K, 28.9 -> 27.9 at
-    // 83 K.  With one tile, where a sweep is short, sharing gives the shorter step: 286 us either way at 8.3
-    // K rows, 20.4 against 21.7 at 1.8 K.  (Loading 16 or 32 scores ahead of the exponentials
-    // measured the same or, where it spilled, less.)
-    // Only the last tile of a launch can reach past the sequence, so the steps before it need no masking;
-    // shared steps are written out per half so that barrier and tensor-memory addresses are constants of
-    // the loop.
-    constexpr bool kWide = kTiles == 2;
-    auto sweep = [&](auto exps) {
-      auto step = [&](int j, int h, bool may_mask) -> bool {
-        if (!mbar_wait_warp(&bars->s_full[t][h], j & 1, ctl)) return false;
-        tc_fence_after();
+    // Phases that go on from job to job, a bit each: of half 0's and half 1's barriers when a job starts, of the job's own
+    // barriers;
+    uint32_t turn = 0;  // and from bit 4 on the CTA's jobs so far
+    auto next_job = [&](int id) -> int {  // the first from `id` on that has rows in this tile
+      while (id < id_end && !tile_live(id, t)) {
+        id = job_after(turn >> 4, false, ok);
+        turn += 16u;
+      }
+      return id;
+    };
+    const int barrier_id = 1 + t * 4 + (int)quarter;
+    auto meet = [&]() -> bool {
+      pair_barrier(barrier_id);
+      return __all_sync(0xffffffffu, *ctl.abort_flag == 0u ? 1 : 0) != 0;
+    };
+    int id = next_job(id0);
+    float score_bound = 0.0f;
+    if (id < id_end) {
+      uint32_t qreg[16];
+      score_bound = load_q(job_at(id), qreg);
+      hand_q(qreg);
+    }
+    while (id < id_end) {
+      const FaTiles kv = tiles_at(id);
+      const int n_keys = keys_of(kv), n_steps = steps_of(kv), last = kv.end - kv.begin - 1;
+      const bool warp_live = kTiles * 128 * job_at(id).q_block + t * 128 + (int)quarter * 32 < seq_len;
+      // both warps of a pair vote over the same 32 rows, so they agree on the form they run
+      const bool fixed_ref = __all_sync(0xffffffffu, score_bound <= kFaFixedRefLimit ? 1 : 0) != 0;
+      float m_ref = -INFINITY;  // reference, in the scores' own (base-2) units
+      auto masked = [&](uint32_t (&s)[32], int valid) {
 #pragma unroll
-        for (int i = 0; i < (kWide ? 2 : 1); ++i) {
-          const int g = kWide ? i : c;  // columns [32 g, 32 g + 32) of the half
-          const uint32_t addr = s_addr + h * 64 + g * 32;
-          uint32_t s[32], packed[16];
-          tmem_ld32(addr, s);
-          tmem_ld_wait();
-          const int valid = may_mask ? seq_len - ((tile_begin + j) * 2 + h) * 64 - g * 32 : 32;
-          if (may_mask && valid < 32) {
-#pragma unroll
-            for (int k = 0; k < 32; ++k)
-              if (k >= valid) s[k] = 0xff800000u;  // -inf: probability 0
-            exps(s, packed, std::true_type{});
-          } else {
-            exps(s, packed, std::false_type{});
-          }
-          tmem_st16(addr, packed);  // over the start of the columns just read
-        }
+        for (int k = 0; k < 32; ++k)
+          if (k >= valid) s[k] = 0xff800000u;  // -inf: probability 0
+      };
+      auto scores_in = [&](int h, uint32_t parity) -> bool { return mbar_wait_warp(&bars->s_full[t][h], parity & 1u, ctl); };
+      // of half h of the job's key tile j
+      auto scores_of = [&](int h, int j) -> bool { return scores_in(h, kJobs ? (turn >> h) ^ (uint32_t)j : (uint32_t)j); };
+      auto give_p = [&](int h, uint32_t count) {
         tmem_st_wait();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_count(&bars->p_ready[t][h], kWide ? 2 : 1);
-        return true;
+        if (lane == 0) mbar_arrive_count(&bars->p_ready[t][h], count);
       };
-      if constexpr (kWide) {
-        for (int j = 0; j + 1 < n_kv && ok; ++j) ok = step(j, c, false);
-        if (ok && n_kv > 0 && !(half_tail && c == 1)) ok = step(n_kv - 1, c, true);
-      } else {
-        for (int j = 0; j + 1 < n_kv && ok; ++j) ok = step(j, 0, false) && step(j, 1, false);
-        if (ok && n_kv > 0) ok = step(n_kv - 1, 0, true) && (half_tail || step(n_kv - 1, 1, true));
-      }
-    };
-    if (q0 + t * 128 + (int)quarter * 32 >= seq_len) {
-      // ---- no live row in this warp (nor in its partner): the issuer needs the hand-over, nobody the result
-      pair_syncs = n_steps;
-      for (int n = 0; n < n_steps && ok; ++n) {
-        ok = mbar_wait_warp(&bars->s_full[t][n & 1], (uint32_t)(n >> 1) & 1u, ctl);
-        if (ok && lane == 0) mbar_arrive(&bars->p_ready[t][n & 1]);
-      }
-    } else if (fixed_ref) {
-      // ---- fixed reference.  The scores all lie inside [-score_bound, score_bound]; the constant
-      // 2^-score_bound that would bring the exponents to [-2 score_bound, 0] cancels between numerator
-      // and row sum, so it is not applied: reference 0, and the scores go into the exponential as
-      // they come out of the tensor core.
-      m_ref = 0.0f;
-      pair_syncs = n_steps;  // this form has no pair barriers
-      sweep([](const uint32_t (&s)[32], uint32_t (&packed)[16], auto masked) {
-        exp2_chunk<decltype(masked)::value ? 0 : kFaPolyPairs>(s, packed);  // (the polynomial cannot take -inf)
-      });
-    } else {
-    // ---- a reference that is not zero.  The first step's scores are looked at once (they stay where
-    // they are for the sweep): their maximum is a lower bound of the row maximum, score_bound an upper one.
-    bool shifted = false;
-    if (mbar_wait_warp(&bars->s_full[t][0], 0, ctl)) {
-      tc_fence_after();
-      uint32_t s[32];
-      tmem_ld32(s_addr + c * 32, s);
-      tmem_ld_wait();
-      const int valid = seq_len - tile_begin * 128 - c * 32;
-      if (valid < 32) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-          if (i >= valid) s[i] = 0xff800000u;  // -inf
-      }
-      const float mx_own = max32(s);
-      xchg->row_max[1][t][c][row_in_tile] = mx_own;  // the sweep's first exchange uses the other slot
-      pair_barrier(barrier_id);
-      const float mx_first = fmaxf(mx_own, xchg->row_max[1][t][c ^ 1][row_in_tile]);
-      const float m = ceilf(fmaxf(score_bound - kFaShiftUp, mx_first));
-      shifted = __all_sync(0xffffffffu, m - mx_first <= shift_down && fabsf(m) <= 1048576.0f ? 1 : 0) != 0;
-      if (shifted) m_ref = m;
-    } else {
-      xchg->row_max[1][t][c][row_in_tile] = INFINITY;  // sends the partner to the form that keeps meeting this warp
-      pair_barrier(barrier_id);
-      ok = false;
-    }
-    if (shifted) {
-    // ---- shifted reference, kept for the whole launch: a whole number m (see kFaShiftUp) under which
-    // nothing overflows and the row's largest probability is not small, so no running maximum is
-    // needed.
-    pair_syncs = n_steps;
-    const float m = m_ref;
-    sweep([m](const uint32_t (&s)[32], uint32_t (&packed)[16], auto masked) {
-      exp2_chunk_shifted<decltype(masked)::value ? 0 : kFaShiftPolyPairs>(s, m, packed);
-    });
-    } else if (ok) {
-    // ---- online form; the same two written-out halves per key tile as above
-    auto step = [&](int j, int h, bool may_mask) -> bool {
-      if (!mbar_wait_warp(&bars->s_full[t][h], j & 1, ctl)) return false;
-      tc_fence_after();
-      uint32_t s[32];
-      tmem_ld32(s_addr + h * 64 + c * 32, s);
-      tmem_ld_wait();
-      if (may_mask) {
-        const int valid = seq_len - ((tile_begin + j) * 2 + h) * 64 - c * 32;
-        if (valid < 32) {
-#pragma unroll
-          for (int i = 0; i < 32; ++i)
-            if (i >= valid) s[i] = 0xff800000u;  // -inf
-        }
-      }
-      const float mx_own = max32(s);
-      // swap with the thread that holds the other 32 scores of this row
-      xchg->row_max[h][t][c][row_in_tile] = mx_own;
-      pair_barrier(barrier_id);
-      ++pair_syncs;
-      const float mx_scaled = fmaxf(mx_own, xchg->row_max[h][t][c ^ 1][row_in_tile]);
-      if ((j | h) == 0) {
-        m_ref = mx_scaled;
-      } else {
-        const bool grow = mx_scaled > m_ref + kFaRescaleThreshold;
-        if (__any_sync(0xffffffffu, grow ? 1 : 0)) {
-          // O_t may still be the target of the previous step's P V.  The issuer follows that P V
-          // with the Q K^T that refills the other half's scores, so their arrival tells that it
-          // has retired; where nothing follows (the last key tile, a half that does not exist), pv_done does.
-          const int jp = h == 1 ? j : j - 1;  // key tile of step n-1 (its half is h^1)
-          const bool waited = 2 * (jp + 1) + (h ^ 1) < n_steps
-                                  ? mbar_wait_warp(&bars->s_full[t][h ^ 1], (uint32_t)(jp + 1) & 1u, ctl)
-                                  : mbar_wait_warp(&bars->pv_done[t], 0, ctl);
-          if (!waited) return false;
+      // The sweep of a row whose reference stays what it is: `exps` turns 32 scores into 16 bf16 pairs.  The two
+      // warps of a pair need nothing from each other here, so in the CTA of two tiles (kWide) each takes every
+      // other step whole - one wait and one hand-over for 64 scores a thread where sharing a step pays for
+      // both twice: 1.85 -> 1.79 ms at 22 K rows, 3.73 -> 3.62 at 32 K, 11.2 -> 10.7 at 52 K, 28.9 -> 27.9 at
+      // 83 K.  With one tile, where a sweep is short, sharing gives the shorter step: 286 us either way at 8.3
+      // K rows, 20.4 against 21.7 at 1.8 K.  (Loading 16 or 32 scores ahead of the exponentials
+      // measured the same or, where it spilled, less.)
+      // Only the last tile of a job can reach past the sequence, so the steps before it need no masking;
+      // shared steps are written out per half so that barrier and tensor-memory addresses are constants of
+      // the loop.
+      constexpr bool kWide = kTiles == 2;
+      auto sweep = [&](auto exps) {
+        auto step = [&](uint32_t parity, int h, bool may_mask) -> bool {
+          if (!scores_in(h, parity)) return false;
           tc_fence_after();
-          const float m_new = grow ? mx_scaled : m_ref;
-          const float alpha = fast_exp2(m_ref - m_new);
-          m_ref = m_new;
-          uint32_t acc[32];  // this thread's 32 of the row's 64 output channels
-          tmem_ld32(o_addr, acc);
-          tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 32; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * alpha);
-          tmem_st32(o_addr, acc);
-          if (c == 1) {  // and the row sum, which is one more accumulator column
-            uint32_t sum[16];
-            tmem_ld16(l_addr, sum);
+          for (int i = 0; i < (kWide ? 2 : 1); ++i) {
+            const int g = kWide ? i : c;  // columns [32 g, 32 g + 32) of the half
+            const uint32_t addr = s_addr + h * 64 + g * 32;
+            uint32_t s[32], packed[16];
+            tmem_ld32(addr, s);
             tmem_ld_wait();
-            sum[0] = __float_as_uint(__uint_as_float(sum[0]) * alpha);
-            tmem_st16(l_addr, sum);
+            const int valid = may_mask ? n_keys - (2 * last + h) * 64 - g * 32 : 32;
+            if (may_mask && valid < 32) {
+              masked(s, valid);
+              exps(s, packed, std::true_type{});
+            } else {
+              exps(s, packed, std::false_type{});
+            }
+            tmem_st16(addr, packed);  // over the start of the columns just read
           }
+          give_p(h, kWide ? 2 : 1);
+          return true;
+        };
+        if constexpr (kWide) {
+          // the counter carries the parity
+          uint32_t j = (turn >> c) & 1u;
+          const uint32_t end = j + (uint32_t)last;
+          for (; j < end && ok; ++j) ok = step(j, c, false);
+          if (ok && 2 * last + c < n_steps) ok = step(end, c, true);
+        } else {
+          for (uint32_t j = 0; j < (uint32_t)last && ok; ++j) ok = step(j, 0, false) && step(j, 1, false);
+          if (ok) ok = step(last, 0, true) && (2 * last + 1 == n_steps || step(last, 1, true));
+        }
+      };
+      if (!warp_live) {
+        // ---- no live row in this warp (nor in its partner): the issuer needs the hand-over, nobody the result
+        for (int n = c; n < n_steps && ok; n += 2) {
+          ok = scores_of(c, n >> 1);
+          if (ok && lane == 0) mbar_arrive_count(&bars->p_ready[t][c], 2);
+        }
+      } else if (fixed_ref) {
+        // ---- fixed reference.  The scores all lie inside [-score_bound, score_bound]; the constant
+        // 2^-score_bound that would bring the exponents to [-2 score_bound, 0] cancels between numerator
+        // and row sum, so it is not applied: reference 0, and the scores go into the exponential as
+        // they come out of the tensor core.
+        m_ref = 0.0f;
+        sweep([](const uint32_t (&s)[32], uint32_t (&packed)[16], auto mask) {
+          exp2_chunk<decltype(mask)::value ? 0 : kFaPolyPairs>(s, packed);  // (the polynomial cannot take -inf)
+        });
+      } else {
+        // ---- a reference that is not zero.  The first step's scores are looked at once (they stay where
+        // they are for the sweep): their maximum is a lower bound of the row maximum, score_bound an upper one.
+        bool shifted = false;
+        ok = scores_of(0, 0);
+        if (ok) {
+          tc_fence_after();
+          uint32_t s[32];
+          tmem_ld32(s_addr + c * 32, s);
+          tmem_ld_wait();
+          masked(s, n_keys - c * 32);
+          const float mx_own = max32(s);
+          pairs->first_max[t][c][row_in_tile] = mx_own;
+          ok = meet();
+          const float mx_first = fmaxf(mx_own, pairs->first_max[t][c ^ 1][row_in_tile]);
+          const float m = ceilf(fmaxf(score_bound - kFaShiftUp, mx_first));
+          shifted = __all_sync(0xffffffffu, m - mx_first <= shift_down && fabsf(m) <= 1048576.0f ? 1 : 0) != 0;
+          if (shifted) m_ref = m;
+        }
+        if (ok && shifted) {
+          // ---- shifted reference, kept for the whole launch: a whole number m (see kFaShiftUp) under which
+          // nothing overflows and the row's largest probability is not small, so no running maximum is
+          // needed.
+          const float m = m_ref;
+          sweep([m](const uint32_t (&s)[32], uint32_t (&packed)[16], auto mask) {
+            exp2_chunk_shifted<decltype(mask)::value ? 0 : kFaShiftPolyPairs>(s, m, packed);
+          });
+        } else if (ok) {
+          // ---- online form.  Both threads of a row share every step, half of its scores each, and tell each other their
+          // maxima.
+          auto step = [&](int j, int h, bool may_mask) -> bool {
+            if (!scores_of(h, j)) return false;
+            tc_fence_after();
+            const uint32_t addr = s_addr + h * 64 + c * 32;
+            // (the scores are read once for the maximum and once more for the exponentials: the registers that this form
+            // takes are the kernel's)
+            auto load = [&](uint32_t (&s)[32]) {
+              tmem_ld32(addr, s);
+              tmem_ld_wait();
+              if (may_mask) masked(s, n_keys - (2 * j + h) * 64 - c * 32);
+            };
+            float mx_own;
+            {
+              uint32_t s[32];
+              load(s);
+              mx_own = max32(s);
+            }
+            pairs->row_max[h][t][c][row_in_tile] = mx_own;
+            if (!meet()) return false;
+            const float mx = fmaxf(mx_own, pairs->row_max[h][t][c ^ 1][row_in_tile]);
+            if ((j | h) == 0) {
+              m_ref = mx;
+            } else {
+              const bool grow = mx > m_ref + kFaRescaleThreshold;
+              if (__any_sync(0xffffffffu, grow ? 1 : 0)) {
+                // O_t may still be the target of the previous step's P V.  The issuer follows that P V
+                // with the Q K^T that refills the other half's scores, so their arrival tells that it
+                // has retired; where nothing follows (the job's last step), pv_done does.
+                const bool waited = 2 * j + h + 1 < n_steps ? scores_of(h ^ 1, j + h)
+                                                            : mbar_wait_warp(&bars->pv_done[t], (turn >> 2) & 1u, ctl);
+                if (!waited) return false;
+                tc_fence_after();
+                const float m_new = grow ? mx : m_ref;
+                const float alpha = fast_exp2(m_ref - m_new);
+                m_ref = m_new;
+                uint32_t acc[32], sum;  // this thread's 32 of the row's 64 output channels; one of the two has the row sum too
+                tmem_ld32(o_addr, acc);
+                tmem_ld1(o_row + 64, sum);
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * alpha);
+                tmem_st32(o_addr, acc);
+                if (c == 1) tmem_st1(o_row + 64, __float_as_uint(__uint_as_float(sum) * alpha));
+              }
+            }
+            uint32_t s[32], packed[16];
+            load(s);
+            exp2_chunk_shifted<0>(s, m_ref, packed);
+            tmem_st16(addr, packed);  // over the start of the columns just read
+            give_p(h, 1);
+            return true;
+          };
+          for (int j = 0; j < last && ok; ++j) ok = step(j, 0, false) && step(j, 1, false);
+          if (ok) ok = step(last, 0, true) && (2 * last + 1 == n_steps || step(last, 1, true));
         }
       }
-      const float2 neg_m2 = make_float2(-m_ref, -m_ref);
-      uint32_t packed[16];
-      softmax_chunk<0>(s, make_float2(1.0f, 1.0f), neg_m2, packed);
-      tmem_st16(s_addr + h * 64 + c * 32, packed);  // over the start of the columns just read
-      tmem_st_wait();
+      if (!ok) break;
+      // The next job's queries are on their way while the tensor cores finish this one; they take the old ones' place,
+      // and the next scores are under way, before this job's rows are written.
+      if constexpr (kJobs) asm volatile("" : "+r"(id));  // the job is worked out again: nothing of it is held over the sweep
+      const int after = job_after(turn >> 4, false, ok);
+      turn += 16u;
+      const int next_id = next_job(after);
+      if (!ok) break;
+      uint32_t qreg[16];
+      if (next_id < id_end) score_bound = load_q(job_at(next_id), qreg);
+      if (!mbar_wait_warp(&bars->o_done[t], (turn >> 2) & 1u, ctl)) break;
+      tc_fence_after();
+      if (next_id < id_end) hand_q(qreg);
+      uint32_t acc[32], sum;
+      tmem_ld32(o_addr, acc);
+      tmem_ld1(o_row + 64, sum);
+      tmem_ld_wait();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->p_ready[t][h]);
-      return true;
-    };
-    for (int j = 0; j + 1 < n_kv && ok; ++j) ok = step(j, 0, false) && step(j, 1, false);
-    if (ok && n_kv > 0) ok = step(n_kv - 1, 0, true) && (half_tail || step(n_kv - 1, 1, true));
-    }
-    }
-    // a warp that gave up early still meets its partner at every barrier the partner may be in
-    for (; pair_syncs < n_steps; ++pair_syncs) pair_barrier(barrier_id);
-    if (ok && mbar_wait_warp(&bars->o_done[t], 0, ctl)) {
-      tc_fence_after();
-      uint32_t acc[32], sum[16];
-      tmem_ld32(o_addr, acc);
-      tmem_ld16(l_addr, sum);
-      tmem_ld_wait();
-      if (kSplit && job.slot >= 0) {
-        if (row_live) fa_store_part(split, job.slot, t * 128 + row_in_tile, c, acc, 1.0f, m_ref, __uint_as_float(sum[0]));
-      } else if (row_live) {
-        float row_sum = __uint_as_float(sum[0]);
-        // each of the row's two threads keeps its own copy of {reference, row sum} in the state
-        float* ml_mine = ml_state + ((size_t)row * (dim / 64) + head) * 4 + 2 * c;
-        if (!first_chunk) {
-          // add what the earlier chunks left for this row, in fp32 with round-to-nearest: partial
-          // output, row sum, and - online form - their reference (the fixed form's is the same in
-          // every launch, bit for bit)
-          const float m_old = ml_mine[0], l_old = ml_mine[1];
-          float a_old = 1.0f, a_new = 1.0f;
-          if (m_old != m_ref) {
-            const float m_tot = fmaxf(m_old, m_ref);
-            a_old = fast_exp2(m_old - m_tot);
-            a_new = fast_exp2(m_ref - m_tot);
-            m_ref = m_tot;
-          }
-          const uint4* src = reinterpret_cast<const uint4*>(o_state + (size_t)row * dim + head * 64 + c * 32);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const uint4 v = src[i];
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-              acc[4 * i + e] = __float_as_uint(fmaf(__uint_as_float(acc[4 * i + e]), a_new, __uint_as_float(w[e]) * a_old));
-          }
-          row_sum = fmaf(row_sum, a_new, l_old * a_old);
-        }
-        if (last_chunk) {
-          const float inv = 1.0f / row_sum;
-          uint4* dst = reinterpret_cast<uint4*>(o + (size_t)row * dim + head * 64 + c * 32);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            uint4 w;
-            w.x = pack_bf16(__uint_as_float(acc[q * 8 + 0]) * inv, __uint_as_float(acc[q * 8 + 1]) * inv);
-            w.y = pack_bf16(__uint_as_float(acc[q * 8 + 2]) * inv, __uint_as_float(acc[q * 8 + 3]) * inv);
-            w.z = pack_bf16(__uint_as_float(acc[q * 8 + 4]) * inv, __uint_as_float(acc[q * 8 + 5]) * inv);
-            w.w = pack_bf16(__uint_as_float(acc[q * 8 + 6]) * inv, __uint_as_float(acc[q * 8 + 7]) * inv);
-            dst[q] = w;
-          }
+      if (kJobs && lane == 0) mbar_arrive(&bars->o_free[t]);
+      const FaJob job = job_at(id);
+      const int row = job.seq * seq_len + row_of(job);  // global row of qkv / o
+      if (row_of(job) < seq_len) {
+        if (job.slot >= 0) {
+          fa_store_part(jobs, job.slot, t * 128 + row_in_tile, c, acc, 1.0f, m_ref, __uint_as_float(sum));
         } else {
-          // leave the sum over the chunks so far for the next launch
-          uint4* dst = reinterpret_cast<uint4*>(o_state + (size_t)row * dim + head * 64 + c * 32);
+          float row_sum = __uint_as_float(sum);
+          // each of the row's two threads keeps its own copy of {reference, row sum} in the state
+          float* ml_mine = ml_state + ((size_t)row * (dim / 64) + job.head) * 4 + 2 * c;
+          if (!first_chunk) {
+            // add what the earlier chunks left for this row, in fp32 with round-to-nearest: partial
+            // output, row sum, and - online form - their reference (the fixed form's is the same in
+            // every launch, bit for bit)
+            const float m_old = ml_mine[0], l_old = ml_mine[1];
+            float a_old = 1.0f, a_new = 1.0f;
+            if (m_old != m_ref) {
+              const float m_tot = fmaxf(m_old, m_ref);
+              a_old = fast_exp2(m_old - m_tot);
+              a_new = fast_exp2(m_ref - m_tot);
+              m_ref = m_tot;
+            }
+            const uint4* src = reinterpret_cast<const uint4*>(o_state + (size_t)row * dim + job.head * 64 + c * 32);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) dst[i] = make_uint4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
-          ml_mine[0] = m_ref;
-          ml_mine[1] = row_sum;
+            for (int i = 0; i < 8; ++i) {
+              const uint4 v = src[i];
+              const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                acc[4 * i + e] = __float_as_uint(fmaf(__uint_as_float(acc[4 * i + e]), a_new, __uint_as_float(w[e]) * a_old));
+            }
+            row_sum = fmaf(row_sum, a_new, l_old * a_old);
+          }
+          if (last_chunk) {
+            const float inv = 1.0f / row_sum;
+            uint4* dst = reinterpret_cast<uint4*>(o + (size_t)row * dim + job.head * 64 + c * 32);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              uint4 w;
+              w.x = pack_bf16(__uint_as_float(acc[q * 8 + 0]) * inv, __uint_as_float(acc[q * 8 + 1]) * inv);
+              w.y = pack_bf16(__uint_as_float(acc[q * 8 + 2]) * inv, __uint_as_float(acc[q * 8 + 3]) * inv);
+              w.z = pack_bf16(__uint_as_float(acc[q * 8 + 4]) * inv, __uint_as_float(acc[q * 8 + 5]) * inv);
+              w.w = pack_bf16(__uint_as_float(acc[q * 8 + 6]) * inv, __uint_as_float(acc[q * 8 + 7]) * inv);
+              dst[q] = w;
+            }
+          } else {
+            // leave the sum over the chunks so far for the next launch
+            uint4* dst = reinterpret_cast<uint4*>(o_state + (size_t)row * dim + job.head * 64 + c * 32);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) dst[i] = make_uint4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
+            ml_mine[0] = m_ref;
+            ml_mine[1] = row_sum;
+          }
         }
       }
+      const uint32_t steps = (uint32_t)steps_of(tiles_at(id));
+      turn ^= ((steps + 1) >> 1 & 1u) | (steps & 2u) | 4u;
+      id = next_id;
     }
+    if (__any_sync(0xffffffffu, *ctl.abort_flag != 0u ? 1 : 0)) pair_barrier_leave(barrier_id);
   }
 
   tc_fence_before();
@@ -839,6 +933,8 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
 //     every key tile each and pass the reference on from step to step;
 //   * scores are multiplied by scale_q scale_k (K arrives with the softmax scale folded in, which its
 //     per-head scale absorbs), the output by scale_v, in fp32.
+constexpr int kFa8Stages = 4;
+constexpr uint32_t kFa8ColS = 0, kFa8ColO = 256;
 constexpr int kFa8KTileBytes = 128 * 64;           // 128 keys x 64 channel bytes
 constexpr int kFa8VTileBytes = 64 * 128;           // 64 channels x 128 key bytes
 constexpr int kFa8VStageBytes = kFa8VTileBytes + 16 * 128;  // + the ones rows
@@ -846,11 +942,20 @@ constexpr uint32_t kFa8ColQ = 416;                 // Q_0, Q_1: 16 columns of 4 
 constexpr float kFa8Headroom = 8.0f;               // the row maximum maps to 2^8 of E4M3's 448
 // What the two warps of a pair hand each other: the reference of their 32 rows after every step, and the
 // barriers that say so.
+struct Fa8Barriers {
+  uint64_t q_ready;
+  uint64_t k_full[kFa8Stages], k_empty[kFa8Stages];
+  uint64_t v_full[kFa8Stages], v_empty[kFa8Stages];
+  uint64_t s_full[2][2], p_ready[2][2], pv_done[2], o_done[2];
+  uint64_t teardown[2];
+  uint32_t tmem_base;
+  uint32_t abort_flag;
+};
 struct Fa8Refs {
   float m_ref[2][2][128];       // [column of steps][tile][row]
   uint64_t ready[2][2][4];      // [column of steps][tile][quarter]
 };
-constexpr int kFa8SmemBytes = kFaStages * (kFa8KTileBytes + kFa8VStageBytes) + (int)sizeof(Fa8Refs) + 512 + 1024;
+constexpr int kFa8SmemBytes = kFa8Stages * (kFa8KTileBytes + kFa8VStageBytes) + (int)sizeof(Fa8Refs) + 512 + 1024;
 
 // 32 scores -> 32 E4M3 probabilities 2^(s * scale - m), all from the special-function unit.  A polynomial good enough
 // to stand beside it (poly_exp2_pair<true>) saves nothing here: core at 21,984 rows 2.13 ms as it is, 2.12
@@ -875,18 +980,19 @@ __global__ void __launch_bounds__(kFaThreads, 1)
 flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __grid_constant__ CUtensorMap tmap_v8t,
                            const uint8_t* __restrict__ q8, const float* __restrict__ amax, __nv_bfloat16* __restrict__ o,
                            float* __restrict__ o_state, float* __restrict__ ml_state, int seq_len, int dim, int tile_begin,
-                           int tile_end, FaSplit split, uint32_t* status, Stamp stamp) {
+                           int tile_end, FaJobs split, uint32_t* status, Stamp stamp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* smem_k = smem;
-  uint8_t* smem_v = smem_k + kFaStages * kFa8KTileBytes;
-  Fa8Refs* refs = reinterpret_cast<Fa8Refs*>(smem_v + kFaStages * kFa8VStageBytes);
-  FaBarriers<kFaStages>* bars = reinterpret_cast<FaBarriers<kFaStages>*>(refs + 1);
+  uint8_t* smem_v = smem_k + kFa8Stages * kFa8KTileBytes;
+  Fa8Refs* refs = reinterpret_cast<Fa8Refs*>(smem_v + kFa8Stages * kFa8VStageBytes);
+  Fa8Barriers* bars = reinterpret_cast<Fa8Barriers*>(refs + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr bool kSplit = kFirst && kLast;
-  FaJob job{(int)blockIdx.x, (int)blockIdx.y, 0, -1};
-  if constexpr (kSplit) job = fa_job(split, tile_begin, tile_end);
+  const FaJob job = fa_job(split, blockIdx.x);
+  const FaTiles kv = fa_tiles(split, blockIdx.x, tile_begin, tile_end);
+  tile_begin = kv.begin;
+  tile_end = kv.end;
   const int q0 = job.q_block * 256;
   const int head = job.head;
   const int n_kv = tile_end - tile_begin;
@@ -895,7 +1001,7 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
 
   if (threadIdx.x == 0) {
     mbar_init(&bars->q_ready, kFaSoftmaxWarps);
-    for (int s = 0; s < kFaStages; ++s) {
+    for (int s = 0; s < kFa8Stages; ++s) {
       mbar_init(&bars->k_full[s], 1);
       mbar_init(&bars->k_empty[s], 2);
       mbar_init(&bars->v_full[s], 1);
@@ -919,7 +1025,7 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
   }
   // the ones rows behind every V stage: 128 bytes of E4M3 1.0 (0x38), then 15 rows of zeros (a row
   // of equal bytes looks the same under the swizzle)
-  for (int i = threadIdx.x; i < kFaStages * 16 * 128 / 16; i += kFaThreads) {
+  for (int i = threadIdx.x; i < kFa8Stages * 16 * 128 / 16; i += kFaThreads) {
     const int stage = i / 128, piece = i % 128;  // 128 16-byte pieces per stage
     const uint32_t fill = piece < 8 ? 0x38383838u : 0u;
     reinterpret_cast<uint4*>(smem_v + stage * kFa8VStageBytes + kFa8VTileBytes)[piece] = make_uint4(fill, fill, fill, fill);
@@ -941,8 +1047,8 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
     if (elect_one()) {
       uint32_t k_issued = 0, v_issued = 0;
       for (int j = 0; j < n_kv; ++j) {
-        const int stage = j % kFaStages;
-        const uint32_t phase = (uint32_t)(j / kFaStages) & 1u;
+        const int stage = j % kFa8Stages;
+        const uint32_t phase = (uint32_t)(j / kFa8Stages) & 1u;
         if (!mbar_wait(&bars->k_empty[stage], phase ^ 1u, ctl)) break;
         mbar_expect_tx(&bars->k_full[stage], kFa8KTileBytes);
         tma_load_2d(smem_k + stage * kFa8KTileBytes, &tmap_k8, &bars->k_full[stage], head * 64, (tile_begin + j) * 128);
@@ -952,8 +1058,8 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
         tma_load_2d(smem_v + stage * kFa8VStageBytes, &tmap_v8t, &bars->v_full[stage], (tile_begin + j) * 128, head * 64);
         ++v_issued;
       }
-      drain_ring<kFaStages>(bars->k_full, k_issued, status);
-      drain_ring<kFaStages>(bars->v_full, v_issued, status);
+      drain_ring<kFa8Stages>(bars->k_full, k_issued, status);
+      drain_ring<kFa8Stages>(bars->v_full, v_issued, status);
     }
   } else if (warp == 16 || warp == 18) {
     // ------------------------------------------------------------------ MMA issuer of tile t
@@ -961,8 +1067,8 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
       const int t = warp == 16 ? 0 : 1;
       constexpr uint32_t idesc_qk = umma_idesc_e4m3(128, 64);
       constexpr uint32_t idesc_pv = umma_idesc_e4m3(128, kFaOCols);
-      const uint32_t s_col = tmem_base + kFaColS + t * 128;
-      const uint32_t o_col = tmem_base + kFaColO + t * kFaOCols;
+      const uint32_t s_col = tmem_base + kFa8ColS + t * 128;
+      const uint32_t o_col = tmem_base + kFa8ColO + t * kFaOCols;
       const uint32_t q_col = tmem_base + kFa8ColQ + t * 16;
       // S_h = Q x K[64h .. 64h+63]^T: 64 rows of 64 bytes = 4096 bytes per half, 32 channels per instruction
       auto issue_qk = [&](int h, int stage) {
@@ -984,7 +1090,7 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
       for (int j = 0; j < n_kv && ok; ++j) {
         int next_stage = stage + 1;
         uint32_t next_phase = phase;
-        if (next_stage == kFaStages) { next_stage = 0; next_phase ^= 1u; }
+        if (next_stage == kFa8Stages) { next_stage = 0; next_phase ^= 1u; }
         const bool last = j + 1 == n_kv;
         if (!mbar_wait(&bars->v_full[stage], phase, ctl)) { ok = false; break; }
         if (!last && !mbar_wait(&bars->k_full[next_stage], next_phase, ctl)) { ok = false; break; }
@@ -1029,9 +1135,9 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
     const int row_local = q0 + t * 128 + row_in_tile;
     const bool row_live = row_local < seq_len;
     const int row = row_local;
-    const uint32_t s_addr = tmem_base + lane_base + kFaColS + t * 128;
-    const uint32_t o_row = tmem_base + lane_base + kFaColO + t * kFaOCols, o_addr = o_row + c * 32;
-    const uint32_t l_addr = tmem_base + lane_base + kFaColO + t * kFaOCols + 64;
+    const uint32_t s_addr = tmem_base + lane_base + kFa8ColS + t * 128;
+    const uint32_t o_row = tmem_base + lane_base + kFa8ColO + t * kFaOCols, o_addr = o_row + c * 32;
+    const uint32_t l_addr = tmem_base + lane_base + kFa8ColO + t * kFaOCols + 64;
     {
       // this thread's 32 channels (32 bytes) of its query row
       uint32_t qreg[8];
@@ -1136,7 +1242,7 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
       tmem_ld32(o_addr, acc);
       tmem_ld16(l_addr, sum);
       tmem_ld_wait();
-      if (kSplit && job.slot >= 0) {
+      if (job.slot >= 0) {
         if (row_live) fa_store_part(split, job.slot, t * 128 + row_in_tile, c, acc, scale_v, m_ref, __uint_as_float(sum[0]));
       } else if (row_live) {
         float row_sum = __uint_as_float(sum[0]);
@@ -1195,9 +1301,9 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
 // Rows of the split jobs: the parts brought to a common reference and added in the order of their keys.
 constexpr int kCombineRows = 32;  // a block's rows; a thread has 8 channels of one
 __global__ void __launch_bounds__(kCombineRows * 8)
-combine_parts_kernel(FaSplit split, __nv_bfloat16* __restrict__ o, int seq_len, int dim, Stamp stamp) {
+combine_parts_kernel(FaJobs split, __nv_bfloat16* __restrict__ o, int seq_len, int dim, Stamp stamp) {
   const Span span(stamp);
-  const int job = split.full + blockIdx.x, q_block = job % split.q_blocks, head = job / split.q_blocks;
+  const int job = split.full + blockIdx.x, q_block = split.q_first + job % split.q_blocks, head = job / split.q_blocks;
   const int r = blockIdx.y * kCombineRows + (threadIdx.x >> 3), ch = (threadIdx.x & 7) * 8;
   const int row = q_block * 256 + r;
   if (row >= seq_len) return;
@@ -1233,38 +1339,47 @@ combine_parts_kernel(FaSplit split, __nv_bfloat16* __restrict__ o, int seq_len, 
 // (21,984 rows: 1376 jobs = 9 waves and 44 jobs, three parts each, 1.776 -> 1.718 ms; in the E4M3 form, when it
 // took part of its exponentials from a polynomial, 2.14 -> 2.07; 31,751 rows, shifted, 4.36 -> 4.17 with its
 // exponentials of that time.)  Sequences of several key chunks have hundreds of waves and are left alone.
-static FaSplit split_plan(long long seq_len, int n_seq, int heads, int num_sms) {
-  const long long n_tiles = (seq_len + 127) / 128, q_blocks = (seq_len + 255) / 256, jobs = q_blocks * heads;
-  FaSplit best{(int)q_blocks, 0, 0, nullptr, nullptr};
-  if (n_seq != 1 || seq_len <= kFaOneTileRows || n_tiles > kFaChunkTiles) return best;
-  const long long rest = jobs % num_sms;
-  if (rest == 0) return best;
+static FaJobs split_plan(long long seq_len, long long rows, int n_seq, int heads, int num_sms, int block_rows) {
+  const long long n_tiles = (seq_len + kFaTileKeys - 1) / kFaTileKeys, q_blocks = (rows + block_rows - 1) / block_rows;
+  const long long count = q_blocks * heads * n_seq;
+  FaJobs jobs{0, (int)q_blocks, heads, (int)count, (int)count, 1, nullptr, nullptr, nullptr};
+  if (n_seq != 1 || seq_len <= kFaOneTileRows || n_tiles > kFaChunkTiles) return jobs;
+  const long long rest = count % num_sms;
+  if (rest == 0) return jobs;
   float best_us = 8.0f + 1.05f * (float)n_tiles;
   for (int parts = 2; parts <= 16 && n_tiles / parts >= 4; ++parts) {
     const float us = 8.0f + (float)((rest * parts + num_sms - 1) / num_sms) * (8.0f + 1.05f * (float)n_tiles / (float)parts);
     if (us < best_us) {
       best_us = us;
-      best.parts = parts;
-      best.full = (int)(jobs - rest);
+      jobs.parts = parts;
     }
   }
-  return best;
+  if (jobs.parts > 1) {
+    jobs.full = (int)(count - rest);
+    jobs.count = jobs.full + (int)rest * jobs.parts;
+  }
+  return jobs;
 }
-static long long split_slots(const FaSplit& split, int heads) {
-  return split.parts == 0 ? 0 : ((long long)split.q_blocks * heads - split.full) * split.parts;
+static long long split_slots(const FaJobs& jobs) { return jobs.count - jobs.full; }
+// The jobs of a launch over query rows [row0, row1), their parts in the context's state buffers; a context without
+// room for them (none, another sequence length, more parts than the whole sequence has) splits nothing.
+static FaJobs jobs_for(const litevggt_ctx* ctx, long long seq_len, long long row0, long long row1, int n_seq, int block_rows) {
+  const int heads = ctx->sz.heads, sms = ctx->num_sms;
+  FaJobs jobs = split_plan(seq_len, row1 - row0, n_seq, heads, sms, block_rows);
+  if (ctx->ws.attn_o_state == nullptr || seq_len != ctx->sz.n_merged ||
+      split_slots(jobs) > split_slots(split_plan(seq_len, seq_len, n_seq, heads, sms, block_rows))) {
+    jobs.count = jobs.full = jobs.q_blocks * heads * n_seq;
+    jobs.parts = 1;
+  }
+  jobs.q_first = (int)(row0 / block_rows);
+  jobs.o = ctx->ws.attn_o_state;
+  jobs.ml = ctx->ws.attn_ml_state;
+  return jobs;
 }
-// Points the plan at the context's state buffers; a context without them (or of another size) splits nothing.
-static FaSplit split_for(const litevggt_ctx* ctx, long long seq_len, int n_seq) {
-  FaSplit split = split_plan(seq_len, n_seq, ctx->sz.heads, ctx->num_sms);
-  if (ctx->ws.attn_o_state == nullptr || seq_len != ctx->sz.n_merged) split.parts = 0;
-  split.o = ctx->ws.attn_o_state;
-  split.ml = ctx->ws.attn_ml_state;
-  return split;
-}
-static cudaError_t launch_combine(const litevggt_ctx* ctx, const FaSplit& split, __nv_bfloat16* o, long long seq_len, cudaStream_t s,
+static cudaError_t launch_combine(const litevggt_ctx* ctx, const FaJobs& split, __nv_bfloat16* o, long long seq_len, cudaStream_t s,
                                   int* launches) {
   ++*launches;
-  return launch(combine_parts_kernel, dim3((unsigned)(split.q_blocks * ctx->sz.heads - split.full), 256 / kCombineRows),
+  return launch(combine_parts_kernel, dim3((unsigned)(split_slots(split) / split.parts), 256 / kCombineRows),
                 kCombineRows * 8, 0, s, split, o, (int)seq_len, ctx->sz.dim, next_stamp(ctx));
 }
 
@@ -1279,7 +1394,7 @@ cudaError_t launch_flash_attention_fp8(litevggt_ctx* ctx, long long m, __nv_bflo
       !make_tmap_u8_2d(ctx->encode_tiled, &tmap_v, ws.v8t, (uint64_t)m_pad, (uint64_t)dim, (uint64_t)m_pad, 128, 64))
     return cudaErrorInvalidValue;
   using Kernel = void (*)(const CUtensorMap, const CUtensorMap, const uint8_t*, const float*, __nv_bfloat16*, float*,
-                          float*, int, int, int, int, FaSplit, uint32_t*, Stamp);
+                          float*, int, int, int, int, FaJobs, uint32_t*, Stamp);
   const Kernel kernels[2][2] = {{flash_attention_fp8_kernel<false, false>, flash_attention_fp8_kernel<false, true>},
                                 {flash_attention_fp8_kernel<true, false>, flash_attention_fp8_kernel<true, true>}};
   static std::atomic<unsigned long long> smem_set[2][2];
@@ -1288,35 +1403,35 @@ cudaError_t launch_flash_attention_fp8(litevggt_ctx* ctx, long long m, __nv_bflo
       cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(kernels[a][b]), kFa8SmemBytes, smem_set[a][b]);
       if (e != cudaSuccess) return e;
     }
-  const FaSplit split = split_for(ctx, m, 1);
-  const dim3 grid = split.parts > 0 ? dim3((unsigned)(split.full + split_slots(split, ctx->sz.heads)))
-                                    : dim3((unsigned)((m + 255) / 256), (unsigned)ctx->sz.heads, 1);
-  const int n_tiles = (int)((m + 127) / 128);
+  const FaJobs split = jobs_for(ctx, m, 0, m, 1, 256);
+  const dim3 grid((unsigned)split.count);
+  const int n_tiles = (int)((m + kFaTileKeys - 1) / kFaTileKeys);
   const int n_chunks = (n_tiles + kFaChunkTiles - 1) / kFaChunkTiles;
   const int per_chunk = (n_tiles + n_chunks - 1) / n_chunks;
   if (n_chunks > 1 && (ws.attn_o_state == nullptr || ws.attn_ml_state == nullptr)) return cudaErrorInvalidValue;
   for (int begin = 0; begin < n_tiles; begin += per_chunk) {
     const int end = begin + per_chunk < n_tiles ? begin + per_chunk : n_tiles;
-    cudaError_t e = launch_clusters(1, false, kernels[begin == 0][end == n_tiles], grid, kFaThreads, kFa8SmemBytes, s, tmap_k, tmap_v, ws.q8,
+    cudaError_t e = launch(kernels[begin == 0][end == n_tiles], grid, kFaThreads, kFa8SmemBytes, s, tmap_k, tmap_v, ws.q8,
                            ws.qkv_amax, o, ws.attn_o_state, ws.attn_ml_state, (int)m, dim, begin, end, split,
                            ws.status, next_stamp(ctx));
     if (e != cudaSuccess) return e;
     ++*launches;
   }
-  return split.parts > 0 ? launch_combine(ctx, split, o, m, s, launches) : cudaSuccess;
+  return split.parts > 1 ? launch_combine(ctx, split, o, m, s, launches) : cudaSuccess;
 }
 
-cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long seq_len, int n_seq,
-                                   __nv_bfloat16* o, cudaStream_t s, int* launches) {
-  if (seq_len == 0 || n_seq == 0) return cudaSuccess;
+// `first_counter`: of the job counters that the projection has zeroed, the first that is free
+static cudaError_t launch_rows(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long seq_len, long long row0, long long row1, int n_seq,
+                               int first_counter, __nv_bfloat16* o, cudaStream_t s, int* launches) {
+  if (seq_len == 0 || row0 == row1 || n_seq == 0) return cudaSuccess;
   const int dim = ctx->sz.dim;
   if (dim != 1024 || ctx->ws.attn_kmax == nullptr) return cudaErrorInvalidValue;
   const long long rows = seq_len * n_seq;
   CUtensorMap tmap;
-  if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap, qkv, (uint64_t)3 * dim, (uint64_t)rows, (uint64_t)3 * dim, 64, 128))
+  if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap, qkv, (uint64_t)3 * dim, (uint64_t)rows, (uint64_t)3 * dim, 64, kFaTileKeys))
     return cudaErrorInvalidValue;
   using Kernel = void (*)(const CUtensorMap, const __nv_bfloat16*, __nv_bfloat16*, float*, float*, const float*, float, int,
-                          int, int, int, FaSplit, uint32_t*, Stamp);
+                          int, int, int, FaJobs, uint32_t*, Stamp);
   // [query tiles of a CTA - 1][first chunk][last chunk]
   const Kernel kernels[2][2][2] = {
       {{flash_attention_kernel<1, false, false>, flash_attention_kernel<1, false, true>},
@@ -1328,41 +1443,53 @@ cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, 
   const int tiles = seq_len <= kFaOneTileRows ? 1 : 2;
   // balanced chunks of at most kFaChunkTiles key tiles; more than one needs the state buffers (which
   // are sized for the single long sequence of the global layer)
-  const int n_tiles = (int)((seq_len + 127) / 128);
+  const int n_tiles = (int)((seq_len + kFaTileKeys - 1) / kFaTileKeys);
   const int n_chunks = (n_tiles + kFaChunkTiles - 1) / kFaChunkTiles;
   const int per_chunk = (n_tiles + n_chunks - 1) / n_chunks;
   if (n_chunks > 1 && (n_seq != 1 || ctx->ws.attn_o_state == nullptr || ctx->ws.attn_ml_state == nullptr))
     return cudaErrorInvalidValue;
-  const FaSplit split = split_for(ctx, seq_len, n_seq);
-  const dim3 grid = split.parts > 0 ? dim3((unsigned)(split.full + split_slots(split, ctx->sz.heads)))
-                                    : dim3((unsigned)((n_tiles + tiles - 1) / tiles), (unsigned)ctx->sz.heads, (unsigned)n_seq);
+  FaJobs split = jobs_for(ctx, seq_len, row0, row1, n_seq, 128 * tiles);
+  if (tiles == 2 && (ctx->ws.attn_taken == nullptr || first_counter + n_chunks > kAttnCounters)) return cudaErrorInvalidValue;
+  split.taken = ctx->ws.attn_taken + first_counter;
+  const dim3 grid = tiles == 2 ? dim3((unsigned)(split.count < ctx->num_sms ? split.count : ctx->num_sms))
+                               : dim3((unsigned)split.q_blocks, (unsigned)ctx->sz.heads, (unsigned)n_seq);
   const int threads = tiles == 2 ? FaShape<2>::kThreads : FaShape<1>::kThreads;
+  // CTAs of one tile that set themselves up under the projection's last blocks would sit two to an SM on the first SMs
+  // to become free (four small frames: 9.9 us against 6.2).  Where there is an SM for each, they ask for one
+  // of their own; where there is not, they wait.
+  const bool early = tiles == 2 || (long long)grid.x * grid.y * grid.z <= ctx->num_sms;
+  const int smem = tiles == 1 && early ? kFaAloneBytes : smem_bytes[tiles - 1];
   for (int begin = 0; begin < n_tiles; begin += per_chunk) {
     const int end = begin + per_chunk < n_tiles ? begin + per_chunk : n_tiles;
     const int a = tiles - 1, b = begin == 0, c = end == n_tiles;
-    cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(kernels[a][b][c]), smem_bytes[a], smem_set[a][b][c]);
+    cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(kernels[a][b][c]), a == 0 ? kFaAloneBytes : smem_bytes[a],
+                                              smem_set[a][b][c]);
     if (e != cudaSuccess) return e;
-    // not before the projection has ended: CTAs that came early would sit two to an SM on the first SMs to
-    // become free (four small frames: 9.9 us against 6.2)
-    e = launch_clusters(1, false, kernels[a][b][c], grid, threads, smem_bytes[a], s, tmap, qkv, o, ctx->ws.attn_o_state, ctx->ws.attn_ml_state,
+    e = launch_clusters(1, early, kernels[a][b][c], grid, threads, smem, s, tmap, qkv, o, ctx->ws.attn_o_state, ctx->ws.attn_ml_state,
                ctx->ws.attn_kmax, fa_shift_down(seq_len), (int)seq_len, dim, begin, end, split, ctx->ws.status, next_stamp(ctx));
     if (e != cudaSuccess) return e;
     ++*launches;
+    ++split.taken;
   }
-  return split.parts > 0 ? launch_combine(ctx, split, o, seq_len, s, launches) : cudaSuccess;
+  return split.parts > 1 ? launch_combine(ctx, split, o, seq_len, s, launches) : cudaSuccess;
+}
+
+cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long seq_len, int n_seq,
+                                   __nv_bfloat16* o, cudaStream_t s, int* launches) {
+  return launch_rows(ctx, qkv, seq_len, 0, seq_len, n_seq, 0, o, s, launches);
 }
 
 // What passes between launches: for several key chunks rows of fp32 partial output and of {reference, row
 // sum} x 2 per head (one copy per thread of a row), for a split last wave the parts' rows; zero where
 // neither happens.
 size_t attention_state_bytes(long long m, int dim, int heads, int num_sms, size_t* ml_offset) {
-  const long long n_tiles = (m + 127) / 128;
+  const long long n_tiles = (m + kFaTileKeys - 1) / kFaTileKeys;
   size_t o_bytes = 0, ml_bytes = 0;
   if (n_tiles > kFaChunkTiles) {
     o_bytes = (size_t)round_up(m * dim * 4, 256);
     ml_bytes = (size_t)round_up(m * heads * 16, 256);
   } else {
-    const long long slots = split_slots(split_plan(m, 1, heads, num_sms), heads);
+    const long long slots = split_slots(split_plan(m, m, 1, heads, num_sms, 256));
     o_bytes = (size_t)slots * 256 * 64 * 4;
     ml_bytes = (size_t)slots * 256 * 2 * 4;
   }

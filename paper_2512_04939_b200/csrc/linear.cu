@@ -84,7 +84,9 @@ cudaError_t launch_linear_scaled(litevggt_ctx* ctx, const __nv_bfloat16* a, long
   epi.stat_kind = stat.key_norm != nullptr ? kStatKeyNorm : stat.amax != nullptr ? kStatAmax : kStatNone;
   epi.seq_len = (int)stat.seq_len;
   epi.stat = stat.key_norm != nullptr ? stat.key_norm : stat.amax;
-  return launch_gemm_out(ctx, a, m, k, w, n, out, epi, ZeroWords{}, s, launches);
+  // (a context without counters runs attention launches that need none)
+  const ZeroWords taken{reinterpret_cast<uint32_t*>(ctx->ws.attn_taken), ctx->ws.attn_taken != nullptr ? kAttnCounters : 0};
+  return launch_gemm_out(ctx, a, m, k, w, n, out, epi, taken, s, launches);
 }
 
 // out = act(a w^T + bias) + residual, the two layers of the transformer MLP (fc1: GELU, no residual;

@@ -48,6 +48,9 @@ constexpr float kKeyScaleLog2e = 0.125f * 1.4426950408889634f;
 
 constexpr long long kMlpChunkRows = 131072;  // rows of the 4D-wide hidden activations held at a time (1 GiB)
 
+// one counter per launch of an attention core: the key chunks of at most 4 Mi keys
+constexpr int kAttnCounters = 64;
+
 // One device allocation carved into named regions.
 struct Workspace {
   uint8_t* base = nullptr;
@@ -72,6 +75,7 @@ struct Workspace {
   __nv_bfloat16* attn_o = nullptr; // [M, D]
   float* attn_o_state = nullptr;   // [M, D] running output between key chunks (long sequences), or split parts
   float* attn_ml_state = nullptr;  // [M, heads, 4] references and partial row sums, or those of the parts
+  int* attn_taken = nullptr;       // [kAttnCounters] jobs taken by an attention launch's CTAs; every Q/K/V projection zeroes them
   float* attn_kmax = nullptr;      // [max(frames, 1), heads] largest |k|^2 per sequence and head
   // E4M3 variant of the attention operands (qkv_dtype = 1)
   uint8_t* q8 = nullptr;           // [M, D] bytes

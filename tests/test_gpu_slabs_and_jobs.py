@@ -1,0 +1,82 @@
+"""Attention CTAs that work off several jobs and the ranks of a small frame's scores, at the sizes where each can go wrong."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from helpers import check_bf16, to_f64, unfold_k
+from synthdata import WORKLOADS, make_attention_weights
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lib():
+    import paper_2512_04939_b200 as pkg
+
+    return pkg
+
+
+def _tokens(n, seed):
+    # a common part, as a frame's tokens have: outputs do not average out to their rounding noise
+    g = torch.Generator().manual_seed(seed)
+    return (torch.randn(1, 1024, generator=g) + 0.5 * torch.randn(n, 1024, generator=g)).to(torch.bfloat16)
+
+
+def _check_core(name, got, qkv, rows):
+    """got[i] is row rows[i] of the attention core over qkv.  The probabilities are rounded to bf16, each off by at most
+    2^-9 relative, and the row sum is formed from the rounded values: an output moves by 2^-9 sum_i d_i p_i (v_i - o),
+    |d_i| <= 1; Hoeffding's inequality for independent d_i, where 1e7 entries together exceed it with a chance
+    of 1e-6 (a factor sqrt(2 ln 2e13) = 7.8)."""
+    ref, u, worst = O.attention_core(unfold_k(qkv), heads=16, rows=rows), unfold_k(qkv), 0.0
+    for h in range(16):
+        q, k, v = (u[:, i * 1024 + h * 64:i * 1024 + h * 64 + 64] for i in range(3))
+        s = q[rows] @ k.T / 8.0
+        p = np.exp(s - s.max(1, keepdims=True))
+        p2 = (p / p.sum(1, keepdims=True)) ** 2
+        o = ref[:, h * 64:h * 64 + 64]
+        worst = max(worst, float((p2 @ (v * v) - 2 * o * (p2 @ v) + o * o * p2.sum(1, keepdims=True)).max()))
+    noise = 7.8 * 2.0 ** -9 * np.sqrt(worst) / float(np.sqrt(np.mean(ref * ref)))
+    check_bf16(name, got, ref, noise=noise, sampled=True)
+
+
+@pytest.mark.parametrize("sharpness", [1.0, 16.0, 64.0])
+@pytest.mark.parametrize("frames,grid", [(1, (65, 64)), (2, (64, 64)), (3, (67, 62)), (4, (67, 61))])
+def test_sequences_of_several_rounds_of_jobs(lib, frames, grid, sharpness):
+    """Frame attention over 4,161 to 4,165 tokens a frame and the global layer over all of them: 17 query blocks, the last with
+    one live tile of two, times 16 heads times the frames make 1.8 to 7.4 rounds of 148 CTAs; key tiles with
+    and without a second half; all three forms of the softmax, in one CTA after the other."""
+    ctx = lib.LiteVGGT(frames, grid[0], grid[1], 0.0)
+    n, t = ctx.n_tokens, ctx.n_tokens // frames
+    x = _tokens(n, 11 * frames + grid[1])
+    w_qkv, b_qkv, w_o, b_o = make_attention_weights(WORKLOADS["C1"], 6)
+    w_qkv[:1024] *= sharpness
+    dev = [v.cuda() for v in (w_qkv, b_qkv, w_o, b_o)]
+    ctx.global_attn(x.cuda(), *dev)
+    ctx.poll()
+    qkv, core = to_f64(ctx.debug_buffer(0)), to_f64(ctx.debug_buffer(1))
+    rows = np.r_[0:8, n // 2:n // 2 + 8, n - 70:n]
+    _check_core(f"global core, {n} rows, sharpness {sharpness}", core[rows], qkv, rows)
+    eye = torch.eye(1024, dtype=torch.bfloat16).cuda()  # the output projection hands the core through
+    out = to_f64(ctx.frame_attn(x.cuda(), dev[0], dev[1], eye, None))
+    ctx.poll()
+    rows = np.r_[0:4, t - 70:t]
+    for f in range(frames):
+        _check_core(f"frame core {f} of {frames}, {t} rows, sharpness {sharpness}", out[f * t + rows], qkv[f * t:(f + 1) * t], rows)
+    ctx.close()
+
+
+@pytest.mark.parametrize("grid,keep", [((1, 1), 0.1), ((16, 16), 0.1), ((16, 16), 0.9), ((4, 64), 0.5), ((7, 37), 0.1), ((6, 43), 0.3)])
+def test_ranks_of_a_small_frames_scores(lib, grid, keep):
+    """Frames of 1, 256, 258 and 259 patches: up to 256 every patch is ranked against the others, above a search finds
+    the threshold.  Scores in few steps, so that ties decide, and frames whose scores are not numbers."""
+    ctx = lib.LiteVGGT(4, grid[0], grid[1], 0.3, ga_keep_frac=keep)
+    g = torch.Generator().manual_seed(grid[0] * 100 + grid[1])
+    x = torch.randn(13, 1024, generator=g)[torch.randint(0, 13, (ctx.n_tokens,), generator=g)].to(torch.bfloat16)
+    grad = torch.randint(0, 4, (4, *grid), generator=g).float()
+    plan = ctx.merge_plan(x.cuda(), grad.cuda())
+    ctx.poll()
+    ex = ctx.plan_export(plan)
+    assert np.array_equal(ex["cls"], O.partition(ex["ga"], ga_keep_frac=keep))
+    plan.destroy()
+    ctx.close()
