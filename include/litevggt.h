@@ -238,11 +238,14 @@ litevggt_status litevggt_global_layer_host(litevggt_ctx* ctx, litevggt_plan** pl
  * device-to-host copy of its output run on two copy streams of the context, with double-buffered
  * staging, so they overlap the neighbouring calls' kernels instead of adding to them (at 1000
  * frames the two copies are 2 x 2.13 GB, about 6 % of a layer).  Kernels run on `stream`, in call
- * order.  Arguments as in litevggt_global_layer_host; both host buffers should be pinned.
+ * order, but for those that write to out_host.  Arguments as in litevggt_global_layer_host; both host buffers should be pinned.
  *   - x_host must stay unchanged, and out_host is NOT complete, until litevggt_host_drain has been
  *     called on `stream` after this call and that point of the stream has been reached.
  *   - A call does not wait for the output copies of earlier calls: feeding one call's out_host to
  *     the next call's x_host needs a drain in between (or the plain entry point, which is ordered).
+ *   - Where out_host is page-locked and 16-byte aligned, tokens may be written to it as soon as their rows are
+ *     done, in any order.  The attention's rows are then shared out differently over the chip than in
+ *     litevggt_global_layer_host, whose results this call's equal up to rounding.
  *   - The first call allocates the second pair of staging buffers (2 x N x D bf16) and creates the
  *     streams and events. */
 litevggt_status litevggt_global_layer_host_pipelined(litevggt_ctx* ctx, litevggt_plan** plan_inout,

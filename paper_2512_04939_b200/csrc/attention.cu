@@ -1479,6 +1479,22 @@ cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, 
   return launch_rows(ctx, qkv, seq_len, 0, seq_len, n_seq, 0, o, s, launches);
 }
 
+// Query rows of so many rounds of CTAs, in whole query blocks of every head.
+static long long rounds_rows(const litevggt_ctx* ctx, int rounds) { return (long long)rounds * ctx->num_sms / ctx->sz.heads * 256; }
+// One round, so that the first rows are soon there, then two at a time.
+long long flash_attention_slab_end(const litevggt_ctx* ctx, long long m, long long row0) {
+  if (m <= kFaOneTileRows || (m + kFaTileKeys - 1) / kFaTileKeys > kFaChunkTiles) return m;
+  const long long end = row0 + rounds_rows(ctx, row0 == 0 ? 1 : 2);
+  return end < m ? end : m;
+}
+
+cudaError_t launch_flash_attention_rows(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long m, long long row0, long long row1,
+                                        __nv_bfloat16* o, cudaStream_t s, int* launches) {
+  const long long first = rounds_rows(ctx, 1), slab = rounds_rows(ctx, 2), index = row0 == 0 ? 0 : 1 + (row0 - first) / slab;
+  if (row0 < 0 || row0 % 256 != 0 || row1 != flash_attention_slab_end(ctx, m, row0)) return cudaErrorInvalidValue;
+  return launch_rows(ctx, qkv, m, row0, row1, 1, (int)index, o, s, launches);
+}
+
 // What passes between launches: for several key chunks rows of fp32 partial output and of {reference, row
 // sum} x 2 per head (one copy per thread of a row), for a split last wave the parts' rows; zero where
 // neither happens.

@@ -1,0 +1,102 @@
+// What the files behind the C ABI share on the host side: argument checks, stopwatch slots, the workspace that
+// is allocated on first use, the state of the key norms.
+#pragma once
+
+#include "runtime.h"
+
+namespace lv {
+
+struct DeviceGuard {
+  int prev = -1;
+  bool ok = false;
+  explicit DeviceGuard(int dev) {
+    if (cudaGetDevice(&prev) != cudaSuccess) return;
+    ok = cudaSetDevice(dev) == cudaSuccess;
+  }
+  ~DeviceGuard() {
+    if (prev >= 0) cudaSetDevice(prev);
+  }
+};
+
+inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+inline bool ctx_ok(const litevggt_ctx* c) { return c != nullptr && c->magic == kCtxMagic; }
+inline bool plan_ok(const litevggt_plan* p) { return p != nullptr && p->magic == kPlanMagic; }
+
+inline void bump(litevggt_ctx* ctx, int n) { ctx->launches += n; }
+
+// Hands the launches of one step the stopwatch slot that their kernels write; `launches` and `e` are what
+// the step counts its launches in and ends with.
+struct StepTimer {
+  litevggt_ctx* ctx;
+  int which, slot;
+  const int& launches;
+  const int before;
+  const cudaError_t& e;
+  StepTimer(litevggt_ctx* c, int w, const int& n, const cudaError_t& err)
+      : ctx(c), which(w), slot(c->timers.used[w] % kTimerSlots), launches(n), before(n), e(err) {
+    unsigned long long* stamps = c->timers.stamps + 2 * (w * kTimerSlots + slot);
+    c->step.start = stamps;
+    c->step.stop = stamps + 1;
+  }
+  ~StepTimer() {
+    ctx->step = Stamp{};
+    ctx->timers.empty[which][slot] = launches == before || e != cudaSuccess;
+    ++ctx->timers.used[which];
+  }
+};
+
+inline litevggt_status cuda_status(cudaError_t e) {
+  if (e == cudaSuccess) return LITEVGGT_OK;
+  (void)cudaGetLastError();
+  return e == cudaErrorMemoryAllocation ? LITEVGGT_ERR_ALLOC : LITEVGGT_ERR_CUDA;
+}
+
+inline litevggt_status ensure_staging(litevggt_ctx* ctx) {
+  if (ctx->ws.stage_x != nullptr) return LITEVGGT_OK;
+  const Sizes& z = ctx->sz;
+  DeviceGuard g(ctx->device);
+  if (!g.ok) return LITEVGGT_ERR_CUDA;
+  const size_t big = (size_t)z.n_tokens * z.dim * 2, small = (size_t)z.n_merged * z.dim * 2;
+  uint8_t* base = nullptr;
+  const size_t total = 2 * (size_t)round_up((long long)big, 256) + 2 * (size_t)round_up((long long)small, 256);
+  if (cudaMalloc(&base, total) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return LITEVGGT_ERR_ALLOC;
+  }
+  size_t off = 0;
+  ctx->ws.stage_x = reinterpret_cast<__nv_bfloat16*>(base + off); off += (size_t)round_up((long long)big, 256);
+  ctx->ws.stage_out = reinterpret_cast<__nv_bfloat16*>(base + off); off += (size_t)round_up((long long)big, 256);
+  ctx->ws.stage_xm = reinterpret_cast<__nv_bfloat16*>(base + off); off += (size_t)round_up((long long)small, 256);
+  ctx->ws.stage_ym = reinterpret_cast<__nv_bfloat16*>(base + off);
+  ctx->ws.bytes += total;
+  return LITEVGGT_OK;
+}
+
+// The key norms of `sequences` sequences, which an output projection leaves zero for the next layer.
+inline ZeroWords kmax_words(const litevggt_ctx* ctx, long long sequences) {
+  return ZeroWords{reinterpret_cast<uint32_t*>(ctx->ws.attn_kmax), sequences * ctx->sz.heads};
+}
+
+// Before a call raises the key norms: they are zero unless an earlier call failed half-way.
+inline cudaError_t begin_norms(litevggt_ctx* ctx, cudaStream_t s) {
+  if (ctx->norms_left) {
+    const cudaError_t e = cudaMemsetAsync(ctx->ws.attn_kmax, 0, sizeof(float) * (size_t)ctx->sz.frames * ctx->sz.heads, s);
+    if (e != cudaSuccess) return e;
+  }
+  ctx->norms_left = true;  // until the output projection is enqueued
+  return cudaSuccess;
+}
+
+// What the global layer's attention core needs to know about Q, K and V before it starts.
+inline LinearStat core_stat(const litevggt_ctx* ctx, long long m) {
+  LinearStat st;
+  if (ctx->cfg.qkv_dtype == 1) {
+    st.amax = ctx->ws.qkv_amax;
+  } else {
+    st.key_norm = ctx->ws.attn_kmax;
+    st.seq_len = m;
+  }
+  return st;
+}
+
+}  // namespace lv

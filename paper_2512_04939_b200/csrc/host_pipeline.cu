@@ -1,0 +1,214 @@
+// The whole layer from and to host memory, call after call (litevggt_global_layer_host_pipelined): copies on the
+// context's own streams, double-buffered staging, and an output that leaves while the layer still computes.
+//
+// Device to host is what such a pass waits for longest: 90 MB at 32 frames of 37 x 37 take 1.65 ms of PCIe behind 1.9
+// ms of kernels.  A token's output needs one merged row, its own or its anchor's, so the attention runs in
+// slabs of query rows, and when a slab has been projected a kernel on the copy stream adds its rows to their
+// tokens' residuals and writes the tokens straight into the pinned buffer, under the next slab's
+// attention: 3.72 -> 2.66 to 2.83 ms a pass.  What bounds it now is PCIe, both ways at once (the next call's input comes in
+// meanwhile), at 45 GB/s out.  The first slab is one round of the attention's CTAs, so that PCIe starts early, the
+// others two, which lose 3 % of a round at their end.  Output buffers that the device cannot write (pageable memory, odd
+// addresses), E4M3 contexts, sequences of up to 4096 rows and those of several key chunks, whose copies are
+// 6 % of a pass or less, take the copy behind the layer.
+#include "host_common.h"
+
+using namespace lv;
+
+namespace {
+
+// Copy streams, events and the second pair of [N, D] staging buffers of the pipelined host entry.
+litevggt_status ensure_host_pipe(litevggt_ctx* ctx) {
+  litevggt_status st = ensure_staging(ctx);
+  if (st != LITEVGGT_OK) return st;
+  HostPipe& hp = ctx->pipe;
+  if (hp.created) return LITEVGGT_OK;
+  DeviceGuard g(ctx->device);
+  if (!g.ok) return LITEVGGT_ERR_CUDA;
+  const Sizes& z = ctx->sz;
+  const size_t big = (size_t)round_up(z.n_tokens * z.dim * 2, 256);
+  const size_t index = (size_t)(round_up(4 * z.n_tokens, 256) + 2 * round_up(4 * z.n_merged, 256) +
+                                round_up(4 * (z.n_merged + 1), 256) + round_up(4 * (z.n_remove + 1), 256));
+  if (cudaMalloc(&hp.extra, 2 * (big + index)) != cudaSuccess) {
+    (void)cudaGetLastError();
+    hp.extra = nullptr;
+    return LITEVGGT_ERR_ALLOC;
+  }
+  cudaError_t e = cudaStreamCreateWithFlags(&hp.copy_in, cudaStreamNonBlocking);
+  // ahead of the next kernels on the caller's stream, which wait for an SM of their own while these fit beside what runs
+  int least = 0, greatest = 0;
+  if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+  if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&hp.copy_out, cudaStreamNonBlocking, greatest);
+  cudaEvent_t* sets[4] = {hp.in_ready, hp.x_free, hp.out_ready, hp.out_free};
+  for (int k = 0; k < 4 && e == cudaSuccess; ++k)
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&sets[k][i], cudaEventDisableTiming);
+  if (e != cudaSuccess) {
+    // partial set-up is released at destroy time only if `created`; release it here instead
+    if (hp.copy_in) cudaStreamDestroy(hp.copy_in);
+    if (hp.copy_out) cudaStreamDestroy(hp.copy_out);
+    for (int k = 0; k < 4; ++k)
+      for (int i = 0; i < 2; ++i)
+        if (sets[k][i]) cudaEventDestroy(sets[k][i]);
+    cudaFree(hp.extra);
+    hp = HostPipe();
+    return cuda_status(e);
+  }
+  hp.x[0] = ctx->ws.stage_x;
+  hp.out[0] = ctx->ws.stage_out;
+  hp.x[1] = reinterpret_cast<__nv_bfloat16*>(hp.extra);
+  hp.out[1] = reinterpret_cast<__nv_bfloat16*>(hp.extra + big);
+  for (int i = 0; i < 2; ++i) hp.index[i] = reinterpret_cast<int*>(hp.extra + 2 * big + i * index);
+  ctx->ws.bytes += 2 * (big + index);
+  hp.created = true;
+  return LITEVGGT_OK;
+}
+
+// Where the device writes `bytes` of page-locked host memory, or nothing: 16-byte units must fit.
+void* device_view(void* host, size_t bytes) {
+  cudaPointerAttributes first, last;
+  if (cudaPointerGetAttributes(&first, host) != cudaSuccess ||
+      cudaPointerGetAttributes(&last, static_cast<uint8_t*>(host) + bytes - 1) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  if (first.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || first.devicePointer == nullptr ||
+      static_cast<uint8_t*>(last.devicePointer) - static_cast<uint8_t*>(first.devicePointer) != (ptrdiff_t)bytes - 1)
+    return nullptr;
+  return aligned16(first.devicePointer) ? first.devicePointer : nullptr;
+}
+
+// The attention layer and the unmerge in slabs of query rows, the finished tokens written to `out`.
+cudaError_t layer_in_slabs(litevggt_ctx* ctx, const litevggt_plan* plan, int slot, const void* w_qkv, const void* b_qkv, const void* w_o, const void* b_o, __nv_bfloat16* out, cudaStream_t s,
+                           bool* started) {
+  const Sizes& z = ctx->sz;
+  Workspace& ws = ctx->ws;
+  HostPipe& hp = ctx->pipe;
+  const long long m = z.n_merged;
+  const int d = z.dim;
+  int n = 0;
+  cudaError_t e = begin_norms(ctx, s);
+  if (e == cudaSuccess) {
+    StepTimer t(ctx, 6, n, e);
+    e = launch_linear_scaled(ctx, ws.stage_xm, m, d, static_cast<const __nv_bfloat16*>(w_qkv), 3 * d,
+                             static_cast<const __nv_bfloat16*>(b_qkv), d, 2 * d, kKeyScaleLog2e, core_stat(ctx, m), ws.qkv, s, &n);
+  }
+  // this slot's rows and indices may still be on their way out, two calls ago
+  if (e == cudaSuccess && hp.used[slot]) e = cudaStreamWaitEvent(s, hp.out_free[slot], 0);
+  // the writers' own copy of the indices: the plan may be rebuilt as soon as this call has returned
+  // (a plan's arrays lie in one allocation, in this order)
+  const size_t index_bytes = reinterpret_cast<uint8_t*>(plan->seg_src + z.n_remove) - reinterpret_cast<uint8_t*>(plan->dst_of);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(hp.index[slot], plan->dst_of, index_bytes, cudaMemcpyDeviceToDevice, s);
+  auto copied = [&](const int* array) { return hp.index[slot] + (array - plan->dst_of); };
+  __nv_bfloat16* ym = hp.out[slot];  // (the staged output is not needed: M <= N rows of it hold the merged ones)
+  for (long long row0 = 0, row1; row0 < m && e == cudaSuccess; row0 = row1) {
+    row1 = flash_attention_slab_end(ctx, m, row0);
+    {
+      StepTimer t(ctx, 7, n, e);
+      e = launch_flash_attention_rows(ctx, ws.qkv, m, row0, row1, ws.attn_o, s, &n);
+    }
+    if (e == cudaSuccess) {
+      StepTimer t(ctx, 8, n, e);
+      e = launch_linear(ctx, ws.attn_o + row0 * d, row1 - row0, d, static_cast<const __nv_bfloat16*>(w_o), d,
+                        static_cast<const __nv_bfloat16*>(b_o), row1 == m ? kmax_words(ctx, 1) : ZeroWords{}, ym + row0 * d, s, &n);
+    }
+    if (e == cudaSuccess) e = cudaEventRecord(hp.out_ready[slot], s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(hp.copy_out, hp.out_ready[slot], 0);
+    if (e == cudaSuccess) {
+      StepTimer t(ctx, 9, n, e);
+      e = launch_unmerge_rows(ctx, copied(plan->dst_of), copied(plan->kept_idx), copied(plan->seg_off), copied(plan->seg_src), ym,
+                              hp.x[slot], out, row0, row1, hp.copy_out, &n);
+      *started = true;
+    }
+  }
+  if (e == cudaSuccess) ctx->norms_left = false;
+  bump(ctx, n);
+  return e;
+}
+
+}  // namespace
+
+extern "C" {
+
+litevggt_status litevggt_global_layer_host_pipelined(litevggt_ctx* ctx, litevggt_plan** plan_inout, const float* grad,
+                                                     const void* x_host, const void* w_qkv, const void* b_qkv,
+                                                     const void* w_o, const void* b_o, void* out_host, void* stream) {
+  if (!ctx_ok(ctx) || plan_inout == nullptr || x_host == nullptr || out_host == nullptr) return LITEVGGT_ERR_NULL;
+  if (grad == nullptr) {
+    const litevggt_plan* plan = *plan_inout;
+    if (!plan_ok(plan) || plan->owner != ctx || !plan->built) return LITEVGGT_ERR_STALE_PLAN;
+  }
+  litevggt_status st = ensure_host_pipe(ctx);
+  if (st != LITEVGGT_OK) return st;
+  DeviceGuard g(ctx->device);
+  if (!g.ok) return LITEVGGT_ERR_CUDA;
+  const Sizes& z = ctx->sz;
+  Workspace& ws = ctx->ws;
+  HostPipe& hp = ctx->pipe;
+  cudaStream_t s = (cudaStream_t)stream;
+  const size_t bytes = (size_t)z.n_tokens * z.dim * 2;
+  const int slot = (int)(hp.calls & 1ull);
+  // copy-in stream: the buffer is free once the unmerge two calls ago has read its residual from it
+  cudaError_t e = cudaSuccess;
+  if (hp.used[slot]) e = cudaStreamWaitEvent(hp.copy_in, hp.x_free[slot], 0);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(hp.x[slot], x_host, bytes, cudaMemcpyHostToDevice, hp.copy_in);
+  if (e == cudaSuccess) e = cudaEventRecord(hp.in_ready[slot], hp.copy_in);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(s, hp.in_ready[slot], 0);
+  if (e != cudaSuccess) return cuda_status(e);
+  if (grad != nullptr) {
+    st = litevggt_merge_plan(ctx, hp.x[slot], grad, plan_inout, stream);
+    if (st != LITEVGGT_OK) return st;
+  }
+  const litevggt_plan* plan = *plan_inout;
+  st = litevggt_merge(ctx, plan, hp.x[slot], ws.stage_xm, stream);
+  const bool apart = ctx->cfg.qkv_dtype == 0 && flash_attention_slab_end(ctx, z.n_merged, 0) < z.n_merged;
+  void* direct = st == LITEVGGT_OK && apart ? device_view(out_host, bytes) : nullptr;
+  if (direct != nullptr) {
+    bool started = false;
+    // what a call's kernels check of their pointers; an argument they refuse stays refused
+    if (w_qkv == nullptr || w_o == nullptr) return LITEVGGT_ERR_NULL;
+    if (!aligned16(w_qkv) || !aligned16(w_o) || (b_qkv != nullptr && !aligned16(b_qkv)) || (b_o != nullptr && !aligned16(b_o)))
+      return LITEVGGT_ERR_ALIGN;
+    e = layer_in_slabs(ctx, plan, slot, w_qkv, b_qkv, w_o, b_o, static_cast<__nv_bfloat16*>(direct), s, &started);
+    if (started) {  // also where a later launch failed: what has begun still uses the slot
+      cudaError_t done = cudaEventRecord(hp.x_free[slot], hp.copy_out);
+      if (done == cudaSuccess) done = cudaEventRecord(hp.out_free[slot], hp.copy_out);
+      if (done == cudaSuccess) {
+        hp.used[slot] = true;
+        ++hp.calls;
+      }
+      if (e == cudaSuccess) e = done;
+    }
+    return cuda_status(e);
+  }
+  if (st == LITEVGGT_OK)
+    st = litevggt_global_attn(ctx, ws.stage_xm, z.n_merged, w_qkv, b_qkv, w_o, b_o, ws.stage_ym, stream);
+  if (st != LITEVGGT_OK) return st;
+  // the output buffer is free once the copy-out two calls ago has drained it
+  if (hp.used[slot]) e = cudaStreamWaitEvent(s, hp.out_free[slot], 0);
+  if (e != cudaSuccess) return cuda_status(e);
+  st = litevggt_unmerge(ctx, plan, ws.stage_ym, hp.x[slot], hp.out[slot], stream);
+  if (st != LITEVGGT_OK) return st;
+  e = cudaEventRecord(hp.out_ready[slot], s);
+  if (e == cudaSuccess) e = cudaEventRecord(hp.x_free[slot], s);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(hp.copy_out, hp.out_ready[slot], 0);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(out_host, hp.out[slot], bytes, cudaMemcpyDeviceToHost, hp.copy_out);
+  if (e == cudaSuccess) e = cudaEventRecord(hp.out_free[slot], hp.copy_out);
+  if (e == cudaSuccess) {
+    hp.used[slot] = true;
+    ++hp.calls;
+  }
+  return cuda_status(e);
+}
+
+litevggt_status litevggt_host_drain(litevggt_ctx* ctx, void* stream) {
+  if (!ctx_ok(ctx)) return LITEVGGT_ERR_NULL;
+  HostPipe& hp = ctx->pipe;
+  if (!hp.created) return LITEVGGT_OK;
+  DeviceGuard g(ctx->device);
+  if (!g.ok) return LITEVGGT_ERR_CUDA;
+  cudaError_t e = cudaSuccess;
+  for (int slot = 0; slot < 2 && e == cudaSuccess; ++slot)
+    if (hp.used[slot]) e = cudaStreamWaitEvent((cudaStream_t)stream, hp.out_free[slot], 0);
+  return cuda_status(e);
+}
+
+}  // extern "C"

@@ -129,6 +129,69 @@ unmerge_kernel(const __nv_bfloat16* __restrict__ ym, const int* __restrict__ dst
   }
 }
 
+// The unmerge of merged rows [row0, row1) only: to their own tokens and to the src tokens of their segments, into memory that
+// may be the host's.  PCIe bounds it (2 KB a token at about 50 GB/s), so few warps do; what matters is that they are all
+// busy to the end (a token each, not a row: some anchors stand for hundreds) and how they get on with the attention
+// beside them.  Its CTA leaves 1024 registers of every scheduler free: one block of four warps on 32 registers, a warp
+// half a token at a time.  Where stores queue up for PCIe the attention's warps on that SM wait behind them, so
+// the blocks are no more than it takes (pass of 32 frames of 37 x 37: 12 blocks 2.73 ms, 16: 2.71, 20: 2.69, 24: 2.66,
+// 32: 2.80, 48: 2.81; a slab's attention 355 us beside 16 of them, 380 beside 24, 480 beside 48).
+constexpr int kOutThreads = 128;
+constexpr int kOutBlocks = 24;
+__global__ void __launch_bounds__(kOutThreads, 16)
+unmerge_rows_kernel(const __nv_bfloat16* __restrict__ ym, const int* __restrict__ dst_of, const int* __restrict__ kept_idx,
+                    const int* __restrict__ seg_off, const int* __restrict__ seg_src, const __nv_bfloat16* __restrict__ residual,
+                    __nv_bfloat16* __restrict__ out, int row0, int row1, int n_tokens, int n_merged, int n_remove, uint32_t* status,
+                    Stamp stamp) {
+  const Span span(stamp);
+  const int lane = threadIdx.x & 31, step = gridDim.x * (kOutThreads / 32);
+  int first = seg_off[row0], last = seg_off[row1];
+  if (first < 0 || last < first || last > n_remove) {
+    if (threadIdx.x == 0) atomicOr(status, kStatusBounds);
+    first = last = 0;
+  }
+  const int rows = row1 - row0, count = rows + (last - first);
+  auto token_at = [&](int i) { return i >= count ? 0 : i < rows ? kept_idx[row0 + i] : seg_src[first + i - rows]; };
+  int i = blockIdx.x * (kOutThreads / 32) + (int)(threadIdx.x >> 5);
+  int ahead = token_at(i);
+  for (; i < count; i += step) {
+    const int token = ahead;
+    ahead = token_at(i + step);
+    const int row = token >= 0 && token < n_tokens ? dst_of[token] : -1;
+    if (row < 0 || row >= n_merged) {
+      if (lane == 0) atomicOr(status, kStatusBounds);
+      continue;
+    }
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+      const int at = half * 64 + lane;  // in 16-byte units
+      const uint4* rp = reinterpret_cast<const uint4*>(residual + (long long)token * 1024) + at;
+      const uint4* yp = reinterpret_cast<const uint4*>(ym + (long long)row * 1024) + at;
+      const uint4 r0 = rp[0], r1 = rp[32], y0 = yp[0], y1 = yp[32];
+      uint4* o = reinterpret_cast<uint4*>(out + (long long)token * 1024) + at;
+      auto sum = [](uint32_t a, uint32_t b) { return pack_bf16(bf16_lo(a) + bf16_lo(b), bf16_hi(a) + bf16_hi(b)); };
+      o[0] = make_uint4(sum(y0.x, r0.x), sum(y0.y, r0.y), sum(y0.z, r0.z), sum(y0.w, r0.w));
+      o[32] = make_uint4(sum(y1.x, r1.x), sum(y1.y, r1.y), sum(y1.z, r1.z), sum(y1.w, r1.w));
+    }
+  }
+}
+
+cudaError_t launch_unmerge_rows(const litevggt_ctx* ctx, const int* dst_of, const int* kept_idx, const int* seg_off,
+                                const int* seg_src, const __nv_bfloat16* ym, const __nv_bfloat16* residual, __nv_bfloat16* out,
+                                long long row0, long long row1, cudaStream_t s, int* launches) {
+  const Sizes& z = ctx->sz;
+  // Shared memory for whoever comes beside it: an SM that this kernel reaches first would be set up with little, and keep
+  // the attention's CTA away until it is done.
+  static std::atomic<unsigned long long> carveout_set{0};
+  const cudaError_t e = set_attribute_once(reinterpret_cast<const void*>(unmerge_rows_kernel), cudaFuncAttributePreferredSharedMemoryCarveout,
+                                           cudaSharedmemCarveoutMaxShared, carveout_set);
+  if (e != cudaSuccess) return e;
+  ++*launches;
+  return launch_clusters(1, false, unmerge_rows_kernel, dim3(kOutBlocks), kOutThreads, 0, s, ym, dst_of, kept_idx, seg_off, seg_src,
+                         residual, out, (int)row0, (int)row1, (int)z.n_tokens, (int)z.n_merged, (int)z.n_remove, ctx->ws.status,
+                         next_stamp(ctx));
+}
+
 // LayerNorm over the 1024 channels of every row (the pre-norm of the transformer blocks, Sec. 3.1):
 // y = (x - mean) / sqrt(var + eps) * gamma + beta, population variance, two passes over the row held
 // in registers, fp32, one rounding.  One warp per row like the kernels above.

@@ -27,17 +27,20 @@ struct Sizes {
 
 inline long long round_up(long long v, long long a) { return (v + a - 1) / a * a; }
 
-// Raises a kernel's dynamic shared-memory limit once per device (`done` holds one bit per device,
-// one object per kernel), so that a launcher's later calls only enqueue work.
-inline cudaError_t set_max_dynamic_smem_once(const void* kernel, int bytes, std::atomic<unsigned long long>& done) {
+// Sets an attribute of a kernel once per device (`done` holds one bit per device, one object per kernel), so that
+// a launcher's later calls only enqueue work.
+inline cudaError_t set_attribute_once(const void* kernel, cudaFuncAttribute attribute, int value, std::atomic<unsigned long long>& done) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const unsigned long long bit = 1ull << (dev & 63);
   if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  e = cudaFuncSetAttribute(kernel, attribute, value);
   if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
   return e;
+}
+inline cudaError_t set_max_dynamic_smem_once(const void* kernel, int bytes, std::atomic<unsigned long long>& done) {
+  return set_attribute_once(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes, done);
 }
 
 // The attention kernels take the exponentials in base 2 of scores that already carry the softmax
@@ -48,7 +51,7 @@ constexpr float kKeyScaleLog2e = 0.125f * 1.4426950408889634f;
 
 constexpr long long kMlpChunkRows = 131072;  // rows of the 4D-wide hidden activations held at a time (1 GiB)
 
-// one counter per launch of an attention core: the key chunks of at most 4 Mi keys
+// one counter per launch of an attention core: the key chunks of at most 4 Mi keys, or the slabs of one chunk
 constexpr int kAttnCounters = 64;
 
 // One device allocation carved into named regions.
@@ -122,7 +125,8 @@ struct HostPipe {
   unsigned long long calls = 0;
   __nv_bfloat16* x[2] = {nullptr, nullptr};    // [N, D] each
   __nv_bfloat16* out[2] = {nullptr, nullptr};  // [N, D] each
-  uint8_t* extra = nullptr;                     // allocation that holds x[1] and out[1]
+  int* index[2] = {nullptr, nullptr};          // a plan's arrays, as a call found them
+  uint8_t* extra = nullptr;                     // allocation that holds x[1], out[1] and both index
 };
 
 struct litevggt_ctx {
@@ -246,6 +250,11 @@ cudaError_t launch_merge(const litevggt_ctx* ctx, const litevggt_plan* plan, con
                          __nv_bfloat16* xm, cudaStream_t s, int* launches);
 cudaError_t launch_unmerge(const litevggt_ctx* ctx, const litevggt_plan* plan, const __nv_bfloat16* ym,
                            const __nv_bfloat16* residual, __nv_bfloat16* out, cudaStream_t s, int* launches);
+// merged rows [row0, row1) to all tokens that they stand for, residual added: out may be host memory.  The index arrays are
+// a plan's; the blocks fit beside the attention kernel's.
+cudaError_t launch_unmerge_rows(const litevggt_ctx* ctx, const int* dst_of, const int* kept_idx, const int* seg_off,
+                                const int* seg_src, const __nv_bfloat16* ym, const __nv_bfloat16* residual, __nv_bfloat16* out,
+                                long long row0, long long row1, cudaStream_t s, int* launches);
 
 // linear.cu
 cudaError_t launch_linear(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k, const __nv_bfloat16* w,
@@ -289,6 +298,11 @@ cudaError_t launch_qk_embed(const litevggt_ctx* ctx, __nv_bfloat16* qkv, const i
 // K last: the projection or qk_embed)
 cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long seq_len, int n_seq,
                                    __nv_bfloat16* o, cudaStream_t s, int* launches);
+// The same for a slab of the one sequence's m query rows: rows [row0, row1) with row1 = flash_attention_slab_end(row0), which is m at
+// once for a sequence that is not to be taken apart.
+long long flash_attention_slab_end(const litevggt_ctx* ctx, long long m, long long row0);
+cudaError_t launch_flash_attention_rows(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long m, long long row0, long long row1,
+                                        __nv_bfloat16* o, cudaStream_t s, int* launches);
 size_t attention_state_bytes(long long m, int dim, int heads, int num_sms, size_t* ml_offset);
 // E4M3 variant: quantised copies of Q, K, V by the per-head magnitudes in ctx->ws.qkv_amax - taken from
 // qkv here first unless the projection has left them there - (fp8_quant.cu), then the attention core on

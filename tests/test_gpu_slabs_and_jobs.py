@@ -1,4 +1,5 @@
-"""Attention CTAs that work off several jobs and the ranks of a small frame's scores, at the sizes where each can go wrong."""
+"""Attention CTAs that work off several jobs, the layer that leaves for host memory slab by slab, and the ranks of a
+small frame's scores, at the sizes where each can go wrong."""
 import numpy as np
 import pytest
 import torch
@@ -63,6 +64,49 @@ def test_sequences_of_several_rounds_of_jobs(lib, frames, grid, sharpness):
     rows = np.r_[0:4, t - 70:t]
     for f in range(frames):
         _check_core(f"frame core {f} of {frames}, {t} rows, sharpness {sharpness}", out[f * t + rows], qkv[f * t:(f + 1) * t], rows)
+    ctx.close()
+
+
+@pytest.mark.parametrize("frames,grid,ratio", [
+    (3, (37, 37), 0.0),    # 4,122 rows: the fewest that leave in slabs, two of them
+    (5, (37, 37), 0.3),    # a second slab of two rounds, not full
+    (9, (37, 37), 0.45),   # anchors of the first frame that stand for many tokens
+    (16, (37, 28), 0.42)])  # several whole slabs
+def test_output_that_leaves_in_slabs(lib, frames, grid, ratio):
+    """Calls in a row, the plan rebuilt in place right behind each: every output is the ordered entry's for the plan
+    the call was given (jobs of the last round are split elsewhere: one rounding of y and one of the output apart),
+    also into pageable memory and at an address that 16-byte stores do not fit."""
+    ctx = lib.LiteVGGT(frames, grid[0], grid[1], ratio)
+    n = ctx.n_tokens
+    w = [v.cuda() for v in make_attention_weights(WORKLOADS["C1"], 2)]
+    g = torch.Generator().manual_seed(n)
+    grads = [torch.rand(frames, *grid, generator=g).cuda() for _ in range(3)]
+    xs = [_tokens(n, n + i).pin_memory() for i in range(3)]
+    expected = []
+    plan = None
+    for x, grad in zip(xs, grads):
+        out = torch.empty_like(x).pin_memory()
+        plan = ctx.global_layer_host(plan, x, *w, out, grad=grad)
+        ctx.poll()
+        expected.append(out)
+    odd = torch.zeros(n * 1024 + 1, dtype=torch.bfloat16).pin_memory()[1:].view(n, 1024)
+    outs = [torch.zeros_like(xs[0]).pin_memory(), odd, torch.zeros_like(xs[0])]
+    for order in ((0, 1, 2), (2, 0, 1)):
+        for x, grad, k in zip(xs, grads, order):
+            outs[k].zero_()
+            ctx.global_layer_host_pipelined(plan, x, *w, outs[k], grad=grad)
+            if outs[k].is_pinned():
+                ctx.merge_plan(_tokens(n, 7).cuda(), grads[0], plan)  # what is still on its way keeps the plan it had
+        ctx.host_drain()
+        ctx.poll()
+        for i, k in enumerate(order):
+            got, ref = outs[k].float(), expected[i].float()
+            gap = (got - ref).abs()
+            # a bf16 unit of either value, and of the attention output before the residual was added
+            unit = 2.0 ** -7 * torch.maximum(ref.abs(), (ref - xs[i].float()).abs())
+            assert bool((gap <= 2 * unit + 1e-3).all()), f"call {i}: {gap.max()}"
+            assert float((gap != 0).float().mean()) < 0.2
+    plan.destroy()
     ctx.close()
 
 
