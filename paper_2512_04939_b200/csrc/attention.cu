@@ -10,8 +10,8 @@
 // 128) tiles and not for an even number of them.  What a sequence of 1041 rows (a 28 x 37 frame) spends
 // outside its nine key tiles bounded it; the frame-local layer of 200 such frames, projections
 // included, went from 3.09 to 2.58 ms.  The pair of tiles reads every K/V tile once for 256 rows and
-// is the faster one when the sweep is longer: 286 us (one tile) against 279 at 8.3 K rows, 80 each at
-// 4.2 K.  Warp roles of the pair (19 warps):
+// is the faster one when the sweep is longer: 41 us (one tile) against 49 at 2.6 K rows, 67 each at 3.6 K, 121 against 118
+// at 5.2 K.  Warp roles of the pair (19 warps):
 //   warps 0-15  softmax.  Warp w works on query tile t = w / 8 and TMEM lane quarter w % 4 (one
 //               thread = one query row); the two warps of a (tile, quarter), c = (w / 4) % 2, either
 //               take every other step whole or share each, 32 of its 64 scores per row and warp
@@ -90,12 +90,12 @@
 // between the tensor core's scores and the exponential.
 // Rows with larger B need a reference other than zero, but seldom a running one: the largest score s0
 // among the first 64 keys bounds the row maximum from below as B does from above, and wherever a
-// whole number m lies close enough to both (kFaShiftUp, fa_shift_down) it serves the whole sweep - the
+// whole number m lies close enough to both (fa_shift_up, fa_shift_down) it serves the whole sweep - the
 // shifted form, at the cost of a subtraction or a clamp per score, both of which the bound spares the
 // fixed form.  Trained projections attend that sharply (query weights x 16 on the generator's tokens:
 // B up to 213): 31,751 rows went from 4.81 to 4.41 ms there.
 // What remains takes the online form: base-2 softmax with a lazily updated reference
-// maximum, the running output rescaled only when a row maximum grows by more than 2^8 over the
+// maximum, the running output rescaled only when a row maximum grows by more than 2^32 over the
 // reference (the threads then first wait until the tile's last P V has retired).  All three equal
 // the plain softmax up to rounding.
 #include <type_traits>
@@ -111,7 +111,9 @@ constexpr int kFaThreads = (kFaSoftmaxWarps + 3) * 32;
 constexpr int kFaTileBytes = kFaTileKeys * 64 * 2;
 constexpr int kFaOnesBytes = 16 * 128;  // 16 key rows of the ones column block
 constexpr uint32_t kFaOCols = 80;  // 64 output channels, the row sum, 15 unused columns
-constexpr float kFaRescaleThreshold = 8.0f;
+// How far a row maximum may grow over the reference of the online form before the row is rescaled.  Probabilities up to 2^32 lose
+// nothing (sums over 2^22 keys times |v| <= 2^20 stay below 2^74); a warp rescales when one of its 32 rows has to.
+constexpr float kFaRescaleThreshold = 32.0f;
 // Largest Cauchy-Schwarz bound B on the base-2 scores of a row for which the fixed reference is
 // used.  With the reference left out the probabilities lie in [2^-B, 2^B]: at B = 80 their products
 // with |v| >= 2^-20 are normal fp32 numbers (>= 2^-100), and a row sum over 2^20 keys times
@@ -138,17 +140,20 @@ constexpr int kFaPolyPairs = LV_FA_POLY_PAIRS;
 #define LV_FA_SHIFT_POLY_PAIRS 2
 #endif
 constexpr int kFaShiftPolyPairs = LV_FA_SHIFT_POLY_PAIRS;
-// Shifted reference m of a row with score bound B and a known score s0.  B - m <= kFaShiftUp: row sums over the 2^22
-// keys that a sequence may have, times |v| <= 2^20, stay below 2^126.  m - s0 <= fa_shift_down(keys): what lies more
-// than 126 under m is off by up to 2^-126 a key (flushed to zero by the special-function unit, held up at
+// Shifted reference m of a row with score bound B and a known score s0, both limits by the sequence's length.  B - m <=
+// fa_shift_up(keys): row sums over that many keys, times |v| <= 2^20, stay below 2^126.  m - s0 <= fa_shift_down(keys): what
+// lies more than 126 under m is off by up to 2^-126 a key (flushed to zero by the special-function unit, held up at
 // 2^-126 by the polynomial's clamp), the row's largest probability is at least 2^-fa_shift_down, so all such keys
-// together are off by 2^-24 of the row's mass at most - no more than one fp32 rounding of the row sum.
-constexpr float kFaShiftUp = 84.0f;
-static float fa_shift_down(long long keys) {
+// together are off by 2^-24 of the row's mass at most - no more than one fp32 rounding of the row sum.  (With 84 up, the
+// limit of 2^22 keys, at every length, a seventh of the 256-row tiles of 31,751 rows at query weights x 16 had a row in
+// the online form, a tenth with 91: 4.53 -> 4.49 ms.)
+static float key_bits(long long keys) {
   int bits = 0;
   while ((1ll << bits) < keys) ++bits;
-  return (float)(126 - 24 - bits);
+  return (float)bits;
 }
+static float fa_shift_up(long long keys) { return 126.0f - 20.0f - key_bits(keys); }
+static float fa_shift_down(long long keys) { return 126.0f - 24.0f - key_bits(keys); }
 // Sequences of at most this many rows take CTAs of one query tile, two to an SM (figures at the top).
 #ifndef LV_FA_ONE_TILE_ROWS
 #define LV_FA_ONE_TILE_ROWS 4096
@@ -345,8 +350,8 @@ __device__ __forceinline__ float max32(const uint32_t (&s)[32]) {
   return fmaxf(fmax3(mx[0], mx[1], mx[2]), mx[3]);
 }
 
-// The two warps of one (tile, lane quarter).  A warp that gives up arrives once more without waiting, so a partner who comes to
-// the barrier passes it - and then finds the abort flag up and gives up too.
+// The two warps of one (tile, lane quarter).  A warp that gives up arrives once more without waiting, so a partner who is at
+// the barrier, or comes to it, passes - and finds the abort flag up before the next one.
 __device__ __forceinline__ void pair_barrier(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
 __device__ __forceinline__ void pair_barrier_leave(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
 
@@ -356,7 +361,7 @@ template <int kTiles, bool kFirst, bool kLast>
 __global__ void __launch_bounds__(FaShape<kTiles>::kThreads, kTiles == 2 ? 1 : 2)
 flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_bfloat16* __restrict__ qkv,
                        __nv_bfloat16* __restrict__ o, float* __restrict__ o_state, float* __restrict__ ml_state,
-                       const float* __restrict__ k_norm2_max, float shift_down, int seq_len, int dim, int tile_begin,
+                       const float* __restrict__ k_norm2_max, float shift_up, float shift_down, int seq_len, int dim, int tile_begin,
                        int tile_end, FaJobs jobs, uint32_t* status, Stamp stamp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -649,10 +654,9 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       return id;
     };
     const int barrier_id = 1 + t * 4 + (int)quarter;
-    auto meet = [&]() -> bool {
-      pair_barrier(barrier_id);
-      return __all_sync(0xffffffffu, *ctl.abort_flag == 0u ? 1 : 0) != 0;
-    };
+    // Asked for in good time before a pair barrier, not behind it: who is passed through by a warp that gave up finds out
+    // before the next one.
+    auto given_up = [&] { return *ctl.abort_flag != 0u; };  // (one read for the whole warp)
     int id = next_job(id0);
     float score_bound = 0.0f;
     if (id < id_end) {
@@ -753,15 +757,17 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
           tmem_ld_wait();
           masked(s, n_keys - c * 32);
           const float mx_own = max32(s);
+          ok = !given_up();
+          if (!ok) break;
           pairs->first_max[t][c][row_in_tile] = mx_own;
-          ok = meet();
+          pair_barrier(barrier_id);
           const float mx_first = fmaxf(mx_own, pairs->first_max[t][c ^ 1][row_in_tile]);
-          const float m = ceilf(fmaxf(score_bound - kFaShiftUp, mx_first));
+          const float m = ceilf(fmaxf(score_bound - shift_up, mx_first));
           shifted = __all_sync(0xffffffffu, m - mx_first <= shift_down && fabsf(m) <= 1048576.0f ? 1 : 0) != 0;
           if (shifted) m_ref = m;
         }
         if (ok && shifted) {
-          // ---- shifted reference, kept for the whole launch: a whole number m (see kFaShiftUp) under which
+          // ---- shifted reference, kept for the whole launch: a whole number m (see fa_shift_up) under which
           // nothing overflows and the row's largest probability is not small, so no running maximum is
           // needed.
           const float m = m_ref;
@@ -774,6 +780,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
           auto step = [&](int j, int h, bool may_mask) -> bool {
             if (!scores_of(h, j)) return false;
             tc_fence_after();
+            const bool gone = given_up();
             const uint32_t addr = s_addr + h * 64 + c * 32;
             // (the scores are read once for the maximum and once more for the exponentials: the registers that this form
             // takes are the kernel's)
@@ -789,7 +796,8 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
               mx_own = max32(s);
             }
             pairs->row_max[h][t][c][row_in_tile] = mx_own;
-            if (!meet()) return false;
+            if (gone) return false;
+            pair_barrier(barrier_id);
             const float mx = fmaxf(mx_own, pairs->row_max[h][t][c ^ 1][row_in_tile]);
             if ((j | h) == 0) {
               m_ref = mx;
@@ -1430,7 +1438,7 @@ static cudaError_t launch_rows(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long
   CUtensorMap tmap;
   if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap, qkv, (uint64_t)3 * dim, (uint64_t)rows, (uint64_t)3 * dim, 64, kFaTileKeys))
     return cudaErrorInvalidValue;
-  using Kernel = void (*)(const CUtensorMap, const __nv_bfloat16*, __nv_bfloat16*, float*, float*, const float*, float, int,
+  using Kernel = void (*)(const CUtensorMap, const __nv_bfloat16*, __nv_bfloat16*, float*, float*, const float*, float, float, int,
                           int, int, int, FaJobs, uint32_t*, Stamp);
   // [query tiles of a CTA - 1][first chunk][last chunk]
   const Kernel kernels[2][2][2] = {
@@ -1466,7 +1474,7 @@ static cudaError_t launch_rows(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long
                                               smem_set[a][b][c]);
     if (e != cudaSuccess) return e;
     e = launch_clusters(1, early, kernels[a][b][c], grid, threads, smem, s, tmap, qkv, o, ctx->ws.attn_o_state, ctx->ws.attn_ml_state,
-               ctx->ws.attn_kmax, fa_shift_down(seq_len), (int)seq_len, dim, begin, end, split, ctx->ws.status, next_stamp(ctx));
+               ctx->ws.attn_kmax, fa_shift_up(seq_len), fa_shift_down(seq_len), (int)seq_len, dim, begin, end, split, ctx->ws.status, next_stamp(ctx));
     if (e != cudaSuccess) return e;
     ++*launches;
     ++split.taken;

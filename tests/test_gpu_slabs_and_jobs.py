@@ -5,7 +5,7 @@ import pytest
 import torch
 
 import oracle as O
-from helpers import check_bf16, to_f64, unfold_k
+from helpers import K_FOLD, check_bf16, to_f64, unfold_k
 from synthdata import WORKLOADS, make_attention_weights
 
 pytestmark = pytest.mark.gpu
@@ -123,4 +123,44 @@ def test_ranks_of_a_small_frames_scores(lib, grid, keep):
     ex = ctx.plan_export(plan)
     assert np.array_equal(ex["cls"], O.partition(ex["ga"], ga_keep_frac=keep))
     plan.destroy()
+    ctx.close()
+
+
+@pytest.mark.parametrize("above", [88.5, 95.0, 97.5])
+def test_reference_that_serves_a_whole_sweep_at_its_limits(lib, above):
+    """16,384 rows: one reference serves score bounds up to 92 over it, and a known score up to 88 under it.  Keys 0 and 1
+    score 0, the highest; key 1 is long, across the queries, so that the bound lies 84 + `above` over it: under 96 the reference
+    serves, above the running maximum has to.  The other keys sit 40 binades down with V = 1 where keys 0 and 1
+    have V = 0: the output is what they hold together, 2^-27, and an error of 2^-24 of the row's mass is allowed."""
+    rows = 16384
+    ctx = lib.LiteVGGT(4, 64, 64, 0.0, n_special=0)
+    assert ctx.n_merged == rows
+    x, w_qkv, b_qkv, w_o, b_o = (torch.zeros(*s, dtype=torch.bfloat16) for s in ((rows, 1024), (3072, 1024), (3072,), (1024, 1024), (1024,)))
+    x[2:, 0], x[1, 1], x[2:, 2] = -40.0 / 16 / K_FOLD, (84 + above) / 16 / K_FOLD, 1.0
+    for h in range(16):
+        b_qkv[64 * h] = 16.0
+        w_qkv[1024 + 64 * h, 0] = w_qkv[1024 + 64 * h + 1, 1] = w_qkv[2048 + 64 * h, 2] = 1.0
+    ctx.global_attn(x.cuda(), w_qkv.cuda(), b_qkv.cuda(), w_o.cuda(), b_o.cuda())
+    ctx.poll()
+    out = to_f64(ctx.debug_buffer(1))[:, ::64]
+    assert np.isfinite(out).all() and np.abs(out - (rows - 2) * 2.0 ** -41).max() <= 2.0 ** -24
+    ctx.close()
+
+
+@pytest.mark.parametrize("bound", [170.0, 179.0, 185.0])
+def test_reference_far_below_the_scores_does_not_overflow(lib, bound):
+    """16,384 rows whose first 64 keys score 0 and all others `bound`, the largest that the lengths allow: the reference
+    lies 92 under them (or is a running one, above 180), their probabilities of 2^92 and values of 2^20 add up to 2^126
+    before the division, and the output is 2^20."""
+    rows = 16384
+    ctx = lib.LiteVGGT(4, 64, 64, 0.0, n_special=0)
+    x, w_qkv, b_qkv, w_o, b_o = (torch.zeros(*s, dtype=torch.bfloat16) for s in ((rows, 1024), (3072, 1024), (3072,), (1024, 1024), (1024,)))
+    x[64:, 0], x[64:, 2] = bound / 16 / K_FOLD, 2.0 ** 20
+    for h in range(16):
+        b_qkv[64 * h] = 16.0
+        w_qkv[1024 + 64 * h, 0] = w_qkv[2048 + 64 * h, 2] = 1.0
+    ctx.global_attn(x.cuda(), w_qkv.cuda(), b_qkv.cuda(), w_o.cuda(), b_o.cuda())
+    ctx.poll()
+    out = to_f64(ctx.debug_buffer(1))[:, ::64]
+    assert np.isfinite(out).all() and np.abs(out / 2.0 ** 20 - 1).max() <= 2.0 ** -8
     ctx.close()
