@@ -246,8 +246,8 @@ litevggt_status litevggt_global_layer_host(litevggt_ctx* ctx, litevggt_plan** pl
  *   - Where out_host is page-locked and 16-byte aligned, tokens may be written to it as soon as their rows are
  *     done, in any order.  The attention's rows are then shared out differently over the chip than in
  *     litevggt_global_layer_host, whose results this call's equal up to rounding.
- *   - The first call allocates the second pair of staging buffers (2 x N x D bf16) and creates the
- *     streams and events. */
+ *   - The first call allocates two pairs of staging buffers (4 x N x D bf16 in all; the plain entry point has
+ *     buffers of its own, so calls of either may follow one another) and creates the streams and events. */
 litevggt_status litevggt_global_layer_host_pipelined(litevggt_ctx* ctx, litevggt_plan** plan_inout,
                                                      const float* grad, const void* x_host,
                                                      const void* w_qkv, const void* b_qkv,

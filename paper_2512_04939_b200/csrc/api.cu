@@ -328,9 +328,10 @@ litevggt_status litevggt_destroy(litevggt_ctx* ctx) {
       cudaEventDestroy(ctx->pipe.out_ready[i]);
       cudaEventDestroy(ctx->pipe.out_free[i]);
     }
-    if (ctx->pipe.extra != nullptr) cudaFree(ctx->pipe.extra);
+    cudaFree(ctx->pipe.base);
   }
   if (ctx->ws.stage_x != nullptr) cudaFree(ctx->ws.stage_x);
+  if (ctx->ws.stage_xm != nullptr) cudaFree(ctx->ws.stage_xm);
   if (ctx->ws.blk_qkv != nullptr) cudaFree(ctx->ws.blk_qkv);
   if (ctx->ws.base != nullptr) cudaFree(ctx->ws.base);
   (void)cudaGetLastError();
@@ -652,7 +653,8 @@ litevggt_status litevggt_global_layer_host(litevggt_ctx* ctx, litevggt_plan** pl
     const litevggt_plan* plan = *plan_inout;
     if (!plan_ok(plan) || plan->owner != ctx || !plan->built) return LITEVGGT_ERR_STALE_PLAN;
   }
-  litevggt_status st = ensure_staging(ctx);
+  litevggt_status st = ensure_merged_staging(ctx);
+  if (st == LITEVGGT_OK) st = ensure_row_pair(ctx, ctx->sz.n_tokens, &ctx->ws.stage_x, &ctx->ws.stage_out);
   if (st != LITEVGGT_OK) return st;
   const Sizes& z = ctx->sz;
   Workspace& ws = ctx->ws;

@@ -51,25 +51,25 @@ inline litevggt_status cuda_status(cudaError_t e) {
   return e == cudaErrorMemoryAllocation ? LITEVGGT_ERR_ALLOC : LITEVGGT_ERR_CUDA;
 }
 
-inline litevggt_status ensure_staging(litevggt_ctx* ctx) {
-  if (ctx->ws.stage_x != nullptr) return LITEVGGT_OK;
-  const Sizes& z = ctx->sz;
+// Two buffers of `rows` token rows in one allocation, whose address is the first one's; once per context.
+inline litevggt_status ensure_row_pair(litevggt_ctx* ctx, long long rows, __nv_bfloat16** first, __nv_bfloat16** second) {
+  if (*first != nullptr) return LITEVGGT_OK;
   DeviceGuard g(ctx->device);
   if (!g.ok) return LITEVGGT_ERR_CUDA;
-  const size_t big = (size_t)z.n_tokens * z.dim * 2, small = (size_t)z.n_merged * z.dim * 2;
+  const size_t each = (size_t)round_up(rows * ctx->sz.dim * 2, 256);
   uint8_t* base = nullptr;
-  const size_t total = 2 * (size_t)round_up((long long)big, 256) + 2 * (size_t)round_up((long long)small, 256);
-  if (cudaMalloc(&base, total) != cudaSuccess) {
+  if (cudaMalloc(&base, 2 * each) != cudaSuccess) {
     (void)cudaGetLastError();
     return LITEVGGT_ERR_ALLOC;
   }
-  size_t off = 0;
-  ctx->ws.stage_x = reinterpret_cast<__nv_bfloat16*>(base + off); off += (size_t)round_up((long long)big, 256);
-  ctx->ws.stage_out = reinterpret_cast<__nv_bfloat16*>(base + off); off += (size_t)round_up((long long)big, 256);
-  ctx->ws.stage_xm = reinterpret_cast<__nv_bfloat16*>(base + off); off += (size_t)round_up((long long)small, 256);
-  ctx->ws.stage_ym = reinterpret_cast<__nv_bfloat16*>(base + off);
-  ctx->ws.bytes += total;
+  *first = reinterpret_cast<__nv_bfloat16*>(base);
+  *second = reinterpret_cast<__nv_bfloat16*>(base + each);
+  ctx->ws.bytes += 2 * each;
   return LITEVGGT_OK;
+}
+// The layer's input and output in merged rows, which both host entries use in the order of the caller's stream.
+inline litevggt_status ensure_merged_staging(litevggt_ctx* ctx) {
+  return ensure_row_pair(ctx, ctx->sz.n_merged, &ctx->ws.stage_xm, &ctx->ws.stage_ym);
 }
 
 // The key norms of `sequences` sequences, which an output projection leaves zero for the next layer.

@@ -16,9 +16,11 @@ using namespace lv;
 
 namespace {
 
-// Copy streams, events and the second pair of [N, D] staging buffers of the pipelined host entry.
+// Copy streams, events and both pairs of [N, D] staging buffers of the pipelined host entry.  None of them is the ordered
+// entry's: that one overwrites its own on the caller's stream, where nothing waits for what a pipelined call has left to
+// the copy streams - and a wait for their events would not go into a graph that captures the ordered entry.
 litevggt_status ensure_host_pipe(litevggt_ctx* ctx) {
-  litevggt_status st = ensure_staging(ctx);
+  litevggt_status st = ensure_merged_staging(ctx);
   if (st != LITEVGGT_OK) return st;
   HostPipe& hp = ctx->pipe;
   if (hp.created) return LITEVGGT_OK;
@@ -28,9 +30,9 @@ litevggt_status ensure_host_pipe(litevggt_ctx* ctx) {
   const size_t big = (size_t)round_up(z.n_tokens * z.dim * 2, 256);
   const size_t index = (size_t)(round_up(4 * z.n_tokens, 256) + 2 * round_up(4 * z.n_merged, 256) +
                                 round_up(4 * (z.n_merged + 1), 256) + round_up(4 * (z.n_remove + 1), 256));
-  if (cudaMalloc(&hp.extra, 2 * (big + index)) != cudaSuccess) {
+  if (cudaMalloc(&hp.base, 2 * (2 * big + index)) != cudaSuccess) {
     (void)cudaGetLastError();
-    hp.extra = nullptr;
+    hp.base = nullptr;
     return LITEVGGT_ERR_ALLOC;
   }
   cudaError_t e = cudaStreamCreateWithFlags(&hp.copy_in, cudaStreamNonBlocking);
@@ -48,16 +50,17 @@ litevggt_status ensure_host_pipe(litevggt_ctx* ctx) {
     for (int k = 0; k < 4; ++k)
       for (int i = 0; i < 2; ++i)
         if (sets[k][i]) cudaEventDestroy(sets[k][i]);
-    cudaFree(hp.extra);
+    cudaFree(hp.base);
     hp = HostPipe();
     return cuda_status(e);
   }
-  hp.x[0] = ctx->ws.stage_x;
-  hp.out[0] = ctx->ws.stage_out;
-  hp.x[1] = reinterpret_cast<__nv_bfloat16*>(hp.extra);
-  hp.out[1] = reinterpret_cast<__nv_bfloat16*>(hp.extra + big);
-  for (int i = 0; i < 2; ++i) hp.index[i] = reinterpret_cast<int*>(hp.extra + 2 * big + i * index);
-  ctx->ws.bytes += 2 * (big + index);
+  for (int i = 0; i < 2; ++i) {
+    uint8_t* slot = hp.base + i * (2 * big + index);
+    hp.x[i] = reinterpret_cast<__nv_bfloat16*>(slot);
+    hp.out[i] = reinterpret_cast<__nv_bfloat16*>(slot + big);
+    hp.index[i] = reinterpret_cast<int*>(slot + 2 * big);
+  }
+  ctx->ws.bytes += 2 * (2 * big + index);
   hp.created = true;
   return LITEVGGT_OK;
 }

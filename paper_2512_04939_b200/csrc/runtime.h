@@ -86,10 +86,10 @@ struct Workspace {
   uint8_t* v8t = nullptr;          // [D, round_up(M, 128)] bytes: V transposed, head-major rows
   float* qkv_amax = nullptr;       // [3, heads] largest magnitude of Q, K, V per head
   // whole-layer-from-host staging
-  __nv_bfloat16* stage_x = nullptr;   // [N, D]
+  __nv_bfloat16* stage_x = nullptr;   // [N, D], the ordered entry's
+  __nv_bfloat16* stage_out = nullptr; // [N, D], behind it
   __nv_bfloat16* stage_xm = nullptr;  // [M, D]
-  __nv_bfloat16* stage_ym = nullptr;  // [M, D]
-  __nv_bfloat16* stage_out = nullptr; // [N, D]
+  __nv_bfloat16* stage_ym = nullptr;  // [M, D], behind it
   // block workspace of the frame-local attention and the MLP (allocated on first use)
   __nv_bfloat16* blk_qkv = nullptr;   // [N, 3D]
   __nv_bfloat16* blk_o = nullptr;     // [N, D]
@@ -116,7 +116,7 @@ struct Timers {
 };
 }  // namespace lv
 
-// Streams, events and the second pair of staging buffers behind litevggt_global_layer_host_pipelined.
+// Streams, events and staging buffers behind litevggt_global_layer_host_pipelined.
 struct HostPipe {
   bool created = false;
   cudaStream_t copy_in = nullptr, copy_out = nullptr;
@@ -126,7 +126,7 @@ struct HostPipe {
   __nv_bfloat16* x[2] = {nullptr, nullptr};    // [N, D] each
   __nv_bfloat16* out[2] = {nullptr, nullptr};  // [N, D] each
   int* index[2] = {nullptr, nullptr};          // a plan's arrays, as a call found them
-  uint8_t* extra = nullptr;                     // allocation that holds x[1], out[1] and both index
+  uint8_t* base = nullptr;                      // allocation that holds them all
 };
 
 struct litevggt_ctx {

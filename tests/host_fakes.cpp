@@ -1,10 +1,11 @@
 // Stand-ins for the CUDA runtime and for the kernel launchers, so that the host side of the library (api.cu,
-// attn_static.cu) can be linked and driven without a GPU.  "Device" memory is host memory; launchers only
+// attn_static.cu, host_pipeline.cu) can be linked and driven without a GPU.  "Device" memory is host memory; launchers only
 // do what the host code can see: count, note, and fail where the test asks for it.
 #include <stdlib.h>
 #include <string.h>
 
 #include <functional>
+#include <map>
 #include <vector>
 
 #include "../paper_2512_04939_b200/csrc/runtime.h"
@@ -25,6 +26,54 @@ static void finish_default_stream() {
   g_default_stream.clear();
 }
 extern "C" int fake_default_stream_pending() { return (int)g_default_stream.size(); }
+
+// Which memory the work on a stream touches, and what of it nothing orders: a vector clock per stream, joined
+// where a stream waits for an event and where the host has waited for a stream.
+using Clock = std::map<const void*, long>;
+struct Access {
+  const char *begin, *end;
+  bool writes;
+  const void* stream;
+  long time;
+};
+static std::map<const void*, Clock> g_stream_clocks;
+static std::map<const void*, Clock> g_events;
+static Clock g_host_clock;
+static std::vector<Access> g_accesses;
+static int g_races = 0;
+static void join(Clock& to, const Clock& from) {
+  for (const auto& c : from)
+    if (to[c.first] < c.second) to[c.first] = c.second;
+}
+static Clock& clock_of(cudaStream_t s) {
+  Clock& c = g_stream_clocks[s];
+  join(c, g_host_clock);
+  return c;
+}
+struct Range {
+  const void* p;
+  long long bytes;
+};
+static void touch(cudaStream_t s, std::vector<Range> reads, std::vector<Range> writes) {
+  Clock& now = clock_of(s);
+  const long time = ++now[s];
+  for (int w = 0; w < 2; ++w)
+    for (const Range& r : w ? writes : reads) {
+      if (r.p == nullptr || r.bytes <= 0) continue;
+      const Access a{static_cast<const char*>(r.p), static_cast<const char*>(r.p) + r.bytes, w == 1, s, time};
+      for (const Access& b : g_accesses)
+        if (b.begin < a.end && a.begin < b.end && (a.writes || b.writes) && now[b.stream] < b.time) ++g_races;
+      g_accesses.push_back(a);
+    }
+}
+extern "C" int fake_races() { return g_races; }
+extern "C" void fake_forget_accesses() {
+  g_stream_clocks.clear();
+  g_events.clear();
+  g_host_clock.clear();
+  g_accesses.clear();
+  g_races = 0;
+}
 
 // ---- CUDA runtime
 extern "C" {
@@ -51,18 +100,42 @@ cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
   memcpy(d, s, n);
   return cudaSuccess;
 }
-cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) { memcpy(d, s, n); return cudaSuccess; }
-cudaError_t cudaDeviceSynchronize() { finish_default_stream(); return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t s) {
-  if (s == nullptr) finish_default_stream();
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t stream) {
+  touch(stream, {{s, (long long)n}}, {{d, (long long)n}});
+  memcpy(d, s, n);
   return cudaSuccess;
 }
-cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = reinterpret_cast<cudaStream_t>(64); return cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() {
+  finish_default_stream();
+  for (const auto& c : g_stream_clocks) join(g_host_clock, c.second);
+  return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+  if (s == nullptr) finish_default_stream();
+  join(g_host_clock, clock_of(s));
+  return cudaSuccess;
+}
+static long long g_handles = 64;  // streams and events
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = reinterpret_cast<cudaStream_t>(g_handles++); return cudaSuccess; }
+cudaError_t cudaStreamCreateWithPriority(cudaStream_t* s, unsigned, int) { return cudaStreamCreateWithFlags(s, 0); }
+cudaError_t cudaDeviceGetStreamPriorityRange(int* least, int* greatest) { *least = 0; *greatest = -5; return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
-cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { *e = nullptr; return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
+  join(clock_of(s), g_events[e]);
+  return cudaSuccess;
+}
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { *e = reinterpret_cast<cudaEvent_t>(g_handles++); return cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
+  g_events[e] = clock_of(s);
+  return cudaSuccess;
+}
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {  // every host buffer is page-locked
+  memset(a, 0, sizeof(*a));
+  a->type = cudaMemoryTypeHost;
+  a->devicePointer = a->hostPointer = const_cast<void*>(p);
+  return cudaSuccess;
+}
 cudaError_t cudaGetSymbolAddress(void** p, const void* symbol) { *p = const_cast<void*>(symbol); return cudaSuccess; }
 }
 
@@ -87,12 +160,31 @@ cudaError_t launch_var_map(const litevggt_ctx* c, const __nv_bfloat16*, float*, 
 cudaError_t launch_partition(const litevggt_ctx* c, const float*, const float*, float*, uint8_t*, cudaStream_t, int* n) { return ran(c, n); }
 cudaError_t launch_build_lists(const litevggt_ctx* c, const uint8_t*, cudaStream_t, int* n) { return ran(c, n); }
 cudaError_t launch_match(litevggt_ctx* c, const __nv_bfloat16*, cudaStream_t, int* n) { return ran(c, n); }
-cudaError_t launch_index_build(litevggt_ctx* c, litevggt_plan*, cudaStream_t, int* n) { return ran(c, n); }
-cudaError_t launch_merge(const litevggt_ctx* c, const litevggt_plan*, const __nv_bfloat16*, __nv_bfloat16*, cudaStream_t, int* n) { return ran(c, n); }
-cudaError_t launch_unmerge(const litevggt_ctx* c, const litevggt_plan*, const __nv_bfloat16*, const __nv_bfloat16*, __nv_bfloat16*,
-                           cudaStream_t, int* n) { return ran(c, n); }
-cudaError_t launch_linear_scaled(litevggt_ctx* c, const __nv_bfloat16*, long long m, long long, const __nv_bfloat16*, long long,
-                                 const __nv_bfloat16*, int, int, float, const LinearStat& st, __nv_bfloat16*, cudaStream_t, int* n) {
+static Range rows(const void* p, long long n) { return {p, n * 1024 * 2}; }
+cudaError_t launch_index_build(litevggt_ctx* c, litevggt_plan* p, cudaStream_t s, int* n) {
+  const Sizes& z = c->sz;
+  touch(s, {}, {{p->dst_of, 4 * z.n_tokens}, {p->kept_idx, 4 * z.n_merged}, {p->seg_off, 4 * (z.n_merged + 1)}, {p->seg_src, 4 * z.n_remove}});
+  return ran(c, n);
+}
+cudaError_t launch_merge(const litevggt_ctx* c, const litevggt_plan* p, const __nv_bfloat16* x, __nv_bfloat16* xm, cudaStream_t s, int* n) {
+  touch(s, {rows(x, c->sz.n_tokens), {p->kept_idx, 4 * c->sz.n_merged}}, {rows(xm, c->sz.n_merged)});
+  return ran(c, n);
+}
+cudaError_t launch_unmerge(const litevggt_ctx* c, const litevggt_plan* p, const __nv_bfloat16* ym, const __nv_bfloat16* res, __nv_bfloat16* out,
+                           cudaStream_t s, int* n) {
+  touch(s, {rows(ym, c->sz.n_merged), rows(res, c->sz.n_tokens), {p->dst_of, 4 * c->sz.n_tokens}}, {rows(out, c->sz.n_tokens)});
+  return ran(c, n);
+}
+cudaError_t launch_unmerge_rows(const litevggt_ctx* c, const int* dst_of, const int* kept, const int* off, const int* src, const __nv_bfloat16* ym,
+                                const __nv_bfloat16* res, __nv_bfloat16* out, long long row0, long long row1, cudaStream_t s, int* n) {
+  const Sizes& z = c->sz;
+  touch(s, {rows(ym + row0 * 1024, row1 - row0), rows(res, z.n_tokens), {dst_of, 4 * z.n_tokens}, {kept, 4 * z.n_merged}, {off, 4 * (z.n_merged + 1)},
+            {src, 4 * z.n_remove}}, {rows(out, z.n_tokens)});
+  return ran(c, n);
+}
+cudaError_t launch_linear_scaled(litevggt_ctx* c, const __nv_bfloat16* a, long long m, long long, const __nv_bfloat16*, long long,
+                                 const __nv_bfloat16*, int, int, float, const LinearStat& st, __nv_bfloat16* out, cudaStream_t s, int* n) {
+  touch(s, {rows(a, m)}, {rows(out, 3 * m)});
   if (st.key_norm != nullptr) {  // raises every norm to 4, as an atomic maximum would
     const long long words = m / st.seq_len * 16;
     g_norm_seen = st.key_norm[0];
@@ -109,8 +201,9 @@ static cudaError_t output_projection(litevggt_ctx* c, const ZeroWords& z, int* n
   zero_words(z);
   return ran(c, n);
 }
-cudaError_t launch_linear(litevggt_ctx* c, const __nv_bfloat16*, long long, long long, const __nv_bfloat16*, long long,
-                          const __nv_bfloat16*, const ZeroWords& z, __nv_bfloat16*, cudaStream_t, int* n) {
+cudaError_t launch_linear(litevggt_ctx* c, const __nv_bfloat16* a, long long m, long long, const __nv_bfloat16*, long long,
+                          const __nv_bfloat16*, const ZeroWords& z, __nv_bfloat16* out, cudaStream_t s, int* n) {
+  touch(s, {rows(a, m)}, {rows(out, m)});
   return output_projection(c, z, n);
 }
 cudaError_t launch_linear_mlp(litevggt_ctx* c, const __nv_bfloat16*, long long, long long, const __nv_bfloat16*, long long,
@@ -131,7 +224,18 @@ cudaError_t launch_qk_embed(const litevggt_ctx* c, __nv_bfloat16*, const int*, l
                             const __nv_bfloat16*, const __nv_bfloat16*, float, int rope, float, float*, cudaStream_t, int* n) {
   return g == nullptr && !rope ? cudaSuccess : ran(c, n);
 }
-cudaError_t launch_flash_attention(litevggt_ctx* c, const __nv_bfloat16*, long long, int, __nv_bfloat16*, cudaStream_t, int* n) { return ran(c, n); }
+cudaError_t launch_flash_attention(litevggt_ctx* c, const __nv_bfloat16* qkv, long long m, int n_seq, __nv_bfloat16* o, cudaStream_t s, int* n) {
+  touch(s, {rows(qkv, 3 * m * n_seq)}, {rows(o, m * n_seq)});
+  return ran(c, n);
+}
+long long flash_attention_slab_end(const litevggt_ctx*, long long m, long long row0) {
+  return m <= 4096 ? m : row0 + 2304 < m ? row0 + 2304 : m;
+}
+cudaError_t launch_flash_attention_rows(litevggt_ctx* c, const __nv_bfloat16* qkv, long long m, long long row0, long long row1, __nv_bfloat16* o,
+                                        cudaStream_t s, int* n) {
+  touch(s, {rows(qkv, 3 * m)}, {rows(o + row0 * 1024, row1 - row0)});
+  return ran(c, n);
+}
 cudaError_t launch_qkv_quantize(litevggt_ctx* c, const __nv_bfloat16*, long long, bool, cudaStream_t, int* n) { return ran(c, n); }
 cudaError_t launch_flash_attention_fp8(litevggt_ctx* c, long long, __nv_bfloat16*, cudaStream_t, int* n) { return ran(c, n); }
 }  // namespace lv

@@ -110,6 +110,33 @@ def test_output_that_leaves_in_slabs(lib, frames, grid, ratio):
     ctx.close()
 
 
+def test_host_entries_in_turn_without_a_drain(lib):
+    """An ordered call right behind a pipelined one, and the other way round, as often as there are buffers: every output is
+    what the same entry gives alone."""
+    frames, grid = 5, (37, 37)
+    ctx = lib.LiteVGGT(frames, *grid, 0.3)
+    n = ctx.n_tokens
+    w = [v.cuda() for v in make_attention_weights(WORKLOADS["C1"], 2)]
+    g = torch.Generator().manual_seed(n)
+    xs = [_tokens(n, n + i).pin_memory() for i in range(6)]
+    plan = ctx.merge_plan(xs[0].cuda(), torch.rand(frames, *grid, generator=g).cuda())
+    calls = (ctx.global_layer_host_pipelined, ctx.global_layer_host)
+    for order in ((0, 1, 0, 1, 1, 0), (1, 0, 0, 1, 0, 0)):
+        alone, behind = ([torch.zeros_like(x).pin_memory() for x in xs] for _ in range(2))
+        for outs in (alone, behind):
+            for k, x, out in zip(order, xs, outs):
+                calls[k](plan, x, *w, out)
+                if outs is alone:
+                    ctx.host_drain()
+                    ctx.poll()
+            ctx.host_drain()
+            ctx.poll()
+        for i, (a, b) in enumerate(zip(alone, behind)):
+            assert torch.equal(a, b), f"call {i} of {order}"
+    plan.destroy()
+    ctx.close()
+
+
 @pytest.mark.parametrize("grid,keep", [((1, 1), 0.1), ((16, 16), 0.1), ((16, 16), 0.9), ((4, 64), 0.5), ((7, 37), 0.1), ((6, 43), 0.3)])
 def test_ranks_of_a_small_frames_scores(lib, grid, keep):
     """Frames of 1, 256, 258 and 259 patches: up to 256 every patch is ranked against the others, above a search finds

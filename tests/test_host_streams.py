@@ -1,0 +1,64 @@
+"""What the host entry points leave to their streams and events: the host side of the library linked against
+stand-ins that keep track of which memory every stream's work touches and of what nothing orders (host_fakes.cpp)."""
+import ctypes as C
+import os
+import subprocess
+
+import pytest
+
+from paper_2512_04939_b200.binding import Config
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2512_04939_b200", "csrc")
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("host") / "libhost.so")
+    sources = [os.path.join(CSRC, f) for f in ("api.cu", "attn_static.cu", "host_pipeline.cu")] + [os.path.join(HERE, "host_fakes.cpp")]
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-w", "-Wl,-Bsymbolic", "-I/usr/local/cuda/include", "-x", "c++",
+                    *sources, "-o", so], check=True)
+    return C.CDLL(so)
+
+
+class Layer:
+    """A context of three 37 x 37 frames, a plan and page-locked buffers, every call on another pair of them."""
+
+    def __init__(self, lib, ratio=0.0, frames=3):
+        cfg = Config()
+        assert lib.litevggt_default_config(frames, 37, 37, C.c_float(ratio), C.byref(cfg)) == 0
+        self.lib, self.h, self.plan = lib, C.c_void_p(), C.c_void_p()
+        assert lib.litevggt_create(C.byref(cfg), 0, C.byref(self.h)) == 0
+        n = C.c_int64()
+        lib.litevggt_sizes(self.h, C.byref(n), None, None, None, None)
+        self.n, self.kept = n.value, []
+        self.p = self.buffer(1 << 12)
+        lib.fake_forget_accesses()
+        assert lib.litevggt_merge_plan(self.h, self.buffer(2048 * self.n), self.p, C.byref(self.plan), None) == 0
+
+    def buffer(self, size):
+        self.kept.append(C.create_string_buffer(size + 256))
+        return C.c_void_p((C.addressof(self.kept[-1]) + 255) & ~255)
+
+    def call(self, entry, grad=False):
+        p, x, out = self.p, self.buffer(2048 * self.n), self.buffer(2048 * self.n)
+        return getattr(self.lib, entry)(self.h, C.byref(self.plan), p if grad else None, x, p, p, p, p, out, None)
+
+    def close(self):
+        self.lib.litevggt_plan_destroy(self.plan)
+        self.lib.litevggt_destroy(self.h)
+
+
+PIPED, ORDERED = "litevggt_global_layer_host_pipelined", "litevggt_global_layer_host"
+
+
+@pytest.mark.parametrize("ratio", [0.0, 0.4])  # 4,122 merged rows leave in slabs, 2,474 behind the layer
+@pytest.mark.parametrize("calls", [(PIPED, ORDERED), (ORDERED, PIPED), (PIPED, PIPED, PIPED, PIPED), (PIPED, PIPED, ORDERED, PIPED, ORDERED, PIPED)])
+def test_nothing_unordered_between_host_entries(host, calls, ratio):
+    """The pipelined entry's copies and writers run on streams of their own; whatever the next call does, of either entry,
+    on a plan that it rebuilds in place, must not meet them in memory."""
+    layer = Layer(host, ratio)
+    for entry in calls:
+        assert layer.call(entry, grad=True) == 0
+    assert host.fake_races() == 0
+    layer.close()
