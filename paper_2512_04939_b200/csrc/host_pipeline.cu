@@ -65,18 +65,20 @@ litevggt_status ensure_host_pipe(litevggt_ctx* ctx) {
   return LITEVGGT_OK;
 }
 
-// Where the device writes `bytes` of page-locked host memory, or nothing: 16-byte units must fit.
+// Where the device writes `bytes` of page-locked host memory, or nothing: one allocation or registration must hold them
+// all (two that hold the ends may have pages between them that the device cannot reach), and 16-byte units must fit.
 void* device_view(void* host, size_t bytes) {
-  cudaPointerAttributes first, last;
-  if (cudaPointerGetAttributes(&first, host) != cudaSuccess ||
-      cudaPointerGetAttributes(&last, static_cast<uint8_t*>(host) + bytes - 1) != cudaSuccess) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
     (void)cudaGetLastError();
     return nullptr;
   }
-  if (first.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || first.devicePointer == nullptr ||
-      static_cast<uint8_t*>(last.devicePointer) - static_cast<uint8_t*>(first.devicePointer) != (ptrdiff_t)bytes - 1)
+  if (at.type != cudaMemoryTypeHost || at.devicePointer == nullptr || !aligned16(at.devicePointer)) return nullptr;
+  const uint8_t *first = static_cast<const uint8_t*>(at.devicePointer), *begin = nullptr;
+  size_t size = 0;
+  if (!allocation_of(first, &begin, &size) || begin > first || (size_t)(first - begin) > size || size - (size_t)(first - begin) < bytes)
     return nullptr;
-  return aligned16(first.devicePointer) ? first.devicePointer : nullptr;
+  return at.devicePointer;
 }
 
 // The attention layer and the unmerge in slabs of query rows, the finished tokens written to `out`.

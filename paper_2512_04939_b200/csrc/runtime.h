@@ -220,6 +220,8 @@ struct ZeroWords {
 
 // tensor_map.cu
 bool resolve_encode_tiled(void** fn);
+// The allocation or registration that an address which the device can use lies in.
+bool allocation_of(const void* device_ptr, const uint8_t** begin, size_t* bytes);
 // 2-D bf16 tensor [outer, inner] row-major with row pitch `pitch_elems`; box [box_outer, box_inner],
 // 128-byte swizzle, zero fill outside the tensor.
 bool make_tmap_bf16_2d(void* encode_fn, CUtensorMap* out, const void* base, uint64_t inner, uint64_t outer,

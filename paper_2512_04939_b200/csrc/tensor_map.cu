@@ -1,20 +1,35 @@
-// Tensor-map (TMA descriptor) encoding on the host.  The driver entry point is resolved
-// at run time so the library carries no link-time dependency on libcuda.
+// What the host side asks the driver itself: tensor-map (TMA descriptor) encoding, and how far an address's allocation
+// reaches.  The entry points are resolved at run time so the library carries no link-time dependency on libcuda.
 #include <cudaTypedefs.h>
 
 #include "runtime.h"
 
 namespace lv {
 
-bool resolve_encode_tiled(void** fn) {
+static bool resolve(const char* name, void** fn) {
   void* p = nullptr;
   cudaDriverEntryPointQueryResult q;
-  cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q);
+  cudaError_t e = cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &q);
   if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || p == nullptr) {
     (void)cudaGetLastError();
     return false;
   }
   *fn = p;
+  return true;
+}
+
+bool resolve_encode_tiled(void** fn) { return resolve("cuTensorMapEncodeTiled", fn); }
+
+bool allocation_of(const void* device_ptr, const uint8_t** begin, size_t* bytes) {
+  void* fn = nullptr;
+  if (!resolve("cuPointerGetAttribute", &fn)) return false;
+  auto attribute = reinterpret_cast<PFN_cuPointerGetAttribute_v4000>(fn);
+  const CUdeviceptr p = reinterpret_cast<CUdeviceptr>(device_ptr);
+  CUdeviceptr start = 0;
+  if (attribute(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, p) != CUDA_SUCCESS ||
+      attribute(bytes, CU_POINTER_ATTRIBUTE_RANGE_SIZE, p) != CUDA_SUCCESS)
+    return false;
+  *begin = reinterpret_cast<const uint8_t*>(start);
   return true;
 }
 

@@ -66,6 +66,18 @@ static void touch(cudaStream_t s, std::vector<Range> reads, std::vector<Range> w
       g_accesses.push_back(a);
     }
 }
+// Page-locked host memory: all of it, unless a test says which.
+static const Range kAll{nullptr, 1ll << 62};
+static std::vector<Range> g_locked;
+static const Range* page_locked(const void* p) {
+  for (const Range& r : g_locked)
+    if (p >= r.p && p < static_cast<const char*>(r.p) + r.bytes) return &r;
+  return g_locked.empty() ? &kAll : nullptr;
+}
+static int g_rows_written = 0;  // launches that write rows to their tokens in host memory
+extern "C" void fake_page_lock(const void* p, long long bytes) { g_locked.push_back({p, bytes}); }
+extern "C" void fake_page_lock_all() { g_locked.clear(); }
+extern "C" int fake_rows_written() { return g_rows_written; }
 extern "C" int fake_races() { return g_races; }
 extern "C" void fake_forget_accesses() {
   g_stream_clocks.clear();
@@ -130,10 +142,12 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
   g_events[e] = clock_of(s);
   return cudaSuccess;
 }
-cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {  // every host buffer is page-locked
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
   memset(a, 0, sizeof(*a));
+  a->hostPointer = const_cast<void*>(p);
+  if (page_locked(p) == nullptr) return cudaSuccess;
   a->type = cudaMemoryTypeHost;
-  a->devicePointer = a->hostPointer = const_cast<void*>(p);
+  a->devicePointer = a->hostPointer;
   return cudaSuccess;
 }
 cudaError_t cudaGetSymbolAddress(void** p, const void* symbol) { *p = const_cast<void*>(symbol); return cudaSuccess; }
@@ -153,6 +167,13 @@ static cudaError_t ran(const litevggt_ctx* ctx, int* launches) {  // one kernel 
 static void zero_words(const ZeroWords& z) { if (z.count > 0) memset(z.words, 0, (size_t)z.count * 4); }
 
 bool resolve_encode_tiled(void** fn) { *fn = reinterpret_cast<void*>(1); return true; }
+bool allocation_of(const void* p, const uint8_t** begin, size_t* bytes) {
+  const Range* r = page_locked(p);
+  if (r == nullptr) return false;
+  *begin = static_cast<const uint8_t*>(r->p);
+  *bytes = (size_t)r->bytes;
+  return true;
+}
 long long index_scratch_words(const Sizes&) { return 1; }
 size_t attention_state_bytes(long long, int, int, int, size_t* ml) { *ml = 0; return 0; }
 cudaError_t launch_grad_map(const litevggt_ctx* c, const float*, float*, cudaStream_t, int* n) { return ran(c, n); }
@@ -178,6 +199,7 @@ cudaError_t launch_unmerge(const litevggt_ctx* c, const litevggt_plan* p, const 
 cudaError_t launch_unmerge_rows(const litevggt_ctx* c, const int* dst_of, const int* kept, const int* off, const int* src, const __nv_bfloat16* ym,
                                 const __nv_bfloat16* res, __nv_bfloat16* out, long long row0, long long row1, cudaStream_t s, int* n) {
   const Sizes& z = c->sz;
+  ++g_rows_written;
   touch(s, {rows(ym + row0 * 1024, row1 - row0), rows(res, z.n_tokens), {dst_of, 4 * z.n_tokens}, {kept, 4 * z.n_merged}, {off, 4 * (z.n_merged + 1)},
             {src, 4 * z.n_remove}}, {rows(out, z.n_tokens)});
   return ran(c, n);

@@ -40,8 +40,8 @@ class Layer:
         self.kept.append(C.create_string_buffer(size + 256))
         return C.c_void_p((C.addressof(self.kept[-1]) + 255) & ~255)
 
-    def call(self, entry, grad=False):
-        p, x, out = self.p, self.buffer(2048 * self.n), self.buffer(2048 * self.n)
+    def call(self, entry, grad=False, out=None):
+        p, x, out = self.p, self.buffer(2048 * self.n), out or self.buffer(2048 * self.n)
         return getattr(self.lib, entry)(self.h, C.byref(self.plan), p if grad else None, x, p, p, p, p, out, None)
 
     def close(self):
@@ -61,4 +61,24 @@ def test_nothing_unordered_between_host_entries(host, calls, ratio):
     for entry in calls:
         assert layer.call(entry, grad=True) == 0
     assert host.fake_races() == 0
+    layer.close()
+
+
+@pytest.mark.parametrize("locked,direct", [
+    ([(0, 1)], True), ([(-4096, 2)], True),                             # one range, from the buffer's start or before
+    ([(0, 0.999)], False), ([(4096, 1)], False),                        # its end or its beginning is not in it
+    ([(0, 0.25), (0.75, 0.25)], False), ([(0, 0.5), (0.5, 0.5)], False),  # both ends are, in two ranges
+    ([(0, -1)], False)])                                                # nothing is page-locked
+def test_only_a_buffer_in_one_page_locked_range_is_written_by_kernels(host, locked, direct):
+    """Kernels write the output only where one page-locked range holds all of it; any other buffer gets a copy."""
+    layer = Layer(host)
+    size = 2048 * layer.n
+    out = layer.buffer(size)
+    for at, length in locked:
+        begin = out.value + int(at if abs(at) > 1 else at * size)
+        host.fake_page_lock(C.c_void_p(begin), C.c_longlong(int(length * size)))
+    before = host.fake_rows_written()
+    assert layer.call(PIPED, out=out) == 0
+    assert (host.fake_rows_written() > before) == direct
+    host.fake_page_lock_all()
     layer.close()
