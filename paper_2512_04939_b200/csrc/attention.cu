@@ -270,13 +270,6 @@ __device__ __forceinline__ float2 poly_exp2_pair(float2 x) {
   return poly_exp2_pair<false>(x, make_float2(12582912.0f, 12582912.0f), make_float2(-12582912.0f, -12582912.0f));
 }
 
-// The larger of the two, NaN if either is.
-__device__ __forceinline__ float fmax_nan(float a, float b) {
-  float r;
-  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-  return r;
-}
-
 // Wait until the most recent loads into a ring (up to one per stage) have landed.
 // `issued` counts the loads issued into the ring so far; load i uses stage i % kStages and
 // completes the phase with parity (i / kStages) & 1.  Not sensitive to the abort flag: the

@@ -464,10 +464,11 @@ struct LinearEpilogue {
 // negative side has no cancellation and neither side a branch.  Two values at a time, in packed arithmetic, 1 / sqrt 2
 // and the 1/2 in the constants: about 9 issue slots a value where the scalar form took 16, in an epilogue that shares
 // them with nobody but draws on the same power (MLP of 208,200 rows 2.75 -> 2.68 ms, of 3,360 rows 55.6 -> 54.8 us;
-// largest error against 64 bits over [-12, 12] 3.3e-7, scalar 4.2e-7).
+// largest error against 64 bits over [-12, 12] 3.3e-7, scalar 4.2e-7).  |x| counts as 64 at most, where h is long zero, so
+// that an infinite x meets no infinity times zero; a NaN stays one.
 __device__ __forceinline__ float2 gelu_erf(float2 x) {
   auto both = [](float c) { return make_float2(c, c); };
-  const float2 m = make_float2(-fabsf(x.x), -fabsf(x.y));  // -|x|
+  const float2 m = make_float2(fmax_nan(-fabsf(x.x), -64.0f), fmax_nan(-fabsf(x.y), -64.0f));  // -|x|
   const float2 d = __ffma2_rn(m, both(-0.3275911f * 0.70710678118654752f), both(1.0f));
   float2 t, ex;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t.x) : "f"(d.x));

@@ -749,6 +749,36 @@ def test_layernorm_frame_attention_and_mlp(lib, wl):
     ctx.close()
 
 
+@pytest.mark.parametrize("rows", [40, 1044])
+def test_gelu_of_values_that_are_not_ordinary(lib, rows):
+    """One hidden unit of the MLP takes infinities, NaN, the largest finite values and where the tails end; the
+    others are zero.  The second layer hands it through, so a row is gelu(its value), rounded twice to bf16."""
+    ctx = _ctx(lib, WORKLOADS["C1"])
+    big = 2.0 ** 64
+    hidden = [np.inf, -np.inf, np.nan, 3.0 * 2.0 ** 126, -3.0 * 2.0 ** 126, 2.0 ** 100, -2.0 ** 100, 0.0, 2.0 ** -60, -2.0 ** -60]
+    hidden += [s * v for v in (0.5, 1.0, 5.5, 12.0, 13.0, 18.0, 63.5, 64.0, 64.5, 70.0, 300.0) for s in (1.0, -1.0)]
+    x = torch.zeros(rows, 1024, dtype=torch.bfloat16)
+    # (infinities as products that overflow)
+    factor = [np.copysign(2.0 ** 65, v) if np.isinf(v) else v / big for v in hidden]
+    x[:len(hidden), 0] = torch.tensor(factor, dtype=torch.float64).to(torch.bfloat16)
+    w1, w2 = torch.zeros(4096, 1024, dtype=torch.bfloat16), torch.zeros(1024, 4096, dtype=torch.bfloat16)
+    w1[0, 0] = big
+    w2[:, 0] = 1.0
+    y = ctx.mlp(x.cuda(), w1.cuda(), None, w2.cuda(), None).cpu().double().numpy()
+    ctx.poll()
+    for r, v in enumerate(hidden):
+        if np.isnan(v):
+            assert np.isnan(y[r]).all()
+        elif np.isinf(v):
+            assert (y[r] == max(v, 0.0)).all()  # the limits
+        else:  # two roundings to bf16, and the rational approximation's 1.5e-7 of |v| / 2 where its tail is not zero
+            ref = float(O.gelu(np.array([v]))[0])
+            bound = 2.0 ** -7 * abs(ref) + (0.75e-7 * abs(v) if abs(v) < 64.0 else 0.0) + 2.0 ** -133
+            assert np.abs(y[r] - ref).max() <= bound, (v, ref, y[r][0])
+    assert (y[len(hidden):] == 0.0).all()
+    ctx.close()
+
+
 # ------------------------------------------------------------------ whole layer
 def test_whole_layer_c1_and_host_entry(lib):
     wl = WORKLOADS["C1"]
