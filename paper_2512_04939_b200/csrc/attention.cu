@@ -95,7 +95,7 @@
 // fixed form.  Trained projections attend that sharply (query weights x 16 on the generator's tokens:
 // B up to 213): 31,751 rows went from 4.81 to 4.41 ms there.
 // What remains takes the online form: base-2 softmax with a lazily updated reference
-// maximum, the running output rescaled only when a row maximum grows by more than 2^32 over the
+// maximum, the running output rescaled only when a row maximum grows by more than 2^8 over the
 // reference (the threads then first wait until the tile's last P V has retired).  All three equal
 // the plain softmax up to rounding.
 #include <type_traits>
@@ -111,9 +111,11 @@ constexpr int kFaThreads = (kFaSoftmaxWarps + 3) * 32;
 constexpr int kFaTileBytes = kFaTileKeys * 64 * 2;
 constexpr int kFaOnesBytes = 16 * 128;  // 16 key rows of the ones column block
 constexpr uint32_t kFaOCols = 80;  // 64 output channels, the row sum, 15 unused columns
-// How far a row maximum may grow over the reference of the online form before the row is rescaled.  Probabilities up to 2^32 lose
-// nothing (sums over 2^22 keys times |v| <= 2^20 stay below 2^74); a warp rescales when one of its 32 rows has to.
-constexpr float kFaRescaleThreshold = 32.0f;
+// How far a row maximum may grow over the reference of the online form before the row is rescaled (a warp rescales when one of
+// its 32 rows has to).  Low enough that parts of a row can be weighed against each other, see part_weight; 32 measured
+// the same time.
+constexpr float kFaRescaleThreshold = 8.0f;
+static_assert(126.0f + kFaRescaleThreshold < 149.0f, "part_weight reaches down to 2^-149");
 // Largest Cauchy-Schwarz bound B on the base-2 scores of a row for which the fixed reference is
 // used.  With the reference left out the probabilities lie in [2^-B, 2^B]: at B = 80 their products
 // with |v| >= 2^-20 are normal fp32 numbers (>= 2^-100), and a row sum over 2^20 keys times
@@ -232,6 +234,15 @@ static_assert(kFaAloneBytes >= FaShape<1>::kSmemBytes, "");
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// What a part of a row counts for beside another whose reference is the higher one by -x: below 2^-126 too, where fast_exp2
+// gives zero.  A part in the online form may hold 2^kFaRescaleThreshold a key, one in the shifted form only
+// 2^-fa_shift_down in all, so what the lower one holds is lost to the row's 24 bits only beyond 2^-(126 + kFaRescaleThreshold).
+__device__ __forceinline__ float part_weight(float x) {
+  float y;
+  asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 
@@ -865,8 +876,8 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
             float a_old = 1.0f, a_new = 1.0f;
             if (m_old != m_ref) {
               const float m_tot = fmaxf(m_old, m_ref);
-              a_old = fast_exp2(m_old - m_tot);
-              a_new = fast_exp2(m_ref - m_tot);
+              a_old = part_weight(m_old - m_tot);
+              a_new = part_weight(m_ref - m_tot);
               m_ref = m_tot;
             }
             const uint4* src = reinterpret_cast<const uint4*>(o_state + (size_t)row * dim + job.head * 64 + c * 32);
@@ -1253,8 +1264,8 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
           float a_old = 1.0f, a_new = 1.0f;
           if (m_old != m_ref) {
             const float m_tot = fmaxf(m_old, m_ref);
-            a_old = fast_exp2(m_old - m_tot);
-            a_new = fast_exp2(m_ref - m_tot);
+            a_old = part_weight(m_old - m_tot);
+            a_new = part_weight(m_ref - m_tot);
             m_ref = m_tot;
           }
           const uint4* src = reinterpret_cast<const uint4*>(o_state + (size_t)row * dim + head * 64 + c * 32);
@@ -1316,7 +1327,7 @@ combine_parts_kernel(FaJobs split, __nv_bfloat16* __restrict__ o, int seq_len, i
   for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
   for (int p = 0; p < split.parts; ++p) {
     const float2 ml = *reinterpret_cast<const float2*>(split.ml + ((slot0 + p) * 256 + r) * 2);
-    const float w = ml.x == m ? 1.0f : fast_exp2(ml.x - m);
+    const float w = ml.x == m ? 1.0f : part_weight(ml.x - m);
     sum = fmaf(ml.y, w, sum);
     const float4* src = reinterpret_cast<const float4*>(split.o + ((slot0 + p) * 256 + r) * 64 + ch);
     const float4 a = src[0], b = src[1];

@@ -67,6 +67,34 @@ def test_sequences_of_several_rounds_of_jobs(lib, frames, grid, sharpness):
     ctx.close()
 
 
+@pytest.mark.parametrize("frames,many,top,bound", [(2, 3900, 63.0, 243.0), (17, 30000, 66.0, 239.0)])
+def test_parts_of_a_row_under_references_far_apart(lib, frames, many, top, bound):
+    """8,192 rows, where some jobs are split in two along the keys, and 69,632 in two key chunks.  The first half scores 20 in
+    its first 64 keys, so that the running maximum has to serve, and 51 in `many` later ones; the second half's first key scores
+    `top` and one reference, 130 over the first half's, serves it.  The first half holds about a third of every row, the only part with
+    V = 1.  Scores are equal within a half, so an output is off by the rounding of two probabilities and its own: 3 x 2^-9 of it."""
+    ctx = lib.LiteVGGT(frames, 64, 64, 0.0, n_special=0)
+    rows = ctx.n_merged
+    half = rows // 2
+    x, w_qkv, b_qkv, w_o, b_o = (torch.zeros(*s, dtype=torch.bfloat16) for s in ((rows, 1024), (3072, 1024), (3072,), (1024, 1024), (1024,)))
+    score = torch.full((rows,), -50.0)
+    score[0], score[64:64 + many], score[half] = 20.0, 51.0, top
+    x[:, 0] = score / 16 / K_FOLD
+    x[5, 1] = (bound ** 2 - 50.0 ** 2) ** 0.5 / 16 / K_FOLD  # a long key, across the queries but for its score of -50
+    x[64:64 + many, 2] = 1.0
+    for h in range(16):
+        b_qkv[64 * h] = 16.0
+        w_qkv[1024 + 64 * h, 0] = w_qkv[1024 + 64 * h + 1, 1] = w_qkv[2048 + 64 * h, 2] = 1.0
+    ctx.global_attn(x.cuda(), w_qkv.cuda(), b_qkv.cuda(), w_o.cuda(), b_o.cuda())
+    ctx.poll()
+    s = 16.0 * to_f64(ctx.debug_buffer(0)[:, 1024:1025])[:, 0]  # the scores that the kernel had, in base 2
+    p = np.exp2(s - s.max())
+    ref = p[64:64 + many].sum() / p.sum()
+    out = to_f64(ctx.debug_buffer(1)[:, ::64])
+    assert 0.2 < ref < 0.6 and np.abs(out / ref - 1.0).max() <= 3 * 2.0 ** -9
+    ctx.close()
+
+
 @pytest.mark.parametrize("frames,grid,ratio", [
     (3, (37, 37), 0.0),    # 4,122 rows: the fewest that leave in slabs, two of them
     (5, (37, 37), 0.3),    # a second slab of two rounds, not full
