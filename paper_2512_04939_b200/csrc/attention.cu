@@ -105,7 +105,6 @@
 
 namespace lv {
 
-constexpr int kFaTileKeys = 128;  // keys of a K/V tile, two steps
 constexpr int kFaSoftmaxWarps = 16;
 constexpr int kFaThreads = (kFaSoftmaxWarps + 3) * 32;
 constexpr int kFaTileBytes = kFaTileKeys * 64 * 2;
@@ -124,10 +123,6 @@ static_assert(126.0f + kFaRescaleThreshold < 149.0f, "part_weight reaches down t
 #define LV_FA_FIXED_REF_LIMIT 80.0f
 #endif
 constexpr float kFaFixedRefLimit = LV_FA_FIXED_REF_LIMIT;
-#ifndef LV_FA_CHUNK_TILES
-#define LV_FA_CHUNK_TILES 512
-#endif
-constexpr int kFaChunkTiles = LV_FA_CHUNK_TILES;  // 65536 keys: K and V of one head = 16 MiB
 // Of the 16 pairs of scores a thread handles per step, this many take the polynomial exponential
 // (fixed-reference form only, where every argument lies in [-kFaFixedRefLimit, kFaFixedRefLimit]).
 #ifndef LV_FA_POLY_PAIRS
@@ -156,11 +151,6 @@ static float key_bits(long long keys) {
 }
 static float fa_shift_up(long long keys) { return 126.0f - 20.0f - key_bits(keys); }
 static float fa_shift_down(long long keys) { return 126.0f - 24.0f - key_bits(keys); }
-// Sequences of at most this many rows take CTAs of one query tile, two to an SM (figures at the top).
-#ifndef LV_FA_ONE_TILE_ROWS
-#define LV_FA_ONE_TILE_ROWS 4096
-#endif
-constexpr long long kFaOneTileRows = LV_FA_ONE_TILE_ROWS;
 
 // The jobs of a launch, one query block of one head of one sequence each, query blocks fastest.  Those that the last
 // round would leave alone on the chip are split along the keys: ids from `full` on are (job, part) with
@@ -1491,20 +1481,11 @@ cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, 
   return launch_rows(ctx, qkv, seq_len, 0, seq_len, n_seq, 0, o, s, launches);
 }
 
-// Query rows of so many rounds of CTAs, in whole query blocks of every head.
-static long long rounds_rows(const litevggt_ctx* ctx, int rounds) { return (long long)rounds * ctx->num_sms / ctx->sz.heads * 256; }
-// One round, so that the first rows are soon there, then two at a time.
-long long flash_attention_slab_end(const litevggt_ctx* ctx, long long m, long long row0) {
-  if (m <= kFaOneTileRows || (m + kFaTileKeys - 1) / kFaTileKeys > kFaChunkTiles) return m;
-  const long long end = row0 + rounds_rows(ctx, row0 == 0 ? 1 : 2);
-  return end < m ? end : m;
-}
-
 cudaError_t launch_flash_attention_rows(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long m, long long row0, long long row1,
                                         __nv_bfloat16* o, cudaStream_t s, int* launches) {
-  const long long first = rounds_rows(ctx, 1), slab = rounds_rows(ctx, 2), index = row0 == 0 ? 0 : 1 + (row0 - first) / slab;
-  if (row0 < 0 || row0 % 256 != 0 || row1 != flash_attention_slab_end(ctx, m, row0)) return cudaErrorInvalidValue;
-  return launch_rows(ctx, qkv, m, row0, row1, 1, (int)index, o, s, launches);
+  const int sms = ctx->num_sms, heads = ctx->sz.heads;
+  if (row0 < 0 || row0 % 256 != 0 || row1 != attention_slab_end(m, row0, sms, heads)) return cudaErrorInvalidValue;
+  return launch_rows(ctx, qkv, m, row0, row1, 1, attention_slab_index(row0, sms, heads), o, s, launches);
 }
 
 // What passes between launches: for several key chunks rows of fp32 partial output and of {reference, row

@@ -105,7 +105,7 @@ cudaError_t layer_in_slabs(litevggt_ctx* ctx, const litevggt_plan* plan, int slo
   auto copied = [&](const int* array) { return hp.index[slot] + (array - plan->dst_of); };
   __nv_bfloat16* ym = hp.out[slot];  // (the staged output is not needed: M <= N rows of it hold the merged ones)
   for (long long row0 = 0, row1; row0 < m && e == cudaSuccess; row0 = row1) {
-    row1 = flash_attention_slab_end(ctx, m, row0);
+    row1 = attention_slab_end(m, row0, ctx->num_sms, z.heads);
     {
       StepTimer t(ctx, 7, n, e);
       e = launch_flash_attention_rows(ctx, ws.qkv, m, row0, row1, ws.attn_o, s, &n);
@@ -164,7 +164,7 @@ litevggt_status litevggt_global_layer_host_pipelined(litevggt_ctx* ctx, litevggt
   }
   const litevggt_plan* plan = *plan_inout;
   st = litevggt_merge(ctx, plan, hp.x[slot], ws.stage_xm, stream);
-  const bool apart = ctx->cfg.qkv_dtype == 0 && flash_attention_slab_end(ctx, z.n_merged, 0) < z.n_merged;
+  const bool apart = ctx->cfg.qkv_dtype == 0 && attention_slab_end(z.n_merged, 0, ctx->num_sms, z.heads) < z.n_merged;
   void* direct = st == LITEVGGT_OK && apart ? device_view(out_host, bytes) : nullptr;
   if (direct != nullptr) {
     bool started = false;

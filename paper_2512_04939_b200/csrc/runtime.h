@@ -11,6 +11,7 @@
 #include <atomic>
 
 #include "../../include/litevggt.h"
+#include "attn_slabs.h"
 
 namespace lv {
 
@@ -50,9 +51,6 @@ inline cudaError_t set_max_dynamic_smem_once(const void* kernel, int bytes, std:
 constexpr float kKeyScaleLog2e = 0.125f * 1.4426950408889634f;
 
 constexpr long long kMlpChunkRows = 131072;  // rows of the 4D-wide hidden activations held at a time (1 GiB)
-
-// one counter per launch of an attention core: the key chunks of at most 4 Mi keys, or the slabs of one chunk
-constexpr int kAttnCounters = 64;
 
 // One device allocation carved into named regions.
 struct Workspace {
@@ -300,9 +298,7 @@ cudaError_t launch_qk_embed(const litevggt_ctx* ctx, __nv_bfloat16* qkv, const i
 // K last: the projection or qk_embed)
 cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long seq_len, int n_seq,
                                    __nv_bfloat16* o, cudaStream_t s, int* launches);
-// The same for a slab of the one sequence's m query rows: rows [row0, row1) with row1 = flash_attention_slab_end(row0), which is m at
-// once for a sequence that is not to be taken apart.
-long long flash_attention_slab_end(const litevggt_ctx* ctx, long long m, long long row0);
+// The same for a slab of the one sequence's m query rows: rows [row0, row1) with row1 = attention_slab_end(row0).
 cudaError_t launch_flash_attention_rows(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long m, long long row0, long long row1,
                                         __nv_bfloat16* o, cudaStream_t s, int* launches);
 size_t attention_state_bytes(long long m, int dim, int heads, int num_sms, size_t* ml_offset);

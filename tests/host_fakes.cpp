@@ -77,6 +77,10 @@ static const Range* page_locked(const void* p) {
 static int g_rows_written = 0;  // launches that write rows to their tokens in host memory
 extern "C" void fake_page_lock(const void* p, long long bytes) { g_locked.push_back({p, bytes}); }
 extern "C" void fake_page_lock_all() { g_locked.clear(); }
+extern "C" long long fake_slab_end(long long m, long long row0, int sms) { return attention_slab_end(m, row0, sms, 16); }
+extern "C" int fake_slab_index(long long row0, int sms) { return attention_slab_index(row0, sms, 16); }
+static int g_sms = 148;
+extern "C" void fake_sms(int n) { g_sms = n; }
 extern "C" int fake_rows_written() { return g_rows_written; }
 extern "C" int fake_races() { return g_races; }
 extern "C" void fake_forget_accesses() {
@@ -95,7 +99,7 @@ cudaError_t cudaGetDeviceCount(int* n) { *n = 1; return cudaSuccess; }
 cudaError_t cudaGetDeviceProperties(cudaDeviceProp* p, int) {
   memset(p, 0, sizeof(*p));
   p->major = 10;
-  p->multiProcessorCount = 148;
+  p->multiProcessorCount = g_sms;
   return cudaSuccess;
 }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
@@ -249,9 +253,6 @@ cudaError_t launch_qk_embed(const litevggt_ctx* c, __nv_bfloat16*, const int*, l
 cudaError_t launch_flash_attention(litevggt_ctx* c, const __nv_bfloat16* qkv, long long m, int n_seq, __nv_bfloat16* o, cudaStream_t s, int* n) {
   touch(s, {rows(qkv, 3 * m * n_seq)}, {rows(o, m * n_seq)});
   return ran(c, n);
-}
-long long flash_attention_slab_end(const litevggt_ctx*, long long m, long long row0) {
-  return m <= 4096 ? m : row0 + 2304 < m ? row0 + 2304 : m;
 }
 cudaError_t launch_flash_attention_rows(litevggt_ctx* c, const __nv_bfloat16* qkv, long long m, long long row0, long long row1, __nv_bfloat16* o,
                                         cudaStream_t s, int* n) {

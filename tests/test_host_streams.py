@@ -82,3 +82,33 @@ def test_only_a_buffer_in_one_page_locked_range_is_written_by_kernels(host, lock
     assert (host.fake_rows_written() > before) == direct
     host.fake_page_lock_all()
     layer.close()
+
+
+@pytest.mark.parametrize("sms", [1, 7, 8, 15, 16, 20, 36, 74, 132, 148])
+@pytest.mark.parametrize("rows", [1, 4096, 4097, 22000, 40000, 65535, 65536, 65537, 4000000])
+def test_slabs_cover_a_sequence_on_any_number_of_sms(host, rows, sms):
+    """In order, in whole query blocks, no more of them than there are job counters - or the sequence as a whole."""
+    end = lambda row0: host.fake_slab_end(C.c_longlong(rows), C.c_longlong(row0), sms)
+    host.fake_slab_end.restype = C.c_longlong
+    row0, slabs = 0, 0
+    while row0 < rows:
+        row1 = end(row0)
+        assert row0 < row1 <= rows and slabs < 64
+        if rows > row1 or row0 > 0:
+            assert host.fake_slab_index(C.c_longlong(row0), sms) == slabs and row0 % 256 == 0
+        row0, slabs = row1, slabs + 1
+    if rows <= 4096 or rows > 65536 or sms < 16:
+        assert slabs == 1
+    if sms == 148 and 4096 < rows <= 65536:
+        assert slabs > 1
+
+
+@pytest.mark.parametrize("sms", [12, 20])
+def test_a_layer_of_a_partitioned_gpu_leaves_for_host_memory(host, sms):
+    host.fake_sms(sms)
+    layer = Layer(host)
+    before = host.fake_rows_written()
+    assert layer.call(PIPED) == 0 and layer.call(PIPED, grad=True) == 0
+    assert (host.fake_rows_written() > before) == (sms >= 16) and host.fake_races() == 0
+    layer.close()
+    host.fake_sms(148)
