@@ -243,9 +243,9 @@ litevggt_status litevggt_global_layer_host(litevggt_ctx* ctx, litevggt_plan** pl
  *     called on `stream` after this call and that point of the stream has been reached.
  *   - A call does not wait for the output copies of earlier calls: feeding one call's out_host to
  *     the next call's x_host needs a drain in between (or the plain entry point, which is ordered).
- *   - Where out_host is page-locked and 16-byte aligned, tokens may be written to it as soon as their rows are
- *     done, in any order.  The attention's rows are then shared out differently over the chip than in
- *     litevggt_global_layer_host, whose results this call's equal up to rounding.
+ *   - The first call, and the first after a drain, may write tokens to a page-locked, 16-byte aligned out_host as soon as
+ *     their rows are done, in any order, so that a call by itself takes less time.  The attention's rows are then shared out
+ *     differently over the chip than in litevggt_global_layer_host, whose results this call's equal up to rounding.
  *   - The first call allocates two pairs of staging buffers (4 x N x D bf16 in all; the plain entry point has
  *     buffers of its own, so calls of either may follow one another) and creates the streams and events. */
 litevggt_status litevggt_global_layer_host_pipelined(litevggt_ctx* ctx, litevggt_plan** plan_inout,

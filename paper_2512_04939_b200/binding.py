@@ -305,8 +305,9 @@ class LiteVGGT:
     def global_layer_host_pipelined(self, plan: Plan | None, x_host, w_qkv, b_qkv, w_o, b_o, out_host,
                                     grad=None) -> Plan:
         """global_layer_host for independent calls in a row: the copies run on the context's copy
-        streams and overlap the neighbouring calls' kernels.  ``out_host`` is complete only after
-        ``host_drain()`` and a synchronisation of the current stream."""
+        streams and overlap the neighbouring calls' kernels; a call that follows a drain may write its
+        output while it computes.  ``out_host`` is complete only after ``host_drain()`` and a
+        synchronisation of the current stream."""
         assert x_host.device.type == "cpu" and out_host.device.type == "cpu"
         assert x_host.shape == (self.n_tokens, self.dim) and out_host.shape == x_host.shape
         h = plan.handle if plan is not None else C.c_void_p()

@@ -9,7 +9,11 @@
 // meanwhile), at 45 GB/s out.  The first slab is one round of the attention's CTAs, so that PCIe starts early, the
 // others two, which lose 3 % of a round at their end.  Output buffers that the device cannot write (pageable memory, odd
 // addresses), E4M3 contexts, sequences of up to 4096 rows and those of several key chunks, whose copies are
-// 6 % of a pass or less, take the copy behind the layer.
+// 6 % of a pass or less, take the copy behind the layer.  So does a call with no drain since the one before: in a stream
+// of calls a copy engine moves an output at 55 GB/s under the next call's kernels and takes nothing from them, while the
+// writers do (40 calls in a row and a drain, ms a call: 16 frames of 37 x 37 1.00 by copies, 1.20 in slabs, 32 frames 2.14
+// and 2.55, 44 frames 3.9 and 4.4; a call and its drain 2.22 and 1.98, 5.2 and 4.1, 7.9 and 6.3).  What a call does
+// thus follows from the calls before it and not from how far the device has come: results repeat.
 #include "host_common.h"
 
 using namespace lv;
@@ -164,7 +168,9 @@ litevggt_status litevggt_global_layer_host_pipelined(litevggt_ctx* ctx, litevggt
   }
   const litevggt_plan* plan = *plan_inout;
   st = litevggt_merge(ctx, plan, hp.x[slot], ws.stage_xm, stream);
-  const bool apart = ctx->cfg.qkv_dtype == 0 && attention_slab_end(z.n_merged, 0, ctx->num_sms, z.heads) < z.n_merged;
+  // In a stream of calls the copy of one hides behind the kernels of the next.
+  const bool apart = hp.drained && ctx->cfg.qkv_dtype == 0 && attention_slab_end(z.n_merged, 0, ctx->num_sms, z.heads) < z.n_merged;
+  hp.drained = false;
   void* direct = st == LITEVGGT_OK && apart ? device_view(out_host, bytes) : nullptr;
   if (direct != nullptr) {
     bool started = false;
@@ -213,6 +219,7 @@ litevggt_status litevggt_host_drain(litevggt_ctx* ctx, void* stream) {
   cudaError_t e = cudaSuccess;
   for (int slot = 0; slot < 2 && e == cudaSuccess; ++slot)
     if (hp.used[slot]) e = cudaStreamWaitEvent((cudaStream_t)stream, hp.out_free[slot], 0);
+  if (e == cudaSuccess) hp.drained = true;
   return cuda_status(e);
 }
 

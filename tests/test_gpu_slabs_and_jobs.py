@@ -139,8 +139,8 @@ def test_output_that_leaves_in_slabs(lib, frames, grid, ratio):
 
 
 def test_host_entries_in_turn_without_a_drain(lib):
-    """An ordered call right behind a pipelined one, and the other way round, as often as there are buffers: every output is
-    what the same entry gives alone."""
+    """An ordered call right behind a pipelined one, and the other way round, more often than there are buffers: every output is
+    what the call gives alone.  The first pipelined call leaves in slabs, those behind it as the ordered ones do."""
     frames, grid = 5, (37, 37)
     ctx = lib.LiteVGGT(frames, *grid, 0.3)
     n = ctx.n_tokens
@@ -149,18 +149,26 @@ def test_host_entries_in_turn_without_a_drain(lib):
     xs = [_tokens(n, n + i).pin_memory() for i in range(6)]
     plan = ctx.merge_plan(xs[0].cuda(), torch.rand(frames, *grid, generator=g).cuda())
     calls = (ctx.global_layer_host_pipelined, ctx.global_layer_host)
-    for order in ((0, 1, 0, 1, 1, 0), (1, 0, 0, 1, 0, 0)):
-        alone, behind = ([torch.zeros_like(x).pin_memory() for x in xs] for _ in range(2))
-        for outs in (alone, behind):
-            for k, x, out in zip(order, xs, outs):
-                calls[k](plan, x, *w, out)
-                if outs is alone:
-                    ctx.host_drain()
-                    ctx.poll()
+    alone = []
+    for call in calls:
+        outs = [torch.zeros_like(x).pin_memory() for x in xs]
+        for x, out in zip(xs, outs):
+            before = ctx.launch_count()
+            call(plan, x, *w, out)
+            launches = ctx.launch_count() - before
             ctx.host_drain()
             ctx.poll()
-        for i, (a, b) in enumerate(zip(alone, behind)):
-            assert torch.equal(a, b), f"call {i} of {order}"
+        alone.append((launches, outs))
+    assert alone[0][0] > alone[1][0] and not torch.equal(alone[0][1][0], alone[1][1][0])  # slabs, and a whole
+    for order in ((0, 1, 0, 1, 1, 0), (1, 0, 0, 1, 0, 0)):
+        outs = [torch.zeros_like(x).pin_memory() for x in xs]
+        for k, x, out in zip(order, xs, outs):
+            calls[k](plan, x, *w, out)
+        ctx.host_drain()
+        ctx.poll()
+        first = order.index(0)
+        for i, out in enumerate(outs):
+            assert torch.equal(out, alone[0 if i == first else 1][1][i]), f"call {i} of {order}"
     plan.destroy()
     ctx.close()
 

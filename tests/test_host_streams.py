@@ -44,6 +44,9 @@ class Layer:
         p, x, out = self.p, self.buffer(2048 * self.n), out or self.buffer(2048 * self.n)
         return getattr(self.lib, entry)(self.h, C.byref(self.plan), p if grad else None, x, p, p, p, p, out, None)
 
+    def drain(self):
+        assert self.lib.litevggt_host_drain(self.h, None) == 0
+
     def close(self):
         self.lib.litevggt_plan_destroy(self.plan)
         self.lib.litevggt_destroy(self.h)
@@ -112,3 +115,19 @@ def test_a_layer_of_a_partitioned_gpu_leaves_for_host_memory(host, sms):
     assert (host.fake_rows_written() > before) == (sms >= 16) and host.fake_races() == 0
     layer.close()
     host.fake_sms(148)
+
+
+def test_in_a_stream_of_calls_copies_take_the_output(host):
+    """Kernels write the output of a call that follows a drain (or nothing); without one in between, the copy of a call is
+    hidden behind the next one's kernels and takes no SM from them."""
+    layer = Layer(host)
+    direct = []
+    for drain in (False, False, True, False, True, True, False):
+        before = host.fake_rows_written()
+        assert layer.call(PIPED) == 0
+        direct.append(host.fake_rows_written() > before)
+        if drain:
+            layer.drain()
+    assert direct == [True, False, False, True, False, True, True]
+    assert host.fake_races() == 0
+    layer.close()
