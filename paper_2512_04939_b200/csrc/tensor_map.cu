@@ -21,8 +21,12 @@ static bool resolve(const char* name, void** fn) {
 bool resolve_encode_tiled(void** fn) { return resolve("cuTensorMapEncodeTiled", fn); }
 
 bool allocation_of(const void* device_ptr, const uint8_t** begin, size_t* bytes) {
-  void* fn = nullptr;
-  if (!resolve("cuPointerGetAttribute", &fn)) return false;
+  static std::atomic<void*> resolved{nullptr};
+  void* fn = resolved.load(std::memory_order_acquire);
+  if (fn == nullptr) {
+    if (!resolve("cuPointerGetAttribute", &fn)) return false;
+    resolved.store(fn, std::memory_order_release);
+  }
   auto attribute = reinterpret_cast<PFN_cuPointerGetAttribute_v4000>(fn);
   const CUdeviceptr p = reinterpret_cast<CUdeviceptr>(device_ptr);
   CUdeviceptr start = 0;
