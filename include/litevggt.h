@@ -314,7 +314,8 @@ litevggt_status litevggt_selftest_bounded_wait(litevggt_ctx* ctx, int64_t limit_
  * took no time: which = 0 grad map, 1 var map, 2 partition + token lists, 3 cosine
  * matching (pack + GEMM/argmax), 4 selection + index build, 5 merge, 6 qkv projection,
  * 7 attention core, 8 output projection, 9 unmerge, 10 LayerNorm, 11 frame-local attention layer,
- * 12 MLP, 13 Q/K normalisation + rotary embedding, 14 E4M3 quantisation of Q/K/V.
+ * 12 MLP, 13 Q/K normalisation + rotary embedding, 14 E4M3 quantisation of Q/K/V.  Where a layer leaves for host
+ * memory as it is finished, 7, 8 and 9 take turns; a record is the sum of a layer's turns.
  * litevggt_timers_reset forgets all
  * records; litevggt_timer_read synchronises the device and returns the summed
  * device time (ms) and the number of records (at most 64 are kept per step). */

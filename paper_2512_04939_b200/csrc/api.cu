@@ -273,17 +273,26 @@ static litevggt_status read_stamps(litevggt_ctx* ctx, int which, float (&ms)[kTi
   DeviceGuard g(ctx->device);
   if (!g.ok) return LITEVGGT_ERR_CUDA;
   unsigned long long t[kTimerSlots][2];
+  unsigned long long p[kAttnCounters][2];
   cudaError_t e = cudaDeviceSynchronize();
   if (e == cudaSuccess)
     e = cudaMemcpy(t, ctx->timers.stamps + 2 * kTimerSlots * which, sizeof(t), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_status(e);
-  for (int i = 0; i < *kept; ++i) {
-    const int slot = (used - *kept + i) % kTimerSlots;
-    const unsigned long long* r = t[slot];
-    // a step without kernels took no time
-    ms[i] = !ctx->timers.empty[which][slot] && r[1] > r[0] ? (float)((double)(r[1] - r[0]) * 1e-6) : 0.0f;
+  auto span = [](const unsigned long long (&r)[2]) { return r[1] > r[0] ? (double)(r[1] - r[0]) * 1e-6 : 0.0; };
+  for (int i = 0; i < *kept && e == cudaSuccess; ++i) {
+    const int slot = (used - *kept + i) % kTimerSlots, pieces = ctx->timers.in_pieces[which][slot];
+    double time = 0.0;
+    if (ctx->timers.empty[which][slot]) {
+      // a step without kernels took no time
+    } else if (pieces == 0) {
+      time = span(t[slot]);
+    } else {
+      e = cudaMemcpy(p, ctx->timers.pieces + 2 * kAttnCounters * ((which - kFirstInPieces) * kTimerSlots + slot), sizeof(p[0]) * pieces,
+                     cudaMemcpyDeviceToHost);
+      for (int k = 0; k < pieces; ++k) time += span(p[k]);
+    }
+    ms[i] = (float)time;
   }
-  return LITEVGGT_OK;
+  return cuda_status(e);
 }
 
 litevggt_status litevggt_timer_read(litevggt_ctx* ctx, int which, float* total_ms, int32_t* count) {

@@ -41,6 +41,31 @@ struct StepTimer {
   ~StepTimer() {
     ctx->step = Stamp{};
     ctx->timers.empty[which][slot] = launches == before || e != cudaSuccess;
+    ctx->timers.in_pieces[which][slot] = 0;
+    ++ctx->timers.used[which];
+  }
+};
+
+// The same for a step that is launched in pieces, with other steps between them.  One record; empty unless all went well.
+struct PieceTimer {
+  litevggt_ctx* ctx;
+  const int which, slot;
+  int pieces = 0;
+  const cudaError_t& e;
+  PieceTimer(litevggt_ctx* c, int w, const cudaError_t& err) : ctx(c), which(w), slot(c->timers.used[w] % kTimerSlots), e(err) {}
+  template <class Launch>
+  cudaError_t piece(const Launch& launch) {
+    unsigned long long* stamps = ctx->timers.pieces + 2 * (((which - kFirstInPieces) * kTimerSlots + slot) * kAttnCounters + pieces++);
+    ctx->step.start = stamps;
+    ctx->step.stop = stamps + 1;
+    const cudaError_t result = launch();
+    ctx->step = Stamp{};
+    return result;
+  }
+  ~PieceTimer() {
+    if (pieces == 0) return;  // as a step that was not come to
+    ctx->timers.empty[which][slot] = e != cudaSuccess;
+    ctx->timers.in_pieces[which][slot] = pieces;
     ++ctx->timers.used[which];
   }
 };

@@ -34,7 +34,8 @@ litevggt_status ensure_host_pipe(litevggt_ctx* ctx) {
   const size_t big = (size_t)round_up(z.n_tokens * z.dim * 2, 256);
   const size_t index = (size_t)(round_up(4 * z.n_tokens, 256) + 2 * round_up(4 * z.n_merged, 256) +
                                 round_up(4 * (z.n_merged + 1), 256) + round_up(4 * (z.n_remove + 1), 256));
-  if (cudaMalloc(&hp.base, 2 * (2 * big + index)) != cudaSuccess) {
+  const size_t stamps = sizeof(unsigned long long) * 2 * kStepsInPieces * kTimerSlots * kAttnCounters;
+  if (cudaMalloc(&hp.base, 2 * (2 * big + index) + stamps) != cudaSuccess) {
     (void)cudaGetLastError();
     hp.base = nullptr;
     return LITEVGGT_ERR_ALLOC;
@@ -47,6 +48,8 @@ litevggt_status ensure_host_pipe(litevggt_ctx* ctx) {
   cudaEvent_t* sets[4] = {hp.in_ready, hp.x_free, hp.out_ready, hp.out_free};
   for (int k = 0; k < 4 && e == cudaSuccess; ++k)
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&sets[k][i], cudaEventDisableTiming);
+  unsigned long long* pieces = reinterpret_cast<unsigned long long*>(hp.base + 2 * (2 * big + index));
+  if (e == cudaSuccess) e = cudaMemsetAsync(pieces, 0, stamps, hp.copy_in);  // ahead of the input that all else waits for
   if (e != cudaSuccess) {
     // partial set-up is released at destroy time only if `created`; release it here instead
     if (hp.copy_in) cudaStreamDestroy(hp.copy_in);
@@ -64,7 +67,8 @@ litevggt_status ensure_host_pipe(litevggt_ctx* ctx) {
     hp.out[i] = reinterpret_cast<__nv_bfloat16*>(slot + big);
     hp.index[i] = reinterpret_cast<int*>(slot + 2 * big);
   }
-  ctx->ws.bytes += 2 * (2 * big + index);
+  ctx->timers.pieces = pieces;
+  ctx->ws.bytes += 2 * (2 * big + index) + stamps;
   hp.created = true;
   return LITEVGGT_OK;
 }
@@ -108,23 +112,22 @@ cudaError_t layer_in_slabs(litevggt_ctx* ctx, const litevggt_plan* plan, int slo
   if (e == cudaSuccess) e = cudaMemcpyAsync(hp.index[slot], plan->dst_of, index_bytes, cudaMemcpyDeviceToDevice, s);
   auto copied = [&](const int* array) { return hp.index[slot] + (array - plan->dst_of); };
   __nv_bfloat16* ym = hp.out[slot];  // (the staged output is not needed: M <= N rows of it hold the merged ones)
+  PieceTimer attention(ctx, 7, e), projection(ctx, 8, e), unmerge(ctx, 9, e);
   for (long long row0 = 0, row1; row0 < m && e == cudaSuccess; row0 = row1) {
     row1 = attention_slab_end(m, row0, ctx->num_sms, z.heads);
-    {
-      StepTimer t(ctx, 7, n, e);
-      e = launch_flash_attention_rows(ctx, ws.qkv, m, row0, row1, ws.attn_o, s, &n);
-    }
-    if (e == cudaSuccess) {
-      StepTimer t(ctx, 8, n, e);
-      e = launch_linear(ctx, ws.attn_o + row0 * d, row1 - row0, d, static_cast<const __nv_bfloat16*>(w_o), d,
-                        static_cast<const __nv_bfloat16*>(b_o), row1 == m ? kmax_words(ctx, 1) : ZeroWords{}, ym + row0 * d, s, &n);
-    }
+    e = attention.piece([&] { return launch_flash_attention_rows(ctx, ws.qkv, m, row0, row1, ws.attn_o, s, &n); });
+    if (e == cudaSuccess)
+      e = projection.piece([&] {
+        return launch_linear(ctx, ws.attn_o + row0 * d, row1 - row0, d, static_cast<const __nv_bfloat16*>(w_o), d,
+                             static_cast<const __nv_bfloat16*>(b_o), row1 == m ? kmax_words(ctx, 1) : ZeroWords{}, ym + row0 * d, s, &n);
+      });
     if (e == cudaSuccess) e = cudaEventRecord(hp.out_ready[slot], s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(hp.copy_out, hp.out_ready[slot], 0);
     if (e == cudaSuccess) {
-      StepTimer t(ctx, 9, n, e);
-      e = launch_unmerge_rows(ctx, copied(plan->dst_of), copied(plan->kept_idx), copied(plan->seg_off), copied(plan->seg_src), ym,
-                              hp.x[slot], out, row0, row1, hp.copy_out, &n);
+      e = unmerge.piece([&] {
+        return launch_unmerge_rows(ctx, copied(plan->dst_of), copied(plan->kept_idx), copied(plan->seg_off), copied(plan->seg_src), ym,
+                                   hp.x[slot], out, row0, row1, hp.copy_out, &n);
+      });
       *started = true;
     }
   }

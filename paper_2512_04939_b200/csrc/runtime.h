@@ -107,10 +107,15 @@ struct Stamp {
 // and went, by the device's own clock, kept in a small ring per step.
 constexpr int kNumTimers = 15;
 constexpr int kTimerSlots = 64;
+constexpr int kFirstInPieces = 7, kStepsInPieces = 3;  // attention core, output projection, unmerge
 struct Timers {
   unsigned long long* stamps = nullptr;  // device [kNumTimers][kTimerSlots]{start, stop}, in the workspace
   int used[kNumTimers] = {};             // launches recorded since the last reset
   bool empty[kNumTimers][kTimerSlots] = {};  // the record's step launched nothing (or failed): its stamps are an older one's
+  // A layer that leaves in slabs takes the steps from kFirstInPieces on in turns: stamps of every piece, of which a record
+  // is the sum.
+  unsigned long long* pieces = nullptr;  // device [kStepsInPieces][kTimerSlots][kAttnCounters]{start, stop}, with the host pipeline
+  int in_pieces[kNumTimers][kTimerSlots] = {};  // pieces of a record, 0: it has stamps of its own
 };
 }  // namespace lv
 

@@ -131,3 +131,32 @@ def test_in_a_stream_of_calls_copies_take_the_output(host):
     assert direct == [True, False, False, True, False, True, True]
     assert host.fake_races() == 0
     layer.close()
+
+
+def test_one_stopwatch_record_per_layer_and_step(host):
+    """4,122 rows in two slabs: attention, output projection and unmerge are launched once for each, 500 ns by the stand-ins'
+    clock, and leave one record of both, also when the ring has come round and where whole layers' records come between."""
+    layer = Layer(host)
+
+    def samples(which):
+        one, count = (C.c_float * 64)(), C.c_int32()
+        assert host.litevggt_timer_samples(layer.h, which, one, 64, C.byref(count)) == 0
+        return [round(v * 1e6) for v in one[:count.value]]
+
+    for call in range(3):
+        assert layer.call(PIPED) == 0  # in slabs
+        if call == 1:
+            assert layer.call(ORDERED) == 0
+        layer.drain()
+    for which in (7, 8, 9):
+        assert samples(which) == [1000, 1000, 500, 1000]
+    x, out = layer.buffer(2048 * layer.n), layer.buffer(2048 * layer.n)
+    for _ in range(70):
+        assert host.litevggt_global_layer_host_pipelined(layer.h, C.byref(layer.plan), None, x, *[layer.p] * 4, out, None) == 0
+        layer.drain()
+    for which in (7, 8, 9):
+        assert samples(which) == [1000] * 64
+    host.fake_fail_linear(1)
+    assert layer.call(PIPED) != 0
+    assert samples(7) == [1000] * 63 + [0] and samples(8) == [1000] * 63 + [0] and samples(9) == [1000] * 64
+    layer.close()
