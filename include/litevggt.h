@@ -293,7 +293,8 @@ litevggt_status litevggt_plan_destroy(litevggt_plan* plan);
 litevggt_status litevggt_debug_buffer(litevggt_ctx* ctx, int which, void** dev_ptr, size_t* bytes);
 
 /* Synchronise `stream` and report whether any kernel flagged a bounded-wait timeout or
- * an out-of-range index since the last poll (the flag is cleared). */
+ * an out-of-range index since the last poll (the flag is cleared).  Kernels that a pipelined call has writing to its
+ * out_host are waited for, copies are not. */
 litevggt_status litevggt_poll_device_status(litevggt_ctx* ctx, void* stream);
 
 /* Self-test of the bounded waits (the paper has no counterpart; Sec. 3.4's kernels are this

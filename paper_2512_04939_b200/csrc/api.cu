@@ -812,7 +812,10 @@ litevggt_status litevggt_poll_device_status(litevggt_ctx* ctx, void* stream) {
   if (!ctx_ok(ctx)) return LITEVGGT_ERR_NULL;
   cudaStream_t s = (cudaStream_t)stream;
   uint32_t word = 0;
-  cudaError_t e = cudaMemcpyAsync(&word, ctx->ws.status, sizeof(word), cudaMemcpyDeviceToHost, s);
+  cudaError_t e = cudaSuccess;
+  for (int slot = 0; slot < 2 && e == cudaSuccess; ++slot)  // the kernels of a call that are not on its stream
+    if (ctx->pipe.in_slabs[slot]) e = cudaStreamWaitEvent(s, ctx->pipe.x_free[slot], 0);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&word, ctx->ws.status, sizeof(word), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ws.status, 0, sizeof(word), s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_status(e);

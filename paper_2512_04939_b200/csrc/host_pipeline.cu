@@ -186,7 +186,7 @@ litevggt_status litevggt_global_layer_host_pipelined(litevggt_ctx* ctx, litevggt
       cudaError_t done = cudaEventRecord(hp.x_free[slot], hp.copy_out);
       if (done == cudaSuccess) done = cudaEventRecord(hp.out_free[slot], hp.copy_out);
       if (done == cudaSuccess) {
-        hp.used[slot] = true;
+        hp.used[slot] = hp.in_slabs[slot] = true;
         ++hp.calls;
       }
       if (e == cudaSuccess) e = done;
@@ -208,6 +208,7 @@ litevggt_status litevggt_global_layer_host_pipelined(litevggt_ctx* ctx, litevggt
   if (e == cudaSuccess) e = cudaEventRecord(hp.out_free[slot], hp.copy_out);
   if (e == cudaSuccess) {
     hp.used[slot] = true;
+    hp.in_slabs[slot] = false;
     ++hp.calls;
   }
   return cuda_status(e);

@@ -125,6 +125,7 @@ struct HostPipe {
   cudaStream_t copy_in = nullptr, copy_out = nullptr;
   cudaEvent_t in_ready[2] = {}, x_free[2] = {}, out_ready[2] = {}, out_free[2] = {};
   bool used[2] = {false, false};
+  bool in_slabs[2] = {false, false};            // the slot's last output was written by kernels on copy_out, until x_free
   bool drained = true;                          // nothing has been called since the last drain
   unsigned long long calls = 0;
   __nv_bfloat16* x[2] = {nullptr, nullptr};    // [N, D] each

@@ -205,7 +205,7 @@ cudaError_t launch_unmerge_rows(const litevggt_ctx* c, const int* dst_of, const 
   const Sizes& z = c->sz;
   ++g_rows_written;
   touch(s, {rows(ym + row0 * 1024, row1 - row0), rows(res, z.n_tokens), {dst_of, 4 * z.n_tokens}, {kept, 4 * z.n_merged}, {off, 4 * (z.n_merged + 1)},
-            {src, 4 * z.n_remove}}, {rows(out, z.n_tokens)});
+            {src, 4 * z.n_remove}}, {rows(out, z.n_tokens), {c->ws.status, 4}});  // (its bounds checks)
   return ran(c, n);
 }
 cudaError_t launch_linear_scaled(litevggt_ctx* c, const __nv_bfloat16* a, long long m, long long, const __nv_bfloat16*, long long,

@@ -160,3 +160,14 @@ def test_one_stopwatch_record_per_layer_and_step(host):
     assert layer.call(PIPED) != 0
     assert samples(7) == [1000] * 63 + [0] and samples(8) == [1000] * 63 + [0] and samples(9) == [1000] * 64
     layer.close()
+
+
+def test_a_poll_sees_what_the_writers_of_an_output_have_flagged(host):
+    """The kernels that write an output check their indices on a stream of the context's own; a poll comes after them
+    without a drain.  (An unordered read of the status word would count as a race.)"""
+    layer = Layer(host)
+    for _ in range(2):
+        assert layer.call(PIPED) == 0
+        assert host.litevggt_poll_device_status(layer.h, None) == 0
+    assert host.fake_races() == 0
+    layer.close()
