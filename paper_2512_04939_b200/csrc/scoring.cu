@@ -561,7 +561,10 @@ __device__ __forceinline__ unsigned score_key(float v) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-__global__ void __launch_bounds__(kPartThreads)
+// kRanked: frames of at most kRankPatches patches.  Larger ones come in numbers, and a third CTA on an SM is worth
+// more than registers: 1000 frames of 28 x 37 take 44 us, 51 with the 58 registers that both kinds of frames had in one kernel.
+template <bool kRanked>
+__global__ void __launch_bounds__(kPartThreads, kRanked ? 1 : 3)
 partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, float* __restrict__ ga,
                  uint8_t* cls, int grid_h, int grid_w, int n_special, int n_ga, int cell_h, int cell_w,
                  float alpha, float beta, const ListArgs lists, Stamp stamp) {
@@ -620,7 +623,7 @@ partition_kernel(const float* __restrict__ grad, const float* __restrict__ var, 
   // Up to kRankPatches patches: two threads count how many of the others beat one, three barriers where the search below
   // takes sixteen (four frames of 16 x 16: 6.1 us for the whole kernel, 7.1 with the search and a reduction each
   // for the two minima and maxima).
-  if (p_count <= kRankPatches) {
+  if constexpr (kRanked) {
     unsigned* key = reinterpret_cast<unsigned*>(score);  // in their scores' place; 0, below every key, for who takes no part
     const int p = threadIdx.x >> 1, part = threadIdx.x & 1;
     float sp = 0.0f;
@@ -735,8 +738,9 @@ cudaError_t launch_partition(const litevggt_ctx* ctx, const float* grad, const f
   const Sizes& z = ctx->sz;
   const size_t smem = (size_t)z.patches * (sizeof(float) + 1) + 16;  // at most 41 KB (8192 patches)
   ++*launches;
-  return launch(partition_kernel, dim3(z.frames), kPartThreads, smem, s, grad, var, ga, cls, z.grid_h, z.grid_w, z.n_special,
-                z.n_ga_frame, (int)ctx->cfg.cell_h, (int)ctx->cfg.cell_w, ctx->cfg.alpha, ctx->cfg.beta, list_args(ctx), next_stamp(ctx));
+  return launch(z.patches <= kRankPatches ? partition_kernel<true> : partition_kernel<false>, dim3(z.frames), kPartThreads, smem, s,
+                grad, var, ga, cls, z.grid_h, z.grid_w, z.n_special, z.n_ga_frame, (int)ctx->cfg.cell_h, (int)ctx->cfg.cell_w,
+                ctx->cfg.alpha, ctx->cfg.beta, list_args(ctx), next_stamp(ctx));
 }
 
 constexpr int kListThreads = 256;
