@@ -95,7 +95,7 @@
 // fixed form.  Trained projections attend that sharply (query weights x 16 on the generator's tokens:
 // B up to 213): 31,751 rows went from 4.81 to 4.41 ms there.
 // What remains takes the online form: base-2 softmax with a lazily updated reference
-// maximum, the running output rescaled only when a row maximum grows by more than 2^8 over the
+// maximum, the running output rescaled only when a row maximum grows far over the
 // reference (the threads then first wait until the tile's last P V has retired).  All three equal
 // the plain softmax up to rounding.
 #include <type_traits>
@@ -110,11 +110,13 @@ constexpr int kFaThreads = (kFaSoftmaxWarps + 3) * 32;
 constexpr int kFaTileBytes = kFaTileKeys * 64 * 2;
 constexpr int kFaOnesBytes = 16 * 128;  // 16 key rows of the ones column block
 constexpr uint32_t kFaOCols = 80;  // 64 output channels, the row sum, 15 unused columns
-// How far a row maximum may grow over the reference of the online form before the row is rescaled (a warp rescales when one of
-// its 32 rows has to).  Low enough that parts of a row can be weighed against each other, see part_weight; 32 measured
-// the same time.
-constexpr float kFaRescaleThreshold = 8.0f;
-static_assert(126.0f + kFaRescaleThreshold < 149.0f, "part_weight reaches down to 2^-149");
+// The online form's reference is set kFaAhead over the maximum found so far and serves until the row maximum lies more than
+// kFaRescaleThreshold over it; then the row is rescaled, and its warp with it, which waits for the tensor core and reads
+// and writes its output.  Sums over 2^22 keys times |v| <= 2^20 stay below 2^82; keys more than 126 - 32 under the maximum
+// are lost, 2^-72 of the row at most.  (Layer of 31,751 rows at query weights x 64, all of them online: 5.30 ms with the
+// reference at the maximum and rescaling beyond 2^8, 5.23 beyond 2^22, 5.13 with the reference 16 ahead, 4.95 as it stands.)
+constexpr float kFaRescaleThreshold = 40.0f;
+constexpr float kFaAhead = 32.0f;
 // Largest Cauchy-Schwarz bound B on the base-2 scores of a row for which the fixed reference is
 // used.  With the reference left out the probabilities lie in [2^-B, 2^B]: at B = 80 their products
 // with |v| >= 2^-20 are normal fp32 numbers (>= 2^-100), and a row sum over 2^20 keys times
@@ -205,6 +207,7 @@ template <int kTiles>
 struct FaPairs {
   float first_max[kTiles][2][128];
   float row_max[2][kTiles][2][128];  // of either half of a key tile
+  uint32_t left[kTiles][2][4];       // [tile][warp of the pair][quarter]: has given up and gone
 };
 // What differs between the CTA of two query tiles (one CTA per SM) and that of one (two per SM).
 template <int kTiles>
@@ -227,14 +230,8 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
-// What a part of a row counts for beside another whose reference is the higher one by -x: below 2^-126 too, where fast_exp2
-// gives zero.  A part in the online form may hold 2^kFaRescaleThreshold a key, one in the shifted form only
-// 2^-fa_shift_down in all, so what the lower one holds is lost to the row's 24 bits only beyond 2^-(126 + kFaRescaleThreshold).
-__device__ __forceinline__ float part_weight(float x) {
-  float y;
-  asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
+// 2^d for a whole number d <= 0, exact; zero under 2^-126.
+__device__ __forceinline__ float exp2_whole(float d) { return __uint_as_float((uint32_t)((int)fmaxf(d, -127.0f) + 127) << 23); }
 
 // 2^(x - m) for a pair of arguments on the FMA pipes, `magic` = 1.5 * 2^23 - m with m a whole number.
 // Adding it rounds x to the nearest integer and leaves n = that integer - m in the low mantissa
@@ -344,10 +341,16 @@ __device__ __forceinline__ float max32(const uint32_t (&s)[32]) {
   return fmaxf(fmax3(mx[0], mx[1], mx[2]), mx[3]);
 }
 
-// The two warps of one (tile, lane quarter).  A warp that gives up arrives once more without waiting, so a partner who is at
-// the barrier, or comes to it, passes - and finds the abort flag up before the next one.
+// The two warps of one (tile, lane quarter).  In a job that has such barriers (one, and in the online form one a step) a warp that
+// gives up goes on to meet its partner at all of them, so no step has to ask.  A warp that leaves between jobs says so and
+// arrives without waiting, which lets the partner through the next job's first barrier, behind which it finds out.
 __device__ __forceinline__ void pair_barrier(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
 __device__ __forceinline__ void pair_barrier_leave(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
+
+// (out of line: it runs only where a wait was given up)
+__device__ __noinline__ void meet_partner(int id, int met, int n_steps) {
+  for (; met < n_steps; ++met) pair_barrier(id);
+}
 
 // kFirst / kLast: this launch holds the first / the last key chunk of the sweep.
 // kTiles: query tiles of the CTA.
@@ -417,6 +420,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
     }
     mbar_fence_init();
     bars->abort_flag = 0;
+    for (int i = 0; i < 8 * kTiles; ++i) (&pairs->left[0][0][0])[i] = 0u;
     tma_prefetch_desc(&tmap_qkv);
   }
   // The row sums come out of the second MMA: its B operand is 80 columns wide, V's 64 channels and,
@@ -448,8 +452,9 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
     if constexpr (kJobs) {
       ok = one_lane ? mbar_wait(&bars->job_full[turn & 1u], turn >> 1 & 1u, ctl) : mbar_wait_warp(&bars->job_full[turn & 1u], turn >> 1 & 1u, ctl);
       if (!ok) return id_end;
-      const int id = *reinterpret_cast<volatile int*>(&bars->job[turn & 1u]);
-      if (!one_lane) __syncwarp();
+      int id = *reinterpret_cast<volatile int*>(&bars->job[turn & 1u]);
+      // (from one lane, so that the compiler knows it to be the same in all and a job's loops not to diverge)
+      if (!one_lane) id = __shfl_sync(0xffffffffu, id, 0);
       if (one_lane || lane == 0) mbar_arrive(&bars->job_empty[turn & 1u]);
       return id;
     } else {
@@ -648,9 +653,6 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       return id;
     };
     const int barrier_id = 1 + t * 4 + (int)quarter;
-    // Asked for in good time before a pair barrier, not behind it: who is passed through by a warp that gave up finds out
-    // before the next one.
-    auto given_up = [&] { return *ctl.abort_flag != 0u; };  // (one read for the whole warp)
     int id = next_job(id0);
     float score_bound = 0.0f;
     if (id < id_end) {
@@ -744,22 +746,24 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         // they are for the sweep): their maximum is a lower bound of the row maximum, score_bound an upper one.
         bool shifted = false;
         ok = scores_of(0, 0);
+        float mx_own = INFINITY;  // of a warp that gives up: sends the partner to the form that keeps meeting it
         if (ok) {
           tc_fence_after();
           uint32_t s[32];
           tmem_ld32(s_addr + c * 32, s);
           tmem_ld_wait();
           masked(s, n_keys - c * 32);
-          const float mx_own = max32(s);
-          ok = !given_up();
-          if (!ok) break;
-          pairs->first_max[t][c][row_in_tile] = mx_own;
-          pair_barrier(barrier_id);
-          const float mx_first = fmaxf(mx_own, pairs->first_max[t][c ^ 1][row_in_tile]);
-          const float m = ceilf(fmaxf(score_bound - shift_up, mx_first));
-          shifted = __all_sync(0xffffffffu, m - mx_first <= shift_down && fabsf(m) <= 1048576.0f ? 1 : 0) != 0;
-          if (shifted) m_ref = m;
+          mx_own = max32(s);
         }
+        pairs->first_max[t][c][row_in_tile] = mx_own;
+        pair_barrier(barrier_id);
+        int met = 0;  // pair barriers of the online form that this warp has been at, where it gives up
+        const volatile uint32_t* partner_left = &pairs->left[t][c ^ 1][quarter];
+        if (__any_sync(0xffffffffu, *partner_left != 0u ? 1 : 0)) break;
+        const float mx_first = fmaxf(mx_own, pairs->first_max[t][c ^ 1][row_in_tile]);
+        const float m = ceilf(fmaxf(score_bound - shift_up, mx_first));
+        shifted = __all_sync(0xffffffffu, m - mx_first <= shift_down && fabsf(m) <= 1048576.0f ? 1 : 0) != 0;
+        if (shifted) m_ref = m;
         if (ok && shifted) {
           // ---- shifted reference, kept for the whole launch: a whole number m (see fa_shift_up) under which
           // nothing overflows and the row's largest probability is not small, so no running maximum is
@@ -772,29 +776,25 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
           // ---- online form.  Both threads of a row share every step, half of its scores each, and tell each other their
           // maxima.
           auto step = [&](int j, int h, bool may_mask) -> bool {
-            if (!scores_of(h, j)) return false;
+            if (!scores_of(h, j)) {
+              met = 2 * j + h;
+              return false;
+            }
             tc_fence_after();
-            const bool gone = given_up();
             const uint32_t addr = s_addr + h * 64 + c * 32;
-            // (the scores are read once for the maximum and once more for the exponentials: the registers that this form
-            // takes are the kernel's)
-            auto load = [&](uint32_t (&s)[32]) {
+            uint32_t s[32], packed[16];
+            auto load = [&] {
               tmem_ld32(addr, s);
               tmem_ld_wait();
               if (may_mask) masked(s, n_keys - (2 * j + h) * 64 - c * 32);
             };
-            float mx_own;
-            {
-              uint32_t s[32];
-              load(s);
-              mx_own = max32(s);
-            }
+            load();
+            const float mx_own = max32(s);
             pairs->row_max[h][t][c][row_in_tile] = mx_own;
-            if (gone) return false;
             pair_barrier(barrier_id);
             const float mx = fmaxf(mx_own, pairs->row_max[h][t][c ^ 1][row_in_tile]);
             if ((j | h) == 0) {
-              m_ref = mx;
+              m_ref = ceilf(mx) + kFaAhead;  // whole numbers, like the other forms'
             } else {
               const bool grow = mx > m_ref + kFaRescaleThreshold;
               if (__any_sync(0xffffffffu, grow ? 1 : 0)) {
@@ -803,10 +803,13 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
                 // has retired; where nothing follows (the job's last step), pv_done does.
                 const bool waited = 2 * j + h + 1 < n_steps ? scores_of(h ^ 1, j + h)
                                                             : mbar_wait_warp(&bars->pv_done[t], (turn >> 2) & 1u, ctl);
-                if (!waited) return false;
+                if (!waited) {
+                  met = 2 * j + h + 1;
+                  return false;
+                }
                 tc_fence_after();
-                const float m_new = grow ? mx : m_ref;
-                const float alpha = fast_exp2(m_ref - m_new);
+                const float m_new = grow ? ceilf(mx) + kFaAhead : m_ref;
+                const float alpha = exp2_whole(m_ref - m_new);
                 m_ref = m_new;
                 uint32_t acc[32], sum;  // this thread's 32 of the row's 64 output channels; one of the two has the row sum too
                 tmem_ld32(o_addr, acc);
@@ -816,10 +819,9 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
                 for (int i = 0; i < 32; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * alpha);
                 tmem_st32(o_addr, acc);
                 if (c == 1) tmem_st1(o_row + 64, __float_as_uint(__uint_as_float(sum) * alpha));
+                load();  // again: held beside the output they would spill
               }
             }
-            uint32_t s[32], packed[16];
-            load(s);
             exp2_chunk_shifted<0>(s, m_ref, packed);
             tmem_st16(addr, packed);  // over the start of the columns just read
             give_p(h, 1);
@@ -828,6 +830,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
           for (int j = 0; j < last && ok; ++j) ok = step(j, 0, false) && step(j, 1, false);
           if (ok) ok = step(last, 0, true) && (2 * last + 1 == n_steps || step(last, 1, true));
         }
+        if (!ok && !shifted) meet_partner(barrier_id, met, n_steps);
       }
       if (!ok) break;
       // The next job's queries are on their way while the tensor cores finish this one; they take the old ones' place,
@@ -850,6 +853,16 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       __syncwarp();
       if (kJobs && lane == 0) mbar_arrive(&bars->o_free[t]);
       const FaJob job = job_at(id);
+      // A part of a row leaves with its sum between 1 and 2 and the reference that goes with it: references chosen for a
+      // launch lie up to a hundred binades over or under what a part holds, which would be lost beside another part.
+      if (!(kFirst && kLast) || job.slot >= 0) {
+        const uint32_t e = min(max(sum >> 23 & 255u, 1u), 253u);
+        const float scale = __uint_as_float((254u - e) << 23);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * scale);
+        sum = __float_as_uint(__uint_as_float(sum) * scale);
+        m_ref += (float)((int)e - 127);
+      }
       const int row = job.seq * seq_len + row_of(job);  // global row of qkv / o
       if (row_of(job) < seq_len) {
         if (job.slot >= 0) {
@@ -860,14 +873,13 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
           float* ml_mine = ml_state + ((size_t)row * (dim / 64) + job.head) * 4 + 2 * c;
           if (!first_chunk) {
             // add what the earlier chunks left for this row, in fp32 with round-to-nearest: partial
-            // output, row sum, and - online form - their reference (the fixed form's is the same in
-            // every launch, bit for bit)
+            // output, row sum and their reference; the weights are powers of two
             const float m_old = ml_mine[0], l_old = ml_mine[1];
             float a_old = 1.0f, a_new = 1.0f;
             if (m_old != m_ref) {
               const float m_tot = fmaxf(m_old, m_ref);
-              a_old = part_weight(m_old - m_tot);
-              a_new = part_weight(m_ref - m_tot);
+              a_old = exp2_whole(m_old - m_tot);
+              a_new = exp2_whole(m_ref - m_tot);
               m_ref = m_tot;
             }
             const uint4* src = reinterpret_cast<const uint4*>(o_state + (size_t)row * dim + job.head * 64 + c * 32);
@@ -907,7 +919,10 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       turn ^= ((steps + 1) >> 1 & 1u) | (steps & 2u) | 4u;
       id = next_id;
     }
-    if (__any_sync(0xffffffffu, *ctl.abort_flag != 0u ? 1 : 0)) pair_barrier_leave(barrier_id);
+    if (__any_sync(0xffffffffu, *ctl.abort_flag != 0u ? 1 : 0)) {
+      *const_cast<volatile uint32_t*>(&pairs->left[t][c][quarter]) = 1u;
+      pair_barrier_leave(barrier_id);
+    }
   }
 
   tc_fence_before();
@@ -1254,8 +1269,8 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
           float a_old = 1.0f, a_new = 1.0f;
           if (m_old != m_ref) {
             const float m_tot = fmaxf(m_old, m_ref);
-            a_old = part_weight(m_old - m_tot);
-            a_new = part_weight(m_ref - m_tot);
+            a_old = fast_exp2(m_old - m_tot);
+            a_new = fast_exp2(m_ref - m_tot);
             m_ref = m_tot;
           }
           const uint4* src = reinterpret_cast<const uint4*>(o_state + (size_t)row * dim + head * 64 + c * 32);
@@ -1317,7 +1332,8 @@ combine_parts_kernel(FaJobs split, __nv_bfloat16* __restrict__ o, int seq_len, i
   for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
   for (int p = 0; p < split.parts; ++p) {
     const float2 ml = *reinterpret_cast<const float2*>(split.ml + ((slot0 + p) * 256 + r) * 2);
-    const float w = ml.x == m ? 1.0f : part_weight(ml.x - m);
+    // (the E4M3 form's references are no whole numbers)
+    const float d = ml.x - m, w = ml.x == m ? 1.0f : d == rintf(d) ? exp2_whole(d) : fast_exp2(d);
     sum = fmaf(ml.y, w, sum);
     const float4* src = reinterpret_cast<const float4*>(split.o + ((slot0 + p) * 256 + r) * 64 + ch);
     const float4 a = src[0], b = src[1];

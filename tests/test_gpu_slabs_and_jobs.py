@@ -69,16 +69,17 @@ def test_sequences_of_several_rounds_of_jobs(lib, frames, grid, sharpness):
 
 @pytest.mark.parametrize("frames,many,top,bound", [(2, 3900, 63.0, 243.0), (17, 30000, 66.0, 239.0)])
 def test_parts_of_a_row_under_references_far_apart(lib, frames, many, top, bound):
-    """8,192 rows, where some jobs are split in two along the keys, and 69,632 in two key chunks.  The first half scores 20 in
-    its first 64 keys, so that the running maximum has to serve, and 51 in `many` later ones; the second half's first key scores
-    `top` and one reference, 130 over the first half's, serves it.  The first half holds about a third of every row, the only part with
+    """8,192 rows, where some jobs are split in two along the keys, and 69,632 in two key chunks.  The first half scores -18 in
+    its first 64 keys, so that the running maximum has to serve, and 51 in `many` later ones, which is not beyond what a
+    reference near the first maximum takes; the second half's first key scores `top` and one reference over 130 binades higher
+    serves it.  The first half holds about half of every row, the only part with
     V = 1.  Scores are equal within a half, so an output is off by the rounding of two probabilities and its own: 3 x 2^-9 of it."""
     ctx = lib.LiteVGGT(frames, 64, 64, 0.0, n_special=0)
     rows = ctx.n_merged
     half = rows // 2
     x, w_qkv, b_qkv, w_o, b_o = (torch.zeros(*s, dtype=torch.bfloat16) for s in ((rows, 1024), (3072, 1024), (3072,), (1024, 1024), (1024,)))
     score = torch.full((rows,), -50.0)
-    score[0], score[64:64 + many], score[half] = 20.0, 51.0, top
+    score[0], score[64:64 + many], score[half] = -18.0, 51.0, top
     x[:, 0] = score / 16 / K_FOLD
     x[5, 1] = (bound ** 2 - 50.0 ** 2) ** 0.5 / 16 / K_FOLD  # a long key, across the queries but for its score of -50
     x[64:64 + many, 2] = 1.0
