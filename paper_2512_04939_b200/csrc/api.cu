@@ -193,7 +193,7 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
   size_t ml_off = 0;
   const size_t state_bytes = attention_state_bytes(z.n_merged, z.dim, z.heads, ctx->num_sms, &ml_off);
   const size_t o_state = c.take<uint8_t>((long long)state_bytes);
-  const size_t o_kmax = c.take<float>((long long)z.frames * z.heads);
+  const size_t o_kmax = c.take<float>((long long)z.frames * 2 * z.heads);
   const bool fp8 = cfg->qkv_dtype == 1;
   const long long m_pad = round_up(z.n_merged, 128);
   const size_t o_q8 = c.take<uint8_t>(fp8 ? z.n_merged * z.dim : 0), o_k8 = c.take<uint8_t>(fp8 ? z.n_merged * z.dim : 0);
@@ -242,7 +242,7 @@ litevggt_status litevggt_create(const litevggt_config* cfg, int device, litevggt
   cudaError_t e = cudaStreamCreateWithFlags(&clear, cudaStreamNonBlocking);
   if (e == cudaSuccess) {
     e = cudaMemsetAsync(ws.base + o_var, 0, o_src - o_var, clear);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ws.attn_kmax, 0, sizeof(float) * (size_t)z.frames * z.heads, clear);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws.attn_kmax, 0, sizeof(float) * (size_t)z.frames * 2 * z.heads, clear);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->timers.stamps, 0, o_taken - o_stamps, clear);
     if (e == cudaSuccess) e = cudaMemsetAsync(ws.status, 0, 16, clear);
     if (e == cudaSuccess) e = cudaStreamSynchronize(clear);
@@ -526,7 +526,8 @@ litevggt_status litevggt_global_attn_ext(litevggt_ctx* ctx, const litevggt_plan*
     e = launch_linear_scaled(ctx, static_cast<const __nv_bfloat16*>(x_merged), m, d,
                              static_cast<const __nv_bfloat16*>(w_qkv), 3 * d, static_cast<const __nv_bfloat16*>(b_qkv), d,
                              2 * d, embeds ? 1.0f : kKeyScaleLog2e,  // (the Q/K pass scales K itself, when there is one)
-                             embeds ? LinearStat{} : core_stat(ctx, m), ctx->ws.qkv, s, &n);
+                             !embeds ? core_stat(ctx, m) : fp8 ? LinearStat{} : LinearStat{ctx->ws.attn_kmax, m, nullptr, true},
+                             ctx->ws.qkv, s, &n);
   }
   if (e == cudaSuccess) {
     StepTimer t(ctx, 13, n, e);

@@ -139,20 +139,23 @@ constexpr int kFaPolyPairs = LV_FA_POLY_PAIRS;
 #define LV_FA_SHIFT_POLY_PAIRS 2
 #endif
 constexpr int kFaShiftPolyPairs = LV_FA_SHIFT_POLY_PAIRS;
-// Shifted reference m of a row with score bound B and a known score s0, both limits by the sequence's length.  B - m <=
-// fa_shift_up(keys): row sums over that many keys, times |v| <= 2^20, stay below 2^126.  m - s0 <= fa_shift_down(keys): what
-// lies more than 126 under m is off by up to 2^-126 a key (flushed to zero by the special-function unit, held up at
-// 2^-126 by the polynomial's clamp), the row's largest probability is at least 2^-fa_shift_down, so all such keys
-// together are off by 2^-24 of the row's mass at most - no more than one fp32 rounding of the row sum.  (With 84 up, the
-// limit of 2^22 keys, at every length, a seventh of the 256-row tiles of 31,751 rows at query weights x 16 had a row in
-// the online form, a tenth with 91: 4.53 -> 4.49 ms.)
+// Shifted reference m of a row with score bound B and a known score s0, both limits by the sequence's length (its binary
+// logarithm, rounded up).  B - m <= fa_shift_up: row sums over that many keys, times the head's largest |v| where that is over
+// 2^20, stay below 2^126.  m - s0 <= fa_shift_down: what lies more than 126 under m is off by up to 2^-126 a key (flushed
+// to zero by the special-function unit, held up at 2^-126 by the polynomial's clamp), the row's largest probability
+// is at least 2^-fa_shift_down, so all such keys together are off by 2^-24 of the row's mass at most - no more than one
+// fp32 rounding of the row sum.  (With 84 up, the limit of 2^22 keys and |v| <= 2^20, at every length, a seventh of the
+// 256-row tiles of 31,751 rows at query weights x 16 had a row in the online form, a tenth with 91: 4.53 -> 4.49 ms.)
 static float key_bits(long long keys) {
   int bits = 0;
   while ((1ll << bits) < keys) ++bits;
   return (float)bits;
 }
-static float fa_shift_up(long long keys) { return 126.0f - 20.0f - key_bits(keys); }
-static float fa_shift_down(long long keys) { return 126.0f - 24.0f - key_bits(keys); }
+__device__ __forceinline__ float fa_shift_up(float bits, float v_max) {
+  const int v_bits = (int)(__float_as_uint(v_max) >> 23) - 126;  // |v| < 2^v_bits; 129 where it is infinite
+  return 126.0f - bits - fmaxf((float)v_bits, 20.0f);
+}
+__device__ __forceinline__ float fa_shift_down(float bits) { return 126.0f - 24.0f - bits; }
 
 // The jobs of a launch, one query block of one head of one sequence each, query blocks fastest.  Those that the last
 // round would leave alone on the chip are split along the keys: ids from `full` on are (job, part) with
@@ -358,7 +361,7 @@ template <int kTiles, bool kFirst, bool kLast>
 __global__ void __launch_bounds__(FaShape<kTiles>::kThreads, kTiles == 2 ? 1 : 2)
 flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_bfloat16* __restrict__ qkv,
                        __nv_bfloat16* __restrict__ o, float* __restrict__ o_state, float* __restrict__ ml_state,
-                       const float* __restrict__ k_norm2_max, float shift_up, float shift_down, int seq_len, int dim, int tile_begin,
+                       const float* __restrict__ kv_max, float key_bits, int seq_len, int dim, int tile_begin,
                        int tile_end, FaJobs jobs, uint32_t* status, Stamp stamp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -632,7 +635,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         for (int i = 0; i < 4; ++i) other = square(__ldg(src + 4 * (c ^ 1) + i), other);
       }
       const float q_norm2 = own + other;
-      return sqrtf(q_norm2 * k_norm2_max[job.seq * (dim / 64) + job.head]);
+      return sqrtf(q_norm2 * kv_max[job.seq * 2 * (dim / 64) + job.head]);
     };
     auto hand_q = [&](const uint32_t (&qreg)[16]) {
       tmem_st16(tmem_base + lane_base + Shape::kColQ + t * 32 + c * 16, qreg);
@@ -761,8 +764,10 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         const volatile uint32_t* partner_left = &pairs->left[t][c ^ 1][quarter];
         if (__any_sync(0xffffffffu, *partner_left != 0u ? 1 : 0)) break;
         const float mx_first = fmaxf(mx_own, pairs->first_max[t][c ^ 1][row_in_tile]);
-        const float m = ceilf(fmaxf(score_bound - shift_up, mx_first));
-        shifted = __all_sync(0xffffffffu, m - mx_first <= shift_down && fabsf(m) <= 1048576.0f ? 1 : 0) != 0;
+        const FaJob job = job_at(id);
+        const float v_max = kv_max[(job.seq * 2 + 1) * (dim / 64) + job.head];
+        const float m = ceilf(fmaxf(score_bound - fa_shift_up(key_bits, v_max), mx_first));
+        shifted = __all_sync(0xffffffffu, m - mx_first <= fa_shift_down(key_bits) && fabsf(m) <= 1048576.0f ? 1 : 0) != 0;
         if (shifted) m_ref = m;
         if (ok && shifted) {
           // ---- shifted reference, kept for the whole launch: a whole number m (see fa_shift_up) under which
@@ -1448,7 +1453,7 @@ static cudaError_t launch_rows(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long
   CUtensorMap tmap;
   if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap, qkv, (uint64_t)3 * dim, (uint64_t)rows, (uint64_t)3 * dim, 64, kFaTileKeys))
     return cudaErrorInvalidValue;
-  using Kernel = void (*)(const CUtensorMap, const __nv_bfloat16*, __nv_bfloat16*, float*, float*, const float*, float, float, int,
+  using Kernel = void (*)(const CUtensorMap, const __nv_bfloat16*, __nv_bfloat16*, float*, float*, const float*, float, int,
                           int, int, int, FaJobs, uint32_t*, Stamp);
   // [query tiles of a CTA - 1][first chunk][last chunk]
   const Kernel kernels[2][2][2] = {
@@ -1484,7 +1489,7 @@ static cudaError_t launch_rows(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long
                                               smem_set[a][b][c]);
     if (e != cudaSuccess) return e;
     e = launch_clusters(1, early, kernels[a][b][c], grid, threads, smem, s, tmap, qkv, o, ctx->ws.attn_o_state, ctx->ws.attn_ml_state,
-               ctx->ws.attn_kmax, fa_shift_up(seq_len), fa_shift_down(seq_len), (int)seq_len, dim, begin, end, split, ctx->ws.status, next_stamp(ctx));
+               ctx->ws.attn_kmax, key_bits(seq_len), (int)seq_len, dim, begin, end, split, ctx->ws.status, next_stamp(ctx));
     if (e != cudaSuccess) return e;
     ++*launches;
     ++split.taken;

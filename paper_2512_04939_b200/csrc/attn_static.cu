@@ -22,7 +22,7 @@ constexpr size_t kStatusBytes = 256;
 constexpr size_t kQkvBytes = (size_t)kStaticMaxRows * 3 * kStaticDim * 2;
 constexpr size_t kOBytes = (size_t)kStaticMaxRows * kStaticDim * 2;
 
-// [ status word, 16 floats of per-head key norms at byte 64, padding | qkv bf16 [1024, 3072] |
+// [ status word, 16 floats of per-head key norms and 16 of value magnitudes at byte 64, padding | qkv bf16 [1024, 3072] |
 //   o bf16 [1024, 1024] ]  = 8 MiB + 256 B
 static __device__ __align__(256) unsigned char g_attn_scratch[kStatusBytes + kQkvBytes + kOBytes];
 
@@ -99,7 +99,7 @@ extern "C" litevggt_status litevggt_global_attn_static(const void* x_merged, int
     (void)cudaGetLastError();
     return LITEVGGT_ERR_CUDA;
   }
-  if (dev->norms_left.load() && cudaMemsetAsync(dev->scratch + 64, 0, kStaticHeads * sizeof(float), s) != cudaSuccess) {
+  if (dev->norms_left.load() && cudaMemsetAsync(dev->scratch + 64, 0, 2 * kStaticHeads * sizeof(float), s) != cudaSuccess) {
     (void)cudaGetLastError();
     return LITEVGGT_ERR_CUDA;
   }
@@ -122,7 +122,7 @@ extern "C" litevggt_status litevggt_global_attn_static(const void* x_merged, int
   if (e == cudaSuccess)
     e = lv::launch_linear(&local, o, m, kStaticDim, static_cast<const __nv_bfloat16*>(w_o), kStaticDim,
                           static_cast<const __nv_bfloat16*>(b_o),
-                          lv::ZeroWords{reinterpret_cast<uint32_t*>(local.ws.attn_kmax), kStaticHeads},
+                          lv::ZeroWords{reinterpret_cast<uint32_t*>(local.ws.attn_kmax), 2 * kStaticHeads},
                           static_cast<__nv_bfloat16*>(y_merged), s, &n);
   if (e != cudaSuccess) {
     (void)cudaGetLastError();

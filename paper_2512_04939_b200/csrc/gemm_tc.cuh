@@ -388,7 +388,7 @@ inline long long gemm_cost(long long waves, int bn, long long k, bool pair) {
 // head of one tensor): a pass over the matrix of its own cost 19 us (key norms, 22 K rows) to 66 us
 // (208 K rows, 200 sequences), and 184 us for the magnitudes of 22 K rows, whose atomics met on 48 words.
 // Here a warp reduces its 32 rows and sends one atomic per sequence that they touch.
-enum : int { kStatNone = 0, kStatKeyNorm = 1, kStatAmax = 2 };
+enum : int { kStatNone = 0, kStatKeyNorm = 1, kStatValues = 2, kStatAmax = 3 };
 
 // Epilogue: out[row, col] = bf16(acc + bias[col])
 struct LinearEpilogue {
@@ -399,38 +399,48 @@ struct LinearEpilogue {
   int n_cols;
   int scale_begin, scale_end;  // output columns [scale_begin, scale_end) are multiplied by `scale`
   float scale;
-  // kStatKeyNorm: stat[seq * heads + head] = largest |row|^2 over the head's 64 columns, for the columns
-  //               [scale_begin, scale_end) and sequences of seq_len rows;
+  // kStatKeyNorm: stat[seq][0][head] = largest |row|^2 over the head's 64 columns, for the columns [scale_begin, scale_end)
+  //               (K) and sequences of seq_len rows, stat[seq][1][head] = largest magnitude of as many columns behind them (V);
+  // kStatValues: the magnitudes only;
   // kStatAmax:    stat[col / 64] = largest magnitude of those 64 columns.  Both start at zero.
   int stat_kind;
   int seq_len;
   float* stat;
 
+  __device__ __forceinline__ static float largest(const uint32_t (&packed)[32]) {
+    float a = 0.0f;  // fmaxf drops a NaN
+#pragma unroll
+    for (int i = 0; i < 32; ++i) a = fmaxf(a, fmaxf(fabsf(bf16_lo(packed[i])), fabsf(bf16_hi(packed[i]))));
+    return a;
+  }
   // 64 accumulator columns of one row -> 32 bf16 pairs
   __device__ __forceinline__ void transform(int row, int col0, const uint32_t (&acc)[64], uint32_t (&packed)[32]) const {
     convert(col0, acc, packed);
     if (stat_kind == kStatAmax) {
-      float a = 0.0f;  // fmaxf drops a NaN
-#pragma unroll
-      for (int i = 0; i < 32; ++i) a = fmaxf(a, fmaxf(fabsf(bf16_lo(packed[i])), fabsf(bf16_hi(packed[i]))));
-      const uint32_t best = __reduce_max_sync(0xffffffffu, row < m_rows ? __float_as_uint(a) : 0u);
+      const uint32_t best = __reduce_max_sync(0xffffffffu, row < m_rows ? __float_as_uint(largest(packed)) : 0u);
       if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned int*>(stat) + col0 / 64, best);
-    } else if (stat_kind == kStatKeyNorm && col0 >= scale_begin && col0 < scale_end) {
-      float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    } else if (stat_kind != kStatNone && col0 >= (stat_kind == kStatValues ? scale_end : scale_begin) && col0 < 2 * scale_end - scale_begin) {
+      const bool is_v = col0 >= scale_end;
+      float what;  // (NaN counts as 0)
+      if (is_v) {
+        what = largest(packed);
+      } else {
+        float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        sum[i & 3] = fmaf(bf16_lo(packed[i]), bf16_lo(packed[i]), sum[i & 3]);
-        sum[i & 3] = fmaf(bf16_hi(packed[i]), bf16_hi(packed[i]), sum[i & 3]);
+        for (int i = 0; i < 32; ++i) {
+          sum[i & 3] = fmaf(bf16_lo(packed[i]), bf16_lo(packed[i]), sum[i & 3]);
+          sum[i & 3] = fmaf(bf16_hi(packed[i]), bf16_hi(packed[i]), sum[i & 3]);
+        }
+        what = fmaxf(0.0f, (sum[0] + sum[1]) + (sum[2] + sum[3]));
       }
-      const float norm2 = fmaxf(0.0f, (sum[0] + sum[1]) + (sum[2] + sum[3]));  // NaN counts as 0
       // non-negative floats order like their bit patterns; the warp's first row is live (see the caller)
       const int row0 = row - (int)(threadIdx.x & 31);
       const int mine = row < m_rows ? row / seq_len : -1;
       const int last = (row0 + 31 < m_rows ? row0 + 31 : m_rows - 1) / seq_len;
-      const int heads = (scale_end - scale_begin) / 64, head = (col0 - scale_begin) / 64;
+      const int heads = (scale_end - scale_begin) / 64, at = (col0 - scale_begin) / 64;  // K's heads, then V's
       for (int seq = row0 / seq_len; seq <= last; ++seq) {
-        const uint32_t best = __reduce_max_sync(0xffffffffu, mine == seq ? __float_as_uint(norm2) : 0u);
-        if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned int*>(stat) + seq * heads + head, best);
+        const uint32_t best = __reduce_max_sync(0xffffffffu, mine == seq ? __float_as_uint(what) : 0u);
+        if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned int*>(stat) + seq * 2 * heads + at, best);
       }
     }
   }

@@ -97,15 +97,15 @@ inline litevggt_status ensure_merged_staging(litevggt_ctx* ctx) {
   return ensure_row_pair(ctx, ctx->sz.n_merged, &ctx->ws.stage_xm, &ctx->ws.stage_ym);
 }
 
-// The key norms of `sequences` sequences, which an output projection leaves zero for the next layer.
+// The key norms and value magnitudes of `sequences` sequences, which an output projection leaves zero for the next layer.
 inline ZeroWords kmax_words(const litevggt_ctx* ctx, long long sequences) {
-  return ZeroWords{reinterpret_cast<uint32_t*>(ctx->ws.attn_kmax), sequences * ctx->sz.heads};
+  return ZeroWords{reinterpret_cast<uint32_t*>(ctx->ws.attn_kmax), sequences * 2 * ctx->sz.heads};
 }
 
 // Before a call raises the key norms: they are zero unless an earlier call failed half-way.
 inline cudaError_t begin_norms(litevggt_ctx* ctx, cudaStream_t s) {
   if (ctx->norms_left) {
-    const cudaError_t e = cudaMemsetAsync(ctx->ws.attn_kmax, 0, sizeof(float) * (size_t)ctx->sz.frames * ctx->sz.heads, s);
+    const cudaError_t e = cudaMemsetAsync(ctx->ws.attn_kmax, 0, sizeof(float) * (size_t)ctx->sz.frames * 2 * ctx->sz.heads, s);
     if (e != cudaSuccess) return e;
   }
   ctx->norms_left = true;  // until the output projection is enqueued

@@ -81,7 +81,7 @@ cudaError_t launch_linear_scaled(litevggt_ctx* ctx, const __nv_bfloat16* a, long
   epi.scale_begin = scale_begin;
   epi.scale_end = scale_end;
   epi.scale = scale;
-  epi.stat_kind = stat.key_norm != nullptr ? kStatKeyNorm : stat.amax != nullptr ? kStatAmax : kStatNone;
+  epi.stat_kind = stat.key_norm != nullptr ? (stat.values_only ? kStatValues : kStatKeyNorm) : stat.amax != nullptr ? kStatAmax : kStatNone;
   epi.seq_len = (int)stat.seq_len;
   epi.stat = stat.key_norm != nullptr ? stat.key_norm : stat.amax;
   // (a context without counters runs attention launches that need none)

@@ -77,7 +77,7 @@ struct Workspace {
   float* attn_o_state = nullptr;   // [M, D] running output between key chunks (long sequences), or split parts
   float* attn_ml_state = nullptr;  // [M, heads, 4] references and partial row sums, or those of the parts
   int* attn_taken = nullptr;       // [kAttnCounters] jobs taken by an attention launch's CTAs; every Q/K/V projection zeroes them
-  float* attn_kmax = nullptr;      // [max(frames, 1), heads] largest |k|^2 per sequence and head
+  float* attn_kmax = nullptr;      // [max(frames, 1), 2, heads] largest |k|^2 and largest |v| per sequence and head
   // E4M3 variant of the attention operands (qkv_dtype = 1)
   uint8_t* q8 = nullptr;           // [M, D] bytes
   uint8_t* k8 = nullptr;           // [M, D] bytes
@@ -273,9 +273,10 @@ cudaError_t launch_linear(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m
 // of the rounded output.  Zeroing the key norms takes no launch: they are zero between calls, because
 // the output projection, which runs after their last reader, leaves them so.
 struct LinearStat {
-  float* key_norm = nullptr;  // [sequences, heads] largest |k|^2 over the columns [scale_begin, scale_end) ...
+  float* key_norm = nullptr;  // [sequences, 2, heads] largest |k|^2 over the columns [scale_begin, scale_end) and largest |v| ...
   long long seq_len = 0;      // ... of sequences of this many rows
   float* amax = nullptr;      // [n / 64] largest magnitude of every 64 columns, zeroed here first
+  bool values_only = false;   // of key_norm only |v|: a later pass rounds K
 };
 cudaError_t launch_linear_scaled(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k,
                                  const __nv_bfloat16* w, long long n, const __nv_bfloat16* bias, int scale_begin,
@@ -302,7 +303,7 @@ cudaError_t launch_qk_embed(const litevggt_ctx* ctx, __nv_bfloat16* qkv, const i
                             const __nv_bfloat16* k_beta, float eps, int rope, float rope_base, float* key_norm,
                             cudaStream_t s, int* launches);
 // ctx->ws.attn_kmax holds the largest |k|^2 per sequence and head (left there by whichever pass rounded
-// K last: the projection or qk_embed)
+// K last: the projection or qk_embed) and the largest |v| (by the projection)
 cudaError_t launch_flash_attention(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long long seq_len, int n_seq,
                                    __nv_bfloat16* o, cudaStream_t s, int* launches);
 // The same for a slab of the one sequence's m query rows: rows [row0, row1) with row1 = attention_slab_end(row0).

@@ -211,8 +211,8 @@ cudaError_t launch_unmerge_rows(const litevggt_ctx* c, const int* dst_of, const 
 cudaError_t launch_linear_scaled(litevggt_ctx* c, const __nv_bfloat16* a, long long m, long long, const __nv_bfloat16*, long long,
                                  const __nv_bfloat16*, int, int, float, const LinearStat& st, __nv_bfloat16* out, cudaStream_t s, int* n) {
   touch(s, {rows(a, m)}, {rows(out, 3 * m)});
-  if (st.key_norm != nullptr) {  // raises every norm to 4, as an atomic maximum would
-    const long long words = m / st.seq_len * 16;
+  if (st.key_norm != nullptr) {  // raises every norm and value to 4, as an atomic maximum would
+    const long long words = m / st.seq_len * 2 * 16;
     g_norm_seen = st.key_norm[0];
     g_norm_last_seen = st.key_norm[words - 1];
     for (long long i = 0; i < words; ++i) st.key_norm[i] = st.key_norm[i] > 4.0f ? st.key_norm[i] : 4.0f;

@@ -67,6 +67,38 @@ def test_sequences_of_several_rounds_of_jobs(lib, frames, grid, sharpness):
     ctx.close()
 
 
+@pytest.mark.parametrize("entry", ["global", "normed", "frame"])
+@pytest.mark.parametrize("value", [2.0 ** 20, 2.0 ** 26, 2.0 ** 100])
+def test_large_values_under_a_shifted_reference(lib, entry, value):
+    """All keys but the first 64 score what the bound allows, 120, the first ones -45: one reference near the upper limit serves,
+    unless the sum over 4,096 or 16,384 keys of 2^(120 - m) times V would not be finite.  All V are equal, so that is what
+    every output is."""
+    ctx = lib.LiteVGGT(4, 64, 64, 0.0, n_special=0)
+    rows = ctx.n_merged
+    x, w_qkv, b_qkv = (torch.zeros(*s, dtype=torch.bfloat16) for s in ((rows, 1024), (3072, 1024), (3072,)))
+    u = torch.tensor([1.0, -1.0] * 32)
+    first = u.clone()
+    first[:44] *= -1.0  # 12 of 32 pairs more that point the other way than along
+    x[:, :64], x[:, 64] = u, value
+    x.view(4, -1, 1024)[:, :64, :64] = first
+    scale = 10.375  # times 64 / 8 log2 e = 119.7
+    for h in range(16):
+        w_qkv[1024 + 64 * h + torch.arange(64), torch.arange(64)] = 1.0
+        w_qkv[2048 + 64 * h, 64] = 1.0
+        b_qkv[64 * h:64 * h + 64] = u if entry == "normed" else scale * u
+    eye, one, zero = torch.eye(1024, dtype=torch.bfloat16), torch.ones(64, dtype=torch.bfloat16), torch.zeros(64, dtype=torch.bfloat16)
+    dev = [t.cuda() for t in (x, w_qkv, b_qkv, eye)]
+    if entry == "frame":
+        out = ctx.frame_attn(*dev, None)
+    elif entry == "global":
+        out = ctx.global_attn(*dev, None)
+    else:
+        out = ctx.global_attn_ext(None, *dev, None, q_norm=((scale * one).cuda(), zero.cuda()), k_norm=(one.cuda(), zero.cuda()))
+    ctx.poll()
+    assert (out[:, ::64].float() == value).all()
+    ctx.close()
+
+
 @pytest.mark.parametrize("frames,many,top,bound", [(2, 3900, 63.0, 243.0), (17, 30000, 66.0, 239.0)])
 def test_parts_of_a_row_under_references_far_apart(lib, frames, many, top, bound):
     """8,192 rows, where some jobs are split in two along the keys, and 69,632 in two key chunks.  The first half scores -18 in
