@@ -8,8 +8,8 @@
 // attention: 3.72 -> 2.66 to 2.83 ms a pass.  What bounds it now is PCIe, both ways at once (the next call's input comes in
 // meanwhile), at 45 GB/s out.  The first slab is one round of the attention's CTAs, so that PCIe starts early, the
 // others two, which lose 3 % of a round at their end.  Output buffers that the device cannot write (pageable memory, odd
-// addresses), E4M3 contexts, sequences of up to 4096 rows and those of several key chunks, whose copies are
-// 6 % of a pass or less, take the copy behind the layer.  So does a call with no drain since the one before: in a stream
+// addresses), E4M3 contexts, sequences of up to 4096 rows and some little longer ones (attn_slabs.h) and those of several key
+// chunks, whose copies are 6 % of a pass or less, take the copy behind the layer.  So does a call with no drain since the one before: in a stream
 // of calls a copy engine moves an output at 55 GB/s under the next call's kernels and takes nothing from them, while the
 // writers do (40 calls in a row and a drain, ms a call: 16 frames of 37 x 37 1.00 by copies, 1.20 in slabs, 32 frames 2.14
 // and 2.55, 44 frames 3.9 and 4.4; a call and its drain 2.22 and 1.98, 5.2 and 4.1, 7.9 and 6.3).  What a call does
@@ -172,7 +172,7 @@ litevggt_status litevggt_global_layer_host_pipelined(litevggt_ctx* ctx, litevggt
   const litevggt_plan* plan = *plan_inout;
   st = litevggt_merge(ctx, plan, hp.x[slot], ws.stage_xm, stream);
   // In a stream of calls the copy of one hides behind the kernels of the next.
-  const bool apart = hp.drained && ctx->cfg.qkv_dtype == 0 && attention_slab_end(z.n_merged, 0, ctx->num_sms, z.heads) < z.n_merged;
+  const bool apart = hp.drained && ctx->cfg.qkv_dtype == 0 && attention_slabs_pay(z.n_merged, z.n_tokens, ctx->num_sms, z.heads);
   hp.drained = false;
   void* direct = st == LITEVGGT_OK && apart ? device_view(out_host, bytes) : nullptr;
   if (direct != nullptr) {

@@ -171,3 +171,13 @@ def test_a_poll_sees_what_the_writers_of_an_output_have_flagged(host):
         assert host.litevggt_poll_device_status(layer.h, None) == 0
     assert host.fake_races() == 0
     layer.close()
+
+
+@pytest.mark.parametrize("frames,ratio,direct", [(3, 0.0, True), (5, 0.3, True), (7, 0.55, False), (6, 0.47, False), (3, 0.01, False)])
+def test_short_sequences_of_many_tokens_leave_by_a_copy(host, frames, ratio, direct):
+    """4,122 rows of as many tokens, 4,809 of 6,870 | 4,386 of 9,618, 4,370 of 8,244, 4,081 of 4,122."""
+    layer = Layer(host, ratio, frames)
+    before = host.fake_rows_written()
+    assert layer.call(PIPED) == 0
+    assert (host.fake_rows_written() > before) == direct
+    layer.close()
