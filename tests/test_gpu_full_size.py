@@ -11,7 +11,7 @@ import torch
 import oracle as O
 from synthdata import (WORKLOADS, make_attention_weights, make_block_weights, make_images,
                        make_peaked_attention_inputs, make_tokens)
-from test_gpu_parity import FIXED_REF_LIMIT, SHIFT_UP, shift_down
+from test_gpu_parity import FIXED_REF_LIMIT, shift_down, shift_up
 from helpers import CORE_NOISE, K_FOLD, LAYER_NOISE, bf16_bound, check_bf16, fold_k, rel_err, report, to_f64
 
 pytestmark = pytest.mark.gpu
@@ -230,7 +230,7 @@ def chunk_forms(qkv_h, starts):
     forms = []
     for s in starts:
         first = (q @ k[s:s + 64].T).max(1)
-        shifted = np.logical_and.reduceat(np.ceil(np.maximum(bound - SHIFT_UP, first)) - first <= shift_down(m), warps)
+        shifted = np.logical_and.reduceat(np.ceil(np.maximum(bound - shift_up(m), first)) - first <= shift_down(m), warps)
         forms.append(np.where(fixed, 0, np.where(shifted, 1, 2)))
     return np.stack(forms)
 

@@ -384,7 +384,10 @@ def score_bounds(qkv, heads=16):
 
 
 FIXED_REF_LIMIT = 80.0  # the library's kFaFixedRefLimit
-SHIFT_UP = 84.0  # its kFaShiftUp
+
+
+def shift_up(rows):  # its fa_shift_up, for values below 2^20
+    return 126 - 20 - int(np.ceil(np.log2(rows)))
 
 
 def shift_down(rows):  # and its fa_shift_down
@@ -475,7 +478,7 @@ def softmax_forms(qkv, heads=16, limit=FIXED_REF_LIMIT):
     for h in range(heads):
         q, k = qkv[:, h * 64:h * 64 + 64], qkv[:, d + h * 64:d + h * 64 + 64]
         first = (q @ k[:64].T).max(1)
-        shift = np.ceil(np.maximum(b[:, h] - SHIFT_UP, first)) - first <= shift_down(m)
+        shift = np.ceil(np.maximum(b[:, h] - shift_up(m), first)) - first <= shift_down(m)
         for w in range(0, m, 32):
             if (b[w:w + 32, h] <= limit).all():
                 form = "fixed"
@@ -604,13 +607,13 @@ def test_a_key_that_is_not_a_number_shows_in_every_output(lib, rows, qkv_dtype, 
 
 @pytest.mark.parametrize("above", [87.0, 90.5])
 def test_shifted_reference_loses_nothing_that_fp32_would_keep(lib, above):
-    """Keys 0 and 1 score 0, the highest; key 1 is long, across the queries, so that the score bound lies 84 +
+    """Keys 0 and 1 score 0, the highest; key 1 is long, across the queries, so that the score bound lies 92 +
     `above` over it: at 87 one reference serves (16,384 rows: up to 88 binades over the highest score),
     at 90.5 the running maximum has to.  The other keys sit 40 binades down with V = 1 where keys 0 and 1 have V = 0,
     so the output is what they hold together, 2^-26, and an error of 2^-24 of the row's mass is allowed."""
     rows = 16384
     ctx, (x, w_qkv, b_qkv, w_o, b_o) = uniform_rows_ctx(lib, rows)
-    x[2:, 0], x[1, 1], x[2:, 2] = -40.0 / 16 / K_FOLD, (84 + above) / 16 / K_FOLD, 1.0
+    x[2:, 0], x[1, 1], x[2:, 2] = -40.0 / 16 / K_FOLD, (92 + above) / 16 / K_FOLD, 1.0
     for h in range(16):
         b_qkv[64 * h] = 16.0
         w_qkv[1024 + 64 * h, 0] = w_qkv[1024 + 64 * h + 1, 1] = w_qkv[2048 + 64 * h, 2] = 1.0
@@ -620,7 +623,7 @@ def test_shifted_reference_loses_nothing_that_fp32_would_keep(lib, above):
     assert set(softmax_forms(qkv)) == {"shifted" if above < 88 else "online"}
     ref = O.attention_core(unfold_k(qkv), heads=16, rows=np.arange(4))[:, ::64]
     got = to_f64(ctx.debug_buffer(1))[:, ::64]
-    report(f"keys 40 binades down, bound {84 + above} up", got=float(got.max()), ref=float(ref.max()))
+    report(f"keys 40 binades down, bound {92 + above} up", got=float(got.max()), ref=float(ref.max()))
     assert ref.min() > 2.0 ** -28 and np.abs(got - ref[0]).max() <= 2.0 ** -24
     ctx.close()
 

@@ -209,7 +209,7 @@ def test_host_entries_in_turn_without_a_drain(lib):
 @pytest.mark.parametrize("grid,keep", [((1, 1), 0.1), ((16, 16), 0.1), ((16, 16), 0.9), ((4, 64), 0.5), ((7, 37), 0.1), ((6, 43), 0.3)])
 def test_ranks_of_a_small_frames_scores(lib, grid, keep):
     """Frames of 1, 256, 258 and 259 patches: up to 256 every patch is ranked against the others, above a search finds
-    the threshold.  Scores in few steps, so that ties decide, and frames whose scores are not numbers."""
+    the threshold.  Scores in few steps, so that ties decide."""
     ctx = lib.LiteVGGT(4, grid[0], grid[1], 0.3, ga_keep_frac=keep)
     g = torch.Generator().manual_seed(grid[0] * 100 + grid[1])
     x = torch.randn(13, 1024, generator=g)[torch.randint(0, 13, (ctx.n_tokens,), generator=g)].to(torch.bfloat16)
