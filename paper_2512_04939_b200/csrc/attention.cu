@@ -28,8 +28,8 @@
 // next: a launch is one such CTA per SM, and each works off jobs (256 rows of one head) until they run out.  The
 // K/V ring goes on from job to job; the next job's queries are fetched while the tensor cores finish this one's last
 // step, take the old ones' place as soon as they have, and the next scores are under way before this job's rows are
-// written.  52,050 rows 10.8 -> 10.5 ms, 251,872 rows 241 -> 237 (of which the power cap takes part back); 31,751 rows
-// at fixed reference 3.85 -> 3.78.  Jobs come off a counter, late in the job before: with a fixed stride, or taken a whole
+// written.  Whole layers: 4,386 rows 153 -> 148 us, 15,932 rows 1.15 -> 1.09 ms, 31,751 rows 3.64 -> 3.60; from 83 K rows on, at
+// the power cap, nothing (251,872 rows 241.9 -> 243.4).  Jobs come off a counter, late in the job before: with a fixed stride, or taken a whole
 // job ahead, rows in the online form left 3 % of 31,751 rows' time to a few CTAs at the end.  With one tile, two
 // CTAs an SM run under each other anyway, and jobs measured 3 % slower.
 // Tensor memory (512 columns allocated, 480 used):

@@ -35,7 +35,7 @@ inline long long attention_slab_end(long long m, long long row0, int num_sms, in
 // to (m - first) m, has to hide what is slower about it, in proportion to n (the writers at 45 GB/s, a copy at 55).
 // Calls and drains in a row, ms in slabs / by a copy, by (m - first) m / n: 949 (7 frames of 37 x 37, 4,386 rows) 0.61 /
 // 0.57, 1066 0.58 / 0.54, 1149 0.68 / 0.67 (on another machine 0.64 / 0.67), 1405 0.46 / 0.44 (0.45 / 0.45), 1457 0.41 /
-// 0.42, 1753 0.44 / 0.48, 1818 0.29 / 0.34, 2106 0.78 / 0.84, 15932 rows 2.30 / 2.83.
+// 0.42, 1753 0.44 / 0.48, 1538 0.78 / 0.84, 1818 0.29 / 0.34, 10538 (15,932 rows) 2.30 / 2.83.
 inline bool attention_slabs_pay(long long m, long long n, int num_sms, int heads) {
   const long long first = attention_slab_end(m, 0, num_sms, heads);
   return first < m && (m - first) * m >= 1400 * n;

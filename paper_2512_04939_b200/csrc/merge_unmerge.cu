@@ -130,7 +130,7 @@ unmerge_kernel(const __nv_bfloat16* __restrict__ ym, const int* __restrict__ dst
 }
 
 // The unmerge of merged rows [row0, row1) only: to their own tokens and to the src tokens of their segments, into memory that
-// may be the host's.  PCIe bounds it (2 KB a token at about 50 GB/s), so few warps do; what matters is that they are all
+// may be the host's.  PCIe bounds it (2 KB a token at 45 GB/s by these stores), so few warps do; what matters is that they are all
 // busy to the end (a token each, not a row: some anchors stand for hundreds) and how they get on with the attention
 // beside them.  Its CTA leaves 1024 registers of every scheduler free: one block of four warps on 32 registers, a warp
 // half a token at a time.  Where stores queue up for PCIe the attention's warps on that SM wait behind them, so
