@@ -128,6 +128,15 @@ def test_parts_of_a_row_under_references_far_apart(lib, frames, many, top, bound
     ctx.close()
 
 
+def _check_up_to_rounding(name, got, ref, x):
+    got, ref = got.float(), ref.float()
+    gap = (got - ref).abs()
+    # a bf16 unit of either value, and of the attention output before the residual was added
+    unit = 2.0 ** -7 * torch.maximum(ref.abs(), (ref - x.float()).abs())
+    assert bool((gap <= 2 * unit + 1e-3).all()), f"{name}: {gap.max()}"
+    assert float((gap != 0).float().mean()) < 0.2
+
+
 @pytest.mark.parametrize("frames,grid,ratio", [
     (3, (37, 37), 0.0),    # 4,122 rows: the fewest that leave in slabs, two of them
     (5, (37, 37), 0.3),    # a second slab of two rounds, not full
@@ -161,12 +170,7 @@ def test_output_that_leaves_in_slabs(lib, frames, grid, ratio):
         ctx.host_drain()
         ctx.poll()
         for i, k in enumerate(order):
-            got, ref = outs[k].float(), expected[i].float()
-            gap = (got - ref).abs()
-            # a bf16 unit of either value, and of the attention output before the residual was added
-            unit = 2.0 ** -7 * torch.maximum(ref.abs(), (ref - xs[i].float()).abs())
-            assert bool((gap <= 2 * unit + 1e-3).all()), f"call {i}: {gap.max()}"
-            assert float((gap != 0).float().mean()) < 0.2
+            _check_up_to_rounding(f"call {i}", outs[k], expected[i], xs[i])
     plan.destroy()
     ctx.close()
 
@@ -193,6 +197,8 @@ def test_host_entries_in_turn_without_a_drain(lib):
             ctx.poll()
         alone.append((launches, outs))
     assert alone[0][0] > alone[1][0] and not torch.equal(alone[0][1][0], alone[1][1][0])  # slabs, and a whole
+    for i, (a, b) in enumerate(zip(alone[0][1], alone[1][1])):  # out of either of the two buffers
+        _check_up_to_rounding(f"call {i} and its drain", a, b, xs[i])
     for order in ((0, 1, 0, 1, 1, 0), (1, 0, 0, 1, 0, 0)):
         outs = [torch.zeros_like(x).pin_memory() for x in xs]
         for k, x, out in zip(order, xs, outs):
