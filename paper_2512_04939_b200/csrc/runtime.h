@@ -70,7 +70,7 @@ struct Workspace {
   unsigned long long* match_keys = nullptr;  // [|Src|] best (cosine, anchor) so far, as one ordered word
   // index build
   int* src_pos = nullptr;        // [N] a token's index in src_list, -1 for tokens of the other classes
-  int* index_scratch = nullptr;  // histograms, counts and the merged tokens on their way (index_build.cu)
+  int* index_scratch = nullptr;  // keys, counts and the merged tokens on their way (index_build.cu)
   // attention
   __nv_bfloat16* qkv = nullptr;    // [M, 3D]
   __nv_bfloat16* attn_o = nullptr; // [M, D]
@@ -249,8 +249,6 @@ cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, cudaStream_t
 // index_build.cu
 cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStream_t s, int* launches);
 long long index_scratch_words(const Sizes& z);
-// the part of the scratch array that has to be zero before launch_index_build; the matching sees to it
-ZeroWords index_zero_words(const litevggt_ctx* ctx);
 
 // merge_unmerge.cu
 cudaError_t launch_merge(const litevggt_ctx* ctx, const litevggt_plan* plan, const __nv_bfloat16* x,

@@ -177,6 +177,44 @@ def test_index_build_bit_exact_given_same_matches(lib, wl):
     ctx.close()
 
 
+@pytest.mark.parametrize("frames,grid,ratio,cell,kind", [
+    (38, (16, 16), 0.3, 2, "random"),   # one block: 204,720 of its 204,800 bytes, five chunks of tokens
+    (7, (19, 25), 0.45, 2, "tied"),     # ties at the threshold, one block
+    (35, (16, 16), 0.45, 2, "tied"),    # 204,992 bytes: the smallest cluster; ties across its blocks
+    (31, (28, 37), 0.3, 2, "random"),   # 32,271 tokens: the largest
+    (31, (28, 37), 0.0, 2, "random"),   # nothing merged
+    (14, (37, 37), 0.5, 16, "equal"),   # one segment of 9,618 tokens
+    (24, (37, 37), 0.3, 2, "tied"),     # 32,976 tokens: the smallest as launches
+    (24, (37, 37), 1.0, 2, "random"),   # every src token merged
+    (24, (37, 37), 0.0, 2, "random"),
+    (30, (37, 37), 0.5, 16, "equal")])  # one segment of 20,610 tokens
+def test_index_arrays_at_the_limits_of_their_forms(lib, frames, grid, ratio, cell, kind):
+    """Numbers and sizes against the oracle's on the library's own matches; segments by a merge, whose sums show their order."""
+    ctx = lib.LiteVGGT(frames, grid[0], grid[1], ratio, cell_h=cell, cell_w=cell)
+    n = ctx.n_tokens
+    g = torch.Generator().manual_seed(n + frames)
+    if kind == "random":
+        x = torch.randn(n, 1024, generator=g)
+    elif kind == "tied":
+        x = torch.randn(13, 1024, generator=g)[torch.randint(0, 13, (n,), generator=g)]
+    else:  # one direction, so that the first anchor takes all
+        x = torch.ones(n, 1024) * 2.0 ** torch.randint(-3, 4, (n, 1), generator=g)
+    x = x.to(torch.bfloat16).cuda()
+    plan = ctx.merge_plan(x, torch.rand(frames, *grid, generator=g).cuda())
+    ctx.merge_plan(x, torch.rand(frames, *grid, generator=g).cuda(), plan)
+    ctx.poll()
+    ex = ctx.plan_export(plan)
+    dst_of, size, kept = O.select_and_index(ex["cls"], ex["best_dst"], ex["best_sim"], n - ctx.n_merged)
+    assert np.array_equal(ex["dst_of"], dst_of) and np.array_equal(ex["size"], size) and np.array_equal(ex["kept_idx"], kept)
+    rows = x[:, :32].float().cpu().numpy()
+    total, rest = rows[kept], np.setdiff1d(np.arange(n), kept)
+    np.add.at(total, dst_of[rest], rows[rest])  # one after the other, in ascending order
+    want = torch.from_numpy(total / size[:, None].astype(np.float32)).to(torch.bfloat16)
+    assert torch.equal(ctx.merge(plan, x)[:, :32].cpu(), want)
+    plan.destroy()
+    ctx.close()
+
+
 @pytest.mark.parametrize("frames,grid,ratio,cell,keep,kind", [
     (1, (5, 7), 0.5, 2, 0.1, "random"),     # no src token
     (2, (9, 9), 0.3, 2, 0.6, "random"),     # few src tokens, all of them merged
