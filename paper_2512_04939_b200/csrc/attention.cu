@@ -42,8 +42,8 @@
 //              MMA's B operand carries a column of ones next to V, so the tensor core adds up
 //              exactly the bf16 probabilities that it multiplies with V - and 15 unused columns)
 //   [416,480)  Q_0, Q_1 (bf16 pairs, 32 columns each), written once by the softmax threads
-//              straight from global memory: Q is the A operand of the first MMA from tensor
-//              memory, so only K and V tiles travel through shared memory.
+//              (from global memory; with one tile from a TMA load): Q is the A operand of the first MMA from
+//              tensor memory, so the MMAs read only K and V tiles from shared memory.
 // The two halves of a tile double-buffer the scores: while the softmax threads work on
 // half h the tensor core already runs O += P V of the other half and the next Q K^T into
 // it.  The MMAs are issued in order, which is what makes the S/P aliasing safe: Q K^T for
@@ -200,6 +200,7 @@ struct FaBarriers {
   uint64_t v_full[kStages], v_empty[kStages];
   uint64_t q_ready[kTiles], s_full[kTiles][2], p_ready[kTiles][2], pv_done[kTiles], o_done[kTiles], o_free[kTiles];
   uint64_t teardown[kTiles];
+  uint64_t q_full;  // (one tile)
   uint64_t job_full[2], job_empty[2];
   int job[2];  // the CTA's next jobs
   uint32_t tmem_base;
@@ -370,6 +371,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
   constexpr int kStages = Shape::kStages;
   uint8_t* smem_v = smem_k + kStages * kFaTileBytes;
   uint8_t* smem_ones = smem_v + kStages * kFaTileBytes;  // see below
+  uint8_t* smem_q = smem_ones - kFaTileBytes;  // one tile's queries on their way, until V needs its last stage
   FaPairs<kTiles>* pairs = reinterpret_cast<FaPairs<kTiles>*>(smem_ones + kFaOnesBytes);
   FaBarriers<kTiles, kStages>* bars = reinterpret_cast<FaBarriers<kTiles, kStages>*>(pairs + 1);
 
@@ -421,6 +423,8 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       mbar_init(&bars->job_full[i], 1);
       mbar_init(&bars->job_empty[i], Shape::kSoftmaxWarps + kTiles);
     }
+    mbar_fence_init();
+    mbar_init(&bars->q_full, 1);
     mbar_fence_init();
     bars->abort_flag = 0;
     for (int i = 0; i < 8 * kTiles; ++i) (&pairs->left[0][0][0])[i] = 0u;
@@ -476,6 +480,10 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         const FaTiles kv = tiles_at(id);
         int next_id = id_end;
         const int row0 = job.seq * seq_len, col = job.head * 64;
+        if constexpr (!kJobs) {
+          mbar_expect_tx(&bars->q_full, kFaTileBytes);
+          tma_load_2d(smem_q, &tmap_qkv, &bars->q_full, col, row0 + job.q_block * 128);
+        }
         for (int j = kv.begin; j < kv.end; ++j) {
           if (kJobs && j == max(kv.begin, kv.end - 2)) {
             // The next job, to everybody; late, so that it is not kept waiting here while another CTA has nothing to do, and
@@ -491,6 +499,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
           tma_load_2d(smem_k + stage * kFaTileBytes, &tmap_qkv, &bars->k_full[stage], dim + col, row0 + j * kFaTileKeys);
           ++k_issued;
           if (!mbar_wait(&bars->v_empty[stage], phase ^ 1u, ctl)) { ok = false; break; }
+          if (!kJobs && v_issued == kStages - 1 && !mbar_wait(&bars->q_ready[0], 0, ctl)) { ok = false; break; }  // the queries lie there
           mbar_expect_tx(&bars->v_full[stage], kFaTileBytes);
           tma_load_2d(smem_v + stage * kFaTileBytes, &tmap_qkv, &bars->v_full[stage], 2 * dim + col, row0 + j * kFaTileKeys);
           ++v_issued;
@@ -498,6 +507,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         }
         id = next_id;
       }
+      if constexpr (!kJobs) drain_ring<1>(&bars->q_full, 1, status);
       // every load issued by this thread must have landed before the CTA may exit
       drain_ring<kStages>(bars->k_full, k_issued, status);
       drain_ring<kStages>(bars->v_full, v_issued, status);
@@ -637,6 +647,28 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       const float q_norm2 = own + other;
       return sqrtf(q_norm2 * kv_max[job.seq * 2 * (dim / 64) + job.head]);
     };
+    // The same for the CTA of one tile, whose queries come by TMA, where the ring's last V tile will be: loaded row by row
+    // every load of a warp touches 32 lines, 2048 in all, and they were the last to arrive (four frames of 16 x 16, M = 543: layer 32.3 -> 31.7 us;
+    // local half of 100 frames of 20 x 20 969 -> 954, of 200 of 28 x 37 5.18 -> 5.15 ms).  A CTA that goes from job to job
+    // fetches the next ones behind its last steps and has no stage to spare.
+    auto read_q = [&](const FaJob& job, uint32_t (&qreg)[16]) -> float {
+      const float k_norm2 = kv_max[job.seq * 2 * (dim / 64) + job.head];
+      if (!mbar_wait_warp(&bars->q_full, 0, ctl)) return -1.0f;
+      const bool live = row_of(job) < seq_len;
+      float q_norm2 = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {  // in the same order in both threads of a row, so that they find the same bound
+        uint4 v = *reinterpret_cast<const uint4*>(smem_q + row_in_tile * 128 + ((i ^ (row_in_tile & 7)) << 4));
+        if (!live) v = make_uint4(0u, 0u, 0u, 0u);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          q_norm2 = fmaf(bf16_hi(w[e]), bf16_hi(w[e]), fmaf(bf16_lo(w[e]), bf16_lo(w[e]), q_norm2));
+          if (i < 4 || c == 1) qreg[4 * (i & 3) + e] = w[e];
+        }
+      }
+      return sqrtf(q_norm2 * k_norm2);
+    };
     auto hand_q = [&](const uint32_t (&qreg)[16]) {
       tmem_st16(tmem_base + lane_base + Shape::kColQ + t * 32 + c * 16, qreg);
       tmem_st_wait();
@@ -660,8 +692,10 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
     float score_bound = 0.0f;
     if (id < id_end) {
       uint32_t qreg[16];
-      score_bound = load_q(job_at(id), qreg);
-      hand_q(qreg);
+      if constexpr (kJobs) score_bound = load_q(job_at(id), qreg);
+      else score_bound = read_q(job_at(id), qreg);
+      if (score_bound < 0.0f) id = id_end;  // given up
+      else hand_q(qreg);
     }
     while (id < id_end) {
       const FaTiles kv = tiles_at(id);

@@ -67,6 +67,29 @@ def test_sequences_of_several_rounds_of_jobs(lib, frames, grid, sharpness):
     ctx.close()
 
 
+@pytest.mark.parametrize("sharpness", [1.0, 16.0, 64.0])
+@pytest.mark.parametrize("grid", [(1, 2), (2, 61), (12, 21), (19, 20), (16, 31), (25, 41)])
+def test_queries_that_arrive_where_values_will(lib, grid, sharpness):
+    """Frames of 7, 127, 257, 385, 501 and 1030 tokens: one to nine key tiles, whose third takes the place of the queries; last
+    query tiles of 1 to 127 rows, before the next frame's; all three forms, for which both threads of a row find the same bound."""
+    ctx = lib.LiteVGGT(3, grid[0], grid[1], 0.0)
+    n, t = ctx.n_tokens, ctx.n_tokens // 3
+    x = _tokens(n, 7 * grid[0] + grid[1])
+    w_qkv, b_qkv, w_o, b_o = make_attention_weights(WORKLOADS["C1"], 6)
+    w_qkv[:1024] *= sharpness
+    dev = [v.cuda() for v in (w_qkv, b_qkv, w_o, b_o)]
+    ctx.global_attn(x.cuda(), *dev)
+    qkv, core = to_f64(ctx.debug_buffer(0)), to_f64(ctx.debug_buffer(1))
+    out = to_f64(ctx.frame_attn(x.cuda(), dev[0], dev[1], torch.eye(1024, dtype=torch.bfloat16).cuda(), None))
+    ctx.poll()
+    rows = np.unique(np.r_[0:min(n, 40), max(0, n - 70):n])
+    _check_core(f"global core, {n} rows, sharpness {sharpness}", core[rows], qkv, rows)
+    rows = np.unique(np.r_[0:min(t, 20), t // 2, max(0, t - 70):t])
+    for f in range(3):
+        _check_core(f"frame core {f} of 3, {t} rows, sharpness {sharpness}", out[f * t + rows], qkv[f * t:(f + 1) * t], rows)
+    ctx.close()
+
+
 @pytest.mark.parametrize("entry", ["global", "normed", "frame"])
 @pytest.mark.parametrize("value", [2.0 ** 20, 2.0 ** 26, 2.0 ** 100])
 def test_large_values_under_a_shifted_reference(lib, entry, value):
