@@ -32,6 +32,11 @@ __device__ __forceinline__ void load_row(uint4 (&v)[4], const __nv_bfloat16* row
   for (int q = 0; q < 4; ++q) v[q] = p[q * 32 + lane];
 }
 
+// kRows: absorbed rows in flight.  Few blocks last as long as their longest row, a chain of loads, and four shorten it; many
+// are bound by HBM and want warps, of which 96 registers leave 16 an SM where two rows' 64 leave 32 (us, two / four: 543
+// merged rows 4.7 / 3.9, 2,520 5.6 / 4.7, 5,205 6.3 / 7.2, 83,280 107 / 145).
+constexpr unsigned kMergeFewBlocks = 148 * 5 / 2;
+template <int kRows>
 __global__ void __launch_bounds__(kRowThreads)
 merge_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ kept_idx, const int* __restrict__ seg_off,
              const int* __restrict__ seg_src, __nv_bfloat16* __restrict__ xm, long long n_merged,
@@ -60,27 +65,40 @@ merge_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ kept_i
   for (int i = 0; i < 32; ++i) acc[i] = 0.0f;
   add_row(acc, v);
   int s = s0;
-  for (; s + 1 < s1; s += 2) {  // two rows in flight
-    long long t0 = seg_src[s], t1 = seg_src[s + 1];
-    if (t0 < 0 || t0 >= n_tokens || t1 < 0 || t1 >= n_tokens) {
+  for (; s + kRows <= s1; s += kRows) {  // kRows rows in flight
+    long long t[kRows];
+    bool inside = true;
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+      t[i] = seg_src[s + i];
+      inside = inside && t[i] >= 0 && t[i] < n_tokens;
+    }
+    if (!inside) {
       if (lane == 0) atomicOr(status, kStatusBounds);
       continue;
     }
-    uint4 a[4], b[4];
-    load_row(a, x + t0 * 1024, lane);
-    load_row(b, x + t1 * 1024, lane);
-    add_row(acc, a);
-    add_row(acc, b);
+    uint4 a[kRows][4];
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) load_row(a[i], x + t[i] * 1024, lane);
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) add_row(acc, a[i]);
   }
-  if (s < s1) {
-    const long long t0 = seg_src[s];
-    if (t0 < 0 || t0 >= n_tokens) {
-      if (lane == 0) atomicOr(status, kStatusBounds);
-    } else {
-      uint4 a[4];
-      load_row(a, x + t0 * 1024, lane);
-      add_row(acc, a);
+  if (s < s1) {  // the rest together too
+    uint4 a[kRows - 1][4];
+#pragma unroll
+    for (int i = 0; i < kRows - 1; ++i) {
+      const long long t = s + i < s1 ? seg_src[s + i] : -1;
+      if (s + i < s1 && t >= 0 && t < n_tokens) {
+        load_row(a[i], x + t * 1024, lane);
+      } else {
+        if (s + i < s1 && lane == 0) atomicOr(status, kStatusBounds);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[i][q] = make_uint4(0u, 0u, 0u, 0u);
+      }
     }
+#pragma unroll
+    for (int i = 0; i < kRows - 1; ++i)
+      if (s + i < s1) add_row(acc, a[i]);
   }
   const float denom = (float)(1 + s1 - s0);
 #pragma unroll
@@ -260,7 +278,7 @@ cudaError_t launch_merge(const litevggt_ctx* ctx, const litevggt_plan* plan, con
   const Sizes& z = ctx->sz;
   const unsigned blocks = (unsigned)((z.n_merged + kRowsPerCta - 1) / kRowsPerCta);
   ++*launches;
-  return launch(merge_kernel, dim3(blocks), kRowThreads, 0, s, x, plan->kept_idx, plan->seg_off, plan->seg_src, xm, z.n_merged,
+  return launch(blocks <= kMergeFewBlocks ? merge_kernel<4> : merge_kernel<2>, dim3(blocks), kRowThreads, 0, s, x, plan->kept_idx, plan->seg_off, plan->seg_src, xm, z.n_merged,
                 z.n_tokens, z.n_remove, ctx->ws.status, next_stamp(ctx));
 }
 
