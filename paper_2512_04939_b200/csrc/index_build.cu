@@ -27,7 +27,7 @@
 namespace lv {
 
 // Every step ends in scans and barriers whose instructions all warps issue, so fewer are sooner through: a block of 512 threads where
-// it has few tokens (3,360 tokens in one block 50.4 us, 51.4 with 1024, 56.3 with 256), 1024 where it has many.
+// it has few tokens (577 tokens in one block 31.0 us, 32.0 with 1024, 3,360 50.4, 51.4, 56.3 with 256), 1024 where it has many.
 constexpr int kIdxThreads = 512;
 constexpr int kIdxWideThreads = 1024;
 constexpr int kScanItems = 4;
@@ -429,7 +429,7 @@ __device__ __forceinline__ void order_long_segments(int block, int blocks, const
 
 // kLocal: one block, which keeps in shared memory what the steps hand on.  kNumber: as far as the numbers of the tokens.
 template <bool kLocal, bool kNumber>
-__global__ void __launch_bounds__(kNumber ? kIdxWideThreads : kIdxThreads, 1) index_build_kernel(const IndexArgs args) {
+__global__ void __launch_bounds__(kLocal || kNumber ? kIdxWideThreads : kIdxThreads, 1) index_build_kernel(const IndexArgs args) {
   IndexArgs a = args;
   extern __shared__ int local_words[];
   if constexpr (kLocal) lay_scratch(a, local_words, true);
@@ -567,6 +567,7 @@ long long index_scratch_words(const Sizes& z) {
 //   launches behind the numbers of the tokens: 43,968 tokens 581 -> 568 (in the cluster 572), 66,624 1158 -> 1148 (1159), from
 //     100,000 on level with ten launches and less than 1 % of the plan.
 constexpr int kLocalBytes = 200 * 1024;
+constexpr long long kWideTokens = 4096;  // (kIdxThreads above; 4,164 tokens 56.4 -> 54.9, 6,050 72.0 -> 70.4)
 constexpr long long kClusterTokens = 32768;
 
 // Blocks of the cluster: 16 SMs where the device has that many together (more than the eight that every one has to offer).
@@ -622,7 +623,7 @@ cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStrea
     static std::atomic<unsigned long long> smem_set{0};
     const cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(index_build_kernel<true, false>), kLocalBytes, smem_set);
     if (e != cudaSuccess) return e;
-    return launch(index_build_kernel<true, false>, dim3(1), kIdxThreads, (size_t)local_bytes, s, stamped());
+    return launch(index_build_kernel<true, false>, dim3(1), a.n_tokens > kWideTokens ? kIdxWideThreads : kIdxThreads, (size_t)local_bytes, s, stamped());
   }
   const bool wide = a.n_tokens > kClusterTokens;
   const auto build = wide ? index_build_kernel<false, true> : index_build_kernel<false, false>;
