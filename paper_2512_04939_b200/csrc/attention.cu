@@ -26,10 +26,14 @@
 //               thread cannot feed both tiles)
 // One CTA of two tiles sits on an SM, so nothing would run under the set-up, the first loads and the write-back of the
 // next: a launch is one such CTA per SM, and each works off jobs (256 rows of one head) until they run out.  The
-// K/V ring goes on from job to job; the next job's queries are fetched while the tensor cores finish this one's last
-// step, take the old ones' place as soon as they have, and the next scores are under way before this job's rows are
+// K/V ring goes on from job to job; the next job's queries have come to shared memory by the time the last scores of this one
+// have, take the old ones' place in tensor memory then, and the next scores are under way before this job's rows are
 // written.  Whole layers: 4,386 rows 153 -> 148 us, 15,932 rows 1.15 -> 1.09 ms, 31,751 rows 3.64 -> 3.60; from 83 K rows on, at
-// the power cap, nothing (251,872 rows 241.9 -> 243.4).  Jobs come off a counter, late in the job before: with a fixed stride, or taken a whole
+// the power cap, nothing (251,872 rows 241.9 -> 243.4).  What the softmax warps do themselves between two jobs is what is left: with
+// queries and rows going row by row between global memory and registers (4096 and 2048 lines for the load unit, twice
+// that for a part's rows) 4.3 us from a job's last probabilities to the next one's first scores, 3.4 as it is, and the first job's
+// queries in 2.1 us, not 3.4: the core at 5,205 rows 109.5 -> 105.7 us, at 8,244 250.5 -> 242.6, whole layers
+// 180.9 -> 178.9, 346.3 -> 339.8, 10,410 rows 492.7 -> 487.9, 31,751 (query weights x 16) 4.27 -> 4.21 ms.  Jobs come off a counter, late in the job before: with a fixed stride, or taken a whole
 // job ahead, rows in the online form left 3 % of 31,751 rows' time to a few CTAs at the end.  With one tile, two
 // CTAs an SM run under each other anyway, and jobs measured 3 % slower.
 // Tensor memory (512 columns allocated, 480 used):
@@ -41,9 +45,9 @@
 //   [256,416)  O_0, O_1 (fp32, 80 columns each: 64 output channels, then the row sum - the second
 //              MMA's B operand carries a column of ones next to V, so the tensor core adds up
 //              exactly the bf16 probabilities that it multiplies with V - and 15 unused columns)
-//   [416,480)  Q_0, Q_1 (bf16 pairs, 32 columns each), written once by the softmax threads
-//              (from global memory; with one tile from a TMA load): Q is the A operand of the first MMA from
-//              tensor memory, so the MMAs read only K and V tiles from shared memory.
+//   [416,480)  Q_0, Q_1 (bf16 pairs, 32 columns each), written once by the softmax threads:
+//              Q is the A operand of the first MMA from tensor memory, so the MMAs read only K and V tiles
+//              from shared memory.
 // The two halves of a tile double-buffer the scores: while the softmax threads work on
 // half h the tensor core already runs O += P V of the other half and the next Q K^T into
 // it.  The MMAs are issued in order, which is what makes the S/P aliasing safe: Q K^T for
@@ -61,8 +65,8 @@
 // thread handles per step; 7 measured best in the kernel (on register data alone, 4 warps per
 // scheduler: 6 pairs take 182 clocks per 32 scores against 257 with the special-function unit only,
 // 8 pairs 220).
-// Shared memory: K ring, V ring, and behind the V ring a 2 KB block that holds the ones column of
-// the P V operand (see the kernel).
+// Shared memory: K ring, V ring, behind the V ring a 2 KB block that holds the ones column of
+// the P V operand (see the kernel), and with two tiles room for the next queries and the rows on their way out.
 //
 // Key chunks.  All CTAs of a head stream the same K/V, but they drift apart, so their combined
 // working set is the head's whole K/V; beyond about a quarter of the L2 that no longer stays
@@ -162,7 +166,7 @@ __device__ __forceinline__ float fa_shift_down(float bits) { return 126.0f - 24.
 // `parts` parts to a job, and leave partial rows for combine_parts_kernel.
 struct FaJobs {
   int q_first, q_blocks, heads, count, full, parts;
-  float* o;   // [slot][256][64] partial output rows, slot = id - full
+  float* o;   // [slot][16][256][4] partial output rows, four channels at a time, slot = id - full
   float* ml;  // [slot][256]{reference, row sum}
   int* taken; // how many jobs beyond the CTAs' first ones have been taken; zero when the launch starts
 };
@@ -183,13 +187,14 @@ __device__ __forceinline__ FaJob fa_job(const FaJobs& jobs, int id) {
   const int rest = job / jobs.q_blocks;
   return FaJob{jobs.q_first + job % jobs.q_blocks, rest % jobs.heads, rest / jobs.heads, slot};
 }
-// This thread's 32 channels of row r (0..255) of the job.
+// This thread's 32 channels of row r (0..255) of the job; rows side by side, 4 channels of each at a time, so that a warp's store
+// is 512 bytes in a row (a row of its own after the other they took 2.4 to 3.8 us).
 __device__ __forceinline__ void fa_store_part(const FaJobs& split, int slot, int r, int c, const uint32_t (&acc)[32], float scale,
                                               float m_ref, float row_sum) {
-  float4* dst = reinterpret_cast<float4*>(split.o + ((size_t)slot * 256 + r) * 64 + c * 32);
+  float4* dst = reinterpret_cast<float4*>(split.o) + ((size_t)slot * 16 + c * 8) * 256 + r;
 #pragma unroll
   for (int i = 0; i < 8; ++i)
-    dst[i] = make_float4(__uint_as_float(acc[4 * i]) * scale, __uint_as_float(acc[4 * i + 1]) * scale,
+    dst[i * 256] = make_float4(__uint_as_float(acc[4 * i]) * scale, __uint_as_float(acc[4 * i + 1]) * scale,
                          __uint_as_float(acc[4 * i + 2]) * scale, __uint_as_float(acc[4 * i + 3]) * scale);
   if (c == 0) *reinterpret_cast<float2*>(split.ml + ((size_t)slot * 256 + r) * 2) = make_float2(m_ref, row_sum);
 }
@@ -200,7 +205,7 @@ struct FaBarriers {
   uint64_t v_full[kStages], v_empty[kStages];
   uint64_t q_ready[kTiles], s_full[kTiles][2], p_ready[kTiles][2], pv_done[kTiles], o_done[kTiles], o_free[kTiles];
   uint64_t teardown[kTiles];
-  uint64_t q_full;  // (one tile)
+  uint64_t q_full[kTiles], q_empty[kTiles];  // the queries' way through shared memory
   uint64_t job_full[2], job_empty[2];
   int job[2];  // the CTA's next jobs
   uint32_t tmem_base;
@@ -221,8 +226,11 @@ struct FaShape {
   static constexpr int kStages = kTiles == 2 ? 4 : 3;
   static constexpr uint32_t kTmemCols = 256 * kTiles;
   static constexpr uint32_t kColS = 0, kColO = 128 * kTiles, kColQ = (128 + 80) * kTiles;
+  // queries on their way in and rows on their way out: where V and K tiles will be and have been, or, where the ring goes on
+  // from job to job, of their own
+  static constexpr int kRowBytes = kTiles == 2 ? 2 * kTiles * kFaTileBytes : 0;
   static constexpr int kSmemBytes =
-      2 * kStages * kFaTileBytes + kFaOnesBytes + (int)sizeof(FaPairs<kTiles>) + 512 + 1024;
+      2 * kStages * kFaTileBytes + kRowBytes + kFaOnesBytes + (int)sizeof(FaPairs<kTiles>) + 512 + 1024;
 };
 
 constexpr int kFaAloneBytes = 120 * 1024;  // shared memory that keeps a second CTA off the SM
@@ -371,8 +379,10 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
   constexpr int kStages = Shape::kStages;
   uint8_t* smem_v = smem_k + kStages * kFaTileBytes;
   uint8_t* smem_ones = smem_v + kStages * kFaTileBytes;  // see below
-  uint8_t* smem_q = smem_ones - kFaTileBytes;  // one tile's queries on their way, until V needs its last stage
-  FaPairs<kTiles>* pairs = reinterpret_cast<FaPairs<kTiles>*>(smem_ones + kFaOnesBytes);
+  uint8_t* smem_rows = smem_ones + kFaOnesBytes;
+  uint8_t* smem_q = kTiles == 2 ? smem_rows : smem_ones - kFaTileBytes;  // [tile], queries; with one tile until V needs its last stage
+  uint8_t* smem_o = kTiles == 2 ? smem_rows + kTiles * kFaTileBytes : smem_k;  // [warp] 32 rows of 64 bytes
+  FaPairs<kTiles>* pairs = reinterpret_cast<FaPairs<kTiles>*>(smem_rows + Shape::kRowBytes);
   FaBarriers<kTiles, kStages>* bars = reinterpret_cast<FaBarriers<kTiles, kStages>*>(pairs + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -413,9 +423,11 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       mbar_init(&bars->q_ready[t], 8);
       mbar_init(&bars->o_done[t], 1);
       mbar_init(&bars->teardown[t], 1);
+      mbar_init(&bars->q_full[t], 1);
     } else {
       mbar_init(&bars->o_free[t], 8);
       mbar_init(&bars->pv_done[t], 1);
+      mbar_init(&bars->q_empty[t], 8);
     }
     mbar_fence_init();
   } else if (threadIdx.x == 96) {
@@ -423,8 +435,6 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       mbar_init(&bars->job_full[i], 1);
       mbar_init(&bars->job_empty[i], Shape::kSoftmaxWarps + kTiles);
     }
-    mbar_fence_init();
-    mbar_init(&bars->q_full, 1);
     mbar_fence_init();
     bars->abort_flag = 0;
     for (int i = 0; i < 8 * kTiles; ++i) (&pairs->left[0][0][0])[i] = 0u;
@@ -475,15 +485,26 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
       int stage = 0;
       bool ok = true;
       uint32_t turn = 0;
+      uint32_t q_sent[kTiles] = {};
+      // A job's queries, of the tiles that have rows, once the ones before have been read.
+      auto send_q = [&](int id) -> bool {
+        const FaJob job = job_at(id);
+#pragma unroll
+        for (int t = 0; t < kTiles; ++t) {
+          if (!tile_live(id, t)) continue;
+          if (q_sent[t] != 0 && !mbar_wait(&bars->q_empty[t], (q_sent[t] - 1) & 1u, ctl)) return false;
+          mbar_expect_tx(&bars->q_full[t], kFaTileBytes);
+          tma_load_2d(smem_q + t * kFaTileBytes, &tmap_qkv, &bars->q_full[t], job.head * 64, job.seq * seq_len + (job.q_block * kTiles + t) * 128);
+          ++q_sent[t];
+        }
+        return true;
+      };
+      if (id0 < id_end) ok = send_q(id0);
       for (int id = id0; id < id_end && ok;) {
         const FaJob job = job_at(id);
         const FaTiles kv = tiles_at(id);
         int next_id = id_end;
         const int row0 = job.seq * seq_len, col = job.head * 64;
-        if constexpr (!kJobs) {
-          mbar_expect_tx(&bars->q_full, kFaTileBytes);
-          tma_load_2d(smem_q, &tmap_qkv, &bars->q_full, col, row0 + job.q_block * 128);
-        }
         for (int j = kv.begin; j < kv.end; ++j) {
           if (kJobs && j == max(kv.begin, kv.end - 2)) {
             // The next job, to everybody; late, so that it is not kept waiting here while another CTA has nothing to do, and
@@ -493,6 +514,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
             bars->job[turn & 1u] = next_id;
             mbar_arrive(&bars->job_full[turn & 1u]);
             ++turn;
+            if (next_id < id_end && !send_q(next_id)) { ok = false; break; }
           }
           if (!mbar_wait(&bars->k_empty[stage], phase ^ 1u, ctl)) { ok = false; break; }
           mbar_expect_tx(&bars->k_full[stage], kFaTileBytes);
@@ -507,7 +529,8 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         }
         id = next_id;
       }
-      if constexpr (!kJobs) drain_ring<1>(&bars->q_full, 1, status);
+#pragma unroll
+      for (int t = 0; t < kTiles; ++t) drain_ring<1>(&bars->q_full[t], q_sent[t], status);
       // every load issued by this thread must have landed before the CTA may exit
       drain_ring<kStages>(bars->k_full, k_issued, status);
       drain_ring<kStages>(bars->v_full, v_issued, status);
@@ -621,44 +644,19 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
     const uint32_t o_row = tmem_base + lane_base + Shape::kColO + t * kFaOCols, o_addr = o_row + c * 32;
 
     auto row_of = [&](const FaJob& job) { return job.q_block * (128 * kTiles) + t * 128 + row_in_tile; };  // within the sequence
-    // This thread's half (32 channels) of its query row, and the Cauchy-Schwarz bound on the whole row's scores (K
-    // carries the softmax scale, so they are in base-2 units already); both threads of the row find the same |q|^2.
-    auto load_q = [&](const FaJob& job, uint32_t (&qreg)[16]) -> float {
-      float own = 0.0f, other = 0.0f;
-#pragma unroll
-      for (int i = 0; i < 16; ++i) qreg[i] = 0u;
-      if (row_of(job) < seq_len) {
-        const uint4* src = reinterpret_cast<const uint4*>(qkv + (size_t)(job.seq * seq_len + row_of(job)) * 3 * dim + job.head * 64);
-        auto square = [](const uint4& v, float sum) {
-          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) sum = fmaf(bf16_hi(w[e]), bf16_hi(w[e]), fmaf(bf16_lo(w[e]), bf16_lo(w[e]), sum));
-          return sum;
-        };
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const uint4 v = __ldg(src + 4 * c + i);
-          own = square(v, own);
-          qreg[4 * i] = v.x; qreg[4 * i + 1] = v.y; qreg[4 * i + 2] = v.z; qreg[4 * i + 3] = v.w;
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) other = square(__ldg(src + 4 * (c ^ 1) + i), other);
-      }
-      const float q_norm2 = own + other;
-      return sqrtf(q_norm2 * kv_max[job.seq * 2 * (dim / 64) + job.head]);
-    };
-    // The same for the CTA of one tile, whose queries come by TMA, where the ring's last V tile will be: loaded row by row
-    // every load of a warp touches 32 lines, 2048 in all, and they were the last to arrive (four frames of 16 x 16, M = 543: layer 32.3 -> 31.7 us;
-    // local half of 100 frames of 20 x 20 969 -> 954, of 200 of 28 x 37 5.18 -> 5.15 ms).  A CTA that goes from job to job
-    // fetches the next ones behind its last steps and has no stage to spare.
-    auto read_q = [&](const FaJob& job, uint32_t (&qreg)[16]) -> float {
+    // The queries come by TMA: loaded row by row, every load of a warp touches 32 lines, 4096 in all for two tiles, 2 us (a CTA of
+    // one tile, four frames of 16 x 16: layer 32.3 -> 31.7 us; local half of 200 frames of 28 x 37 5.18 -> 5.15 ms).  This thread's half (32 channels) of its row goes to tensor memory, in the place of the queries before, all
+    // of whose Q K^T must have retired.  Returns the Cauchy-Schwarz bound on the whole row's scores (K carries the
+    // softmax scale, so they are in base-2 units already), or -1 where a wait was given up.
+    auto take_q = [&](const FaJob& job, uint32_t parity) -> float {
       const float k_norm2 = kv_max[job.seq * 2 * (dim / 64) + job.head];
-      if (!mbar_wait_warp(&bars->q_full, 0, ctl)) return -1.0f;
+      if (!mbar_wait_warp(&bars->q_full[t], parity, ctl)) return -1.0f;
       const bool live = row_of(job) < seq_len;
+      uint32_t qreg[16];
       float q_norm2 = 0.0f;
 #pragma unroll
       for (int i = 0; i < 8; ++i) {  // in the same order in both threads of a row, so that they find the same bound
-        uint4 v = *reinterpret_cast<const uint4*>(smem_q + row_in_tile * 128 + ((i ^ (row_in_tile & 7)) << 4));
+        uint4 v = *reinterpret_cast<const uint4*>(smem_q + t * kFaTileBytes + row_in_tile * 128 + ((i ^ (row_in_tile & 7)) << 4));
         if (!live) v = make_uint4(0u, 0u, 0u, 0u);
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -667,14 +665,15 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
           if (i < 4 || c == 1) qreg[4 * (i & 3) + e] = w[e];
         }
       }
-      return sqrtf(q_norm2 * k_norm2);
-    };
-    auto hand_q = [&](const uint32_t (&qreg)[16]) {
       tmem_st16(tmem_base + lane_base + Shape::kColQ + t * 32 + c * 16, qreg);
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->q_ready[t]);
+      if (lane == 0) {
+        mbar_arrive(&bars->q_ready[t]);
+        if (kJobs) mbar_arrive(&bars->q_empty[t]);
+      }
+      return sqrtf(q_norm2 * k_norm2);
     };
     bool ok = true;
     // Phases that go on from job to job, a bit each: of half 0's and half 1's barriers when a job starts, of the job's own
@@ -691,11 +690,8 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
     int id = next_job(id0);
     float score_bound = 0.0f;
     if (id < id_end) {
-      uint32_t qreg[16];
-      if constexpr (kJobs) score_bound = load_q(job_at(id), qreg);
-      else score_bound = read_q(job_at(id), qreg);
-      if (score_bound < 0.0f) id = id_end;  // given up
-      else hand_q(qreg);
+      score_bound = take_q(job_at(id), 0u);
+      if (score_bound < 0.0f) id = id_end;
     }
     while (id < id_end) {
       const FaTiles kv = tiles_at(id);
@@ -872,18 +868,22 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         if (!ok && !shifted) meet_partner(barrier_id, met, n_steps);
       }
       if (!ok) break;
-      // The next job's queries are on their way while the tensor cores finish this one; they take the old ones' place,
-      // and the next scores are under way, before this job's rows are written.
+      // The next job's queries take the old ones' place, and the next scores are under way, while the tensor cores finish this
+      // one's last P V and its rows are written.
       if constexpr (kJobs) asm volatile("" : "+r"(id));  // the job is worked out again: nothing of it is held over the sweep
       const int after = job_after(turn >> 4, false, ok);
       turn += 16u;
       const int next_id = next_job(after);
       if (!ok) break;
-      uint32_t qreg[16];
-      if (next_id < id_end) score_bound = load_q(job_at(next_id), qreg);
+      if (next_id < id_end) {
+        const int last_step = steps_of(tiles_at(id)) - 1;  // its scores came behind all others
+        if (!scores_of(last_step & 1, last_step >> 1)) break;
+        tc_fence_after();
+        score_bound = take_q(job_at(next_id), ((turn >> 2) & 1u) ^ 1u);
+        if (score_bound < 0.0f) break;
+      }
       if (!mbar_wait_warp(&bars->o_done[t], (turn >> 2) & 1u, ctl)) break;
       tc_fence_after();
-      if (next_id < id_end) hand_q(qreg);
       uint32_t acc[32], sum;
       tmem_ld32(o_addr, acc);
       tmem_ld1(o_row + 64, sum);
@@ -903,6 +903,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
         m_ref += (float)((int)e - 127);
       }
       const int row = job.seq * seq_len + row_of(job);  // global row of qkv / o
+      uint8_t* my_rows = smem_o + warp * 2048;  // 32 rows of 64 bytes, 16-byte unit u of row r at u ^ (r / 2 mod 4)
       if (row_of(job) < seq_len) {
         if (job.slot >= 0) {
           fa_store_part(jobs, job.slot, t * 128 + row_in_tile, c, acc, 1.0f, m_ref, __uint_as_float(sum));
@@ -934,7 +935,6 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
           }
           if (last_chunk) {
             const float inv = 1.0f / row_sum;
-            uint4* dst = reinterpret_cast<uint4*>(o + (size_t)row * dim + job.head * 64 + c * 32);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               uint4 w;
@@ -942,7 +942,7 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
               w.y = pack_bf16(__uint_as_float(acc[q * 8 + 2]) * inv, __uint_as_float(acc[q * 8 + 3]) * inv);
               w.z = pack_bf16(__uint_as_float(acc[q * 8 + 4]) * inv, __uint_as_float(acc[q * 8 + 5]) * inv);
               w.w = pack_bf16(__uint_as_float(acc[q * 8 + 6]) * inv, __uint_as_float(acc[q * 8 + 7]) * inv);
-              dst[q] = w;
+              *reinterpret_cast<uint4*>(my_rows + lane * 64 + ((q ^ (lane >> 1 & 3)) << 4)) = w;
             }
           } else {
             // leave the sum over the chunks so far for the next launch
@@ -953,6 +953,18 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_
             ml_mine[1] = row_sum;
           }
         }
+      }
+      if (last_chunk && job.slot < 0) {
+        // four lanes a row: a store of the warp's covers 8 lines, where a row of its own for every lane makes it 32
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = i * 8 + (lane >> 2), in_seq = job.q_block * (128 * kTiles) + t * 128 + (int)quarter * 32 + r;
+          const uint4 v = *reinterpret_cast<const uint4*>(my_rows + r * 64 + (((lane & 3) ^ (r >> 1 & 3)) << 4));
+          if (in_seq < seq_len)
+            *reinterpret_cast<uint4*>(o + (size_t)(job.seq * seq_len + in_seq) * dim + job.head * 64 + c * 32 + (lane & 3) * 8) = v;
+        }
+        __syncwarp();
       }
       const uint32_t steps = (uint32_t)steps_of(tiles_at(id));
       turn ^= ((steps + 1) >> 1 & 1u) | (steps & 2u) | 4u;
@@ -1356,26 +1368,29 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
 
 // Rows of the split jobs: the parts brought to a common reference and added in the order of their keys.
 constexpr int kCombineRows = 32;  // a block's rows; a thread has 8 channels of one
+constexpr int kCombineAwayBytes = 28 * 1024;
+static_assert(kCombineAwayBytes + FaShape<2>::kSmemBytes > 226 * 1024, "");
 __global__ void __launch_bounds__(kCombineRows * 8)
 combine_parts_kernel(FaJobs split, __nv_bfloat16* __restrict__ o, int seq_len, int dim, Stamp stamp) {
   const Span span(stamp);
   const int job = split.full + blockIdx.x, q_block = split.q_first + job % split.q_blocks, head = job / split.q_blocks;
-  const int r = blockIdx.y * kCombineRows + (threadIdx.x >> 3), ch = (threadIdx.x & 7) * 8;
-  const int row = q_block * 256 + r;
-  if (row >= seq_len) return;
+  __shared__ uint4 tile[kCombineRows][9];  // (a column beside the eight, against bank conflicts)
+  const int r = blockIdx.y * kCombineRows + (threadIdx.x & 31), ch = (threadIdx.x >> 5) * 8;  // a lane a row, as the parts lie
   const size_t slot0 = (size_t)blockIdx.x * split.parts;
   float m = -INFINITY;
+#pragma unroll 4
   for (int p = 0; p < split.parts; ++p) m = fmaxf(m, split.ml[((slot0 + p) * 256 + r) * 2]);
   float acc[8], sum = 0.0f;
 #pragma unroll
   for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
+#pragma unroll 4
   for (int p = 0; p < split.parts; ++p) {
     const float2 ml = *reinterpret_cast<const float2*>(split.ml + ((slot0 + p) * 256 + r) * 2);
     // (the E4M3 form's references are no whole numbers)
     const float d = ml.x - m, w = ml.x == m ? 1.0f : d == rintf(d) ? exp2_whole(d) : fast_exp2(d);
     sum = fmaf(ml.y, w, sum);
-    const float4* src = reinterpret_cast<const float4*>(split.o + ((slot0 + p) * 256 + r) * 64 + ch);
-    const float4 a = src[0], b = src[1];
+    const float4* src = reinterpret_cast<const float4*>(split.o) + ((slot0 + p) * 16 + ch / 4) * 256 + r;
+    const float4 a = src[0], b = src[256];
     acc[0] = fmaf(a.x, w, acc[0]);
     acc[1] = fmaf(a.y, w, acc[1]);
     acc[2] = fmaf(a.z, w, acc[2]);
@@ -1386,9 +1401,12 @@ combine_parts_kernel(FaJobs split, __nv_bfloat16* __restrict__ o, int seq_len, i
     acc[7] = fmaf(b.w, w, acc[7]);
   }
   const float inv = 1.0f / sum;
-  *reinterpret_cast<uint4*>(o + (size_t)row * dim + head * 64 + ch) =
+  tile[threadIdx.x & 31][threadIdx.x >> 5] =
       make_uint4(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv), pack_bf16(acc[4] * inv, acc[5] * inv),
                  pack_bf16(acc[6] * inv, acc[7] * inv));
+  __syncthreads();
+  const int row = q_block * 256 + blockIdx.y * kCombineRows + (threadIdx.x >> 3);
+  if (row < seq_len) *reinterpret_cast<uint4*>(o + (size_t)row * dim + head * 64 + (threadIdx.x & 7) * 8) = tile[threadIdx.x >> 3][threadIdx.x & 7];
 }
 
 // How the jobs that do not fill a wave of one CTA an SM are split: into so many parts that their waves end
@@ -1436,8 +1454,10 @@ static FaJobs jobs_for(const litevggt_ctx* ctx, long long seq_len, long long row
 static cudaError_t launch_combine(const litevggt_ctx* ctx, const FaJobs& split, __nv_bfloat16* o, long long seq_len, cudaStream_t s,
                                   int* launches) {
   ++*launches;
+  // (as much shared memory as does not fit beside the attention's: blocks that were on the first SMs early would all stay there,
+  // 7.9 us where they take 5.1 spread over the chip)
   return launch(combine_parts_kernel, dim3((unsigned)(split_slots(split) / split.parts), 256 / kCombineRows),
-                kCombineRows * 8, 0, s, split, o, (int)seq_len, ctx->sz.dim, next_stamp(ctx));
+                kCombineRows * 8, kCombineAwayBytes, s, split, o, (int)seq_len, ctx->sz.dim, next_stamp(ctx));
 }
 
 cudaError_t launch_flash_attention_fp8(litevggt_ctx* ctx, long long m, __nv_bfloat16* o, cudaStream_t s, int* launches) {
