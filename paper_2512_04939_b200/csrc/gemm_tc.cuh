@@ -127,6 +127,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   constexpr int kStages = Shape::kStages;
   constexpr bool kPair = kCtas == 2;
   static_assert(kPair || Epi::kTileOut, "the row-state epilogue runs on pairs");
+  static_assert(!kPair || (kBN % 32 == 0 && kBN <= 256), "columns of an instruction of a pair");
+  static_assert(kBN % kGemmOutChunkCols == 0 || (kBN % kGemmOutChunkCols == 32 && Epi::kTileOut), "");
   extern __shared__ uint8_t smem_raw[];
   // the same offset in both CTAs of a pair: the leader's descriptors address the other CTA's tiles too
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -291,14 +293,26 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         const int warp_row0 = row0 + (int)quarter * 32;
         uint8_t* block = smem_out + (warp - 2) * kGemmOutBlockBytes;
 #pragma unroll 1
-        for (int c = half; c < kBN / kGemmOutChunkCols; c += 2) {
+        for (int c = half; c < (kBN + kGemmOutChunkCols - 1) / kGemmOutChunkCols; c += 2) {
           const int col0 = tile.nt * kBN + c * kGemmOutChunkCols;
           if (col0 >= n_cols || warp_row0 >= m_rows) break;  // nothing of this block exists (warp-uniform)
-          uint32_t acc[64];
+          uint32_t acc[64];  // (where the tile ends before, what lies behind it is read and not used)
           tmem_ld32(t_addr + c * 64, reinterpret_cast<uint32_t(&)[32]>(acc[0]));
           tmem_ld32(t_addr + c * 64 + 32, reinterpret_cast<uint32_t(&)[32]>(acc[32]));
           tmem_ld_wait();
           uint32_t packed[32];
+          if constexpr (kBN % kGemmOutChunkCols != 0) {
+            // The end of such a tile, or of the matrix within one: 32 columns, two whole sectors that the row's thread stores.
+            if (min(kBN - c * kGemmOutChunkCols, n_cols - col0) < kGemmOutChunkCols) {
+              epi.template convert<4>(row, col0, acc, packed);
+              if (row < m_rows) {
+                uint4* dst = reinterpret_cast<uint4*>(epi.out + (long long)row * n_cols + col0);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) dst[q] = make_uint4(packed[4 * q], packed[4 * q + 1], packed[4 * q + 2], packed[4 * q + 3]);
+              }
+              continue;
+            }
+          }
           epi.transform(row, col0, acc, packed);
           // The previous store out of this warp's staging block must be done reading it.
           if (chunk_iter != 0) {
@@ -395,6 +409,7 @@ struct LinearEpilogue {
   static constexpr bool kTileOut = true;
   struct State {};
   const __nv_bfloat16* bias;  // may be null
+  __nv_bfloat16* out;
   int m_rows;
   int n_cols;
   int scale_begin, scale_end;  // output columns [scale_begin, scale_end) are multiplied by `scale`
@@ -415,7 +430,7 @@ struct LinearEpilogue {
   }
   // 64 accumulator columns of one row -> 32 bf16 pairs
   __device__ __forceinline__ void transform(int row, int col0, const uint32_t (&acc)[64], uint32_t (&packed)[32]) const {
-    convert(col0, acc, packed);
+    convert<8>(row, col0, acc, packed);
     if (stat_kind == kStatAmax) {
       const uint32_t best = __reduce_max_sync(0xffffffffu, row < m_rows ? __float_as_uint(largest(packed)) : 0u);
       if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned int*>(stat) + col0 / 64, best);
@@ -444,12 +459,14 @@ struct LinearEpilogue {
       }
     }
   }
-  __device__ __forceinline__ void convert(int col0, const uint32_t (&acc)[64], uint32_t (&packed)[32]) const {
+  // the first kEights x 8 of them, which lie on one side of the scale's borders
+  template <int kEights>
+  __device__ __forceinline__ void convert(int, int col0, const uint32_t (&acc)[64], uint32_t (&packed)[32]) const {
     const float sc = (col0 >= scale_begin && col0 < scale_end) ? scale : 1.0f;
     if (bias != nullptr) {
       const uint4* bp = reinterpret_cast<const uint4*>(bias + col0);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
+      for (int q = 0; q < kEights; ++q) {
         const uint4 b = __ldg(bp + q);
         const uint32_t bw[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
@@ -461,7 +478,7 @@ struct LinearEpilogue {
       }
     } else {
 #pragma unroll
-      for (int i = 0; i < 32; ++i)
+      for (int i = 0; i < 4 * kEights; ++i)
         packed[i] = pack_bf16(__uint_as_float(acc[2 * i]) * sc, __uint_as_float(acc[2 * i + 1]) * sc);
     }
   }
@@ -503,18 +520,23 @@ struct MlpEpilogue {
   struct State {};
   const __nv_bfloat16* bias;      // may be null
   const __nv_bfloat16* residual;  // may be null, same shape as the output with pitch ld_res
+  __nv_bfloat16* out;
   int m_rows;
   int n_cols;
   long long ld_res;
   int gelu;
 
-  __device__ __forceinline__ void transform(int row, int col0, const uint32_t (&acc)[64],
-                                            uint32_t (&packed)[32]) const {
+  __device__ __forceinline__ void transform(int row, int col0, const uint32_t (&acc)[64], uint32_t (&packed)[32]) const {
+    convert<8>(row, col0, acc, packed);
+  }
+  // the first kEights x 8 columns
+  template <int kEights>
+  __device__ __forceinline__ void convert(int row, int col0, const uint32_t (&acc)[64], uint32_t (&packed)[32]) const {
     const bool has_res = residual != nullptr && row < m_rows;
     const uint4* bp = reinterpret_cast<const uint4*>(bias + col0);
     const uint4* rp = reinterpret_cast<const uint4*>(residual + (long long)row * ld_res + col0);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < kEights; ++q) {
       float v[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(acc[q * 8 + i]);

@@ -401,6 +401,39 @@ def test_linear(lib, m, k, n):
     ctx.close()
 
 
+@pytest.mark.parametrize("m,k,n", [(1848, 1024, 1344), (2305, 512, 2112), (3360, 1024, 2048), (3700, 1024, 4096), (3700, 4096, 832)])
+def test_linear_on_tiles_that_end_within_64_columns(lib, m, k, n):
+    """Tiles of 160 and 224 columns: 64, 32, 32, 64 and 160 are left for the last one, whole chunks of 64 and halves."""
+    ctx = _ctx(lib, WORKLOADS["C1"])
+    g = torch.Generator().manual_seed(m + n)
+    a = torch.randn(m, k, generator=g).to(torch.bfloat16)
+    w = (0.05 * torch.randn(n, k, generator=g)).to(torch.bfloat16)
+    b = (0.1 * torch.randn(n, generator=g)).to(torch.bfloat16)
+    rows = np.unique(np.r_[0:40, 100:160, 250:260, m - 70:m])
+    for bias in (b, None):
+        got = ctx.linear(a.cuda(), w.cuda(), None if bias is None else bias.cuda())
+        ctx.poll()
+        ref = to_f64(a)[rows] @ to_f64(w).T + (0 if bias is None else to_f64(bias))
+        check_bf16(f"linear {m}x{k}x{n}", to_f64(got)[rows], ref, sampled=True)
+    ctx.close()
+
+
+def test_mlp_in_place_on_tiles_that_end_within_64_columns(lib):
+    """3,360 rows, whose second layer has tiles of 224 columns; the residual where the output goes."""
+    ctx = lib.LiteVGGT(7, 19, 25, 0.45)
+    g = torch.Generator().manual_seed(5)
+    x = torch.randn(3360, 1024, generator=g).to(torch.bfloat16)
+    w1, w2 = (0.02 * torch.randn(4096, 1024, generator=g)).to(torch.bfloat16), (0.02 * torch.randn(1024, 4096, generator=g)).to(torch.bfloat16)
+    b1, b2 = (0.1 * torch.randn(4096, generator=g)).to(torch.bfloat16), (0.1 * torch.randn(1024, generator=g)).to(torch.bfloat16)
+    y = x.cuda()
+    ctx.mlp(y, w1.cuda(), b1.cuda(), w2.cuda(), b2.cuda(), residual=y, out=y)
+    ctx.poll()
+    rows = np.r_[0:20, 120:136, 3320:3360]
+    ref = O.mlp(to_f64(x)[rows], *[to_f64(v) for v in (w1, b1, w2, b2)]) + to_f64(x)[rows]
+    check_bf16("mlp in place, 3360 rows", to_f64(y)[rows], ref, noise=LAYER_NOISE, sampled=True)
+    ctx.close()
+
+
 # ------------------------------------------------------------------ a7-a9 attention
 # Tolerances of the attention layer.  Each stage is judged on the GPU's own upstream result, so the
 # stated bound (1e-2 of the RMS, or the output's own rounding floor + 2e-3) applies as it is: the
