@@ -137,10 +137,11 @@ constexpr float kFaFixedRefLimit = LV_FA_FIXED_REF_LIMIT;
 constexpr int kFaPolyPairs = LV_FA_POLY_PAIRS;
 // The same in the shifted-reference form, whose polynomial pairs also need a clamp and whose other
 // pairs a subtraction, and which takes the polynomial of degree 6 (the running maximum that served these
-// rows before is as good as the special-function unit).  Core at 31,751 rows, query weights x 16: 0 pairs 4.61 ms, 2: 4.52,
-// 3: 4.57, 4: 4.58; x 8: 4.21, 4.13, 4.14, 4.12; with a cubic, which moves probabilities by 7.5e-5, less still.
+// rows before is as good as the special-function unit).  Layers at query weights x 16, 2 / 3 / 4 / 5 pairs: 10,410 rows 557 / 543 /
+// 544 / 541 us, 31,751 4.17 / 4.07 ms, 62,460 16.10 / 15.84 / 16.14 / 16.00; x 8: 31,751 3.83 / 3.80, 62,460 14.56 / 14.51 / 14.61 /
+// 14.61.  (Three measured no better than two while the waits had their loops in line.)
 #ifndef LV_FA_SHIFT_POLY_PAIRS
-#define LV_FA_SHIFT_POLY_PAIRS 2
+#define LV_FA_SHIFT_POLY_PAIRS 3
 #endif
 constexpr int kFaShiftPolyPairs = LV_FA_SHIFT_POLY_PAIRS;
 // Shifted reference m of a row with score bound B and a known score s0, both limits by the sequence's length (its binary
