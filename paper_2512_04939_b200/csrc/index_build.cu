@@ -11,7 +11,7 @@
 // each, of which there were ten) are barriers (0.7 us) of one cluster of blocks, each with a run of the src tokens (and the
 // tokens from its first to the next block's first) and a run of the rows.  A short sequence is the work of one block
 // that holds in its shared memory what one step hands to the next (four frames of 16 x 16: 9.7 us, 6 so); in a long one the
-// steps behind the numbers of its tokens are launches over the chip.  (launch_index_build has the figures.)
+// steps behind the numbers of its tokens are launches over the chip, in a very long one all are.  (launch_index_build has the figures.)
 //   select    the R-th largest cosine by its ordered bits, eight of them at a time: every block makes a
 //             histogram of its own keys in shared memory, and after a barrier adds up those of all blocks
 //             and finds the bin that holds the R-th for itself.  What the histograms of the blocks before it hold
@@ -35,6 +35,11 @@ constexpr int kSelBins = 256;
 constexpr int kSelPasses = 4;
 constexpr int kIdxMaxBlocks = 16, kIdxPortableBlocks = 8;  // of a cluster
 constexpr int kIdxParts = 128;     // runs of rows of a long sequence
+// Sequences of more tokens than this are numbered by launches over the chip too, their keys selected 11 + 11 + 10 bits at a
+// time by histograms in global memory: what the cluster's 16 SMs do for all tokens grows beyond five launches (index build, us,
+// cluster / launches: 66,624 tokens 37 / 44, 189,000 58 / 48, 208,200 67 / 50, 1,041,000 238 / 77).
+constexpr long long kManyTokens = 98304;
+constexpr int kLongBins = 2048, kLongThreads = 1024, kLongChunk = kLongThreads * kScanItems;  // <= 4 Mi tokens in <= 1024 chunks
 // A token's rank in a segment of up to this many tokens comes from comparing it with each of them, at
 // most R x 1024 loads; longer ones, of which there are at most R / 1024, each take a block that walks
 // over all R merged tokens in order.
@@ -95,6 +100,9 @@ struct IndexArgs {
   int* long_rows;                       // [0] number of long segments, then their rows
   int* count;                           // [M] merged tokens of a row
   int* part_sums;                       // [kIdxParts] merged tokens by run of rows, where the steps are launches
+  unsigned* hist;                       // [3][kLongBins], zero when the build of a very long sequence starts
+  Selection* sel;                       // [3] its selection after every pass
+  unsigned long long* token_sums;       // its counts of every kLongChunk tokens
   int *rem_token, *rem_anchor, *rem_row, *rem_slot, *seg_tmp;  // [R] merged tokens; tokens by slot
   int *row_of, *offset, *anchor_of;     // dst_of, seg_off and best_dst, for reading: copies where the block keeps such in shared memory
   long long n_src, n_dst, n_tokens, n_merged, n_remove;
@@ -114,6 +122,9 @@ __host__ __device__ inline long long lay_scratch(IndexArgs& a, int* words, bool 
   a.long_rows = take(1 + a.n_remove / kLongSegment + 1);
   a.count = take(a.n_merged);
   a.part_sums = take(kIdxParts);
+  a.hist = reinterpret_cast<unsigned*>(take(a.n_tokens > kManyTokens ? 3 * kLongBins : 0));
+  a.sel = reinterpret_cast<Selection*>(take(a.n_tokens > kManyTokens ? 3 * 4 : 0));
+  a.token_sums = reinterpret_cast<unsigned long long*>(take(a.n_tokens > kManyTokens ? 2 * (a.n_tokens / kLongChunk + 1) : 0));
   a.key = reinterpret_cast<unsigned*>(take(a.n_src));
   a.rem_token = take(a.n_remove);
   a.rem_anchor = take(a.n_remove);
@@ -209,25 +220,28 @@ __device__ __forceinline__ void hist_add(unsigned* hist, unsigned bin, bool on) 
   }
 }
 
+// The matching's key of src token i taken apart into anchor token and cosine, whose ordered bits it returns.
+template <bool kLocal>
+__device__ __forceinline__ unsigned take_match(const IndexArgs& a, int i, unsigned long long match, float inv_norm) {
+  unsigned col = ~(unsigned)match;
+  if (col >= a.n_dst) {
+    atomicOr(a.status, kStatusBounds);
+    col = 0;
+  }
+  const unsigned v = (unsigned)(match >> 32);  // the cosine before the src row's own norm, as ordered bits
+  const float sim = __uint_as_float((v & 0x80000000u) ? (v & 0x7fffffffu) : ~v) * inv_norm;
+  const int anchor = a.dst_list[col];
+  a.best_dst[i] = anchor;
+  if constexpr (kLocal) a.anchor_of[i] = anchor;
+  a.best_sim[i] = sim;
+  return a.key[i] = sim_bits(sim);
+}
+
 // The block's src tokens [p0, p1): the matching's keys taken apart into anchor token and cosine, whose ordered bits a thread
 // holds for its first kHeld tokens and finds in memory for others; and the first histogram.
 constexpr int kHeld = 4;
 template <bool kLocal>
 __device__ __forceinline__ void read_matches(const IndexArgs& a, int p0, int p1, bool selects, unsigned* hist, unsigned (&held)[kHeld]) {
-  auto take = [&](int i, unsigned long long match, float inv_norm) -> unsigned {
-    unsigned col = ~(unsigned)match;
-    if (col >= a.n_dst) {
-      atomicOr(a.status, kStatusBounds);
-      col = 0;
-    }
-    const unsigned v = (unsigned)(match >> 32);  // the cosine before the src row's own norm, as ordered bits
-    const float sim = __uint_as_float((v & 0x80000000u) ? (v & 0x7fffffffu) : ~v) * inv_norm;
-    const int anchor = a.dst_list[col];
-    a.best_dst[i] = anchor;
-    if constexpr (kLocal) a.anchor_of[i] = anchor;
-    a.best_sim[i] = sim;
-    return a.key[i] = sim_bits(sim);
-  };
   for (int base = p0; base < p1; base += kHeld * threads()) {
     unsigned long long match[kHeld];
     float inv_norm[kHeld];
@@ -241,7 +255,7 @@ __device__ __forceinline__ void read_matches(const IndexArgs& a, int p0, int p1,
     for (int j = 0; j < kHeld; ++j) {
       const int first = base + j * threads(), i = first + (int)threadIdx.x;
       if (first >= p1) break;
-      const unsigned k = i < p1 ? take(i, match[j], inv_norm[j]) : 0u;
+      const unsigned k = i < p1 ? take_match<kLocal>(a, i, match[j], inv_norm[j]) : 0u;
       if (base == p0) held[j] = k;
       if (selects) hist_add(hist, k >> sel_shift(0), i < p1);
     }
@@ -258,9 +272,16 @@ __device__ __forceinline__ void count_keys(const IndexArgs& a, int p0, int p1, c
 #pragma unroll
   for (int j = 0; j < kHeld; ++j)
     if (p0 + j * threads() < p1) count(held[j], p0 + j * threads() + (int)threadIdx.x < p1);
-  for (int base = p0 + kHeld * threads(); base < p1; base += threads()) {
-    const bool on = base + (int)threadIdx.x < p1;
-    count(on ? a.key[base + threadIdx.x] : 0u, on);
+  for (int base = p0 + kHeld * threads(); base < p1; base += kHeld * threads()) {
+    unsigned k[kHeld];
+#pragma unroll
+    for (int j = 0; j < kHeld; ++j) {
+      const int i = base + j * threads() + (int)threadIdx.x;
+      k[j] = i < p1 ? a.key[i] : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < kHeld; ++j)
+      if (base + j * threads() < p1) count(k[j], base + j * threads() + (int)threadIdx.x < p1);
   }
 }
 
@@ -490,8 +511,10 @@ __global__ void __launch_bounds__(kLocal || kNumber ? kIdxWideThreads : kIdxThre
   lay_segments<kLocal>(a, (int)r0, (int)(r1 < a.n_merged ? r1 : a.n_merged), [&]() -> int {
     if (threadIdx.x < 32) {
       unsigned sum = 0;
+      if constexpr (!kLocal) {
 #pragma unroll 8
-      for (int i = threadIdx.x; i < (kLocal ? 0 : blocks * block); i += 32) sum += ld_cluster(mapa_u32(smem_u32(&sh.part[i % block]), i / block));
+        for (int i = threadIdx.x; i < blocks * block; i += 32) sum += ld_cluster(mapa_u32(smem_u32(&sh.part[i % block]), i / block));
+      }
       sum = __reduce_add_sync(0xffffffffu, sum);
       if (threadIdx.x == 0) rows_before = (int)sum;
     }
@@ -504,6 +527,107 @@ __global__ void __launch_bounds__(kLocal || kNumber ? kIdxWideThreads : kIdxThre
   all_blocks<kLocal>();
   for (int i = block * threads() + (int)threadIdx.x; i < a.n_remove; i += blocks * threads()) rank_token(i, a);
   order_long_segments(block, blocks, a);
+}
+
+// ---- the selection and the numbers of very long sequences, launches of kLongThreads threads a block
+__host__ __device__ constexpr int long_shift(int pass) { return pass == 0 ? 21 : pass == 1 ? 10 : 0; }
+__host__ __device__ constexpr int long_bins(int pass) { return pass == 2 ? 1024 : 2048; }
+
+// Fixes the bits of pass `pass` from its histogram.
+template <int kShift, int kBins>
+__device__ __forceinline__ Selection long_select_bin(const unsigned* hist, const Selection& before) {
+  __shared__ unsigned scratch[32];
+  __shared__ Selection found;
+  constexpr int per = kBins / kLongThreads;
+  unsigned c[per], sum = 0;
+#pragma unroll
+  for (int i = 0; i < per; ++i) {  // from the highest bin downwards
+    c[i] = hist[kBins - 1 - (threadIdx.x * per + i)];
+    sum += c[i];
+  }
+  unsigned above = block_scan_inclusive(sum, scratch) - sum;
+#pragma unroll
+  for (int i = 0; i < per; ++i) {
+    if (above < before.need && above + c[i] >= before.need)
+      found = Selection{before.prefix | (unsigned)(kBins - 1 - (threadIdx.x * per + i)) << kShift, before.need - above, 0u, 0u};
+    above += c[i];
+  }
+  __syncthreads();
+  return found;
+}
+
+// kShift, kBins: this pass's; kShiftBefore, kBinsBefore: those of the one before, or 0 in the first, which takes the matching's
+// keys apart.
+template <int kPass, int kShift, int kBins, int kShiftBefore, int kBinsBefore>
+__global__ void __launch_bounds__(kLongThreads) index_select_kernel(const IndexArgs a) {
+  const Span span(a.stamp);
+  __shared__ unsigned bins[kLongBins];
+  const bool selects = a.n_remove > 0 && a.n_remove < a.n_src;
+  for (int i = threadIdx.x; i < kLongBins; i += kLongThreads) bins[i] = 0u;
+  Selection so_far{0u, (unsigned)a.n_remove, 0u, 0u};
+  if constexpr (kPass > 0) {
+    if constexpr (kPass == 2) so_far = a.sel[0];
+    so_far = long_select_bin<kShiftBefore, kBinsBefore>(a.hist + (kPass - 1) * kLongBins, so_far);
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.sel[kPass - 1] = so_far;
+  } else {
+    for (long long i = (long long)blockIdx.x * kLongThreads + threadIdx.x; i < a.n_merged; i += (long long)gridDim.x * kLongThreads) a.count[i] = 0;
+    if (blockIdx.x == 0 && threadIdx.x < kIdxParts) a.part_sums[threadIdx.x] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.long_rows[0] = 0;
+  }
+  __syncthreads();
+  for (long long base = (long long)blockIdx.x * kLongThreads; base < a.n_src; base += (long long)gridDim.x * kLongThreads) {
+    const int i = (int)base + (int)threadIdx.x;
+    bool on = i < a.n_src;
+    unsigned k = 0;
+    if (on) {
+      if constexpr (kPass == 0) {
+        k = take_match<false>(a, i, a.match_key[i], a.inv_norm_src[i]);
+      } else {
+        k = a.key[i];
+        on = (k >> kShiftBefore) == (so_far.prefix >> kShiftBefore);
+      }
+    }
+    if (selects) hist_add(bins, (k >> kShift) & (unsigned)(kBins - 1), on);
+  }
+  if (!selects) return;
+  __syncthreads();
+  for (int i = threadIdx.x; i < kBins; i += kLongThreads)
+    if (bins[i] != 0u) atomicAdd(&a.hist[kPass * kLongBins + i], bins[i]);
+}
+
+// Threshold (from the last histogram; below all keys where every src token is merged) and the counts of every chunk of tokens.
+__global__ void __launch_bounds__(kLongThreads) index_count_kernel(const IndexArgs a) {
+  const Span span(a.stamp);
+  __shared__ unsigned long long scratch[32];
+  const Selection s = a.n_remove == a.n_src ? Selection{0u, (unsigned)a.n_src, 0u, 0u}
+                                            : long_select_bin<long_shift(2), long_bins(2)>(a.hist + 2 * kLongBins, a.sel[1]);
+  if (blockIdx.x == 0 && threadIdx.x == 0) a.sel[2] = s;
+  TokenKeys t;
+  t.load_places(a, blockIdx.x * kLongChunk, (int)a.n_tokens);
+  t.load_keys(a);
+  unsigned long long sum = 0ull;
+#pragma unroll
+  for (int i = 0; i < kScanItems; ++i)
+    sum += t.pos[i] < 0 ? 0ull : t.key[i] > s.prefix ? 1ull : t.key[i] == s.prefix ? 1ull << 32 : 0ull;
+  const unsigned long long incl = block_scan_inclusive(sum, scratch);
+  if (threadIdx.x == kLongThreads - 1) a.token_sums[blockIdx.x] = incl;
+}
+
+__global__ void __launch_bounds__(kLongThreads) index_number_kernel(const IndexArgs a) {
+  const Span span(a.stamp);
+  __shared__ unsigned long long scratch[32];
+  Selection s{};
+  unsigned long long before = 0ull;
+  if (a.n_remove > 0) {
+    s = a.sel[2];
+    block_scan_inclusive((int)threadIdx.x < (int)blockIdx.x ? a.token_sums[threadIdx.x] : 0ull, scratch);
+    before = scratch[31];
+  }
+  TokenKeys t;
+  const int first = blockIdx.x * kLongChunk;
+  t.load_places(a, first, (int)a.n_tokens);
+  t.load_keys(a);
+  number_tokens<false>(a, first, (int)min((long long)first + kLongChunk, a.n_tokens), s.prefix, s.need, before, t);
 }
 
 // The steps behind the numbers as launches over the chip.
@@ -564,8 +688,8 @@ long long index_scratch_words(const Sizes& z) {
 //     56.5 -> 50.4, 6,050 87.2 -> 70.8 (the cluster there 70.4, at 3,360 56.8);
 //   one cluster, while what its 16 SMs do for all tokens is less than the launches: 9,408 tokens 98.9 -> 75.8, 12,600 134 -> 120
 //     (as launches 122);
-//   launches behind the numbers of the tokens: 43,968 tokens 581 -> 568 (in the cluster 572), 66,624 1158 -> 1148 (1159), from
-//     100,000 on level with ten launches and less than 1 % of the plan.
+//   launches behind the numbers of the tokens: 43,968 tokens 581 -> 568 (in the cluster 572), 66,624 1158 -> 1148 (1159);
+//   launches throughout, from kManyTokens on.
 constexpr int kLocalBytes = 200 * 1024;
 constexpr long long kWideTokens = 4096;  // (kIdxThreads above; 4,164 tokens 56.4 -> 54.9, 6,050 72.0 -> 70.4)
 constexpr long long kClusterTokens = 32768;
@@ -594,6 +718,13 @@ static int cluster_blocks(const void* kernel, int threads, std::atomic<unsigned 
     asked.fetch_or(bit, std::memory_order_release);
   }
   return (fits.load(std::memory_order_acquire) & bit) != 0 ? kIdxMaxBlocks : kIdxPortableBlocks;
+}
+
+// The histograms of a very long sequence, which have to be zero before launch_index_build; the matching sees to it.
+ZeroWords index_zero_words(const litevggt_ctx* ctx) {
+  IndexArgs a = index_sizes(ctx->sz);
+  lay_scratch(a, ctx->ws.index_scratch, false);
+  return a.n_tokens > kManyTokens ? ZeroWords{a.hist, 3 * kLongBins} : ZeroWords{};
 }
 
 cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStream_t s, int* launches) {
@@ -625,12 +756,31 @@ cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStrea
     if (e != cudaSuccess) return e;
     return launch(index_build_kernel<true, false>, dim3(1), a.n_tokens > kWideTokens ? kIdxWideThreads : kIdxThreads, (size_t)local_bytes, s, stamped());
   }
-  const bool wide = a.n_tokens > kClusterTokens;
+  const bool wide = a.n_tokens > kClusterTokens, many = a.n_tokens > kManyTokens;
   const auto build = wide ? index_build_kernel<false, true> : index_build_kernel<false, false>;
   const int threads = wide ? kIdxWideThreads : kIdxThreads;
   static std::atomic<unsigned long long> asked[2], fits[2];
   const int cluster = cluster_blocks(reinterpret_cast<const void*>(build), threads, asked[wide], fits[wide]);
-  cudaError_t e = launch_clusters(cluster, true, build, dim3((unsigned)cluster), (unsigned)threads, 0, s, stamped());
+  cudaError_t e = cudaSuccess;
+  if (!many) e = launch_clusters(cluster, true, build, dim3((unsigned)cluster), (unsigned)threads, 0, s, stamped());
+  if (many) {
+    if (a.n_src == 0) {  // no matching ran
+      e = cudaMemsetAsync(a.hist, 0, 3 * kLongBins * sizeof(unsigned), s);
+      if (e != cudaSuccess) return e;
+    }
+    // at most as many blocks as run at a time: each flushes a histogram
+    const bool selects = a.n_remove > 0 && a.n_remove < a.n_src;
+    long long blocks = (a.n_src + 4 * kLongThreads - 1) / (4 * kLongThreads);
+    const dim3 select((unsigned)(blocks < 1 ? 1 : blocks < 2 * ctx->num_sms ? blocks : 2 * ctx->num_sms));
+    const dim3 chunks((unsigned)((a.n_tokens + kLongChunk - 1) / kLongChunk));
+    e = launch(index_select_kernel<0, long_shift(0), long_bins(0), 0, 0>, select, kLongThreads, 0, s, stamped());
+    if (e == cudaSuccess && selects)
+      e = launch(index_select_kernel<1, long_shift(1), long_bins(1), long_shift(0), long_bins(0)>, select, kLongThreads, 0, s, stamped());
+    if (e == cudaSuccess && selects)
+      e = launch(index_select_kernel<2, long_shift(2), long_bins(2), long_shift(1), long_bins(1)>, select, kLongThreads, 0, s, stamped());
+    if (e == cudaSuccess && a.n_remove > 0) e = launch(index_count_kernel, chunks, kLongThreads, 0, s, stamped());
+    if (e == cudaSuccess) e = launch(index_number_kernel, chunks, kLongThreads, 0, s, stamped());
+  }
   if (e != cudaSuccess || !wide) return e;
   const int rows_per_part = (int)((a.n_merged + kIdxParts - 1) / kIdxParts);
   const unsigned blocks = (unsigned)((a.n_remove + kIdxThreads - 1) / kIdxThreads);

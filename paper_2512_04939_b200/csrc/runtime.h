@@ -249,6 +249,8 @@ cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, cudaStream_t
 // index_build.cu
 cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStream_t s, int* launches);
 long long index_scratch_words(const Sizes& z);
+// the part of the scratch array that has to be zero before launch_index_build; the matching sees to it
+ZeroWords index_zero_words(const litevggt_ctx* ctx);
 
 // merge_unmerge.cu
 cudaError_t launch_merge(const litevggt_ctx* ctx, const litevggt_plan* plan, const __nv_bfloat16* x,

@@ -94,7 +94,7 @@ cudaError_t launch_match(litevggt_ctx* ctx, const __nv_bfloat16* x, cudaStream_t
   const long long tiles = row_blocks * ((z.n_dst + bn - 1) / bn);
   // the argmax epilogue writes no matrix: the store map is never read, any valid map fills the slot
   auto run = [&](auto launch) {
-    return launch(tmap_a, tmap_b, tmap_a, z.n_src, z.n_dst, 1024, epi, tiles, ctx->num_sms, ws.status, ZeroWords{}, next_stamp(ctx), s);
+    return launch(tmap_a, tmap_b, tmap_a, z.n_src, z.n_dst, 1024, epi, tiles, ctx->num_sms, ws.status, index_zero_words(ctx), next_stamp(ctx), s);
   };
   e = bn == 256 ? run(gemm_launch<ArgmaxEpilogue, 256, 2>)
                 : bn == 128 ? run(gemm_launch<ArgmaxEpilogue, 128, 2>) : run(gemm_launch<ArgmaxEpilogue, 64, 2>);
