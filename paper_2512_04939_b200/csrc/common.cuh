@@ -149,15 +149,22 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
     }
   }
 }
-// Warp-uniform flavour for warps that go on to execute .sync.aligned instructions.  The first try stands alone in the caller's code,
-// with one vote and one branch; the bounded loop behind it is a function of its own.  With the loop in line, its
-// convergence barriers and clock reads were executed on every wait of the softmax's loop and in the way of its registers: layers of
-// 21,984 rows 1.804 -> 1.785 ms (on E4M3 operands 2.374 -> 2.352), 31,751 rows under sharp queries 4.25 -> 4.16, 83,280 rows, at the
-// power cap, 27.08 -> 26.54, block of 100 frames 14.55 -> 14.26, four frames of 16 x 16 30.8 -> 30.4 us.
+// Warp-uniform flavours for warps that go on to execute .sync.aligned instructions.
+// Where a warp waits once a tile, as the matrix products' epilogue does: all in line.  A call, even one that is hardly ever
+// made, takes registers from code that uses all of its 168: with it, MLP layers in tiles of 128 and 192 columns spilled (both layers
+// of 1,044 rows 29.0 us, 28.6 in line, 1,777 rows 34.5 and 34.0; of 300 to 700 rows, whose tiles make one wave, the call and its
+// spills were hidden and 0.2 us faster).
+__device__ __forceinline__ bool mbar_wait_warp_in_line(uint64_t* bar, uint32_t parity, const WaitCtl& ctl) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, ctl) ? 1 : 0) != 0;
+}
+// Where it waits in every step of a loop, as the softmax does: the first try stands alone in the caller's code, with one vote
+// and one branch; the bounded loop behind it is a function of its own.  With the loop in line, its convergence barriers and
+// clock reads were executed on every wait and in the way of the loop's registers (timed in turn: layers of 21,984 rows 1.804 -> 1.785 ms,
+// on E4M3 operands 2.374 -> 2.352, 31,751 rows under sharp queries 4.25 -> 4.16, 83,280 rows 27.08 -> 26.54).
 __device__ __noinline__ static bool mbar_wait_warp_long(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag,
                                                         uint32_t* status, long long limit) {
   const WaitCtl ctl{abort_flag, status, limit};
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, ctl) ? 1 : 0) != 0;
+  return mbar_wait_warp_in_line(bar, parity, ctl);
 }
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, const WaitCtl& ctl) {
   if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity) ? 1 : 0)) return true;

@@ -286,7 +286,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       }
       const uint32_t ab = tile_iter & 1u;
       const uint32_t ab_phase = (tile_iter >> 1) & 1u;
-      if (!mbar_wait_warp(&bars->tmem_full[ab], ab_phase, ctl)) break;
+      if (!mbar_wait_warp_in_line(&bars->tmem_full[ab], ab_phase, ctl)) break;
       tc_fence_after();
       const uint32_t t_addr = tmem_base + ((quarter * 32u) << 16) + ab * kBN;
       if constexpr (Epi::kTileOut) {
