@@ -296,6 +296,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         for (int c = half; c < (kBN + kGemmOutChunkCols - 1) / kGemmOutChunkCols; c += 2) {
           const int col0 = tile.nt * kBN + c * kGemmOutChunkCols;
           if (col0 >= n_cols || warp_row0 >= m_rows) break;  // nothing of this block exists (warp-uniform)
+          int r = row;
+          // Worked out for every chunk: held over the loop, the row's addresses spill (12 bytes at 224 columns, 8 at 160; both
+          // layers of an MLP of 1,153 rows 30.5 us, 30.0 so, 1,777 34.0 and 33.4).  Other widths have the registers.
+          if constexpr (kBN % kGemmOutChunkCols != 0) asm volatile("" : "+r"(r));
           uint32_t acc[64];  // (where the tile ends before, what lies behind it is read and not used)
           tmem_ld32(t_addr + c * 64, reinterpret_cast<uint32_t(&)[32]>(acc[0]));
           tmem_ld32(t_addr + c * 64 + 32, reinterpret_cast<uint32_t(&)[32]>(acc[32]));
@@ -304,16 +308,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           if constexpr (kBN % kGemmOutChunkCols != 0) {
             // The end of such a tile, or of the matrix within one: 32 columns, two whole sectors that the row's thread stores.
             if (min(kBN - c * kGemmOutChunkCols, n_cols - col0) < kGemmOutChunkCols) {
-              epi.template convert<4>(row, col0, acc, packed);
-              if (row < m_rows) {
-                uint4* dst = reinterpret_cast<uint4*>(epi.out + (long long)row * n_cols + col0);
+              epi.template convert<4>(r, col0, acc, packed);
+              if (r < m_rows) {
+                uint4* dst = reinterpret_cast<uint4*>(epi.out + (long long)r * n_cols + col0);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) dst[q] = make_uint4(packed[4 * q], packed[4 * q + 1], packed[4 * q + 2], packed[4 * q + 3]);
               }
               continue;
             }
           }
-          epi.transform(row, col0, acc, packed);
+          epi.transform(r, col0, acc, packed);
           // The previous store out of this warp's staging block must be done reading it.
           if (chunk_iter != 0) {
             if (lane == 0) bulk_wait_group_read<0>();

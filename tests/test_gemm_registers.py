@@ -20,7 +20,7 @@ def spills(tmp_path_factory):
     return {(epilogue, int(columns), int(ctas)): (int(stores), int(loads)) for epilogue, columns, ctas, stores, loads in found}
 
 
-@pytest.mark.parametrize("columns,ctas", [(64, 2), (128, 2), (192, 2), (256, 2), (256, 1)])
+@pytest.mark.parametrize("columns,ctas", [(64, 2), (128, 2), (160, 2), (192, 2), (224, 2), (256, 2), (256, 1)])
 @pytest.mark.parametrize("epilogue", ["LinearEpilogue", "MlpEpilogue"])
 def test_no_instance_spills(spills, epilogue, columns, ctas):
     assert spills[epilogue, columns, ctas] == (0, 0)
