@@ -46,10 +46,10 @@
 #include <cuda.h>
 
 #include "common.cuh"
+#include "gemm_tiles.h"
 
 namespace lv {
 
-constexpr int kGemmBM = 128;  // rows of a CTA
 constexpr int kGemmBK = 64;
 constexpr int kGemmMaxThreads = 320;  // 2 + 8 warps
 // Threads of a launch: TMA warp + MMA warp + 4 (row-state epilogue) or 8 (matrix epilogue) warps.
@@ -387,17 +387,6 @@ cudaError_t gemm_launch(const CUtensorMap& a, const CUtensorMap& b, const CUtens
   const long long groups = work < num_sms / kCtas ? work : num_sms / kCtas;
   return launch_clusters(kCtas, true, gemm_tc_kernel<Epi, kBN, kCtas>, dim3((unsigned)(kCtas * groups)), gemm_threads<Epi>(),
                          Shape::kSmemBytes, s, a, b, out, (int)m, (int)n, (int)k, epi, status, zero, stamp);
-}
-
-// What a launch costs, in units of what one column of a tile costs per k-block, times k: every wave of pairs pays
-// about 150 columns' worth for the 128 rows of A that each CTA loads, a wave of single CTAs 205, whose B is not
-// shared; a pair about 111 x 1024 more, once, for its cluster-wide hand-overs.  (us at k = 1024, one wave / every
-// further one: a pair at 256 columns 11.3 / 5.3, 192: 9.8 / 4.6, 128: 8.0 / 3.75, 64: 7.6 / 2.8; one CTA at 256
-// columns 10.6 / 6.2, of which the formula gives 6.0 so that two waves of either, equal within 2 %, stay with
-// single CTAs.)  Where finer rows save one wave of many, pairs are still ahead: 52,050 x 1024 x 1024, 11 waves of
-// single CTAs 106 us, 12 of pairs 96; 12,850 x 4096 x 1024, 11 and 12 waves, 95 and 87.
-inline long long gemm_cost(long long waves, int bn, long long k, bool pair) {
-  return pair ? waves * (150 + bn) * k + 90 * 1024 : waves * (205 + bn) * k - 21 * 1024;
 }
 
 // ----------------------------------------------------------------------------------------

@@ -7,36 +7,12 @@
 
 namespace lv {
 
-// Columns of a pair's tile, or 0: CTAs of their own, 256 columns.  Narrower tiles win where wider ones
-// would leave pairs idle in the only or the last wave, CTAs of their own where 128 rows a block save a wave,
-// and below k = 512 (104,100 rows x 128 x 320: 36 us, a pair 50).  Of the multiples of 32 that a pair's tile can have, 224 and
-// 160 cut 1024 columns into five and seven (block of 7 frames of 19 x 25, whose 3,360 rows then make one wave of 70 tiles of
-// the MLP's second layer where they made 56: 254.2 -> 251.4 us).  `heads`: a tile holds whole heads of 64 columns, of which the
-// epilogue takes a statistic.
-static int tile_columns(long long m, long long n, long long k, bool heads, int num_sms) {
-  if (k < 512) return 0;
-  auto waves = [&](int rows, int bn, int groups) {
-    return (((m + rows - 1) / rows) * ((n + bn - 1) / bn) + groups - 1) / groups;
-  };
-  int best = 0;
-  long long best_cost = gemm_cost(waves(kGemmBM, 256, num_sms), 256, k, false);
-  for (const int bn : {256, 224, 192, 160, 128, 64}) {  // (a pair's tile has a multiple of 32)
-    if (heads && bn % 64 != 0) continue;
-    const long long cost = gemm_cost(waves(2 * kGemmBM, bn, num_sms / 2), bn, k, true);
-    if (cost < best_cost) {
-      best = bn;
-      best_cost = cost;
-    }
-  }
-  return best;
-}
-
 // out [m, n] = epi(a [m, k] w [n, k]^T)
 template <class Epi>
 static cudaError_t launch_gemm_out(litevggt_ctx* ctx, const __nv_bfloat16* a, long long m, long long k,
                                    const __nv_bfloat16* w, long long n, __nv_bfloat16* out, const Epi& epi,
                                    bool heads, const ZeroWords& zero, cudaStream_t s, int* launches) {
-  const int columns = tile_columns(m, n, k, heads, ctx->num_sms), bn = columns != 0 ? columns : 256;
+  const int columns = gemm_tile_columns(m, n, k, heads, ctx->num_sms), bn = columns != 0 ? columns : 256;
   CUtensorMap tmap_a, tmap_b, tmap_out;
   if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap_a, a, (uint64_t)k, (uint64_t)m, (uint64_t)k, kGemmBK, kGemmBM) ||
       !make_tmap_bf16_2d(ctx->encode_tiled, &tmap_b, w, (uint64_t)k, (uint64_t)n, (uint64_t)k, kGemmBK, columns != 0 ? bn / 2 : bn) ||

@@ -404,9 +404,11 @@ def test_linear(lib, m, k, n):
     ctx.close()
 
 
-@pytest.mark.parametrize("m,k,n", [(1848, 1024, 1344), (2305, 512, 2112), (3360, 1024, 2048), (3700, 1024, 4096), (3700, 4096, 832)])
+@pytest.mark.parametrize("m,k,n", [(1848, 1024, 1344), (2305, 512, 2112), (3360, 1024, 2048), (3700, 1024, 4096), (3700, 4096, 832),
+                                   (2305, 768, 2112)])
 def test_linear_on_tiles_that_end_within_64_columns(lib, m, k, n):
-    """Tiles of 160 and 224 columns: 64, 32, 32, 64 and 160 are left for the last one, whole chunks of 64 and halves."""
+    """Tiles of 160 and 224 columns: 64, 32, 64, 160 and 32 are left for the last one, whole chunks of 64 and halves (and 192 columns
+    at k = 512)."""
     ctx = _ctx(lib, WORKLOADS["C1"])
     g = torch.Generator().manual_seed(m + n)
     a = torch.randn(m, k, generator=g).to(torch.bfloat16)
