@@ -693,16 +693,17 @@ long long index_scratch_words(const Sizes& z) {
   return lay_scratch(a, nullptr, false);
 }
 
-// Which form, by what a plan's build on new features and the merge behind it take (us; the forms up to here: one block up
-// to 8192 tokens, ten launches beyond):
-//   one block, as long as what it hands on fits into its shared memory (some 9000 tokens): 577 tokens 34.8 -> 31.0, 3,360
-//     56.5 -> 50.4, 6,050 87.2 -> 70.8 (the cluster there 70.4, at 3,360 56.8);
-//   one cluster, while what its 16 SMs do for all tokens is less than the launches: 9,408 tokens 98.9 -> 75.8, 12,600 134 -> 120
-//     (as launches 122);
-//   launches behind the numbers of the tokens: 43,968 tokens 581 -> 568 (in the cluster 572), 66,624 1158 -> 1148 (1159);
+// Which form, by what a plan's build on new features and the merge behind it take (us):
+//   one block up to kLocalTokens, which keep in its shared memory what it hands on (one block / the cluster): 3,360 tokens 47.7 / 53.7, 4,050
+//     55.3 / 58.6, 5,040 68.2 / 68.2, 6,300 69.7 / 67.5, 7,203 78.3 / 74.3, 8,820 93.4 / 82.2; of 40 kinds, each token's rank counted
+//     among many, 5,040 83.9 / 80.1, 6,300 107 / 98, 8,820 155 / 127;
+//   one cluster, while what its 16 SMs do for all tokens is less than the launches: 12,600 tokens 120 (as launches 122);
+//   launches behind the numbers of the tokens: 43,968 tokens 568 (in the cluster 572), 66,624 1148 (1159);
 //   launches throughout, from kManyTokens on.
-constexpr int kLocalBytes = 200 * 1024;
-constexpr long long kWideTokens = 4096;  // (kIdxThreads above; 4,164 tokens 56.4 -> 54.9, 6,050 72.0 -> 70.4)
+constexpr long long kLocalTokens = 5120;
+constexpr int kLocalBytes = 164 * 1024;
+static_assert(kLocalTokens * 8 * 4 + 2048 <= kLocalBytes, "at most eight words a token (all src, all merged) and the fixed ones");
+constexpr long long kWideTokens = 4096;  // (kIdxThreads above; 4,164 tokens 56.4 with 512 threads, 54.9 with 1024)
 constexpr long long kClusterTokens = 32768;
 
 // Blocks of the cluster: 16 SMs where the device has that many together (more than the eight that every one has to offer).
@@ -761,7 +762,7 @@ cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStrea
     ++*launches;
     return a;
   };
-  if (local_bytes <= kLocalBytes) {
+  if (a.n_tokens <= kLocalTokens && local_bytes <= kLocalBytes) {
     static std::atomic<unsigned long long> smem_set{0};
     const cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(index_build_kernel<true, false>), kLocalBytes, smem_set);
     if (e != cudaSuccess) return e;

@@ -178,9 +178,12 @@ def test_index_build_bit_exact_given_same_matches(lib, wl):
 
 
 @pytest.mark.parametrize("frames,grid,ratio,cell,kind", [
-    (38, (16, 16), 0.3, 2, "random"),   # one block: 204,720 of its 204,800 bytes, five chunks of tokens
+    (38, (16, 16), 0.3, 2, "random"),
     (7, (19, 25), 0.45, 2, "tied"),     # ties at the threshold, one block
-    (35, (16, 16), 0.45, 2, "tied"),    # 204,992 bytes: the smallest cluster; ties across its blocks
+    (35, (16, 16), 0.45, 2, "tied"),    # ties across the cluster's blocks
+    (16, (15, 21), 0.45, 2, "tied"),    # 5,120 tokens: the most for one block, two chunks of tokens
+    (16, (15, 21), 1.0, 16, "random"),  # and the most shared memory
+    (3, (46, 37), 0.45, 2, "tied"),     # 5,121: the smallest cluster
     (31, (28, 37), 0.3, 2, "random"),   # 32,271 tokens: the largest
     (31, (28, 37), 0.0, 2, "random"),   # nothing merged
     (14, (37, 37), 0.5, 16, "equal"),   # one segment of 9,618 tokens
