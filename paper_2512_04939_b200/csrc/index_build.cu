@@ -108,6 +108,7 @@ struct IndexArgs {
   long long n_src, n_dst, n_tokens, n_merged, n_remove;
   uint32_t* status;
   Stamp stamp;
+  __host__ __device__ bool selects() const { return n_remove > 0 && n_remove < n_src; }  // else none or all are merged
 };
 
 // Lays what the steps hand on over `words`: [ long segments: count, rows | merged tokens per row | keys | five words a merged
@@ -469,7 +470,7 @@ __global__ void __launch_bounds__(kLocal || kNumber ? kIdxWideThreads : kIdxThre
   __shared__ IndexShared sh;
   __shared__ uint2 sums[2][kSelBins];
   const int block = kLocal ? 0 : blockIdx.x, blocks = kLocal ? 1 : gridDim.x;  // one cluster
-  const bool selects = a.n_remove > 0 && a.n_remove < a.n_src;  // else none or all are merged
+  const bool selects = a.selects();
   for (int i = threadIdx.x; i < kSelPasses * kSelBins; i += threads()) sh.hist[0][i] = 0u;
   if (threadIdx.x < kIdxMaxBlocks) sh.part[threadIdx.x] = 0u;
   __syncthreads();
@@ -574,7 +575,7 @@ template <int kPass, int kShift, int kBins, int kShiftBefore, int kBinsBefore>
 __global__ void __launch_bounds__(kLongThreads) index_select_kernel(const IndexArgs a) {
   const Span span(a.stamp);
   __shared__ unsigned bins[kLongBins];
-  const bool selects = a.n_remove > 0 && a.n_remove < a.n_src;
+  const bool selects = a.selects();
   for (int i = threadIdx.x; i < kLongBins; i += kLongThreads) bins[i] = 0u;
   Selection so_far{0u, (unsigned)a.n_remove, 0u, 0u};
   if constexpr (kPass > 0) {
@@ -733,11 +734,11 @@ static int cluster_blocks(const void* kernel, int threads, std::atomic<unsigned 
   return (fits.load(std::memory_order_acquire) & bit) != 0 ? kIdxMaxBlocks : kIdxPortableBlocks;
 }
 
-// The histograms of a very long sequence, which have to be zero before launch_index_build; the matching sees to it.
+// The histograms of a very long sequence, which have to be zero before launch_index_build where it selects; the matching sees to it.
 ZeroWords index_zero_words(const litevggt_ctx* ctx) {
   IndexArgs a = index_sizes(ctx->sz);
   lay_scratch(a, ctx->ws.index_scratch, false);
-  return a.n_tokens > kManyTokens ? ZeroWords{a.hist, 3 * kLongBins} : ZeroWords{};
+  return a.n_tokens > kManyTokens && a.selects() ? ZeroWords{a.hist, 3 * kLongBins} : ZeroWords{};
 }
 
 cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStream_t s, int* launches) {
@@ -777,12 +778,8 @@ cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStrea
   cudaError_t e = cudaSuccess;
   if (!many) e = launch_clusters(cluster, true, build, dim3((unsigned)cluster), (unsigned)threads, 0, s, stamped());
   if (many) {
-    if (a.n_src == 0) {  // no matching ran
-      e = cudaMemsetAsync(a.hist, 0, 3 * kLongBins * sizeof(unsigned), s);
-      if (e != cudaSuccess) return e;
-    }
     // at most as many blocks as run at a time: each flushes a histogram
-    const bool selects = a.n_remove > 0 && a.n_remove < a.n_src;
+    const bool selects = a.selects();
     long long blocks = (a.n_src + 4 * kLongThreads - 1) / (4 * kLongThreads);
     const dim3 select((unsigned)(blocks < 1 ? 1 : blocks < 2 * ctx->num_sms ? blocks : 2 * ctx->num_sms));
     const dim3 chunks((unsigned)((a.n_tokens + kLongChunk - 1) / kLongChunk));

@@ -194,7 +194,12 @@ def test_index_build_bit_exact_given_same_matches(lib, wl):
     (71, (37, 37), 0.3, 2, "tied"),     # 97,554 tokens: the most that the cluster numbers
     (72, (37, 37), 0.3, 2, "tied"),     # 98,928: the fewest that launches do, ties across chunks
     (72, (37, 37), 1.0, 2, "random"),   # every src token merged
-    (72, (37, 37), 0.5, 16, "equal")])  # one segment of 49,464 tokens, walked by one block
+    (72, (37, 37), 0.5, 16, "equal"),   # one segment of 49,464 tokens, walked by one block
+    (72, (37, 37), 0.0, 2, "random"),   # nothing merged
+    (12, (20, 20), 0.5, 1, "random"),   # every patch an anchor, so no src token: one block,
+    (31, (28, 37), 0.5, 1, "random"),   # one cluster,
+    (24, (37, 37), 0.5, 1, "random"),   # the cluster and launches,
+    (72, (37, 37), 0.5, 1, "random")])  # launches
 def test_index_arrays_at_the_limits_of_their_forms(lib, frames, grid, ratio, cell, kind):
     """Numbers and sizes against the oracle's on the library's own matches; segments by a merge, whose sums show their order."""
     ctx = lib.LiteVGGT(frames, grid[0], grid[1], ratio, cell_h=cell, cell_w=cell)
