@@ -369,10 +369,9 @@ __device__ __noinline__ void meet_partner(int id, int met, int n_steps) {
 // kTiles: query tiles of the CTA.
 template <int kTiles, bool kFirst, bool kLast>
 __global__ void __launch_bounds__(FaShape<kTiles>::kThreads, kTiles == 2 ? 1 : 2)
-flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, const __nv_bfloat16* __restrict__ qkv,
-                       __nv_bfloat16* __restrict__ o, float* __restrict__ o_state, float* __restrict__ ml_state,
-                       const float* __restrict__ kv_max, float key_bits, int seq_len, int dim, int tile_begin,
-                       int tile_end, FaJobs jobs, uint32_t* status, Stamp stamp) {
+flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, __nv_bfloat16* __restrict__ o,
+                       float* __restrict__ o_state, float* __restrict__ ml_state, const float* __restrict__ kv_max,
+                       float key_bits, int seq_len, int dim, int tile_begin, int tile_end, FaJobs jobs, uint32_t* status, Stamp stamp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* smem_k = smem;
@@ -1508,7 +1507,7 @@ static cudaError_t launch_rows(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long
   CUtensorMap tmap;
   if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap, qkv, (uint64_t)3 * dim, (uint64_t)rows, (uint64_t)3 * dim, 64, kFaTileKeys))
     return cudaErrorInvalidValue;
-  using Kernel = void (*)(const CUtensorMap, const __nv_bfloat16*, __nv_bfloat16*, float*, float*, const float*, float, int,
+  using Kernel = void (*)(const CUtensorMap, __nv_bfloat16*, float*, float*, const float*, float, int,
                           int, int, int, FaJobs, uint32_t*, Stamp);
   // [query tiles of a CTA - 1][first chunk][last chunk]
   const Kernel kernels[2][2][2] = {
@@ -1543,7 +1542,7 @@ static cudaError_t launch_rows(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long
     cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(kernels[a][b][c]), a == 0 ? kFaAloneBytes : smem_bytes[a],
                                               smem_set[a][b][c]);
     if (e != cudaSuccess) return e;
-    e = launch_clusters(1, early, kernels[a][b][c], grid, threads, smem, s, tmap, qkv, o, ctx->ws.attn_o_state, ctx->ws.attn_ml_state,
+    e = launch_clusters(1, early, kernels[a][b][c], grid, threads, smem, s, tmap, o, ctx->ws.attn_o_state, ctx->ws.attn_ml_state,
                ctx->ws.attn_kmax, key_bits(seq_len), (int)seq_len, dim, begin, end, split, ctx->ws.status, next_stamp(ctx));
     if (e != cudaSuccess) return e;
     ++*launches;
