@@ -1504,8 +1504,10 @@ static cudaError_t launch_rows(litevggt_ctx* ctx, const __nv_bfloat16* qkv, long
   const int dim = ctx->sz.dim;
   if (dim != 1024 || ctx->ws.attn_kmax == nullptr) return cudaErrorInvalidValue;
   const long long rows = seq_len * n_seq;
+  // (a head's row is 128 bytes; the next head's, brought along, is gone again before its turn: 130,125 rows read 2.39 GB a layer,
+  // 2.13 where only the queries come alone, 1.91 where keys and values do too, in the same time)
   CUtensorMap tmap;
-  if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap, qkv, (uint64_t)3 * dim, (uint64_t)rows, (uint64_t)3 * dim, 64, kFaTileKeys))
+  if (!make_tmap_bf16_2d(ctx->encode_tiled, &tmap, qkv, (uint64_t)3 * dim, (uint64_t)rows, (uint64_t)3 * dim, 64, kFaTileKeys, true))
     return cudaErrorInvalidValue;
   using Kernel = void (*)(const CUtensorMap, __nv_bfloat16*, float*, float*, const float*, float, int,
                           int, int, int, FaJobs, uint32_t*, Stamp);

@@ -228,9 +228,10 @@ bool resolve_encode_tiled(void** fn);
 // The allocation or registration that an address which the device can use lies in.
 bool allocation_of(const void* device_ptr, const uint8_t** begin, size_t* bytes);
 // 2-D bf16 tensor [outer, inner] row-major with row pitch `pitch_elems`; box [box_outer, box_inner],
-// 128-byte swizzle, zero fill outside the tensor.
+// 128-byte swizzle, zero fill outside the tensor.  A load brings 256 bytes of a row into L2, or, where what lies beside the box is
+// not wanted before L2 has lost it (`box_alone`), 128.
 bool make_tmap_bf16_2d(void* encode_fn, CUtensorMap* out, const void* base, uint64_t inner, uint64_t outer,
-                       uint64_t pitch_elems, uint32_t box_inner, uint32_t box_outer);
+                       uint64_t pitch_elems, uint32_t box_inner, uint32_t box_outer, bool box_alone = false);
 bool make_tmap_u8_2d(void* encode_fn, CUtensorMap* out, const void* base, uint64_t inner, uint64_t outer,
                      uint64_t pitch_bytes, uint32_t box_inner, uint32_t box_outer);
 
