@@ -1368,8 +1368,6 @@ flash_attention_fp8_kernel(const __grid_constant__ CUtensorMap tmap_k8, const __
 
 // Rows of the split jobs: the parts brought to a common reference and added in the order of their keys.
 constexpr int kCombineRows = 32;  // a block's rows; a thread has 8 channels of one
-constexpr int kCombineAwayBytes = 28 * 1024;
-static_assert(kCombineAwayBytes + FaShape<2>::kSmemBytes > 226 * 1024, "");
 __global__ void __launch_bounds__(kCombineRows * 8)
 combine_parts_kernel(FaJobs split, __nv_bfloat16* __restrict__ o, int seq_len, int dim, Stamp stamp) {
   const Span span(stamp);
@@ -1454,10 +1452,10 @@ static FaJobs jobs_for(const litevggt_ctx* ctx, long long seq_len, long long row
 static cudaError_t launch_combine(const litevggt_ctx* ctx, const FaJobs& split, __nv_bfloat16* o, long long seq_len, cudaStream_t s,
                                   int* launches) {
   ++*launches;
-  // (as much shared memory as does not fit beside the attention's: blocks that were on the first SMs early would all stay there,
-  // 7.9 us where they take 5.1 spread over the chip)
+  // (its blocks wait until the attention's CTAs leave: 608 threads of 96 registers, in either form of operands, leave no room for 256
+  // of 40.  Blocks that fitted beside them, as they did beside 80, would all sit on the first SMs, 7.9 us where they take 5.1)
   return launch(combine_parts_kernel, dim3((unsigned)(split_slots(split) / split.parts), 256 / kCombineRows),
-                kCombineRows * 8, kCombineAwayBytes, s, split, o, (int)seq_len, ctx->sz.dim, next_stamp(ctx));
+                kCombineRows * 8, 0, s, split, o, (int)seq_len, ctx->sz.dim, next_stamp(ctx));
 }
 
 cudaError_t launch_flash_attention_fp8(litevggt_ctx* ctx, long long m, __nv_bfloat16* o, cudaStream_t s, int* launches) {
