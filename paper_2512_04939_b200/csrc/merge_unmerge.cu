@@ -34,8 +34,7 @@ __device__ __forceinline__ void load_row(uint4 (&v)[4], const __nv_bfloat16* row
 
 // kRows: absorbed rows in flight.  Few blocks last as long as their longest row, a chain of loads, and four shorten it; many
 // are bound by HBM and want warps, of which 96 registers leave 16 an SM where two rows' 64 leave 32 (us, two / four: 543
-// merged rows 4.7 / 3.9, 2,520 5.6 / 4.7, 5,205 6.3 / 7.2, 83,280 107 / 145).
-constexpr unsigned kMergeFewBlocks = 148 * 5 / 2;
+// merged rows 4.7 / 3.9, 2,520 5.6 / 4.7, 5,205 6.3 / 7.2, 83,280 107 / 145; the line is two and a half blocks an SM, 2,960 rows).
 template <int kRows>
 __global__ void __launch_bounds__(kRowThreads)
 merge_kernel(const __nv_bfloat16* __restrict__ x, const int* __restrict__ kept_idx, const int* __restrict__ seg_off,
@@ -278,8 +277,9 @@ cudaError_t launch_merge(const litevggt_ctx* ctx, const litevggt_plan* plan, con
   const Sizes& z = ctx->sz;
   const unsigned blocks = (unsigned)((z.n_merged + kRowsPerCta - 1) / kRowsPerCta);
   ++*launches;
-  return launch(blocks <= kMergeFewBlocks ? merge_kernel<4> : merge_kernel<2>, dim3(blocks), kRowThreads, 0, s, x, plan->kept_idx, plan->seg_off, plan->seg_src, xm, z.n_merged,
-                z.n_tokens, z.n_remove, ctx->ws.status, next_stamp(ctx));
+  const bool few = 2 * (long long)blocks <= 5 * ctx->num_sms;
+  return launch(few ? merge_kernel<4> : merge_kernel<2>, dim3(blocks), kRowThreads, 0, s, x, plan->kept_idx, plan->seg_off,
+                plan->seg_src, xm, z.n_merged, z.n_tokens, z.n_remove, ctx->ws.status, next_stamp(ctx));
 }
 
 cudaError_t launch_unmerge(const litevggt_ctx* ctx, const litevggt_plan* plan, const __nv_bfloat16* ym,
