@@ -26,16 +26,17 @@
 //               thread cannot feed both tiles)
 // One CTA of two tiles sits on an SM, so nothing would run under the set-up, the first loads and the write-back of the
 // next: a launch is one such CTA per SM, and each works off jobs (256 rows of one head) until they run out.  The
-// K/V ring goes on from job to job; the next job's queries have come to shared memory by the time the last scores of this one
-// have, take the old ones' place in tensor memory then, and the next scores are under way before this job's rows are
-// written.  Whole layers: 4,386 rows 153 -> 148 us, 15,932 rows 1.15 -> 1.09 ms, 31,751 rows 3.64 -> 3.60; from 83 K rows on, at
-// the power cap, nothing (251,872 rows 241.9 -> 243.4).  What the softmax warps do themselves between two jobs is what is left: with
-// queries and rows going row by row between global memory and registers (4096 and 2048 lines for the load unit, twice
-// that for a part's rows) 4.3 us from a job's last probabilities to the next one's first scores, 3.4 as it is, and the first job's
-// queries in 2.1 us, not 3.4: the core at 5,205 rows 109.5 -> 105.7 us, at 8,244 250.5 -> 242.6, whole layers
-// 180.9 -> 178.9, 346.3 -> 339.8, 10,410 rows 492.7 -> 487.9, 31,751 (query weights x 16) 4.27 -> 4.21 ms.  Jobs come off a counter, late in the job before: with a fixed stride, or taken a whole
-// job ahead, rows in the online form left 3 % of 31,751 rows' time to a few CTAs at the end.  With one tile, two
-// CTAs an SM run under each other anyway, and jobs measured 3 % slower.
+// K/V ring goes on from job to job; the next job's queries have come to shared memory by the time the last scores of this
+// one have, take the old ones' place in tensor memory then, and the next scores are under way before this job's rows are
+// written.  Whole layers: 4,386 rows 153 -> 148 us, 15,932 rows 1.15 -> 1.09 ms, 31,751 rows 3.64 -> 3.60; from 83 K rows
+// on, at the power cap, nothing (251,872 rows 241.9 -> 243.4).  What the softmax warps do themselves between two jobs is
+// what is left: with queries and rows going row by row between global memory and registers (4096 and 2048 lines for the
+// load unit, twice that for a part's rows) 4.3 us from a job's last probabilities to the next one's first scores, 3.4 as
+// it is, and the first job's queries in 2.1 us, not 3.4: the core at 5,205 rows 109.5 -> 105.7 us, at 8,244 250.5 ->
+// 242.6, whole layers 180.9 -> 178.9, 346.3 -> 339.8, 10,410 rows 492.7 -> 487.9, 31,751 (query weights x 16) 4.27 ->
+// 4.21 ms.  Jobs come off a counter, late in the job before: with a fixed stride, or taken a whole job ahead, rows in the
+// online form left 3 % of 31,751 rows' time to a few CTAs at the end.  With one tile, two CTAs an SM run under each other
+// anyway, and jobs measured 3 % slower.
 // Tensor memory (512 columns allocated, 480 used):
 //   [0,256)    S/P: tile t, half h at column t*128 + h*64.  S_th is 128 x 64 fp32.  A softmax
 //              thread reads its 32 columns and writes its 32 probabilities (16 columns of bf16
@@ -644,9 +645,10 @@ flash_attention_kernel(const __grid_constant__ CUtensorMap tmap_qkv, __nv_bfloat
     const uint32_t o_row = tmem_base + lane_base + Shape::kColO + t * kFaOCols, o_addr = o_row + c * 32;
 
     auto row_of = [&](const FaJob& job) { return job.q_block * (128 * kTiles) + t * 128 + row_in_tile; };  // within the sequence
-    // The queries come by TMA: loaded row by row, every load of a warp touches 32 lines, 4096 in all for two tiles, 2 us (a CTA of
-    // one tile, four frames of 16 x 16: layer 32.3 -> 31.7 us; local half of 200 frames of 28 x 37 5.18 -> 5.15 ms).  This thread's half (32 channels) of its row goes to tensor memory, in the place of the queries before, all
-    // of whose Q K^T must have retired.  Returns the Cauchy-Schwarz bound on the whole row's scores (K carries the
+    // The queries come by TMA: loaded row by row, every load of a warp touches 32 lines, 4096 in all for two tiles, 2 us
+    // (a CTA of one tile, four frames of 16 x 16: layer 32.3 -> 31.7 us; local half of 200 frames of 28 x 37 5.18 -> 5.15
+    // ms).  This thread's half (32 channels) of its row goes to tensor memory, in the place of the queries before, all of
+    // whose Q K^T must have retired.  Returns the Cauchy-Schwarz bound on the whole row's scores (K carries the
     // softmax scale, so they are in base-2 units already), or -1 where a wait was given up.
     auto take_q = [&](const FaJob& job, uint32_t parity) -> float {
       const float k_norm2 = kv_max[job.seq * 2 * (dim / 64) + job.head];

@@ -764,11 +764,12 @@ cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStrea
     ++*launches;
     return a;
   };
-  if (a.n_tokens <= kLocalTokens && local_bytes <= kLocalBytes) {
+  if (a.n_tokens <= kLocalTokens) {
+    const auto build = index_build_kernel<true, false>;
     static std::atomic<unsigned long long> smem_set{0};
-    const cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(index_build_kernel<true, false>), kLocalBytes, smem_set);
+    const cudaError_t e = set_max_dynamic_smem_once(reinterpret_cast<const void*>(build), kLocalBytes, smem_set);
     if (e != cudaSuccess) return e;
-    return launch(index_build_kernel<true, false>, dim3(1), a.n_tokens > kWideTokens ? kIdxWideThreads : kIdxThreads, (size_t)local_bytes, s, stamped());
+    return launch(build, dim3(1), a.n_tokens > kWideTokens ? kIdxWideThreads : kIdxThreads, (size_t)local_bytes, s, stamped());
   }
   const bool wide = a.n_tokens > kClusterTokens, many = a.n_tokens > kManyTokens;
   const auto build = wide ? index_build_kernel<false, true> : index_build_kernel<false, false>;
@@ -796,8 +797,8 @@ cudaError_t launch_index_build(litevggt_ctx* ctx, litevggt_plan* plan, cudaStrea
   const unsigned blocks = (unsigned)((a.n_remove + kIdxThreads - 1) / kIdxThreads);
   if (blocks > 0) e = launch(index_assign_kernel, dim3(blocks), kIdxThreads, 0, s, stamped(), rows_per_part);
   // (1024 threads where they make it one scan a block: 1,041,000 tokens 14.2 -> 8.5 us)
-  if (e == cudaSuccess)
-    e = launch(index_lay_kernel, dim3(kIdxParts), rows_per_part > kIdxThreads * kScanItems ? kIdxWideThreads : kIdxThreads, 0, s, stamped(), rows_per_part);
+  const int lay_threads = rows_per_part > kIdxThreads * kScanItems ? kIdxWideThreads : kIdxThreads;
+  if (e == cudaSuccess) e = launch(index_lay_kernel, dim3(kIdxParts), lay_threads, 0, s, stamped(), rows_per_part);
   if (e == cudaSuccess && blocks > 0) e = launch(index_slot_kernel, dim3(blocks), kIdxThreads, 0, s, stamped());
   if (e == cudaSuccess && blocks > 0)
     e = launch(index_order_kernel, dim3(blocks + (a.n_remove > kLongSegment ? kLongBlocks : 0)), kIdxThreads, 0, s, stamped());
