@@ -40,7 +40,7 @@ METRIC = "frames/s through merge+global-attn+unmerge (plan refreshed every 6th l
 # workload C5, summed over the layer's key-chunk launches, from one single-pass ncu capture
 # (profiles/flash_attention_C5_dram.md).  Reported only while the kernel source is the one that was
 # measured.
-ATTENTION_TRAFFIC_C5 = {"bytes_per_layer": 38.99e9 + 17.60e9, "kernel_sha256": "34a060dcffe5f53f4419a55b87b784b3955253c76f83cb71ed6114138542ed6e"}
+ATTENTION_TRAFFIC_C5 = {"bytes_per_layer": 33.55e9 + 17.60e9, "kernel_sha256": "be1d6883766af8c1e36645c220a371ae88871d81ca4f45dbdc7f738ee52f575c"}
 
 
 def _attention_source_hash() -> str:
