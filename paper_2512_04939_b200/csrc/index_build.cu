@@ -10,7 +10,7 @@
 // steps that need the whole of the step before.  So there is no sort, and what used to be boundaries between launches (4.3 us
 // each, of which there were ten) are barriers (0.7 us) of one cluster of blocks, each with a run of the src tokens (and the
 // tokens from its first to the next block's first) and a run of the rows.  A short sequence is the work of one block
-// that holds in its shared memory what one step hands to the next (four frames of 16 x 16: 9.7 us, 6 so); in a long one the
+// that holds in its shared memory what one step hands to the next (four frames of 16 x 16: 9.7 us, 5 so); in a long one the
 // steps behind the numbers of its tokens are launches over the chip, in a very long one all are.  (launch_index_build has the figures.)
 //   select    the R-th largest cosine by its ordered bits, eight of them at a time: every block makes a
 //             histogram of its own keys in shared memory, and after a barrier adds up those of all blocks
@@ -37,7 +37,7 @@ constexpr int kIdxMaxBlocks = 16, kIdxPortableBlocks = 8;  // of a cluster
 constexpr int kIdxParts = 128;     // runs of rows of a long sequence
 // Sequences of more tokens than this are numbered by launches over the chip too, their keys selected 11 + 11 + 10 bits at a
 // time by histograms in global memory: what the cluster's 16 SMs do for all tokens grows beyond five launches (index build, us,
-// cluster / launches: 66,624 tokens 37 / 44, 189,000 58 / 48, 208,200 67 / 50, 1,041,000 238 / 77).
+// cluster / launches: 66,624 tokens 36 / 44, 189,000 58 / 45, 208,200 67 / 45, 1,041,000 238 / 77).
 constexpr long long kManyTokens = 98304;
 constexpr int kLongBins = 2048, kLongThreads = 1024, kLongChunk = kLongThreads * kScanItems;  // <= 4 Mi tokens in <= 1024 chunks
 // A token's rank in a segment of up to this many tokens comes from comparing it with each of them, at

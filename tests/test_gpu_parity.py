@@ -232,10 +232,10 @@ def test_index_arrays_at_the_limits_of_their_forms(lib, frames, grid, ratio, cel
     (2, (9, 9), 0.3, 2, 0.6, "random"),     # few src tokens, all of them merged
     (5, (9, 11), 0.45, 2, 0.1, "tied"),     # every cosine equal to many others
     (7, (19, 25), 0.45, 2, 0.0, "equal"),   # one anchor takes 1512 tokens: a long segment, single block
-    (6, (35, 39), 0.2, 8, 0.1, "tied"),     # 8,220 tokens: the smallest plan of several launches
-    (9, (37, 37), 0.45, 2, 0.1, "random"),  # four blocks of tokens; 28 row blocks, fewer than pairs: all in column runs
-    (30, (37, 37), 0.5, 2, 0.1, "random"),  # 25,288 src tokens: a whole sweep of the 74 pairs, 25 row blocks in column runs
-    (8, (37, 37), 1.0, 16, 0.0, "equal")])  # one segment of 9,583, every src token merged
+    (6, (35, 39), 0.2, 8, 0.1, "tied"),     # 8,220 tokens: one cluster
+    (9, (37, 37), 0.45, 2, 0.1, "random"),  # one cluster; 28 row blocks, fewer than pairs: all in column runs
+    (30, (37, 37), 0.5, 2, 0.1, "random"),  # cluster and launches; 25,288 src tokens: a whole sweep of the 74 pairs, 25 row blocks in column runs
+    (8, (37, 37), 1.0, 16, 0.0, "equal")])  # one cluster, one segment of 9,583, every src token merged
 def test_partition_and_index_build_on_degenerate_inputs(lib, frames, grid, ratio, cell, keep, kind):
     """Ties everywhere, segments longer than a block ranks by comparison, everything or nothing merged."""
     ctx = lib.LiteVGGT(frames, grid[0], grid[1], ratio, cell_h=cell, cell_w=cell, ga_keep_frac=keep)
